@@ -308,8 +308,10 @@ msf_status msf_kv_resample(msf_plan_t plan, const void* k_win, const void* v_win
  * q, k_win, v_win, out [B, N, H, D]; out may not alias q/k/v. Reads the
  * pyramid the last msf_kv_resample on the same stream produced. bf16 plans
  * run the tcgen05 tensor-core kernel (bf16 operands, fp32 softmax and
- * accumulation); fp32 plans run an fp32 CUDA-core kernel. Errors:
- * INVALID_ARG, STATE, CUDA. */
+ * accumulation); fp32 plans run the tensor cores on three bf16 planes per
+ * value (24 bits), or, for a call with a value that is not finite or not below
+ * 2^127 in magnitude, an fp32 CUDA-core kernel. Errors: INVALID_ARG, STATE,
+ * CUDA. */
 msf_status msf_mssa_forward(msf_plan_t plan, const void* q, const void* k_win, const void* v_win,
                             void* out, void* stream);
 

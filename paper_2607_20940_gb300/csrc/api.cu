@@ -8,6 +8,7 @@
 #include <vector>
 
 #include "attn_bwd_tc.h"
+#include "attn_f32_tc.h"
 #include "attn_tc.h"
 #include "gemm_tc.h"
 #include "msp_tc.h"
@@ -391,7 +392,7 @@ extern "C" msf_status msf_mssa_forward_lse(msf_plan_t plan, const void* q, const
     build_attn_args(p, q, k_win, v_win, out, a);
     a.lse = lse;
     if (p.elem == 2) return msf::launch_attn_tc(plan, a, (cudaStream_t)stream);
-    return cuda_status(msf::launch_attn_simt(a, false, (cudaStream_t)stream));
+    return msf::launch_attn_f32_tc(plan, a, (cudaStream_t)stream);
 }
 
 extern "C" msf_status msf_mssa_forward(msf_plan_t plan, const void* q, const void* k_win,
@@ -403,7 +404,7 @@ extern "C" msf_status msf_mssa_forward(msf_plan_t plan, const void* q, const voi
     msf::AttnArgs a;
     build_attn_args(p, q, k_win, v_win, out, a);
     if (p.elem == 2) return msf::launch_attn_tc(plan, a, (cudaStream_t)stream);
-    return cuda_status(msf::launch_attn_simt(a, false, (cudaStream_t)stream));
+    return msf::launch_attn_f32_tc(plan, a, (cudaStream_t)stream);
 }
 
 extern "C" msf_status msf_mssa_forward_resample(msf_plan_t plan, const void* q, const void* k_win,
@@ -428,7 +429,7 @@ extern "C" msf_status msf_mssa_forward_resample(msf_plan_t plan, const void* q, 
         st = cuda_status(msf::launch_pool(jb, p.B, false, s));
         if (st != MSF_OK) return st;
     }
-    return cuda_status(msf::launch_attn_simt(a, false, s));
+    return msf::launch_attn_f32_tc(plan, a, s);
 }
 
 // Gradient rows of group gi: the context rows that come from the window,

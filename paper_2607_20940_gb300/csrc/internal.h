@@ -36,6 +36,7 @@ struct msf_plan {
     // tensor-core attention scheduling state in the workspace
     int attn_items;     // 256-row query blocks over all groups, streams and heads
     int attn_max_ctas;  // persistent CTAs the partial-result slots are sized for
+    long long f32_tiles;  // fp32 plans: 128 x 128 query-context tiles at full history
     size_t ws_bytes;
     float scale;      // softmax scale
 
@@ -101,6 +102,36 @@ inline size_t tier_codes_bytes(const Plan& p) {
     if (p.d.latent_channels <= 0 || p.d.patch <= 0 || p.elem != 2 || p.d.embed_dim <= 0) return 0;
     return round256((size_t)p.B * p.N * kTierCodeCols * 2);
 }
+// fp32 plans: the tensor-core attention's operands as three bf16 planes,
+// [B, 3, rows, H, D] for q and for k, v of the sink, the ring, each group's
+// pyramid part and the window; the output units of split query tiles, each
+// [128 rows][D] fp32 and the rows' running max and sum; and one flag word per
+// block of the kernel that writes the planes.
+enum : int { kF32Q = 0, kF32Sink = 1, kF32Ring = 2, kF32Pyr = 3, kF32Win = 4 };
+constexpr int kF32MaxSms = 160;
+constexpr int kF32MaxRounds = 6;       // rounds of units per SM when tiles are split
+constexpr int kF32SplitBlocks = 1024;  // grid limit of the split
+inline int f32_part_rows(const Plan& p, int part) {
+    return part == kF32Sink ? p.d.sink_tokens : part == kF32Ring ? p.ring_slots * p.G : part == kF32Pyr ? p.pyr_tokens : p.N;
+}
+inline size_t f32_part_bytes(const Plan& p, int part) {
+    return round256((size_t)3 * p.B * f32_part_rows(p, part) * p.H * p.D * 2);
+}
+inline size_t f32_plane_bytes(const Plan& p) {
+    if (p.elem != 4) return 0;
+    size_t n = f32_part_bytes(p, kF32Q);
+    for (int i = kF32Sink; i <= kF32Win; ++i) n += 2 * f32_part_bytes(p, i);
+    return n;
+}
+// Units are at least half as long as the rounds ask for, so kF32MaxRounds
+// rounds make at most twice as many per SM, and never more than K/V tiles.
+inline int f32_max_slots(const Plan& p) {
+    const long long n = 2ll * kF32MaxRounds * kF32MaxSms;
+    return (int)(p.f32_tiles < n ? p.f32_tiles : n);
+}
+inline size_t f32_partial_bytes(const Plan& p) {
+    return p.elem == 4 ? round256((size_t)f32_max_slots(p) * 128 * (p.D + 2) * 4) + round256(kF32SplitBlocks * 4) : 0;
+}
 // Backward workspace (caller-provided per msf_mssa_backward call):
 // [delta fp32 [B, H, N] | dk_ctx fp32 [B, R, H, D] | dv_ctx fp32 [B, R, H, D]],
 // R = rows of every group's context that come from the window (the rows
@@ -121,7 +152,8 @@ inline size_t bwd_ctx_bytes(const Plan& p) {
 inline size_t bwd_workspace_bytes(const Plan& p) { return bwd_delta_bytes(p) + 2 * bwd_ctx_bytes(p); }
 inline size_t workspace_bytes(const Plan& p) {
     return kStatusBytes + 2 * pyramid_bytes(p) + msp_scratch_bytes(p) + attn_counter_bytes(p) +
-           attn_partial_bytes(p) + msp_split_bytes(p) + tier_codes_bytes(p);
+           attn_partial_bytes(p) + msp_split_bytes(p) + tier_codes_bytes(p) + f32_plane_bytes(p) +
+           f32_partial_bytes(p);
 }
 inline unsigned int* status_word(const Plan& p) { return (unsigned int*)p.ws; }
 inline char* pyr_k(const Plan& p) { return (char*)p.ws + kStatusBytes; }
@@ -140,6 +172,19 @@ inline float* msp_split(const Plan& p) {
     return (float*)((char*)attn_partials(p) + attn_partial_bytes(p));
 }
 inline char* tier_codes(const Plan& p) { return (char*)msp_split(p) + msp_split_bytes(p); }
+inline char* f32_planes(const Plan& p, int part, int which) {  // which: 0 = q or k, 1 = v
+    char* base = tier_codes(p) + tier_codes_bytes(p);
+    if (part == kF32Q) return base;
+    base += f32_part_bytes(p, kF32Q);
+    for (int i = kF32Sink; i < part; ++i) base += 2 * f32_part_bytes(p, i);
+    return base + which * f32_part_bytes(p, part);
+}
+inline float* f32_partials(const Plan& p) {
+    return (float*)(tier_codes(p) + tier_codes_bytes(p) + f32_plane_bytes(p));
+}
+inline unsigned int* f32_flags(const Plan& p) {
+    return (unsigned int*)((char*)f32_partials(p) + round256((size_t)f32_max_slots(p) * 128 * (p.D + 2) * 4));
+}
 
 // Number of context tokens of group gi with the current history count.
 inline int group_nkv(const Plan& p, int gi) {

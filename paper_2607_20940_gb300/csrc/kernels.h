@@ -146,6 +146,9 @@ struct AttnArgs {
     unsigned int* status;
     float* lse;           // optional [B, H, N] row log-sum-exp (natural log); NULL = none
     int N;                // query rows per stream
+    // CUDA-core kernel only: run only if one of these words is set (NULL = run).
+    const unsigned int* run_if;
+    int n_run_if;
 };
 cudaError_t launch_attn_simt(const AttnArgs& a, bool bf16, cudaStream_t st);
 

@@ -141,7 +141,7 @@ extern "C" msf_status msf_plan_create(const msf_plan_desc* desc, msf_plan_t* out
     // Attention work: 256-row query blocks and 128-row context tiles, counted
     // at full history (the most tiles the schedule can ever hold).
     {
-        long long items = 0, tiles = 0;
+        long long items = 0, tiles = 0, f32_tiles = 0;
         for (int gi = 0; gi < ng; ++gi) {
             const msf::Group& g = p->groups[gi];
             long long it = (long long)p->B * p->H * ((g.q_end - g.q_begin + 255) / 256);
@@ -152,12 +152,14 @@ extern "C" msf_status msf_plan_create(const msf_plan_desc* desc, msf_plan_t* out
                 nt += ((long long)(d.history_capacity + g.n_finer) * g.pooled + 127) / 128;
             items += it;
             tiles += it * nt;
+            f32_tiles += (long long)p->B * p->H * ((g.q_end - g.q_begin + 127) / 128) * nt;
         }
         if (items > (1 << 30)) {
             delete p;
             return MSF_ERR_UNSUPPORTED;
         }
         p->attn_items = (int)items;
+        p->f32_tiles = f32_tiles;
         p->attn_max_ctas = (int)(tiles < msf::kAttnMaxCtas ? tiles : msf::kAttnMaxCtas);
     }
     p->ws_bytes = msf::workspace_bytes(*p);

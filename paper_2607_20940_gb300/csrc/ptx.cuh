@@ -397,5 +397,14 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
     return r;
 }
 
+// Two fp32 values as three bf16 pairs each: h = bf16(x), m = bf16(x - h),
+// l = bf16(x - h - m), all rounded to nearest; both differences are exact.
+__device__ __forceinline__ void split_bf16(float x0, float x1, uint32_t& h, uint32_t& m, uint32_t& l) {
+    h = pack_bf16(x0, x1);
+    const float r0 = x0 - __uint_as_float(h << 16), r1 = x1 - __uint_as_float(h & 0xffff0000u);
+    m = pack_bf16(r0, r1);
+    l = pack_bf16(r0 - __uint_as_float(m << 16), r1 - __uint_as_float(m & 0xffff0000u));
+}
+
 }  // namespace ptx
 }  // namespace msf
