@@ -351,7 +351,8 @@ msf_status msf_mssa_forward_lse(msf_plan_t plan, const void* q, const void* k_wi
  * bytes, 16-byte aligned, overwritten. Output buffers may not alias inputs.
  * bf16 plans run tcgen05 tensor-core kernels (one for dq over each query
  * tile's whole context, one per query group for the window rows' dk/dv);
- * fp32 plans run CUDA-core kernels.
+ * fp32 plans run them on three bf16 planes per value (as the forward does),
+ * or CUDA-core kernels where the planes cannot hold a value.
  * Errors: INVALID_ARG, STATE (not bound), WORKSPACE, CUDA. */
 msf_status msf_mssa_backward(msf_plan_t plan, const void* q, const void* k_win, const void* v_win,
                              const void* out, const void* dout, const float* lse, void* dq,

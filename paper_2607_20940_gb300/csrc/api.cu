@@ -20,7 +20,7 @@ using msf::Plan;
 
 namespace msf {
 
-cudaError_t set_smem_attr(const void* fn, int bytes, int carveout) {
+cudaError_t set_smem_attr(const void* fn, int bytes, int carveout, int regs) {
     static std::mutex mu;
     static std::vector<std::pair<const void*, int>> done;  // (kernel, device)
     int dev = 0;
@@ -29,6 +29,12 @@ cudaError_t set_smem_attr(const void* fn, int bytes, int carveout) {
     std::lock_guard<std::mutex> lock(mu);
     for (const auto& d : done)
         if (d.first == fn && d.second == dev) return cudaSuccess;
+    if (regs > 0) {
+        cudaFuncAttributes fa;
+        e = cudaFuncGetAttributes(&fa, fn);
+        if (e == cudaSuccess && fa.numRegs != regs) e = cudaErrorInvalidKernelImage;
+        if (e != cudaSuccess) return e;
+    }
     e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
     if (e == cudaSuccess && carveout >= 0)
         e = cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, carveout);
@@ -576,12 +582,15 @@ static msf_status mssa_backward(msf_plan_t plan, const void* q, const void* k_wi
         msf_status st = msf::launch_bwd_tc(plan, in, s);
         if (st != MSF_OK) return st;
     } else {
-        e = msf::launch_bwd_dq_simt(c, a, dq, bf16, s);
-        if (e != cudaSuccess) return cuda_status(e);
-        for (int gi = 0; gi < p.n_groups; ++gi) {
-            e = msf::launch_bwd_dkdv_simt(c, bg[gi], bf16, s);
-            if (e != cudaSuccess) return cuda_status(e);
+        msf::BwdRunIf run_if;  // the CUDA-core kernels: always, or where the planes cannot hold an operand
+        if (tc) {
+            char* planes = (char*)bwd_ws + msf::bwd_delta_bytes(p) + 2 * msf::bwd_ctx_bytes(p);
+            msf_status st = msf::launch_bwd_f32_tc(plan, c, a, bg, (float*)dq, planes, &run_if, s);
+            if (st != MSF_OK) return st;
         }
+        e = msf::launch_bwd_dq_simt(c, a, dq, bf16, run_if, s);
+        if (e == cudaSuccess) e = msf::launch_bwd_dkdv_simt(c, bg, p.n_groups, bf16, run_if, s);
+        if (e != cudaSuccess) return cuda_status(e);
     }
     return cuda_status(msf::launch_bwd_gather(c, ga, dk_win, dv_win, bf16, s));
 }

@@ -1,4 +1,6 @@
-// MSSA backward on CUDA cores (fp32 arithmetic, bf16 or fp32 storage).
+// MSSA backward on CUDA cores (fp32 arithmetic, bf16 or fp32 storage): the
+// cross-check of the tensor-core kernels, the fp32 path of operands that three
+// bf16 planes cannot hold, and the delta and gather kernels of every path.
 //
 // The gradient of Eq. 4 for a loss with dL/dO = dO, per query group g with
 // context K_g, V_g (sink, history, window; pooled as in the forward):
@@ -87,6 +89,14 @@ __device__ __forceinline__ void stE(__nv_bfloat16* p, const float* x) {
 
 constexpr float kLog2e = 1.4426950408889634f;
 
+// Whether a conditional kernel has to run (every thread of the block).
+__device__ __forceinline__ bool wanted(const BwdRunIf& c) {
+    if (!c.flags) return true;
+    bool f = false;
+    for (int i = threadIdx.x; i < c.n; i += blockDim.x) f |= __ldg(c.flags + i) != 0;
+    return __syncthreads_or(f);
+}
+
 // delta[b, h, t] = sum_d dout * out: a row of D elements is shared by D/8
 // consecutive threads, each loading 8 elements of both tensors (one 16-byte
 // vector each for bf16). One row per thread group: giving a warp several
@@ -121,9 +131,11 @@ __global__ void __launch_bounds__(256) bwd_delta_kernel(const BwdCommon c) {
 // dq: a block owns 32 queries of one (stream, head, group); four threads share
 // a query and hold every fourth element of q, dO and dq.
 template <typename T, int D>
-__global__ void __launch_bounds__(128) bwd_dq_kernel(const BwdCommon c, const AttnArgs a, T* dq) {
+__global__ void __launch_bounds__(128) bwd_dq_kernel(const BwdCommon c, const AttnArgs a, T* dq,
+                                                     const BwdRunIf run_if) {
     ptx::grid_dep_wait();
     ptx::grid_dep_launch();
+    if (!wanted(run_if)) return;
     constexpr int DP = D / 4;
     constexpr int KT = 32;
     __shared__ float Ks[KT][D];
@@ -193,19 +205,33 @@ __global__ void __launch_bounds__(128) bwd_dq_kernel(const BwdCommon c, const At
     for (int i = 0; i < DP; ++i) o[4 * i + cc] = st1<T>(acc[i] * c.scale);
 }
 
-// dk, dv of one group's gradient rows: a block owns 32 rows of one segment of
-// one (stream, head); four threads share a row. The group's queries stream
+// dk, dv of every group's gradient rows: a block owns 32 rows of one segment
+// of one (stream, head); four threads share a row. The group's queries stream
 // through shared memory 32 at a time. Rows go to the context-gradient buffer.
+struct BwdGroups {
+    int n;
+    BwdGroup g[MSF_MAX_GROUPS];
+};
+__host__ __device__ inline int grad_tiles(const BwdGroup& g) {
+    int n = 0;
+    if (g.q_end > g.q_begin)
+        for (int s = 0; s < g.n_gseg; ++s) n += (g.gseg[s].len + 31) / 32;
+    return n;
+}
 template <typename T, int D>
-__global__ void __launch_bounds__(128) bwd_dkdv_kernel(const BwdCommon c, const BwdGroup G) {
+__global__ void __launch_bounds__(128)
+    bwd_dkdv_kernel(const BwdCommon c, const __grid_constant__ BwdGroups groups, const BwdRunIf run_if) {
     ptx::grid_dep_wait();
     ptx::grid_dep_launch();
+    if (!wanted(run_if)) return;
     constexpr int DP = D / 4;
     constexpr int QT = 32;
     __shared__ float Qs[QT][D];
     __shared__ float Gs[QT][D];
     __shared__ float Ls[QT], Ds[QT];
-    int tile = blockIdx.x, si = 0;
+    int tile = blockIdx.x, si = 0, gi = 0;
+    for (int nt; gi + 1 < groups.n && tile >= (nt = grad_tiles(groups.g[gi])); ++gi) tile -= nt;
+    const BwdGroup& G = groups.g[gi];
     while (si < G.n_gseg) {
         int nt = (G.gseg[si].len + 31) / 32;
         if (tile < nt) break;
@@ -363,7 +389,7 @@ cudaError_t launch_bwd_delta(const BwdCommon& c, bool bf16, cudaStream_t st) {
                 : launch_pdl(bwd_delta_kernel<float, 64>, grid, dim3(256), 0, st, c);
 }
 
-cudaError_t launch_bwd_dq_simt(const BwdCommon& c, const AttnArgs& a, void* dq, bool bf16,
+cudaError_t launch_bwd_dq_simt(const BwdCommon& c, const AttnArgs& a, void* dq, bool bf16, BwdRunIf run_if,
                                cudaStream_t st) {
     int tiles = 0;
     for (int gi = 0; gi < a.n_groups; ++gi) tiles += (a.g[gi].q_end - a.g[gi].q_begin + 31) / 32;
@@ -371,24 +397,29 @@ cudaError_t launch_bwd_dq_simt(const BwdCommon& c, const AttnArgs& a, void* dq, 
     dim3 grid((unsigned)tiles, (unsigned)c.H, (unsigned)c.B);
     if (c.D == 128)
         return bf16 ? launch_pdl(bwd_dq_kernel<__nv_bfloat16, 128>, grid, dim3(128), 0, st, c, a,
-                                 (__nv_bfloat16*)dq)
-                    : launch_pdl(bwd_dq_kernel<float, 128>, grid, dim3(128), 0, st, c, a, (float*)dq);
+                                 (__nv_bfloat16*)dq, run_if)
+                    : launch_pdl(bwd_dq_kernel<float, 128>, grid, dim3(128), 0, st, c, a, (float*)dq, run_if);
     return bf16 ? launch_pdl(bwd_dq_kernel<__nv_bfloat16, 64>, grid, dim3(128), 0, st, c, a,
-                             (__nv_bfloat16*)dq)
-                : launch_pdl(bwd_dq_kernel<float, 64>, grid, dim3(128), 0, st, c, a, (float*)dq);
+                             (__nv_bfloat16*)dq, run_if)
+                : launch_pdl(bwd_dq_kernel<float, 64>, grid, dim3(128), 0, st, c, a, (float*)dq, run_if);
 }
 
-cudaError_t launch_bwd_dkdv_simt(const BwdCommon& c, const BwdGroup& g, bool bf16,
+cudaError_t launch_bwd_dkdv_simt(const BwdCommon& c, const BwdGroup* g, int n_groups, bool bf16, BwdRunIf run_if,
                                  cudaStream_t st) {
+    BwdGroups gs;
+    gs.n = n_groups;
     int tiles = 0;
-    for (int s = 0; s < g.n_gseg; ++s) tiles += (g.gseg[s].len + 31) / 32;
-    if (tiles == 0 || g.q_end <= g.q_begin) return cudaSuccess;
+    for (int i = 0; i < n_groups; ++i) {
+        gs.g[i] = g[i];
+        tiles += grad_tiles(g[i]);
+    }
+    if (tiles == 0) return cudaSuccess;
     dim3 grid((unsigned)tiles, (unsigned)c.H, (unsigned)c.B);
     if (c.D == 128)
-        return bf16 ? launch_pdl(bwd_dkdv_kernel<__nv_bfloat16, 128>, grid, dim3(128), 0, st, c, g)
-                    : launch_pdl(bwd_dkdv_kernel<float, 128>, grid, dim3(128), 0, st, c, g);
-    return bf16 ? launch_pdl(bwd_dkdv_kernel<__nv_bfloat16, 64>, grid, dim3(128), 0, st, c, g)
-                : launch_pdl(bwd_dkdv_kernel<float, 64>, grid, dim3(128), 0, st, c, g);
+        return bf16 ? launch_pdl(bwd_dkdv_kernel<__nv_bfloat16, 128>, grid, dim3(128), 0, st, c, gs, run_if)
+                    : launch_pdl(bwd_dkdv_kernel<float, 128>, grid, dim3(128), 0, st, c, gs, run_if);
+    return bf16 ? launch_pdl(bwd_dkdv_kernel<__nv_bfloat16, 64>, grid, dim3(128), 0, st, c, gs, run_if)
+                : launch_pdl(bwd_dkdv_kernel<float, 64>, grid, dim3(128), 0, st, c, gs, run_if);
 }
 
 cudaError_t launch_bwd_gather(const BwdCommon& c, const GatherArgs& g, void* dk, void* dv,

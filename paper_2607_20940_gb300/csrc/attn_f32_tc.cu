@@ -50,24 +50,13 @@ constexpr int kThreads = 384;  // 12 warps
 constexpr int kRing = 4;       // plane tiles in flight
 constexpr int kSBuf = 192;     // TMEM columns of one S / P buffer
 constexpr int kOCol = 2 * kSBuf;
+// 168 registers per thread at launch; the control warpgroup drops to 104 and
+// the two softmax warpgroups rise to 192: 4 x 104 + 8 x 192 <= 12 x 168.
+constexpr int kLaunchRegs = 168, kCtrlRegs = 104, kSoftmaxRegs = 192;
+static_assert(4 * kCtrlRegs + 8 * kSoftmaxRegs <= 12 * kLaunchRegs, "register split");
 constexpr long long kWaitLimit = 2000000000LL;  // ~1 s of SM clock
 
 // ------------------------------------------------------------ plane split
-struct SplitJob {
-    const float* src;     // stream 0
-    __nv_bfloat16* dst;   // stream 0, plane 0
-    long long src_bstride, dst_bstride, dst_plane;  // elements
-    int vecs;             // 8-element vectors per stream
-    long long base;       // first vector of the job (all streams) in the launch
-};
-constexpr int kMaxSplitJobs = 1 + 2 * (3 + MSF_MAX_GROUPS);
-struct SplitParams {
-    SplitJob j[kMaxSplitJobs];
-    int n;
-    long long total;
-    unsigned int* flags;  // one word per block: 1 = a value the planes cannot hold
-};
-
 __global__ void __launch_bounds__(256) split_planes_kernel(const __grid_constant__ SplitParams p) {
     ptx::grid_dep_wait();
     ptx::grid_dep_launch();
@@ -123,12 +112,6 @@ struct FParams {
     unsigned int* status;
     long long wait_limit;
 };
-struct FMaps {
-    CUtensorMap q;
-    CUtensorMap k[kNumMaps];
-    CUtensorMap v[kNumMaps];
-};
-
 template <int D>
 struct FCfg {
     static constexpr int kTile = kBM * D * 2;  // one plane of one 128-row tile
@@ -152,13 +135,13 @@ __device__ __forceinline__ bool any_flag(const unsigned int* flags, int n) {
 
 template <int D>
 __global__ void __launch_bounds__(kThreads, 1)
-    mssa_f32_kernel(const __grid_constant__ FMaps maps, const __grid_constant__ FParams p) {
+    mssa_f32_kernel(const __grid_constant__ F32Maps maps, const __grid_constant__ FParams p) {
     using C = FCfg<D>;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char* smem = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     unsigned char* sQ = smem;                // [3] planes h, m, l
     unsigned char* sR = smem + 3 * C::kTile;  // [kRing]
-    __shared__ uint64_t q_full, full[kRing], empty[kRing], s_full, p_full, o_full, drain_bar;
+    __shared__ uint64_t q_full, full[kRing], empty[kRing], s_full, p_full, o_full, meet_bar, drain_bar;
     __shared__ float sx[2][kBM];  // row maxima, at the end row sums, of the two column halves
     __shared__ uint32_t tmem_base_sh;
     __shared__ int abort_flag;
@@ -187,6 +170,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         ptx::mbar_init(&s_full, 1);
         ptx::mbar_init(&p_full, 8);
         ptx::mbar_init(&o_full, 1);
+        ptx::mbar_init(&meet_bar, 8);
         ptx::mbar_init(&drain_bar, 1);
         ptx::fence_mbar_init();
     }
@@ -214,7 +198,9 @@ __global__ void __launch_bounds__(kThreads, 1)
     };
 
     if (skip) {
-    } else if (warp == 0) {
+    } else if (warp < 4) {
+        ptx::setmaxnreg_dec<kCtrlRegs>();
+        if (warp == 0) {
         // ============================ TMA producer ============================
         if (lane == 0) {
             bool ok = true;
@@ -258,7 +244,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 atomicOr(p.status, kDevTimeout);
             }
         }
-    } else if (warp == 1) {
+        } else if (warp == 1) {
         // ============================= MMA issuer =============================
         constexpr uint32_t idS = ptx::idesc_bf16(kBM, kBM, false, false);
         constexpr uint32_t idO = ptx::idesc_bf16(kBM, D, false, true);
@@ -332,7 +318,9 @@ __global__ void __launch_bounds__(kThreads, 1)
             ptx::mbar_wait_bounded(&drain_bar, 0, &never, kWaitLimit);
             if (lane == 0) atomicOr(p.status, kDevTimeout);
         }
-    } else if (warp >= 4) {
+        }
+    } else {
+        ptx::setmaxnreg_inc<kSoftmaxRegs>();
         // ========== softmax: one thread per query row and column half ==========
         const int half = (warp - 4) / 4, wq = warp % 4;
         const int r = wq * 32 + lane;
@@ -344,6 +332,15 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
         for (int e = 0; e < DH; ++e) acc[e] = 0.f;
         float m = -INFINITY, l = 0.f;
+        // The eight softmax warps meet (bounded, unlike a hardware barrier).
+        uint32_t meets = 0;
+        auto meet = [&]() {
+            __syncwarp();
+            if (lane == 0) ptx::mbar_arrive(&meet_bar);
+            const bool r = ptx::mbar_wait_bounded(&meet_bar, meets & 1u, abort_p, p.wait_limit);
+            ++meets;
+            return (bool)__all_sync(0xffffffffu, r);
+        };
         bool ok = true;
         for (int j = 0; j < n && ok; ++j) {
             int map, row, valid;
@@ -373,7 +370,8 @@ __global__ void __launch_bounds__(kThreads, 1)
             // The halves share the row's maximum; both have read their scores
             // when they meet, so P may overwrite them.
             sx[half][r] = own;
-            ptx::named_bar_sync(1, 256);
+            ok = meet();
+            if (!ok) break;
             const float m_new = fmaxf(m, fmaxf(own, sx[half ^ 1][r]) * sl2);
             const float corr = ex2(m - m_new);
             m = m_new;
@@ -413,7 +411,9 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
         if (ok) {
             sx[half][r] = l;
-            ptx::named_bar_sync(1, 256);
+            ok = meet();
+        }
+        if (ok) {
             l += sx[half ^ 1][r];
             const int q = q_row0 + r;
             float4* dst = nullptr;
@@ -509,11 +509,9 @@ __global__ void __launch_bounds__(256) merge_f32_kernel(const __grid_constant__ 
 
 // ---------------------------------------------------------------- host side
 
-// Units per query tile. T = K/V tiles per SM; a unit costs about two tiles
-// besides its own (Q's planes, the pipeline's start, the read-out and merge),
-// and the last of k rounds of units leaves the SMs half a unit idle on
-// average, T / 2k tiles: k = sqrt(T / 4) rounds. With one round every unit
-// has to start at once, so units grow until they fit.
+// Units per query tile (f32_unit_tiles), within the partial slots; with one
+// round of units per SM every unit has to start at once, so units grow until
+// they fit.
 void choose_splits(FParams& p, int sms, int max_slots) {
     long long total = 0;
     int longest = 0;
@@ -522,10 +520,8 @@ void choose_splits(FParams& p, int sms, int max_slots) {
         longest = p.g[i].n_tiles > longest ? p.g[i].n_tiles : longest;
     }
     const double T = (double)total / sms;
-    int k = (int)(sqrt(T / 4.0) + 0.5);
-    k = k < 1 ? 1 : k > kF32MaxRounds ? kF32MaxRounds : k;
-    int len = (int)ceil(T / k);
-    if (len < 2) len = 2;
+    int len = f32_unit_tiles(T);
+    const bool one_round = len >= T;
     for (;; ++len) {
         long long units = 0, slots = 0;
         for (int i = 0; i < p.n_groups; ++i) {
@@ -535,11 +531,68 @@ void choose_splits(FParams& p, int sms, int max_slots) {
             units += u;
             slots += g.n_split > 1 ? u : 0;
         }
-        if (len >= longest || (slots <= max_slots && (k > 1 || units <= sms))) return;
+        if (len >= longest || (slots <= max_slots && (!one_round || units <= sms))) return;
     }
 }
 
 }  // namespace
+
+// T tiles per SM in all: a unit costs about two tiles besides its own (the
+// resident planes, the pipeline's start, the read-out and merge), and the last
+// of k rounds of units leaves the SMs half a unit idle on average, T / 2k
+// tiles: k = sqrt(T / 4) rounds cost least.
+int f32_unit_tiles(double T) {
+    int k = (int)(sqrt(T / 4.0) + 0.5);
+    k = k < 1 ? 1 : k > kF32MaxRounds ? kF32MaxRounds : k;
+    const int len = (int)ceil(T / k);
+    return len < 2 ? 2 : len;
+}
+
+bool add_planes(const Plan& P, SplitParams& sp, const void* src, long long src_bstride_bytes, char* dst, int alloc,
+                int rows, CUtensorMap* m) {
+    const long long rowe = (long long)P.H * P.D;
+    SplitJob& j = sp.j[sp.n++];
+    j.src = (const float*)src;
+    j.dst = (__nv_bfloat16*)dst;
+    j.src_bstride = src_bstride_bytes / 4;
+    j.dst_plane = alloc * rowe;
+    j.dst_bstride = 3 * j.dst_plane;
+    j.vecs = (int)(rows * rowe / 8);
+    j.base = sp.total;
+    sp.total += (long long)j.vecs * P.B;
+    return encode_rows(m, dst, P.D, P.H, rows, 3 * P.B, j.dst_plane * 2);
+}
+
+bool add_context_planes(const Plan& P, const AttnArgs& a, SplitParams& sp, F32Maps& maps) {
+    const size_t rowe = (size_t)P.H * P.D;
+    if (!add_planes(P, sp, a.q, a.q_bstride, f32_planes(P, kF32Q, 0), P.N, P.N, &maps.q)) return false;
+    bool done[kNumMaps] = {false};
+    for (int gi = 0; gi < a.n_groups; ++gi)
+        for (int s = 0; s < a.g[gi].n_seg; ++s) {
+            const Segment& sg = a.g[gi].seg[s];
+            const bool pyr = sg.map_id == kMapPyr;
+            const int map = pyr ? kMapPyr0 + gi : sg.map_id;
+            if (done[map]) continue;
+            done[map] = true;
+            // rows that the segment's tensor holds: a group's part of the
+            // pyramid, the live slots of the ring, else all of it
+            const int part = pyr ? kF32Pyr : map == kMapSink ? kF32Sink : map == kMapHist ? kF32Ring : kF32Win;
+            const int rows = pyr || map == kMapHist ? sg.len : sg.rows_total;
+            const size_t off = pyr ? (size_t)3 * P.B * P.groups[gi].pyr_offset * rowe * 2 : 0;
+            const int alloc = pyr ? P.groups[gi].pyr_cap : f32_part_rows(P, part);
+            const size_t so = pyr ? (size_t)sg.row0 * rowe * 4 : 0;
+            if (!add_planes(P, sp, sg.k + so, sg.bstride, f32_planes(P, part, 0) + off, alloc, rows, &maps.k[map]) ||
+                !add_planes(P, sp, sg.v + so, sg.bstride, f32_planes(P, part, 1) + off, alloc, rows, &maps.v[map]))
+                return false;
+        }
+    return true;
+}
+
+cudaError_t launch_split_planes(const SplitParams& sp, int* n_flags, cudaStream_t st) {
+    const long long want = (sp.total + 255) / 256;
+    *n_flags = want < kF32SplitBlocks ? (int)want : kF32SplitBlocks;
+    return launch_pdl(split_planes_kernel, dim3((unsigned)*n_flags), dim3(256), 0, st, sp);
+}
 
 msf_status launch_attn_f32_tc(msf_plan_t plan, const AttnArgs& a, cudaStream_t st) {
     const Plan& P = *plan;
@@ -552,40 +605,23 @@ msf_status launch_attn_f32_tc(msf_plan_t plan, const AttnArgs& a, cudaStream_t s
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return fail(e);
     if (sms > kF32MaxSms) sms = kF32MaxSms;
-    const long long rowe = (long long)P.H * P.D;
-
     SplitParams sp;
     memset(&sp, 0, sizeof(sp));
-    FMaps maps;
+    F32Maps maps;
     memset(&maps, 0, sizeof(maps));
     FParams fp;
     memset(&fp, 0, sizeof(fp));
     sp.flags = f32_flags(P);
-    // A [B, rows, H, D] fp32 tensor's first `rows` rows per stream as planes
-    // [B, 3, alloc, H, D] at `dst`, and their tensor map.
-    auto add = [&](const void* src, long long src_bstride_bytes, char* dst, int alloc, int rows, CUtensorMap* m) {
-        SplitJob& j = sp.j[sp.n++];
-        j.src = (const float*)src;
-        j.dst = (__nv_bfloat16*)dst;
-        j.src_bstride = src_bstride_bytes / 4;
-        j.dst_plane = alloc * rowe;
-        j.dst_bstride = 3 * j.dst_plane;
-        j.vecs = (int)(rows * rowe / 8);
-        j.base = sp.total;
-        sp.total += (long long)j.vecs * P.B;
-        return encode_rows(m, dst, P.D, P.H, rows, 3 * P.B, j.dst_plane * 2);
-    };
-    bool ok = add(a.q, a.q_bstride, f32_planes(P, kF32Q, 0), P.N, P.N, &maps.q);
+    if (!add_context_planes(P, a, sp, maps)) return fail(cudaErrorInvalidValue);
     fp.n_groups = a.n_groups;
-    bool done[kNumMaps] = {false};
-    for (int gi = 0; gi < a.n_groups && ok; ++gi) {
+    for (int gi = 0; gi < a.n_groups; ++gi) {
         const AttnGroup& ag = a.g[gi];
         FGroup& g = fp.g[gi];
         g.q_begin = ag.q_begin;
         g.q_end = ag.q_end;
         g.n_qt = (ag.q_end - ag.q_begin + kBM - 1) / kBM;
         g.n_seg = ag.n_seg;
-        for (int s = 0; s < ag.n_seg && ok; ++s) {
+        for (int s = 0; s < ag.n_seg; ++s) {
             const Segment& sg = ag.seg[s];
             FSeg& fs = g.seg[s];
             const bool pyr = sg.map_id == kMapPyr;
@@ -594,20 +630,8 @@ msf_status launch_attn_f32_tc(msf_plan_t plan, const AttnArgs& a, cudaStream_t s
             fs.len = sg.len;
             fs.tile0 = g.n_tiles;
             g.n_tiles += (sg.len + kBM - 1) / kBM;
-            if (done[fs.map]) continue;
-            done[fs.map] = true;
-            // rows that the segment's tensor holds: a group's part of the
-            // pyramid, the live slots of the ring, else all of it
-            const int part = pyr ? kF32Pyr : sg.map_id == kMapSink ? kF32Sink : sg.map_id == kMapHist ? kF32Ring : kF32Win;
-            const int rows = pyr || sg.map_id == kMapHist ? sg.len : sg.rows_total;
-            const size_t off = pyr ? (size_t)3 * P.B * P.groups[gi].pyr_offset * rowe * 2 : 0;
-            const int alloc = pyr ? P.groups[gi].pyr_cap : f32_part_rows(P, part);
-            const size_t so = pyr ? (size_t)sg.row0 * rowe * 4 : 0;
-            ok = add(sg.k + so, sg.bstride, f32_planes(P, part, 0) + off, alloc, rows, &maps.k[fs.map]) &&
-                 add(sg.v + so, sg.bstride, f32_planes(P, part, 1) + off, alloc, rows, &maps.v[fs.map]);
         }
     }
-    if (!ok) return fail(cudaErrorInvalidValue);
     fp.H = P.H;
     fp.B = P.B;
     fp.N = P.N;
@@ -641,14 +665,12 @@ msf_status launch_attn_f32_tc(msf_plan_t plan, const AttnArgs& a, cudaStream_t s
     }
     if (units == 0) return MSF_OK;
     if (slots > f32_max_slots(P)) return MSF_ERR_STATE;
-    const long long want = (sp.total + 255) / 256;
-    const int blocks = want < kF32SplitBlocks ? (int)want : kF32SplitBlocks;
-    fp.n_flags = blocks;
-    e = launch_pdl(split_planes_kernel, dim3((unsigned)blocks), dim3(256), 0, st, sp);
+    e = launch_split_planes(sp, &fp.n_flags, st);
     if (e != cudaSuccess) return fail(e);
     const bool d128 = P.D == 128;
     const int smem = d128 ? FCfg<128>::kSmem : FCfg<64>::kSmem < 120 * 1024 ? 120 * 1024 : FCfg<64>::kSmem;
-    e = d128 ? set_smem_attr((const void*)mssa_f32_kernel<128>, smem) : set_smem_attr((const void*)mssa_f32_kernel<64>, smem);
+    const void* fn = d128 ? (const void*)mssa_f32_kernel<128> : (const void*)mssa_f32_kernel<64>;
+    e = set_smem_attr(fn, smem, -1, kLaunchRegs);
     if (e != cudaSuccess) return fail(e);
     const dim3 grid((unsigned)units);
     e = d128 ? launch_pdl(mssa_f32_kernel<128>, grid, dim3(kThreads), smem, st, maps, fp)
@@ -659,7 +681,7 @@ msf_status launch_attn_f32_tc(msf_plan_t plan, const AttnArgs& a, cudaStream_t s
     if (e != cudaSuccess) return fail(e);
     AttnArgs fallback = a;
     fallback.run_if = sp.flags;
-    fallback.n_run_if = blocks;
+    fallback.n_run_if = fp.n_flags;
     e = launch_attn_simt(fallback, false, st);
     return e == cudaSuccess ? MSF_OK : fail(e);
 }

@@ -1,12 +1,46 @@
 // fp32 MSSA attention on the tensor cores (three bf16 planes per fp32 value).
 #pragma once
 
+#include <cuda.h>
+#include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include "attn_tc.h"
 #include "internal.h"
 #include "kernels.h"
 
 namespace msf {
+
+// ---- the operands' planes (attn_f32_tc.cu)
+struct SplitJob {
+    const float* src;    // stream 0
+    __nv_bfloat16* dst;  // stream 0, plane 0
+    long long src_bstride, dst_bstride, dst_plane;  // elements
+    int vecs;            // 8-element vectors per stream
+    long long base;      // first vector of the job (all streams) in the launch
+};
+constexpr int kMaxSplitJobs = 2 + 2 * (3 + MSF_MAX_GROUPS);
+struct SplitParams {
+    SplitJob j[kMaxSplitJobs];
+    int n;
+    long long total;
+    unsigned int* flags;  // one word per block: 1 = a value the planes cannot hold
+};
+struct F32Maps {
+    CUtensorMap q, dout;
+    CUtensorMap k[kNumMaps];
+    CUtensorMap v[kNumMaps];
+};
+// Add the first `rows` rows per stream of a [B, .., H, D] fp32 tensor as planes
+// [B, 3, alloc, H, D] at `dst` to the split, and encode their tensor map.
+bool add_planes(const Plan& P, SplitParams& sp, const void* src, long long src_bstride_bytes, char* dst, int alloc,
+                int rows, CUtensorMap* m);
+// q and the k, v of every context segment of `a`, in the workspace's planes.
+bool add_context_planes(const Plan& P, const AttnArgs& a, SplitParams& sp, F32Maps& maps);
+// Write the planes and the flags; *n_flags is the number of flag words.
+cudaError_t launch_split_planes(const SplitParams& sp, int* n_flags, cudaStream_t st);
+// K/V tiles per unit of work: see the definition.
+int f32_unit_tiles(double tiles_per_sm);
 
 // The fp32 attention of `a` (a plan with fp32 tensors, workspace bound): the
 // operands split into bf16 planes, the tensor-core kernel, the merge of split

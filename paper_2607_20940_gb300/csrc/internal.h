@@ -133,7 +133,8 @@ inline size_t f32_partial_bytes(const Plan& p) {
     return p.elem == 4 ? round256((size_t)f32_max_slots(p) * 128 * (p.D + 2) * 4) + round256(kF32SplitBlocks * 4) : 0;
 }
 // Backward workspace (caller-provided per msf_mssa_backward call):
-// [delta fp32 [B, H, N] | dk_ctx fp32 [B, R, H, D] | dv_ctx fp32 [B, R, H, D]],
+// [delta fp32 [B, H, N] | dk_ctx fp32 [B, R, H, D] | dv_ctx fp32 [B, R, H, D] |
+// fp32 plans: the planes of dout],
 // R = rows of every group's context that come from the window (the rows
 // that receive key/value gradients): N for g = 1, n_finer * G/g^2 + the
 // window suffix for g > 1.
@@ -149,7 +150,9 @@ inline size_t bwd_delta_bytes(const Plan& p) { return round256((size_t)p.B * p.H
 inline size_t bwd_ctx_bytes(const Plan& p) {
     return round256((size_t)p.B * bwd_ctx_rows(p) * p.H * p.D * 4);
 }
-inline size_t bwd_workspace_bytes(const Plan& p) { return bwd_delta_bytes(p) + 2 * bwd_ctx_bytes(p); }
+inline size_t bwd_workspace_bytes(const Plan& p) {
+    return bwd_delta_bytes(p) + 2 * bwd_ctx_bytes(p) + (p.elem == 4 ? f32_part_bytes(p, kF32Q) : 0);
+}
 inline size_t workspace_bytes(const Plan& p) {
     return kStatusBytes + 2 * pyramid_bytes(p) + msp_scratch_bytes(p) + attn_counter_bytes(p) +
            attn_partial_bytes(p) + msp_split_bytes(p) + tier_codes_bytes(p) + f32_plane_bytes(p) +

@@ -13,8 +13,10 @@ namespace msf {
 // carveout >= 0, its preferred shared-memory carveout in percent) on the
 // current device, once per (kernel, device): the attribute belongs to a
 // device's context, so a process that launches on several devices needs it on
-// each. Thread-safe.
-cudaError_t set_smem_attr(const void* fn, int bytes, int carveout = -1);
+// each. `regs` > 0: also refuse (cudaErrorInvalidKernelImage) a kernel that was
+// not compiled to exactly that many registers per thread, which its
+// setmaxnreg split counts on. Thread-safe.
+cudaError_t set_smem_attr(const void* fn, int bytes, int carveout = -1, int regs = 0);
 
 // One block that waits, with the bounded wait of the tcgen05 kernels, on an
 // mbarrier nothing arrives at, then raises the TIMEOUT bit of *status.
@@ -206,11 +208,16 @@ struct GatherArgs {
     int mode;  // msf_resample_mode
 };
 cudaError_t launch_bwd_delta(const BwdCommon& c, bool bf16, cudaStream_t st);
+// Run a kernel only if one of these n words is set (NULL = run).
+struct BwdRunIf {
+    const unsigned int* flags = nullptr;
+    int n = 0;
+};
 // dq for every query of every group (context of each group as in the forward).
-cudaError_t launch_bwd_dq_simt(const BwdCommon& c, const AttnArgs& a, void* dq, bool bf16,
+cudaError_t launch_bwd_dq_simt(const BwdCommon& c, const AttnArgs& a, void* dq, bool bf16, BwdRunIf run_if,
                                cudaStream_t st);
-// Context-row gradients of one group's window-derived rows.
-cudaError_t launch_bwd_dkdv_simt(const BwdCommon& c, const BwdGroup& g, bool bf16,
+// Context-row gradients of every group's window-derived rows.
+cudaError_t launch_bwd_dkdv_simt(const BwdCommon& c, const BwdGroup* g, int n_groups, bool bf16, BwdRunIf run_if,
                                  cudaStream_t st);
 // dk_win, dv_win from the context-row gradients (adjoint of Subsample, sum
 // over groups, one rounding to the dtype).

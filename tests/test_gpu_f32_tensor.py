@@ -99,3 +99,76 @@ def test_f32_tensor_attention_small_and_large_values():
     out, _, _ = _forward(w, x)
     mx, _ = err_stats(out * 2.0 ** 60, oracle_mssa(x, w) * 2.0 ** 60)
     assert mx <= 1.5e-5, mx
+
+
+def _backward(w, x, seed=9):
+    plan = make_plan(w, F32)
+    d = device_inputs(x, w.history_capacity)
+    ws = bind(plan, d)
+    out = torch.empty_like(d["q"])
+    lse = torch.empty((w.batch, w.heads, plan.info.n_tokens), device="cuda")
+    dout = torch.randn(d["q"].shape, generator=torch.Generator().manual_seed(seed))
+    plan.kv_resample(d["k_win"], d["v_win"])
+    plan.mssa_forward_lse(d["q"], d["k_win"], d["v_win"], out, lse)
+    bws = plan.backward_workspace()
+    got = []
+    for fn in (plan.mssa_backward, plan.mssa_backward, plan.mssa_backward_simt):
+        g = [torch.full_like(d["q"], float("nan")) for _ in range(3)]
+        fn(d["q"], d["k_win"], d["v_win"], out, dout.cuda(), lse, *g, bws)
+        got.append(g)
+    torch.cuda.synchronize()
+    assert plan.device_status() == msf().MSF_OK
+    del ws
+    return dout, got
+
+
+# Gradients: sums of up to a few thousand products P * (dP - delta) * k with
+# |P| <= 1 and dP around sqrt(D); fp32 sums of them in any order differ by less
+# than 2^-24 times the terms' absolute sum, well below 1e-5 of the largest
+# gradient (the CUDA-core kernels show up to 2e-6 of it).
+@pytest.mark.parametrize("w", CASES[:7], ids=[f"{w.scales}-{w.grid_h}x{w.grid_w}-h{w.heads}-d{w.head_dim}" for w in CASES[:7]])
+@pytest.mark.parametrize("mode", [0, 1], ids=["avg", "strided"])
+def test_f32_tensor_backward(w, mode):
+    from oracle import mssa_bwd as obwd
+    if mode and max(w.scales) == 1:
+        pytest.skip("no pooling")
+    x = synth.attention_inputs(w, F32)
+    m = msf()
+    desc = m.make_desc(w.scales, w.grid_h, w.grid_w, w.heads, w.head_dim, w.sink_tokens, w.history_frames,
+                       history_capacity=w.history_capacity, batch=w.batch, dtype=m.MSF_DTYPE_F32, resample=mode)
+    plan = m.Plan(desc)
+    d = device_inputs(x, w.history_capacity)
+    ws = bind(plan, d)
+    out = torch.empty_like(d["q"])
+    lse = torch.empty((w.batch, w.heads, plan.info.n_tokens), device="cuda")
+    dout = torch.randn(d["q"].shape, generator=torch.Generator().manual_seed(9))
+    plan.kv_resample(d["k_win"], d["v_win"])
+    plan.mssa_forward_lse(d["q"], d["k_win"], d["v_win"], out, lse)
+    bws = plan.backward_workspace()
+    got = []
+    for _ in range(2):
+        g = [torch.full_like(d["q"], float("nan")) for _ in range(3)]
+        plan.mssa_backward(d["q"], d["k_win"], d["v_win"], out, dout.cuda(), lse, *g, bws)
+        got.append(g)
+    torch.cuda.synchronize()
+    assert plan.device_status() == m.MSF_OK
+    assert all(torch.equal(a, b) for a, b in zip(*got))
+    f = synth.to_f64
+    ref = obwd.mssa_backward(f(x["q"]), f(x["k_win"]), f(x["v_win"]), f(x["k_sink"]), f(x["v_sink"]), f(x["k_hist"]),
+                             f(x["v_hist"]), f(dout), w.scales, w.grid_h, w.grid_w, mode=mode)
+    for g, key in zip(got[0], ("dq", "dk_win", "dv_win")):
+        e = abs(g.double().cpu().numpy() - ref[key]).max() / max(abs(ref[key]).max(), 1e-30)
+        # one key in all (a 1 x 1 window without a cache): dS is 0 in exact arithmetic
+        assert e <= 1e-5 or abs(ref[key]).max() < 1e-12, (key, e)
+    del ws
+
+
+@pytest.mark.parametrize("value", [float("inf"), float("nan"), torch.finfo(F32).min])
+@pytest.mark.parametrize("where", ["q", "k_win", "v_sink"])
+def test_f32_backward_values_the_planes_cannot_hold(value, where):
+    w = CASES[4]
+    x = synth.attention_inputs(w, F32)
+    x[where][1, 3, 1, 5] = value
+    _, (got, _, simt) = _backward(w, x)
+    for a, b in zip(got, simt):
+        assert torch.equal(torch.nan_to_num(a, nan=123.0), torch.nan_to_num(b, nan=123.0))
