@@ -4,24 +4,28 @@
 // forward's row log-sum-exp, P = exp(c S - lse) is rebuilt tile by tile and
 //   dS = P * (dP - delta),  dP = dO V^T,  delta = rowsum(dO * O)
 //   dQ = c dS K,  dK = c dS^T Q,  dV = P^T dO.
-// Two kernels, neither needs atomics:
+// One persistent launch (a CTA per SM) runs two kinds of items, no atomics:
 //
-// bwd_dq_tc_kernel: one CTA per 128-row query tile of one (stream, head,
-//   group). It walks the group's whole context (sink, history or pyramid
-//   part, window suffix) in 128-row K/V tiles:
+// dq item: a 128-row query tile of one (stream, head, group). It walks the
+//   group's whole context (sink, history or pyramid part, window suffix) in
+//   128-row K/V tiles:
 //     S = Q K^T (SS, two buffers), dP = dO V^T (SS)  -> TMEM
-//     softmax warps: P, dS (bf16, over S's columns)   -> TMEM
+//     softmax warps: dS (bf16, over S's columns)      -> TMEM
 //     dQ += dS K (TS, K read MN-major)               -> TMEM
 //   then scales dQ by c and stores it.
-// bwd_dkdv_tc_kernel: one CTA per 128-row tile of context rows that come
-//   from the window, every group in one launch. It walks its group's
-//   queries in 128-row tiles:
+// dk/dv item: a 128-row tile of context rows that come from the window. It
+//   walks its group's queries in 128-row tiles:
 //     S^T = K Q^T (SS), dP^T = V dO^T (SS)            -> TMEM (lanes = keys)
-//     softmax warps: P^T, dS^T (bf16, over S^T/dP^T)  -> TMEM
+//     softmax warps: P^T over S^T, then dS^T over dP^T -> TMEM
 //     dV += P^T dO (TS), dK += dS^T Q (TS)           -> TMEM
 //   then writes c dK and dV (fp32) to its rows of the context-gradient
-//   buffers, staged through shared memory so that every warp stores whole
-//   rows. A gather kernel applies the adjoint of Subsample afterwards.
+//   buffers. A gather kernel applies the adjoint of Subsample afterwards.
+//
+// CTA c takes items c, 2G-1-c, 2G+c, ... of the list sorted by cost (G CTAs,
+// back and forth so that no CTA always gets a round's longest), and its roles
+// run on from item to item: the next item's loads and first MMAs overlap the
+// output of the one before, and tensor memory and barriers are set up once.
+// On the 480p layer an item used to cost 5-9 us besides its tiles.
 //
 // Roles (384 threads): warp 0 TMA producer, warp 1 MMA issuer (warp-wide
 // loop, one elected lane issues), warp 2 TMEM allocation, warps 4-11 the
@@ -29,11 +33,9 @@
 // warps 4-7 columns 0-63, warps 8-11 columns 64-127. Each half writes its
 // bf16 P / dS into its own columns (the MMA that reads them takes its A
 // operand per 16-column step), so the halves never wait for each other.
-// TMEM columns of the dK/dV
-// kernel: S^T [0,128), dP^T [128,256), dV, dK from 256 (the dQ kernel's
-// layout is given with it). The tensor pipe executes MMAs
-// in issue order, so an MMA that overwrites S or dP never overtakes the MMA
-// that reads the bf16 P or dS stored there. Every wait is bounded.
+// The tensor pipe executes MMAs in issue order, so an MMA that overwrites S
+// or dP never overtakes the MMA that reads the bf16 P or dS stored there.
+// Every wait is bounded.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -84,13 +86,15 @@ struct BwdTcParams {
     int R;  // rows per stream of the context-gradient buffers
     unsigned int* status;
     long long wait_limit;
-    // bwd_dq_tc_kernel
+    int dq_v8, ctx_v8;  // 32-byte aligned outputs: 32-byte stores
+    int n_items;
+    // dq work
     int n_groups;
     BGroupQ g[MSF_MAX_GROUPS];
     // dK/dV work
     int n_kgroups;
     BGroupK kg[MSF_MAX_GROUPS];
-    // Block ranges of the one launch, most expensive items first: kind 0 =
+    // Item ranges, most expensive items first: kind 0 =
     // dq items of group g[group], kind 1 = dK/dV items of kg[group].
     int n_ranges;
     struct Range {
@@ -103,14 +107,35 @@ struct BwdMaps {
     CUtensorMap v[kNumMaps];
 };
 
-// Dynamic shared memory of the launch: seven 128 x D bf16 tiles (dq items:
-// Q, dO, a 3-deep K ring and a 2-deep V ring; dK/dV items: K, V, a 2-deep
-// Q/dO ring and the per-query statistics), at least 120 KB so that one CTA
-// (and one 512-column TMEM allocation) sits on an SM.
+// Barriers of the roles; an index counts phases from the launch's start.
+struct BwdBars {
+    // dq items: Q and dO, the K and V rings, S + dP ready, dP read, dS written, dQ complete
+    uint64_t qg_full, qg_empty, k_full[3], k_empty[3], v_full[2], v_empty[2];
+    uint64_t sdp_full, dp_free, ds_full, dq_full;
+    // dk/dv items: K, V, the Q and dO rings, S^T ready, P^T written, dP^T
+    // ready, dS^T written, dV and dK complete; the warps of a half meet
+    uint64_t kst_full, kst_empty, vst_full, vst_empty, q_full[3], q_empty[3], g_full[2], g_empty[2];
+    uint64_t st_full, p_full, dpt_full, dst_full, kv_full, meet[2];
+    uint64_t item_done, drain;
+    uint32_t tmem_base;
+    int abort_flag;
+};
+
+// Dynamic shared memory of the launch (no static part, so that its base is
+// 1024-byte aligned): seven 128 x D bf16 tiles (dq items: Q, dO, a 3-deep K
+// ring and a 2-deep V ring; dk/dv items: K, V, a 3-deep Q ring and a 2-deep
+// dO ring), the per-query statistics of two query tiles, the barriers. At
+// least 120 KB, so that one CTA (and one 512-column TMEM allocation) sits on
+// an SM.
 template <int D>
 struct BCfg {
     static constexpr int kTile = kBM * D * 2;
+    static constexpr int kStats = 7 * kTile;
+    static constexpr int kBars = kStats + 4 * kBM * 4;
+    static constexpr int kUsed = kBars + (int)sizeof(BwdBars);
+    static constexpr int kSmem = kUsed > 120 * 1024 ? kUsed : 120 * 1024;
 };
+static_assert(BCfg<128>::kSmem <= 227 * 1024, "shared memory of the launch");
 
 __device__ __forceinline__ float ex2(float x) {
     float y;
@@ -132,615 +157,637 @@ __device__ __forceinline__ void load_tile(unsigned char* dst, const CUtensorMap*
     for (int c = 0; c < D / 64; ++c) ptx::tma_load_4d(dst + c * (kBM * 128), m, bar, c * 64, h, row, b);
 }
 
-// ============================================================== dQ kernel
-//
-// TMEM: S for even tiles [0,128), S for odd tiles [128,256), dP [256,384),
-// dQ from 384. Smem: Q, dO, a 3-deep K ring, a 2-deep V ring. The softmax
-// warps first copy dP_j into registers and release it, so dP_{j+1} (and
-// S_{j+1}, issued a tile ahead into the other S buffer) run on the tensor
-// pipe while they compute dS_j; dQ_j and S_{j+2} then run while the softmax
-// works on tile j+1.
-
-template <int D>
-struct QCfg {
-    static constexpr int kTile = kBM * D * 2;
-    static constexpr int kSmem = 7 * kTile + 1024 > 120 * 1024 ? 7 * kTile + 1024 : 120 * 1024;
+// The parts of an item that every role needs.
+struct BItem {
+    int kind, gi;
+    int h, b;
+    int n;     // tiles it walks: K/V tiles (dq), query tiles (dk/dv)
+    int row0;  // dq: first query; dk/dv: first context row in its tensor map
+    int map;   // dk/dv: tensor map of K and V
+    int crow;  // dk/dv: first row in the context-gradient buffers
+    int rows;  // valid rows of the own tile
 };
-static_assert(7 * QCfg<128>::kTile + 1024 + 2048 <= 227 * 1024, "shared memory of the launch");
 
+__device__ __forceinline__ BItem item_of(const BwdTcParams& p, int idx) {
+    int r = 0;
+    while (r + 1 < p.n_ranges && idx >= p.range[r + 1].base) ++r;
+    const int local = idx - p.range[r].base;
+    BItem it;
+    it.kind = p.range[r].kind;
+    it.gi = p.range[r].group;
+    if (it.kind == 0) {
+        const BGroupQ& G = p.g[it.gi];
+        const int qt = local % G.n_qt;
+        it.h = (local / G.n_qt) % p.H;
+        it.b = local / (G.n_qt * p.H);
+        it.n = G.n_tiles;
+        it.row0 = G.q_begin + qt * kBM;
+        it.map = 0;
+        it.crow = 0;
+        it.rows = min(kBM, G.q_end - it.row0);
+    } else {
+        const BGroupK& K = p.kg[it.gi];
+        const int kt_all = local % K.n_kt;
+        it.h = (local / K.n_kt) % p.H;
+        it.b = local / (K.n_kt * p.H);
+        int s = 0;
+        while (s + 1 < K.n_grad && kt_all >= K.gr[s + 1].kt0) ++s;
+        const int off = (kt_all - K.gr[s].kt0) * kBM;
+        it.n = K.n_qt;
+        it.row0 = K.gr[s].row0 + off;
+        it.map = K.gr[s].map;
+        it.crow = K.gr[s].crow0 + off;
+        it.rows = min(kBM, K.gr[s].len - off);
+    }
+    return it;
+}
+
+// K/V tile u of a dq item of group G.
+__device__ __forceinline__ void kv_tile(const BGroupQ& G, int u, int& map, int& row, int& valid) {
+    int s = 0;
+    while (s < G.n_seg - 1 && u >= G.seg[s + 1].tile0) ++s;
+    const int kt = u - G.seg[s].tile0;
+    map = G.seg[s].map;
+    row = G.seg[s].row0 + kt * kBM;
+    valid = min(kBM, G.seg[s].len - kt * kBM);
+}
+
+// Item of round k of this CTA: rounds alternate direction.
+__device__ __forceinline__ int round_item(int k) {
+    const int g = (int)gridDim.x, c = (int)blockIdx.x;
+    return k * g + ((k & 1) ? g - 1 - c : c);
+}
+
+// 64 fp32 columns of a row scaled by mul: 32-byte stores when aligned.
+__device__ __forceinline__ void store_f32(float* dst, const uint32_t (&o)[32], float mul, bool v8) {
+    uint32_t x[32];
+#pragma unroll
+    for (int e = 0; e < 32; ++e) x[e] = __float_as_uint(__uint_as_float(o[e]) * mul);
+    if (v8) {
+#pragma unroll
+        for (int e = 0; e < 4; ++e) ptx::st_global_v8(dst + 8 * e, x + 8 * e);
+    } else {
+#pragma unroll
+        for (int e = 0; e < 8; ++e)
+            reinterpret_cast<uint4*>(dst)[e] = make_uint4(x[4 * e], x[4 * e + 1], x[4 * e + 2], x[4 * e + 3]);
+    }
+}
+
+// TMEM columns, dq items: S of even tiles [0,128), of odd tiles [128,256), dP
+// [256,384), dQ from 384. The softmax warps first copy dP_j into registers and
+// release it, so dP_{j+1} (and S_{j+1}, issued a tile ahead into the other S
+// buffer) run on the tensor pipe while they compute dS_j; dQ_j and S_{j+2}
+// then run while the softmax works on tile j+1.
+// dk/dv items: S^T [0,128), dP^T [128,256), dV from 256, dK from 256 + D. Two
+// phases per query tile keep the pipe busy: once P^T_i is written, dV_i and
+// S^T_{i+1} run while the softmax turns dP^T_i into dS^T_i; then dK_i and
+// dP^T_{i+1} run while it turns S^T_{i+1} into P^T_{i+1}. All MMAs are 128
+// columns wide: the two 64-query halves of the version before cost 62.6
+// cycles per 64-wide MMA (shared-memory reads bound it) against 82 per 128.
 template <int D>
-__device__ __forceinline__ void dq_item(const BwdMaps& maps, const BwdTcParams& p, int gi, int local) {
-    using C = QCfg<D>;
-    extern __shared__ __align__(1024) unsigned char smem_raw[];
-    unsigned char* smem = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    unsigned char* sQ = smem;
-    unsigned char* sG = smem + C::kTile;       // dO
-    unsigned char* sK = smem + 2 * C::kTile;   // [3]
-    unsigned char* sV = smem + 5 * C::kTile;   // [2]
-
-    __shared__ uint64_t qg_full, k_full[3], k_empty[3], v_full[2], v_empty[2];
-    __shared__ uint64_t sdp_full, dp_free, ds_full, dq_full, drain_bar;
-    __shared__ uint32_t tmem_base_sh;
-    __shared__ int abort_flag;
-
+__global__ void __launch_bounds__(kThreads, 1)
+    bwd_tc_kernel(const __grid_constant__ BwdMaps maps, const __grid_constant__ BwdTcParams p) {
+    using C = BCfg<D>;
+    extern __shared__ __align__(1024) unsigned char smem[];
+    BwdBars& bar = *reinterpret_cast<BwdBars*>(smem + C::kBars);
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-    const BGroupQ& G = p.g[gi];
-    const int qt = local % G.n_qt;
-    const int h = (local / G.n_qt) % p.H;
-    const int b = local / (G.n_qt * p.H);
-    const int q_row0 = G.q_begin + qt * kBM;
-    const int n = G.n_tiles;
-
+    if (ptx::smem_u32(smem) & 1023u) {  // the swizzled tiles need it
+        if (threadIdx.x == 0) atomicOr(p.status, kDevTimeout);
+        return;
+    }
     if (threadIdx.x == 0) {
-        abort_flag = 0;
-        ptx::mbar_init(&qg_full, 1);
+        bar.abort_flag = 0;
+        uint64_t* one[] = {&bar.qg_full, &bar.qg_empty, &bar.sdp_full, &bar.dq_full, &bar.kst_full, &bar.kst_empty,
+                           &bar.vst_full, &bar.vst_empty, &bar.st_full, &bar.dpt_full, &bar.kv_full, &bar.drain};
+        for (uint64_t* x : one) ptx::mbar_init(x, 1);
         for (int s = 0; s < 3; ++s) {
-            ptx::mbar_init(&k_full[s], 1);
-            ptx::mbar_init(&k_empty[s], 1);
+            ptx::mbar_init(&bar.k_full[s], 1);
+            ptx::mbar_init(&bar.k_empty[s], 1);
+            ptx::mbar_init(&bar.q_full[s], 1);
+            ptx::mbar_init(&bar.q_empty[s], 1);
         }
         for (int s = 0; s < 2; ++s) {
-            ptx::mbar_init(&v_full[s], 1);
-            ptx::mbar_init(&v_empty[s], 1);
+            ptx::mbar_init(&bar.v_full[s], 1);
+            ptx::mbar_init(&bar.v_empty[s], 1);
+            ptx::mbar_init(&bar.g_full[s], 1);
+            ptx::mbar_init(&bar.g_empty[s], 1);
+            ptx::mbar_init(&bar.meet[s], 4);
         }
-        ptx::mbar_init(&sdp_full, 1);
-        ptx::mbar_init(&dp_free, 8);
-        ptx::mbar_init(&ds_full, 8);
-        ptx::mbar_init(&dq_full, 1);
-        ptx::mbar_init(&drain_bar, 1);
+        ptx::mbar_init(&bar.dp_free, 8);
+        ptx::mbar_init(&bar.ds_full, 8);
+        ptx::mbar_init(&bar.p_full, 8);
+        ptx::mbar_init(&bar.dst_full, 8);
+        ptx::mbar_init(&bar.item_done, 8);
         ptx::fence_mbar_init();
     }
     if (warp == 2) {
-        ptx::tmem_alloc(&tmem_base_sh, 512);
+        ptx::tmem_alloc(&bar.tmem_base, 512);
         ptx::tmem_relinquish();
     }
     ptx::tc_fence_before();
     __syncthreads();
     ptx::tc_fence_after();
-    const uint32_t tbase = tmem_base_sh;
-    volatile int* abort_p = &abort_flag;
+    const uint32_t tbase = bar.tmem_base;
+    volatile int* abort_p = &bar.abort_flag;
     volatile int never = 0;
     ptx::grid_dep_wait();
     ptx::grid_dep_launch();
-
-    auto tile_of = [&](int u, int& seg, int& row, int& valid) {
-        int s = 0;
-        while (s < G.n_seg - 1 && u >= G.seg[s + 1].tile0) ++s;
-        const int kt = u - G.seg[s].tile0;
-        seg = s;
-        row = G.seg[s].row0 + kt * kBM;
-        valid = min(kBM, G.seg[s].len - kt * kBM);
-    };
 
     if (warp == 0) {
         // ============================ TMA producer ============================
         if (lane == 0) {
             bool ok = true;
-            ptx::mbar_arrive_expect_tx(&qg_full, 2 * C::kTile);
-            load_tile<D>(sQ, &maps.q, &qg_full, h, q_row0, b);
-            load_tile<D>(sG, &maps.dout, &qg_full, h, q_row0, b);
-            int j = 0, nk = 0, nv = 0;
-            for (; j < n; ++j) {
-                int seg, row, valid;
-                tile_of(j, seg, row, valid);
-                const int ks = j % 3, vs = j & 1;
-                if (!ptx::mbar_wait_bounded(&k_empty[ks], (uint32_t)(((j / 3) & 1) ^ 1), abort_p,
-                                            p.wait_limit)) {
-                    ok = false;
-                    break;
+            // tiles issued so far to each ring, items of each kind
+            int nk = 0, nv = 0, nq = 0, ng = 0, n_dq = 0, n_kst = 0, n_vst = 0;
+            auto take = [&](uint64_t* empty, uint32_t parity) {
+                ok = ok && ptx::mbar_wait_bounded(empty, parity, abort_p, p.wait_limit);
+                return ok;
+            };
+            int prev_kind = -1;
+            for (int k = 0; ok; ++k) {
+                const int idx = round_item(k);
+                if (idx >= p.n_items) break;
+                const BItem it = item_of(p, idx);
+                // The item before the last is done (so that the phases of
+                // item_done are seen one by one); on a change of kind the last
+                // one too, whose tiles this one's overwrite.
+                if (k >= 2 && !take(&bar.item_done, (uint32_t)(k & 1))) break;
+                if (k >= 1 && it.kind != prev_kind && !take(&bar.item_done, (uint32_t)((k - 1) & 1))) break;
+                prev_kind = it.kind;
+                if (it.kind == 0) {
+                    const BGroupQ& G = p.g[it.gi];
+                    if (!take(&bar.qg_empty, (uint32_t)((n_dq & 1) ^ 1))) break;
+                    ptx::mbar_arrive_expect_tx(&bar.qg_full, 2 * C::kTile);
+                    load_tile<D>(smem, &maps.q, &bar.qg_full, it.h, it.row0, it.b);
+                    load_tile<D>(smem + C::kTile, &maps.dout, &bar.qg_full, it.h, it.row0, it.b);
+                    ++n_dq;
+                    for (int j = 0; j < it.n; ++j) {
+                        int map, row, valid;
+                        kv_tile(G, j, map, row, valid);
+                        const int ks = nk % 3, vs = nv & 1;
+                        if (!take(&bar.k_empty[ks], (uint32_t)(((nk / 3) & 1) ^ 1))) break;
+                        ptx::mbar_arrive_expect_tx(&bar.k_full[ks], C::kTile);
+                        load_tile<D>(smem + (2 + ks) * C::kTile, &maps.k[map], &bar.k_full[ks], it.h, row, it.b);
+                        ++nk;
+                        if (!take(&bar.v_empty[vs], (uint32_t)(((nv >> 1) & 1) ^ 1))) break;
+                        ptx::mbar_arrive_expect_tx(&bar.v_full[vs], C::kTile);
+                        load_tile<D>(smem + (5 + vs) * C::kTile, &maps.v[map], &bar.v_full[vs], it.h, row, it.b);
+                        ++nv;
+                    }
+                } else {
+                    const BGroupK& K = p.kg[it.gi];
+                    if (!take(&bar.kst_empty, (uint32_t)((n_kst & 1) ^ 1))) break;
+                    ptx::mbar_arrive_expect_tx(&bar.kst_full, C::kTile);
+                    load_tile<D>(smem, &maps.k[it.map], &bar.kst_full, it.h, it.row0, it.b);
+                    ++n_kst;
+                    for (int i = 0; i < it.n; ++i) {
+                        const int qs = nq % 3, gs = ng & 1, row = K.q_begin + i * kBM;
+                        if (!take(&bar.q_empty[qs], (uint32_t)(((nq / 3) & 1) ^ 1))) break;
+                        ptx::mbar_arrive_expect_tx(&bar.q_full[qs], C::kTile);
+                        load_tile<D>(smem + (2 + qs) * C::kTile, &maps.q, &bar.q_full[qs], it.h, row, it.b);
+                        ++nq;
+                        if (i == 0) {
+                            if (!take(&bar.vst_empty, (uint32_t)((n_vst & 1) ^ 1))) break;
+                            ptx::mbar_arrive_expect_tx(&bar.vst_full, C::kTile);
+                            load_tile<D>(smem + C::kTile, &maps.v[it.map], &bar.vst_full, it.h, it.row0, it.b);
+                            ++n_vst;
+                        }
+                        if (!take(&bar.g_empty[gs], (uint32_t)(((ng >> 1) & 1) ^ 1))) break;
+                        ptx::mbar_arrive_expect_tx(&bar.g_full[gs], C::kTile);
+                        load_tile<D>(smem + (5 + gs) * C::kTile, &maps.dout, &bar.g_full[gs], it.h, row, it.b);
+                        ++ng;
+                    }
                 }
-                ptx::mbar_arrive_expect_tx(&k_full[ks], C::kTile);
-                load_tile<D>(sK + ks * C::kTile, &maps.k[G.seg[seg].map], &k_full[ks], h, row, b);
-                ++nk;
-                if (!ptx::mbar_wait_bounded(&v_empty[vs], (uint32_t)(((j >> 1) & 1) ^ 1), abort_p,
-                                            p.wait_limit)) {
-                    ok = false;
-                    break;
-                }
-                ptx::mbar_arrive_expect_tx(&v_full[vs], C::kTile);
-                load_tile<D>(sV + vs * C::kTile, &maps.v[G.seg[seg].map], &v_full[vs], h, row, b);
-                ++nv;
             }
             if (!ok) {
                 // every copy issued lands before the CTA exits
-                ptx::mbar_wait_bounded(&qg_full, 0, &never, kWaitLimit);
-                for (int jj = (nk > 3 ? nk - 3 : 0); jj < nk; ++jj)
-                    ptx::mbar_wait_bounded(&k_full[jj % 3], (uint32_t)((jj / 3) & 1), &never, kWaitLimit);
-                for (int jj = (nv > 2 ? nv - 2 : 0); jj < nv; ++jj)
-                    ptx::mbar_wait_bounded(&v_full[jj & 1], (uint32_t)((jj >> 1) & 1), &never, kWaitLimit);
+                auto landed = [&](uint64_t* full, int n) {
+                    if (n > 0) ptx::mbar_wait_bounded(full, (uint32_t)((n - 1) & 1), &never, kWaitLimit);
+                };
+                landed(&bar.qg_full, n_dq);
+                landed(&bar.kst_full, n_kst);
+                landed(&bar.vst_full, n_vst);
+                for (int s = 0; s < 3; ++s) {
+                    landed(&bar.k_full[s], (nk + 2 - s) / 3);
+                    landed(&bar.q_full[s], (nq + 2 - s) / 3);
+                }
+                for (int s = 0; s < 2; ++s) {
+                    landed(&bar.v_full[s], (nv + 1 - s) / 2);
+                    landed(&bar.g_full[s], (ng + 1 - s) / 2);
+                }
                 atomicOr(p.status, kDevTimeout);
             }
         }
     } else if (warp == 1) {
         // ============================= MMA issuer =============================
-        constexpr uint32_t idS = ptx::idesc_bf16(kBM, kBM, false, false);
-        constexpr uint32_t idQ = ptx::idesc_bf16(kBM, D, false, true);
-        constexpr uint64_t kTileDesc = (uint64_t)(C::kTile >> 4);
-        const uint64_t q_desc = ptx::sdesc_sw128(ptx::smem_u32(sQ), 16, 1024);
-        const uint64_t g_desc = ptx::sdesc_sw128(ptx::smem_u32(sG), 16, 1024);
-        const uint64_t k_desc = ptx::sdesc_sw128(ptx::smem_u32(sK), 16, 1024);
-        const uint64_t v_desc = ptx::sdesc_sw128(ptx::smem_u32(sV), 16, 1024);
-        const uint64_t kmn_desc = ptx::sdesc_sw128(ptx::smem_u32(sK), kBM * 128, 1024);
-        auto wait_all = [&](uint64_t* bar, uint32_t parity) {
-            const bool r = ptx::mbar_wait_bounded(bar, parity, abort_p, p.wait_limit);
-            return __all_sync(0xffffffffu, r);
-        };
-        auto issue_s = [&](int j) {  // S_j = Q K_j^T into the S buffer of j's parity
-            const uint64_t kd = k_desc + (uint64_t)(j % 3) * kTileDesc;
-#pragma unroll
-            for (int kk = 0; kk < D / 16; ++kk)
-                ptx::mma_ss(tbase + (j & 1) * 128, q_desc + kmajor_step(kk), kd + kmajor_step(kk), idS,
-                            kk > 0 ? 1u : 0u);
-        };
-        auto issue_dp = [&](int j) {  // dP_j = dO V_j^T
-            const uint64_t vd = v_desc + (uint64_t)(j & 1) * kTileDesc;
-#pragma unroll
-            for (int kk = 0; kk < D / 16; ++kk)
-                ptx::mma_ss(tbase + 256, g_desc + kmajor_step(kk), vd + kmajor_step(kk), idS,
-                            kk > 0 ? 1u : 0u);
-            ptx::mma_commit(&v_empty[j & 1]);
-            ptx::mma_commit(&sdp_full);
-        };
-        bool ok = wait_all(&qg_full, 0) && wait_all(&k_full[0], 0) && wait_all(&v_full[0], 0);
-        if (ok) {
-            ptx::tc_fence_after();
-            if (ptx::elect_one_sync()) {
-                issue_s(0);
-                issue_dp(0);
-            }
-            __syncwarp();
-            if (n > 1) {
-                ok = wait_all(&k_full[1], 0);
-                if (ok) {
-                    ptx::tc_fence_after();
-                    if (ptx::elect_one_sync()) issue_s(1);
-                    __syncwarp();
-                }
-            }
-        }
         // Two probe points per tile. A tcgen05.mma holds its issuing thread
         // about as long as the tensor pipe takes to run it, and only ~250
         // cycles of work stay in flight after the last issue, so every
         // barrier check here is pipe time: the probes of each point go out
         // together, and the bounded waits run only if one is not ready.
-        for (int j = 0; j < n && ok; ++j) {
-            const bool next = j + 1 < n, next2 = j + 2 < n;
-            {
-                const bool rd = ptx::mbar_try_wait(&dp_free, (uint32_t)(j & 1));
-                const bool rv = !next || ptx::mbar_try_wait(&v_full[(j + 1) & 1], (uint32_t)(((j + 1) >> 1) & 1));
-                if (!__all_sync(0xffffffffu, rd && rv))
-                    ok = wait_all(&dp_free, (uint32_t)(j & 1)) &&
-                         (!next || wait_all(&v_full[(j + 1) & 1], (uint32_t)(((j + 1) >> 1) & 1)));
-            }
-            if (!ok) break;
-            if (next) {
-                ptx::tc_fence_after();
-                if (ptx::elect_one_sync()) issue_dp(j + 1);
-                __syncwarp();
-            }
-            // dS_j, and K_{j+2} for the S two tiles ahead; if K has not
-            // landed yet, dQ_j goes first and S_{j+2} after its own wait.
-            bool k_ready;
-            {
-                const bool rs = ptx::mbar_try_wait(&ds_full, (uint32_t)(j & 1));
-                k_ready = !next2 || ptx::mbar_try_wait(&k_full[(j + 2) % 3], (uint32_t)(((j + 2) / 3) & 1));
-                k_ready = __all_sync(0xffffffffu, k_ready);
-                if (!__all_sync(0xffffffffu, rs)) ok = wait_all(&ds_full, (uint32_t)(j & 1));
-            }
-            if (!ok) break;
-            ptx::tc_fence_after();
-            if (ptx::elect_one_sync()) {
-                const uint64_t kd = kmn_desc + (uint64_t)(j % 3) * kTileDesc;
-#pragma unroll
-                for (int kk = 0; kk < kBM / 16; ++kk)
-                    ptx::mma_ts(tbase + 384, tbase + (j & 1) * 128 + 64 * (kk / 4) + (kk % 4) * 8,
-                                kd + (uint64_t)(kk * (2048 >> 4)), idQ, (j > 0 || kk > 0) ? 1u : 0u);
-                ptx::mma_commit(&k_empty[j % 3]);
-                if (j + 1 == n) ptx::mma_commit(&dq_full);
-                if (next2 && k_ready) issue_s(j + 2);
-            }
-            __syncwarp();
-            if (next2 && !k_ready) {
-                ok = wait_all(&k_full[(j + 2) % 3], (uint32_t)(((j + 2) / 3) & 1));
-                if (!ok) break;
-                ptx::tc_fence_after();
-                if (ptx::elect_one_sync()) issue_s(j + 2);
-                __syncwarp();
-            }
-        }
-        if (!ok) {
-            if (ptx::elect_one_sync()) ptx::mma_commit(&drain_bar);
-            __syncwarp();
-            ptx::mbar_wait_bounded(&drain_bar, 0, &never, kWaitLimit);
-            if (lane == 0) atomicOr(p.status, kDevTimeout);
-        }
-    } else if (warp >= 4) {
-        // ============ softmax: one thread per query row and column half ============
-        const int half = (warp - 4) / 4;
-        const int wq = warp % 4;
-        const int r = wq * 32 + lane;
-        const uint32_t lane_off = (uint32_t)(wq * 32) << 16;
-        const uint32_t tP = tbase + 256 + 64 * half + lane_off;
-        const int q = q_row0 + r;
-        const bool qv = q < G.q_end;
-        const size_t rix = ((size_t)b * p.H + h) * p.N + (qv ? q : 0);
-        const float nl = qv ? -p.lse[rix] * kLog2e : -INFINITY;  // -lse in log2 units
-        const float dl = qv ? p.delta[rix] : 0.f;
-        const uint64_t sl2x2 = ptx::f2_pack(p.scale_log2, p.scale_log2), nlx2 = ptx::f2_pack(nl, nl);
-        const uint64_t ndlx2 = ptx::f2_pack(-dl, -dl);
-        bool ok = true;
-        for (int j = 0; j < n && ok; ++j) {
-            int seg, row, valid;
-            tile_of(j, seg, row, valid);
-            ok = __all_sync(0xffffffffu, ptx::mbar_wait_bounded(&sdp_full, (uint32_t)(j & 1), abort_p,
-                                                                p.wait_limit));
-            if (!ok) break;
-            ptx::tc_fence_after();
-            // this half's dP_j into registers, then release its columns
-            uint32_t dp[2][32];
-            ptx::tmem_ld32(tP, dp[0]);
-            ptx::tmem_ld32(tP + 32, dp[1]);
-            ptx::tmem_wait_ld();
-            ptx::tc_fence_before();
-            __syncwarp();
-            if (lane == 0) ptx::mbar_arrive(&dp_free);
-            const uint32_t tS = tbase + (j & 1) * 128 + 64 * half + lane_off;
-#pragma unroll
-            for (int c2 = 0; c2 < 2; ++c2) {
-                uint32_t s[32];
-                ptx::tmem_ld32(tS + 32 * c2, s);
-                ptx::tmem_wait_ld();
-                const int lim = valid - (64 * half + 32 * c2);
-                if (lim < 32) {
-                    // keys past the segment's end: score -inf, probability 0
-#pragma unroll
-                    for (int e = 0; e < 32; ++e)
-                        if (e >= lim) s[e] = 0xff800000u;
-                }
-                uint32_t pk[16];
-#pragma unroll
-                for (int e = 0; e < 16; ++e) {
-                    const uint64_t arg = ptx::f2_fma(
-                        ptx::f2_pack(__uint_as_float(s[2 * e]), __uint_as_float(s[2 * e + 1])), sl2x2, nlx2);
-                    float a0, a1;
-                    ptx::f2_unpack(arg, a0, a1);
-                    const uint64_t pp = ptx::f2_pack(ex2(a0), ex2(a1));
-                    const uint64_t dd = ptx::f2_add(
-                        ptx::f2_pack(__uint_as_float(dp[c2][2 * e]), __uint_as_float(dp[c2][2 * e + 1])), ndlx2);
-                    const uint64_t ds = ptx::f2_mul(pp, dd);
-                    float d0, d1;
-                    ptx::f2_unpack(ds, d0, d1);
-                    pk[e] = ptx::pack_bf16(d0, d1);
-                }
-                ptx::tmem_st16(tS + 16 * c2, pk);
-            }
-            ptx::tmem_wait_st();
-            ptx::tc_fence_before();
-            __syncwarp();
-            if (lane == 0) ptx::mbar_arrive(&ds_full);
-        }
-        if (ok) ok = __all_sync(0xffffffffu, ptx::mbar_wait_bounded(&dq_full, 0, abort_p, p.wait_limit));
-        if (ok) {
-            // each half stores D/2 columns of its row
-            ptx::tc_fence_after();
-            constexpr int DH = D / 2;
-            const uint32_t tQ = tbase + 384 + DH * half + lane_off;
-            __nv_bfloat16* dst = p.dq + (((size_t)b * p.N + (qv ? q : 0)) * p.H + h) * D + DH * half;
-#pragma unroll
-            for (int c = 0; c < DH / 32; ++c) {
-                uint32_t o[32];
-                ptx::tmem_ld32(tQ + 32 * c, o);
-                ptx::tmem_wait_ld();
-                uint32_t pk[16];
-#pragma unroll
-                for (int e = 0; e < 16; ++e)
-                    pk[e] = ptx::pack_bf16(__uint_as_float(o[2 * e]) * p.scale,
-                                           __uint_as_float(o[2 * e + 1]) * p.scale);
-                if (qv) {
-                    uint4* d4 = reinterpret_cast<uint4*>(dst + 32 * c);
-#pragma unroll
-                    for (int e = 0; e < 4; ++e)
-                        d4[e] = make_uint4(pk[4 * e], pk[4 * e + 1], pk[4 * e + 2], pk[4 * e + 3]);
-                }
-            }
-        }
-        if (!ok && lane == 0) atomicOr(p.status, kDevTimeout);
-    }
-
-    ptx::tc_fence_before();
-    __syncthreads();
-    if (warp == 2) {
-        ptx::tc_fence_after();
-        ptx::tmem_dealloc(tbase, 512);
-    }
-}
-
-// ============================================================ dK/dV kernel
-
-template <int D>
-__device__ __forceinline__ void dkdv_item(const BwdMaps& maps, const BwdTcParams& p, int kgi,
-                                          int local) {
-    using C = BCfg<D>;
-    extern __shared__ __align__(1024) unsigned char smem_raw[];
-    unsigned char* smem = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    unsigned char* sK = smem;
-    unsigned char* sV = smem + C::kTile;
-    unsigned char* sQ = smem + 2 * C::kTile;   // [2]
-    unsigned char* sG = smem + 4 * C::kTile;   // [2] dO
-
-    __shared__ uint64_t kv_full, qg_full[2], qg_empty[2], st_full[2], pds_full[2], kv_done, drain_bar;
-    __shared__ uint32_t tmem_base_sh;
-    __shared__ int abort_flag;
-    // per-query statistics of the current and the previous query tile, in
-    // the seventh tile of the dynamic shared memory
-    float(*sL)[kBM] = reinterpret_cast<float(*)[kBM]>(smem + 6 * C::kTile);
-    float(*sD)[kBM] = reinterpret_cast<float(*)[kBM]>(smem + 6 * C::kTile + 2 * kBM * 4);
-
-    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-    const BGroupK& KG = p.kg[kgi];
-    const int kt_all = local % KG.n_kt;
-    const int h = (local / KG.n_kt) % p.H;
-    const int b = local / (KG.n_kt * p.H);
-    int gsi = 0;
-    while (gsi + 1 < KG.n_grad && kt_all >= KG.gr[gsi + 1].kt0) ++gsi;
-    const BGrad& gr = KG.gr[gsi];
-    const int kt = kt_all - gr.kt0;
-    const int key_row = gr.row0 + kt * kBM;
-    const int valid_keys = min(kBM, gr.len - kt * kBM);
-    const int nq = KG.n_qt;
-
-    if (threadIdx.x == 0) {
-        abort_flag = 0;
-        ptx::mbar_init(&kv_full, 1);
-        for (int s = 0; s < 2; ++s) {
-            ptx::mbar_init(&qg_full[s], 1);
-            ptx::mbar_init(&qg_empty[s], 1);
-        }
-        for (int s = 0; s < 2; ++s) {
-            ptx::mbar_init(&st_full[s], 1);
-            ptx::mbar_init(&pds_full[s], 4);  // one arrival per warp of the column half
-        }
-        ptx::mbar_init(&kv_done, 1);
-        ptx::mbar_init(&drain_bar, 1);
-        ptx::fence_mbar_init();
-    }
-    if (warp == 2) {
-        ptx::tmem_alloc(&tmem_base_sh, 512);
-        ptx::tmem_relinquish();
-    }
-    ptx::tc_fence_before();
-    __syncthreads();
-    ptx::tc_fence_after();
-    const uint32_t tbase = tmem_base_sh;
-    volatile int* abort_p = &abort_flag;
-    volatile int never = 0;
-    ptx::grid_dep_wait();
-    ptx::grid_dep_launch();
-
-    if (warp == 0) {
-        // ============================ TMA producer ============================
-        if (lane == 0) {
-            bool ok = true;
-            ptx::mbar_arrive_expect_tx(&kv_full, 2 * C::kTile);
-            load_tile<D>(sK, &maps.k[gr.map], &kv_full, h, key_row, b);
-            load_tile<D>(sV, &maps.v[gr.map], &kv_full, h, key_row, b);
-            int i = 0;
-            for (; i < nq; ++i) {
-                const int st = i & 1;
-                if (!ptx::mbar_wait_bounded(&qg_empty[st], (uint32_t)(((i >> 1) & 1) ^ 1), abort_p,
-                                            p.wait_limit)) {
-                    ok = false;
-                    break;
-                }
-                ptx::mbar_arrive_expect_tx(&qg_full[st], 2 * C::kTile);
-                load_tile<D>(sQ + st * C::kTile, &maps.q, &qg_full[st], h, KG.q_begin + i * kBM, b);
-                load_tile<D>(sG + st * C::kTile, &maps.dout, &qg_full[st], h, KG.q_begin + i * kBM, b);
-            }
-            if (!ok) {
-                ptx::mbar_wait_bounded(&kv_full, 0, &never, kWaitLimit);
-                for (int ii = (i > 2 ? i - 2 : 0); ii < i; ++ii)
-                    ptx::mbar_wait_bounded(&qg_full[ii & 1], (uint32_t)((ii >> 1) & 1), &never, kWaitLimit);
-                atomicOr(p.status, kDevTimeout);
-            }
-        }
-    } else if (warp == 1) {
-        // ============================= MMA issuer =============================
+        constexpr uint32_t idS = ptx::idesc_bf16(kBM, kBM, false, false);
         constexpr uint32_t idO = ptx::idesc_bf16(kBM, D, false, true);
         constexpr uint64_t kTileDesc = (uint64_t)(C::kTile >> 4);
-        const uint64_t k_desc = ptx::sdesc_sw128(ptx::smem_u32(sK), 16, 1024);
-        const uint64_t v_desc = ptx::sdesc_sw128(ptx::smem_u32(sV), 16, 1024);
-        const uint64_t q_desc = ptx::sdesc_sw128(ptx::smem_u32(sQ), 16, 1024);
-        const uint64_t g_desc = ptx::sdesc_sw128(ptx::smem_u32(sG), 16, 1024);
-        const uint64_t qmn_desc = ptx::sdesc_sw128(ptx::smem_u32(sQ), kBM * 128, 1024);
-        const uint64_t gmn_desc = ptx::sdesc_sw128(ptx::smem_u32(sG), kBM * 128, 1024);
-        auto wait_all = [&](uint64_t* bar, uint32_t parity) {
-            const bool r = ptx::mbar_wait_bounded(bar, parity, abort_p, p.wait_limit);
+        const uint64_t desc = ptx::sdesc_sw128(ptx::smem_u32(smem), 16, 1024);          // tile 0, K-major
+        const uint64_t desc_mn = ptx::sdesc_sw128(ptx::smem_u32(smem), kBM * 128, 1024);  // tile 0, MN-major
+        auto wait_all = [&](uint64_t* b, uint32_t parity) {
+            const bool r = ptx::mbar_wait_bounded(b, parity, abort_p, p.wait_limit);
             return __all_sync(0xffffffffu, r);
         };
-        // Query tile i is done in two halves of 64 queries: half A's
-        // dV/dK MMAs and the next tile's S^T/dP^T of half A run while the
-        // softmax works on half B, and the other way round.
-        constexpr uint32_t idS64 = ptx::idesc_bf16(kBM, 64, false, false);
-        auto issue_st = [&](int i, int hf) {  // S^T, dP^T of half hf of query tile i
-            const int st = i & 1;
-            const uint64_t qd = q_desc + (uint64_t)st * kTileDesc + (uint64_t)((64 * 128 * hf) >> 4);
-            const uint64_t gd = g_desc + (uint64_t)st * kTileDesc + (uint64_t)((64 * 128 * hf) >> 4);
+        // D[128 x 128] = tile a x tile b^T
+        auto mma_tiles = [&](uint32_t d, int a, int b) {
+            const uint64_t ad = desc + (uint64_t)a * kTileDesc, bd = desc + (uint64_t)b * kTileDesc;
 #pragma unroll
             for (int kk = 0; kk < D / 16; ++kk)
-                ptx::mma_ss(tbase + 64 * hf, k_desc + kmajor_step(kk), qd + kmajor_step(kk), idS64,
-                            kk > 0 ? 1u : 0u);
-#pragma unroll
-            for (int kk = 0; kk < D / 16; ++kk)
-                ptx::mma_ss(tbase + 128 + 64 * hf, v_desc + kmajor_step(kk), gd + kmajor_step(kk), idS64,
-                            kk > 0 ? 1u : 0u);
-            ptx::mma_commit(&st_full[hf]);
+                ptx::mma_ss(d, ad + kmajor_step(kk), bd + kmajor_step(kk), idS, kk > 0 ? 1u : 0u);
         };
-        auto issue_kv = [&](int i, int hf) {  // dV += P^T dO, dK += dS^T Q over half hf
-            const int st = i & 1;
-            const uint64_t gd = gmn_desc + (uint64_t)st * kTileDesc;
-            const uint64_t qd = qmn_desc + (uint64_t)st * kTileDesc;
+        // D[128 x D] (+)= bf16 tile at TMEM column a (64 columns per half) x tile b
+        auto mma_out = [&](uint32_t d, uint32_t a, int b, bool acc) {
+            const uint64_t bd = desc_mn + (uint64_t)b * kTileDesc;
 #pragma unroll
-            for (int kk = 0; kk < 4; ++kk) {
-                const uint64_t roff = (uint64_t)((4 * hf + kk) * (2048 >> 4));
-                ptx::mma_ts(tbase + 256, tbase + 64 * hf + kk * 8, gd + roff, idO,
-                            (i > 0 || hf > 0 || kk > 0) ? 1u : 0u);
-                ptx::mma_ts(tbase + 256 + D, tbase + 128 + 64 * hf + kk * 8, qd + roff, idO,
-                            (i > 0 || hf > 0 || kk > 0) ? 1u : 0u);
-            }
+            for (int kk = 0; kk < kBM / 16; ++kk)
+                ptx::mma_ts(d, a + 64 * (kk / 4) + (kk % 4) * 8, bd + (uint64_t)(kk * (2048 >> 4)), idO,
+                            (acc || kk > 0) ? 1u : 0u);
         };
-        bool ok = wait_all(&kv_full, 0) && wait_all(&qg_full[0], 0);
-        if (ok) {
-            ptx::tc_fence_after();
-            if (ptx::elect_one_sync()) {
-                issue_st(0, 0);
-                issue_st(0, 1);
+        bool ok = true;
+        int nk = 0, nv = 0, nq = 0, ng = 0;  // ring tiles consumed
+        int tq = 0, tk = 0;                  // tiles done of each kind
+        int iq = 0, ik = 0;                  // items done of each kind
+        for (int k = 0; ok; ++k) {
+            const int idx = round_item(k);
+            if (idx >= p.n_items) break;
+            const BItem it = item_of(p, idx);
+            const int n = it.n;
+            if (it.kind == 0) {
+                auto issue_s = [&](int j) { mma_tiles(tbase + (j & 1) * 128, 0, 2 + (nk + j) % 3); };
+                auto issue_dp = [&](int j) {
+                    const int vs = (nv + j) & 1;
+                    mma_tiles(tbase + 256, 1, 5 + vs);
+                    ptx::mma_commit(&bar.v_empty[vs]);
+                    ptx::mma_commit(&bar.sdp_full);
+                    if (j + 1 == n) ptx::mma_commit(&bar.qg_empty);  // the last S went out before
+                };
+                auto k_full = [&](int j) { return &bar.k_full[(nk + j) % 3]; };
+                auto k_par = [&](int j) { return (uint32_t)(((nk + j) / 3) & 1); };
+                auto v_full = [&](int j) { return &bar.v_full[(nv + j) & 1]; };
+                auto v_par = [&](int j) { return (uint32_t)(((nv + j) >> 1) & 1); };
+                ok = wait_all(&bar.qg_full, (uint32_t)(iq & 1)) && wait_all(k_full(0), k_par(0)) &&
+                     wait_all(v_full(0), v_par(0));
+                if (ok) {
+                    ptx::tc_fence_after();
+                    if (ptx::elect_one_sync()) {
+                        issue_s(0);
+                        issue_dp(0);
+                    }
+                    __syncwarp();
+                    if (n > 1) {
+                        ok = wait_all(k_full(1), k_par(1));
+                        if (ok) {
+                            ptx::tc_fence_after();
+                            if (ptx::elect_one_sync()) issue_s(1);
+                            __syncwarp();
+                        }
+                    }
+                }
+                for (int j = 0; j < n && ok; ++j, ++tq) {
+                    const bool next = j + 1 < n, next2 = j + 2 < n;
+                    const uint32_t par = (uint32_t)(tq & 1);
+                    {
+                        const bool rd = ptx::mbar_try_wait(&bar.dp_free, par);
+                        const bool rv = !next || ptx::mbar_try_wait(v_full(j + 1), v_par(j + 1));
+                        if (!__all_sync(0xffffffffu, rd && rv))
+                            ok = wait_all(&bar.dp_free, par) && (!next || wait_all(v_full(j + 1), v_par(j + 1)));
+                    }
+                    if (!ok) break;
+                    if (next) {
+                        ptx::tc_fence_after();
+                        if (ptx::elect_one_sync()) issue_dp(j + 1);
+                        __syncwarp();
+                    }
+                    // dS_j, and K_{j+2} for the S two tiles ahead; if K has not
+                    // landed yet, dQ_j goes first and S_{j+2} after its own wait.
+                    bool k_ready;
+                    {
+                        const bool rs = ptx::mbar_try_wait(&bar.ds_full, par);
+                        k_ready = !next2 || ptx::mbar_try_wait(k_full(j + 2), k_par(j + 2));
+                        k_ready = __all_sync(0xffffffffu, k_ready);
+                        if (!__all_sync(0xffffffffu, rs)) ok = wait_all(&bar.ds_full, par);
+                    }
+                    if (!ok) break;
+                    ptx::tc_fence_after();
+                    if (ptx::elect_one_sync()) {
+                        const int ks = (nk + j) % 3;
+                        mma_out(tbase + 384, tbase + (j & 1) * 128, 2 + ks, j > 0);
+                        ptx::mma_commit(&bar.k_empty[ks]);
+                        if (!next) ptx::mma_commit(&bar.dq_full);
+                        if (next2 && k_ready) issue_s(j + 2);
+                    }
+                    __syncwarp();
+                    if (next2 && !k_ready) {
+                        ok = wait_all(k_full(j + 2), k_par(j + 2));
+                        if (!ok) break;
+                        ptx::tc_fence_after();
+                        if (ptx::elect_one_sync()) issue_s(j + 2);
+                        __syncwarp();
+                    }
+                }
+                nk += n;
+                nv += n;
+                ++iq;
+            } else {
+                auto q_full = [&](int i) { return &bar.q_full[(nq + i) % 3]; };
+                auto q_par = [&](int i) { return (uint32_t)(((nq + i) / 3) & 1); };
+                auto g_full = [&](int i) { return &bar.g_full[(ng + i) & 1]; };
+                auto g_par = [&](int i) { return (uint32_t)(((ng + i) >> 1) & 1); };
+                auto issue_st = [&](int i) {  // S^T = K Q_i^T
+                    mma_tiles(tbase, 0, 2 + (nq + i) % 3);
+                    ptx::mma_commit(&bar.st_full);
+                    if (i + 1 == n) ptx::mma_commit(&bar.kst_empty);
+                };
+                auto issue_dpt = [&](int i) {  // dP^T = V dO_i^T
+                    mma_tiles(tbase + 128, 1, 5 + ((ng + i) & 1));
+                    ptx::mma_commit(&bar.dpt_full);
+                    if (i + 1 == n) ptx::mma_commit(&bar.vst_empty);
+                };
+                ok = wait_all(&bar.kst_full, (uint32_t)(ik & 1)) && wait_all(q_full(0), q_par(0));
+                if (ok) {
+                    ptx::tc_fence_after();
+                    if (ptx::elect_one_sync()) issue_st(0);
+                    __syncwarp();
+                    ok = wait_all(&bar.vst_full, (uint32_t)(ik & 1)) && wait_all(g_full(0), g_par(0));
+                }
+                if (ok) {
+                    ptx::tc_fence_after();
+                    if (ptx::elect_one_sync()) issue_dpt(0);
+                    __syncwarp();
+                }
+                for (int i = 0; i < n && ok; ++i, ++tk) {
+                    const bool next = i + 1 < n;
+                    const uint32_t par = (uint32_t)(tk & 1);
+                    // P^T_i and the next Q: dV_i, S^T_{i+1}
+                    bool ready;
+                    {
+                        const bool rp = ptx::mbar_try_wait(&bar.p_full, par);
+                        ready = !next || ptx::mbar_try_wait(q_full(i + 1), q_par(i + 1));
+                        ready = __all_sync(0xffffffffu, ready);
+                        if (!__all_sync(0xffffffffu, rp)) ok = wait_all(&bar.p_full, par);
+                    }
+                    if (!ok) break;
+                    ptx::tc_fence_after();
+                    if (ptx::elect_one_sync()) {
+                        const int gs = (ng + i) & 1;
+                        mma_out(tbase + 256, tbase, 5 + gs, i > 0);
+                        ptx::mma_commit(&bar.g_empty[gs]);  // dP^T_i went out before
+                        if (next && ready) issue_st(i + 1);
+                    }
+                    __syncwarp();
+                    if (next && !ready) {
+                        ok = wait_all(q_full(i + 1), q_par(i + 1));
+                        if (!ok) break;
+                        ptx::tc_fence_after();
+                        if (ptx::elect_one_sync()) issue_st(i + 1);
+                        __syncwarp();
+                    }
+                    // dS^T_i and the next dO: dK_i, dP^T_{i+1}
+                    {
+                        const bool rs = ptx::mbar_try_wait(&bar.dst_full, par);
+                        ready = !next || ptx::mbar_try_wait(g_full(i + 1), g_par(i + 1));
+                        ready = __all_sync(0xffffffffu, ready);
+                        if (!__all_sync(0xffffffffu, rs)) ok = wait_all(&bar.dst_full, par);
+                    }
+                    if (!ok) break;
+                    ptx::tc_fence_after();
+                    if (ptx::elect_one_sync()) {
+                        const int qs = (nq + i) % 3;
+                        mma_out(tbase + 256 + D, tbase + 128, 2 + qs, i > 0);
+                        ptx::mma_commit(&bar.q_empty[qs]);
+                        if (!next)
+                            ptx::mma_commit(&bar.kv_full);
+                        else if (ready)
+                            issue_dpt(i + 1);
+                    }
+                    __syncwarp();
+                    if (next && !ready) {
+                        ok = wait_all(g_full(i + 1), g_par(i + 1));
+                        if (!ok) break;
+                        ptx::tc_fence_after();
+                        if (ptx::elect_one_sync()) issue_dpt(i + 1);
+                        __syncwarp();
+                    }
+                }
+                nq += n;
+                ng += n;
+                ++ik;
             }
-            __syncwarp();
-        }
-        for (int i = 0; i < nq && ok; ++i) {
-            const int st = i & 1;
-            const bool more = i + 1 < nq;
-            // P/dS of half 0 and the next query tile's Q/dO, probed together
-            // (each barrier check of this thread is pipe time); if Q/dO has
-            // not landed, half 0's dV/dK go first.
-            bool q_ready;
-            {
-                const bool rp = ptx::mbar_try_wait(&pds_full[0], (uint32_t)(i & 1));
-                q_ready = !more || ptx::mbar_try_wait(&qg_full[st ^ 1], (uint32_t)(((i + 1) >> 1) & 1));
-                q_ready = __all_sync(0xffffffffu, q_ready);
-                if (!__all_sync(0xffffffffu, rp)) ok = wait_all(&pds_full[0], (uint32_t)(i & 1));
-            }
-            if (!ok) break;
-            ptx::tc_fence_after();
-            if (ptx::elect_one_sync()) {
-                issue_kv(i, 0);
-                if (more && q_ready) issue_st(i + 1, 0);
-            }
-            __syncwarp();
-            if (more && !q_ready) {
-                ok = wait_all(&qg_full[st ^ 1], (uint32_t)(((i + 1) >> 1) & 1));
-                if (!ok) break;
-                ptx::tc_fence_after();
-                if (ptx::elect_one_sync()) issue_st(i + 1, 0);
-                __syncwarp();
-            }
-            ok = wait_all(&pds_full[1], (uint32_t)(i & 1));
-            if (!ok) break;
-            ptx::tc_fence_after();
-            if (ptx::elect_one_sync()) {
-                issue_kv(i, 1);
-                ptx::mma_commit(&qg_empty[st]);
-                if (more)
-                    issue_st(i + 1, 1);
-                else
-                    ptx::mma_commit(&kv_done);
-            }
-            __syncwarp();
         }
         if (!ok) {
-            if (ptx::elect_one_sync()) ptx::mma_commit(&drain_bar);
+            if (ptx::elect_one_sync()) ptx::mma_commit(&bar.drain);
             __syncwarp();
-            ptx::mbar_wait_bounded(&drain_bar, 0, &never, kWaitLimit);
+            ptx::mbar_wait_bounded(&bar.drain, 0, &never, kWaitLimit);
             if (lane == 0) atomicOr(p.status, kDevTimeout);
         }
     } else if (warp >= 4) {
-        // ============= softmax: one thread per key row and column half =============
+        // ============== softmax: one thread per own row and column half ==============
         const int half = (warp - 4) / 4;
         const int wq = warp % 4;
         const int r = wq * 32 + lane;
-        const int tix = (warp - 4) * 32 + lane;  // 0..255
         const uint32_t lane_off = (uint32_t)(wq * 32) << 16;
-        const uint32_t tS = tbase + 64 * half + lane_off, tP = tbase + 128 + 64 * half + lane_off;
+        constexpr int DH = D / 2;  // output columns of this thread
         const uint64_t sl2x2 = ptx::f2_pack(p.scale_log2, p.scale_log2);
         bool ok = true;
-        for (int i = 0; i < nq && ok; ++i) {
-            // this half's 64 per-query statistics, shared by its 128 key rows:
-            // threads 0-63 of the half load -lse (log2 units), 64-127 -delta
-            {
-                const int hix = tix & 127;
-                const int qq = 64 * half + (hix & 63);
-                const int q = KG.q_begin + i * kBM + qq;
-                const bool qv = q < KG.q_end;
-                const size_t rix = ((size_t)b * p.H + h) * p.N + (qv ? q : 0);
-                if (hix < 64)
-                    sL[i & 1][qq] = qv ? -p.lse[rix] * kLog2e : -INFINITY;
-                else
-                    sD[i & 1][qq] = qv ? -p.delta[rix] : 0.f;
-            }
-            ptx::named_bar_sync(1 + half, 128);
-            const float* L = sL[i & 1] + 64 * half;
-            const float* ND = sD[i & 1] + 64 * half;
-            ok = __all_sync(0xffffffffu, ptx::mbar_wait_bounded(&st_full[half], (uint32_t)(i & 1), abort_p,
-                                                                p.wait_limit));
-            if (!ok) break;
-            ptx::tc_fence_after();
-#pragma unroll
-            for (int c2 = 0; c2 < 2; ++c2) {
-                uint32_t s[32], dp[32];
-                ptx::tmem_ld32(tS + 32 * c2, s);
-                ptx::tmem_ld32(tP + 32 * c2, dp);
-                ptx::tmem_wait_ld();
-                uint32_t pp[16], pd[16];
-#pragma unroll
-                for (int e = 0; e < 16; ++e) {
-                    const int c0 = 32 * c2 + 2 * e;
-                    const uint64_t arg = ptx::f2_fma(
-                        ptx::f2_pack(__uint_as_float(s[2 * e]), __uint_as_float(s[2 * e + 1])), sl2x2,
-                        ptx::f2_pack(L[c0], L[c0 + 1]));
-                    float a0, a1;
-                    ptx::f2_unpack(arg, a0, a1);
-                    const float p0 = ex2(a0), p1 = ex2(a1);
-                    pp[e] = ptx::pack_bf16(p0, p1);
-                    const uint64_t dd = ptx::f2_add(
-                        ptx::f2_pack(__uint_as_float(dp[2 * e]), __uint_as_float(dp[2 * e + 1])),
-                        ptx::f2_pack(ND[c0], ND[c0 + 1]));
-                    float d0, d1;
-                    ptx::f2_unpack(ptx::f2_mul(ptx::f2_pack(p0, p1), dd), d0, d1);
-                    pd[e] = ptx::pack_bf16(d0, d1);
-                }
-                ptx::tmem_st16(tS + 16 * c2, pp);
-                ptx::tmem_st16(tP + 16 * c2, pd);
-            }
-            ptx::tmem_wait_st();
-            ptx::tc_fence_before();
+        auto wait_all = [&](uint64_t* b, uint32_t parity) {
+            return (bool)__all_sync(0xffffffffu, ptx::mbar_wait_bounded(b, parity, abort_p, p.wait_limit));
+        };
+        auto arrive = [&](uint64_t* b) {
             __syncwarp();
-            if (lane == 0) ptx::mbar_arrive(&pds_full[half]);
-        }
-        if (ok) ok = __all_sync(0xffffffffu, ptx::mbar_wait_bounded(&kv_done, 0, abort_p, p.wait_limit));
-        if (ok) {
-            // Every MMA has completed: the Q/dO ring is free and stages one
-            // fp32 [128][D + 4] tile (dK, then dV); each half fills D/2
-            // columns of its rows, then every warp stores whole rows.
-            ptx::tc_fence_after();
-            float* stage = reinterpret_cast<float*>(sQ);
-            constexpr int kStride = D + 4;
-            constexpr int E = D / 32;
-            constexpr int DH = D / 2;
-            for (int which = 0; which < 2; ++which) {
-                const float mul = which == 0 ? p.scale : 1.f;
+            if (lane == 0) ptx::mbar_arrive(b);
+        };
+        int tq = 0, tk = 0, iq = 0, ik = 0;
+        for (int k = 0; ok; ++k) {
+            const int idx = round_item(k);
+            if (idx >= p.n_items) break;
+            const BItem it = item_of(p, idx);
+            const int n = it.n;
+            const size_t head = ((size_t)it.b * p.H + it.h) * p.N;  // row of lse and delta
+            if (it.kind == 0) {
+                const BGroupQ& G = p.g[it.gi];
+                const uint32_t tP = tbase + 256 + 64 * half + lane_off;
+                const int q = it.row0 + r;
+                const bool qv = r < it.rows;
+                const float nl = qv ? -p.lse[head + q] * kLog2e : -INFINITY;  // -lse in log2 units
+                const float dl = qv ? p.delta[head + q] : 0.f;
+                const uint64_t nlx2 = ptx::f2_pack(nl, nl), ndlx2 = ptx::f2_pack(-dl, -dl);
+                for (int j = 0; j < n; ++j, ++tq) {
+                    int map, row, valid;
+                    kv_tile(G, j, map, row, valid);
+                    ok = wait_all(&bar.sdp_full, (uint32_t)(tq & 1));
+                    if (!ok) break;
+                    ptx::tc_fence_after();
+                    // this half's dP_j into registers, then release its columns
+                    uint32_t dp[2][32];
+                    ptx::tmem_ld32(tP, dp[0]);
+                    ptx::tmem_ld32(tP + 32, dp[1]);
+                    ptx::tmem_wait_ld();
+                    ptx::tc_fence_before();
+                    arrive(&bar.dp_free);
+                    const uint32_t tS = tbase + (j & 1) * 128 + 64 * half + lane_off;
+#pragma unroll
+                    for (int c2 = 0; c2 < 2; ++c2) {
+                        uint32_t s[32];
+                        ptx::tmem_ld32(tS + 32 * c2, s);
+                        ptx::tmem_wait_ld();
+                        const int lim = valid - (64 * half + 32 * c2);
+                        if (lim < 32) {
+                            // keys past the segment's end: score -inf, probability 0
+#pragma unroll
+                            for (int e = 0; e < 32; ++e)
+                                if (e >= lim) s[e] = 0xff800000u;
+                        }
+                        uint32_t pk[16];
+#pragma unroll
+                        for (int e = 0; e < 16; ++e) {
+                            const uint64_t arg = ptx::f2_fma(
+                                ptx::f2_pack(__uint_as_float(s[2 * e]), __uint_as_float(s[2 * e + 1])), sl2x2, nlx2);
+                            float a0, a1;
+                            ptx::f2_unpack(arg, a0, a1);
+                            const uint64_t pp = ptx::f2_pack(ex2(a0), ex2(a1));
+                            const uint64_t dd = ptx::f2_add(
+                                ptx::f2_pack(__uint_as_float(dp[c2][2 * e]), __uint_as_float(dp[c2][2 * e + 1])),
+                                ndlx2);
+                            const uint64_t ds = ptx::f2_mul(pp, dd);
+                            float d0, d1;
+                            ptx::f2_unpack(ds, d0, d1);
+                            pk[e] = ptx::pack_bf16(d0, d1);
+                        }
+                        ptx::tmem_st16(tS + 16 * c2, pk);
+                    }
+                    ptx::tmem_wait_st();
+                    ptx::tc_fence_before();
+                    arrive(&bar.ds_full);
+                }
+                ok = ok && wait_all(&bar.dq_full, (uint32_t)(iq & 1));
+                if (!ok) break;
+                ++iq;
+                // each half stores D/2 columns of its row
+                ptx::tc_fence_after();
+                const uint32_t tQ = tbase + 384 + DH * half + lane_off;
+                __nv_bfloat16* dst = p.dq + (((size_t)it.b * p.N + (qv ? q : 0)) * p.H + it.h) * D + DH * half;
+                uint32_t o[DH / 32][32];
+#pragma unroll
+                for (int c = 0; c < DH / 32; ++c) ptx::tmem_ld32(tQ + 32 * c, o[c]);
+                ptx::tmem_wait_ld();
 #pragma unroll
                 for (int c = 0; c < DH / 32; ++c) {
-                    uint32_t o[32];
-                    ptx::tmem_ld32(tbase + 256 + (which == 0 ? D : 0) + DH * half + 32 * c + lane_off, o);
-                    ptx::tmem_wait_ld();
-                    float4* dst = reinterpret_cast<float4*>(stage + r * kStride + DH * half + 32 * c);
+                    uint32_t pk[16];
 #pragma unroll
-                    for (int e = 0; e < 8; ++e)
-                        dst[e] = make_float4(__uint_as_float(o[4 * e]) * mul, __uint_as_float(o[4 * e + 1]) * mul,
-                                             __uint_as_float(o[4 * e + 2]) * mul,
-                                             __uint_as_float(o[4 * e + 3]) * mul);
+                    for (int e = 0; e < 16; ++e)
+                        pk[e] = ptx::pack_bf16(__uint_as_float(o[c][2 * e]) * p.scale,
+                                               __uint_as_float(o[c][2 * e + 1]) * p.scale);
+                    if (qv && p.dq_v8) {
+                        ptx::st_global_v8(dst + 32 * c, pk);
+                        ptx::st_global_v8(dst + 32 * c + 16, pk + 8);
+                    } else if (qv) {
+                        uint4* d4 = reinterpret_cast<uint4*>(dst + 32 * c);
+#pragma unroll
+                        for (int e = 0; e < 4; ++e)
+                            d4[e] = make_uint4(pk[4 * e], pk[4 * e + 1], pk[4 * e + 2], pk[4 * e + 3]);
+                    }
                 }
-                ptx::named_bar_sync(3, 256);
-                float* base = (which == 0 ? p.dk_ctx : p.dv_ctx);
-                for (int rr = warp - 4; rr < valid_keys; rr += 8) {
-                    const size_t o = (((size_t)b * p.R + gr.crow0 + kt * kBM + rr) * p.H + h) * D + E * lane;
-                    const float* src = stage + rr * kStride + E * lane;
-                    if (E == 4)
-                        *reinterpret_cast<float4*>(base + o) = *reinterpret_cast<const float4*>(src);
-                    else
-                        *reinterpret_cast<float2*>(base + o) = *reinterpret_cast<const float2*>(src);
+            } else {
+                const BGroupK& K = p.kg[it.gi];
+                const uint32_t tS = tbase + 64 * half + lane_off, tP = tbase + 128 + 64 * half + lane_off;
+                float* stats = reinterpret_cast<float*>(smem + C::kStats) + 128 * half;
+                for (int i = 0; i < n; ++i, ++tk) {
+                    const uint32_t par = (uint32_t)(tk & 1);
+                    // This half's 64 per-query statistics, shared by its 128 key
+                    // rows: threads 0-63 of the half load -lse (log2 units),
+                    // 64-127 -delta, into the buffer of the tile's parity.
+                    float* L = stats + 256 * par;
+                    {
+                        const int q = K.q_begin + i * kBM + 64 * half + (r & 63);
+                        const bool qv = q < K.q_end;
+                        if (r < 64)
+                            L[r] = qv ? -p.lse[head + q] * kLog2e : -INFINITY;
+                        else
+                            L[r] = qv ? -p.delta[head + q] : 0.f;
+                    }
+                    arrive(&bar.meet[half]);
+                    ok = wait_all(&bar.meet[half], par) && wait_all(&bar.st_full, par);
+                    if (!ok) break;
+                    ptx::tc_fence_after();
+                    uint64_t pf[32];  // P^T, fp32 pairs
+#pragma unroll
+                    for (int c2 = 0; c2 < 2; ++c2) {
+                        uint32_t s[32], pk[16];
+                        ptx::tmem_ld32(tS + 32 * c2, s);
+                        ptx::tmem_wait_ld();
+#pragma unroll
+                        for (int e = 0; e < 16; ++e) {
+                            const float2 l2 = *reinterpret_cast<const float2*>(L + 32 * c2 + 2 * e);
+                            const uint64_t arg = ptx::f2_fma(
+                                ptx::f2_pack(__uint_as_float(s[2 * e]), __uint_as_float(s[2 * e + 1])), sl2x2,
+                                ptx::f2_pack(l2.x, l2.y));
+                            float a0, a1;
+                            ptx::f2_unpack(arg, a0, a1);
+                            const float p0 = ex2(a0), p1 = ex2(a1);
+                            pf[16 * c2 + e] = ptx::f2_pack(p0, p1);
+                            pk[e] = ptx::pack_bf16(p0, p1);
+                        }
+                        ptx::tmem_st16(tS + 16 * c2, pk);
+                    }
+                    ptx::tmem_wait_st();
+                    ptx::tc_fence_before();
+                    arrive(&bar.p_full);
+                    ok = wait_all(&bar.dpt_full, par);
+                    if (!ok) break;
+                    ptx::tc_fence_after();
+#pragma unroll
+                    for (int c2 = 0; c2 < 2; ++c2) {
+                        uint32_t dp[32], pk[16];
+                        ptx::tmem_ld32(tP + 32 * c2, dp);
+                        ptx::tmem_wait_ld();
+#pragma unroll
+                        for (int e = 0; e < 16; ++e) {
+                            const float2 d2 = *reinterpret_cast<const float2*>(L + 64 + 32 * c2 + 2 * e);
+                            const uint64_t dd = ptx::f2_add(
+                                ptx::f2_pack(__uint_as_float(dp[2 * e]), __uint_as_float(dp[2 * e + 1])),
+                                ptx::f2_pack(d2.x, d2.y));
+                            float d0, d1;
+                            ptx::f2_unpack(ptx::f2_mul(pf[16 * c2 + e], dd), d0, d1);
+                            pk[e] = ptx::pack_bf16(d0, d1);
+                        }
+                        ptx::tmem_st16(tP + 16 * c2, pk);
+                    }
+                    ptx::tmem_wait_st();
+                    ptx::tc_fence_before();
+                    arrive(&bar.dst_full);
                 }
-                ptx::named_bar_sync(3, 256);
+                ok = ok && wait_all(&bar.kv_full, (uint32_t)(ik & 1));
+                if (!ok) break;
+                ++ik;
+                // each half stores D/2 columns of its dK and dV rows
+                ptx::tc_fence_after();
+                const size_t off = (((size_t)it.b * p.R + it.crow + r) * p.H + it.h) * D + DH * half;
+                const bool rv = r < it.rows;
+#pragma unroll
+                for (int which = 0; which < 2; ++which) {
+                    float* dst = (which == 0 ? p.dv_ctx : p.dk_ctx) + off;
+                    const float mul = which == 0 ? 1.f : p.scale;
+                    uint32_t o[DH / 32][32];
+#pragma unroll
+                    for (int c = 0; c < DH / 32; ++c)
+                        ptx::tmem_ld32(tbase + 256 + which * D + DH * half + 32 * c + lane_off, o[c]);
+                    ptx::tmem_wait_ld();
+                    if (rv) {
+#pragma unroll
+                        for (int c = 0; c < DH / 32; ++c) store_f32(dst + 32 * c, o[c], mul, p.ctx_v8 != 0);
+                    }
+                }
             }
+            // the item's accumulators are read: the next item's MMAs may
+            // overwrite them (its first P or dS is written after this)
+            ptx::tc_fence_before();
+            arrive(&bar.item_done);
         }
         if (!ok && lane == 0) atomicOr(p.status, kDevTimeout);
     }
@@ -751,20 +798,6 @@ __device__ __forceinline__ void dkdv_item(const BwdMaps& maps, const BwdTcParams
         ptx::tc_fence_after();
         ptx::tmem_dealloc(tbase, 512);
     }
-}
-
-// One launch for both kinds of work, so that short dK/dV items fill the
-// SMs that long dq items leave idle at the end.
-template <int D>
-__global__ void __launch_bounds__(kThreads, 1)
-    bwd_tc_kernel(const __grid_constant__ BwdMaps maps, const __grid_constant__ BwdTcParams p) {
-    int r = 0;
-    while (r + 1 < p.n_ranges && (int)blockIdx.x >= p.range[r + 1].base) ++r;
-    const int local = (int)blockIdx.x - p.range[r].base;
-    if (p.range[r].kind == 0)
-        dq_item<D>(maps, p, p.range[r].group, local);
-    else
-        dkdv_item<D>(maps, p, p.range[r].group, local);
 }
 
 bool encode_all(BwdMaps& m, const Plan& P, const BwdTcInput& in) {
@@ -932,19 +965,31 @@ msf_status launch_bwd_tc(msf_plan_t plan, const BwdTcInput& in, cudaStream_t st)
         total += rs[i].count;
     }
     tp.n_ranges = nr;
+    tp.n_items = total;
     (void)items;
     (void)kitems;
     if (total == 0) return MSF_OK;
-    const bool d128 = P.D == 128;
-    const int smem = d128 ? QCfg<128>::kSmem : QCfg<64>::kSmem;
-    cudaError_t e = d128 ? set_smem_attr((const void*)bwd_tc_kernel<128>, QCfg<128>::kSmem)
-                         : set_smem_attr((const void*)bwd_tc_kernel<64>, QCfg<64>::kSmem);
+    // Rows of one head are a multiple of 32 bytes, so the bases decide.
+    tp.dq_v8 = (uintptr_t)in.dq % 32 == 0;
+    tp.ctx_v8 = (uintptr_t)in.dk_ctx % 32 == 0 && (uintptr_t)in.dv_ctx % 32 == 0;
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) {
         set_cuda_error((int)e);
         return MSF_ERR_CUDA;
     }
-    e = d128 ? launch_pdl(bwd_tc_kernel<128>, dim3((unsigned)total), dim3(kThreads), smem, st, maps, tp)
-             : launch_pdl(bwd_tc_kernel<64>, dim3((unsigned)total), dim3(kThreads), smem, st, maps, tp);
+    const int grid = total < sms ? total : sms;
+    const bool d128 = P.D == 128;
+    const int smem = d128 ? BCfg<128>::kSmem : BCfg<64>::kSmem;
+    e = d128 ? set_smem_attr((const void*)bwd_tc_kernel<128>, BCfg<128>::kSmem)
+             : set_smem_attr((const void*)bwd_tc_kernel<64>, BCfg<64>::kSmem);
+    if (e != cudaSuccess) {
+        set_cuda_error((int)e);
+        return MSF_ERR_CUDA;
+    }
+    e = d128 ? launch_pdl(bwd_tc_kernel<128>, dim3((unsigned)grid), dim3(kThreads), smem, st, maps, tp)
+             : launch_pdl(bwd_tc_kernel<64>, dim3((unsigned)grid), dim3(kThreads), smem, st, maps, tp);
     if (e != cudaSuccess) {
         set_cuda_error((int)e);
         return MSF_ERR_CUDA;
