@@ -322,7 +322,9 @@ msf_status msf_mssa_forward(msf_plan_t plan, const void* q, const void* k_win, c
  * segment; with fused_append also the history ring, which holds the staged
  * head) waits (bounded) until every CTA's share is written; the pyramid, the
  * staged head and out are
- * exactly those of the two calls. fp32 plans run the two calls. flags:
+ * exactly those of the two calls. fp32 plans and small calls (those whose
+ * attention gives every 128-row query tile its own thread-block cluster) run
+ * the two calls. flags:
  * MSF_RESAMPLE_FULL or MSF_RESAMPLE_WINDOW_ONLY. Errors: INVALID_ARG,
  * UNSUPPORTED (more pooling jobs than one launch takes), STATE (not bound),
  * CUDA; a wait that gives up raises TIMEOUT in the device status. */

@@ -1,6 +1,7 @@
 // MSSA attention on the sm_103a tensor cores (Eq. 4 context, bf16 operands,
 // fp32 online softmax and accumulation).
 //
+// Calls with few query tiles go to the small-call kernel (attn_small_tc.cu).
 // Work: an item is one 256-row query block (two 128-row tiles Q0, Q1) of one
 // (stream, head, query group); it walks that group's context segments (sink,
 // history or pyramid part, window suffix) in 128-row K/V tiles. All items'
@@ -42,6 +43,7 @@
 #include <stdlib.h>
 #include <string.h>
 
+#include "attn_small_tc.h"
 #include "attn_tc.h"
 #include "pool.cuh"
 #include "ptx.cuh"
@@ -77,23 +79,6 @@ constexpr int kMergeBatch = 8;
 // 128-row K/V step costs), and at least the per-wait bound.
 constexpr long long kHelperCyclesPerTile = 1LL << 20;
 
-struct TcSeg {
-    int map;
-    int row0;
-    int len;
-    int tile0;  // first tile of this segment in the item's tile sequence
-};
-struct TcGroup {
-    int q_begin, q_end;
-    int n_qb;        // 256-row query blocks
-    int n_items;     // B * H * n_qb
-    int n_seg;
-    int n_tiles;     // tiles per item
-    int n_virt;      // item stride in the tile sequence: n_tiles + lead tiles
-    long long tile_base;  // first tile of this group in the global sequence
-    int item_base;        // first item index of this group (merge counters)
-    TcSeg seg[kMaxSeg];
-};
 struct TcParams {
     int H, B;
     float scale_log2;
@@ -122,12 +107,6 @@ struct TcParams {
     int pool_ring;  // the batch also writes the history ring (the staged head)
     unsigned int* pyr_sync;
 };
-struct TcMaps {
-    CUtensorMap q;
-    CUtensorMap k[kNumMaps];
-    CUtensorMap v[kNumMaps];
-};
-
 template <int D>
 struct Cfg {
     static constexpr int kChunks = D / 64;                    // 128-byte swizzle chunks per row
@@ -1289,6 +1268,16 @@ msf_status launch_attn_tc(msf_plan_t plan, const AttnArgs& a, cudaStream_t st, c
     tp.total_tiles = total_tiles;
     if (total_tiles == 0) return MSF_OK;
     if (item_base > P.attn_items) return MSF_ERR_STATE;
+    // Small calls: one 128-row query tile per cluster (after the pyramid, if
+    // the launch was to build it).
+    const int cluster = attn_small_cluster(tp.g, tp.n_groups, P.H, P.B, P.D, cache.num_sms);
+    if (cluster > 0) {
+        e = pool ? launch_pool(*pool, P.B, true, st) : cudaSuccess;
+        if (e == cudaSuccess) e = launch_attn_small(cache.maps, tp.g, tp.n_groups, P, a, cluster, st);
+        if (e == cudaSuccess) return MSF_OK;
+        set_cuda_error((int)e);
+        return MSF_ERR_CUDA;
+    }
     long long ncta = cache.num_sms;
     if (ncta > P.attn_max_ctas) ncta = P.attn_max_ctas;
     if (ncta > total_tiles) ncta = total_tiles;

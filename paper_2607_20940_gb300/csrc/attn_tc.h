@@ -16,6 +16,31 @@ enum : int { kMapSink = 0, kMapHist = 1, kMapWin = 2, kMapPyr0 = 3 };
 constexpr int kMapPyr = -1;
 constexpr int kNumMaps = kMapPyr0 + MSF_MAX_GROUPS;
 
+// What the attention kernels know of a query group: its context as 128-row
+// tiles of up to three segments.
+struct TcSeg {
+    int map;
+    int row0;
+    int len;
+    int tile0;  // first tile of this segment in the item's tile sequence
+};
+struct TcGroup {
+    int q_begin, q_end;
+    int n_qb;        // 256-row query blocks
+    int n_items;     // B * H * n_qb
+    int n_seg;
+    int n_tiles;     // tiles per item
+    int n_virt;      // item stride in the tile sequence: n_tiles + lead tiles
+    long long tile_base;  // first tile of this group in the global sequence
+    int item_base;        // first item index of this group (merge counters)
+    TcSeg seg[kMaxSeg];
+};
+struct TcMaps {
+    CUtensorMap q;
+    CUtensorMap k[kNumMaps];
+    CUtensorMap v[kNumMaps];
+};
+
 // With `pool` (bf16 jobs), the launch also builds that K/V pyramid: every CTA
 // pools a share of it first, and tiles of pyramid segments wait until all
 // shares are written.
