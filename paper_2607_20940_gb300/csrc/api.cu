@@ -10,6 +10,7 @@
 #include "attn_bwd_tc.h"
 #include "attn_f32_tc.h"
 #include "attn_tc.h"
+#include "gemm_f32_tc.h"
 #include "gemm_tc.h"
 #include "msp_tc.h"
 #include "internal.h"
@@ -713,14 +714,21 @@ extern "C" msf_status msf_patchify(msf_plan_t plan, const void* latent, const vo
             return MSF_OK;
         }
     }
-    for (int l = 0; l < p.T; ++l) {
-        const int P = p.d.patch * p.d.scales[l];
+    // One problem per run of consecutive states that share a tier: their raw
+    // blocks and output rows are contiguous.
+    msf::GemmArgs runs[MSF_MAX_STATES];
+    int n_runs = 0;
+    bool f32_tc = !bf16;
+    for (int l0 = 0; l0 < p.T;) {
+        int l1 = l0 + 1;
+        while (l1 < p.T && p.d.scales[l1] == p.d.scales[l0] && w_tier[l1] == w_tier[l0]) ++l1;
+        const int P = p.d.patch * p.d.scales[l0];
         const int F = sh.C * P * P;
-        msf::GemmArgs g;
-        g.A = raw + (size_t)l * per * p.elem;
-        g.B = w_tier[l];
-        g.C = (char*)tokens + (size_t)p.st_off[l] * E * p.elem;
-        g.M = p.st_n[l];
+        msf::GemmArgs& g = runs[n_runs++];
+        g.A = raw + (size_t)l0 * per * p.elem;
+        g.B = w_tier[l0];
+        g.C = (char*)tokens + (size_t)p.st_off[l0] * E * p.elem;
+        g.M = p.st_off[l1 - 1] + p.st_n[l1 - 1] - p.st_off[l0];
         g.N = E;
         g.K = F;
         g.lda = F;
@@ -728,7 +736,12 @@ extern "C" msf_status msf_patchify(msf_plan_t plan, const void* latent, const vo
         g.ldc = E;
         g.a_bstride = (long long)p.T * per;
         g.c_bstride = (long long)p.N * E;
-        e = msf::launch_gemm_nt_simt(g, p.B, bf16, s);
+        f32_tc = f32_tc && msf::gemm_f32_tc_supported(g);
+        l0 = l1;
+    }
+    if (f32_tc) return cuda_status(msf::launch_gemm_f32_tc(runs, n_runs, p.B, msf::status_word(p), s));
+    for (int i = 0; i < n_runs; ++i) {
+        e = msf::launch_gemm_nt_simt(runs[i], p.B, bf16, s);
         if (e != cudaSuccess) return cuda_status(e);
     }
     return MSF_OK;
@@ -869,6 +882,11 @@ extern "C" msf_status msf_unpatchify(msf_plan_t plan, int32_t position, const vo
     g.ldc = F;
     g.a_bstride = (long long)p.N * E;
     g.c_bstride = per;
+    if (!bf16 && msf::gemm_f32_tc_supported(g)) {
+        // straight into the latent
+        g.C = latent_out;
+        return cuda_status(msf::launch_gemm_f32_tc(&g, 1, p.B, msf::status_word(p), s, &sh, P));
+    }
     cudaError_t e = msf::launch_gemm_nt_simt(g, p.B, bf16, s);
     if (e != cudaSuccess) return cuda_status(e);
     return cuda_status(msf::launch_unpatchify_raw(raw, latent_out, sh, position, per, 0, p.B, bf16, s));

@@ -1,7 +1,7 @@
 // Bandwidth-bound kernels of the window pass:
 //   - KV pyramid pooling (Eq. 4's Subsample), also used by the history append
 //   - MSP raw patchify / unpatchify (Sec. 4.1 token rearrangement)
-//   - a CUDA-core GEMM for the tier projections of fp32 plans
+//   - a CUDA-core GEMM for tier projections that no tensor-core kernel takes
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 

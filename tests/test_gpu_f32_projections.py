@@ -1,0 +1,88 @@
+"""fp32 patch embedding and de-embedding on the tensor cores: tile edges, K
+chunk remainders, cluster splits, shared and separate tier weights, streams,
+chunks of frames, and operands the bf16 planes cannot hold.
+
+Tolerance against fp64: products are exact to 2^-24 of themselves and sums of K
+unit-variance terms (weights N(0, 1/K)) round to a few 2^-24 of values up to
+~5: 5e-6 covers the worst element.
+"""
+import pytest
+import torch
+
+from helpers import F32, msf
+from paper_2607_20940_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+
+#        scales      grid      E    C  patch batch frames
+SHAPES = [
+    ((1,), (1, 1), 64, 16, 2, 1, 1),        # one token, one K chunk
+    ((1, 2), (6, 22), 192, 3, 2, 2, 1),     # K = 12 and 48: part of a chunk; N a tile and a half
+    ((1, 1, 2, 2, 4), (16, 24), 200, 16, 2, 1, 1),  # N not a tile's multiple, runs of states, K = 1024
+    ((2, 2, 4), (12, 20), 1536, 16, 2, 1, 2),       # coarse only, frames per state
+    ((1, 2, 2), (30, 52), 1536, 16, 2, 2, 1),       # several tiles each way, two streams
+    ((1, 1), (10, 13), 4100, 16, 1, 1, 1),          # de-embedding: 64 tokens' K remainder, N = 16
+]
+
+
+def _run(shape, edit=None):
+    scales, (gh, gw), E, C, patch, B, F = shape
+    w = synth.Workload("p", len(scales), scales, gh, gw, 1, 64, 0, 0, 0, B, 70, latent_channels=C, patch=patch,
+                       embed_dim=E, frames=F)
+    m = msf()
+    plan = m.Plan(m.make_desc(scales, gh, gw, 1, 64, 0, 0, batch=B, dtype=m.MSF_DTYPE_F32, latent_channels=C,
+                              patch=patch, embed_dim=E, frames_per_state=F))
+    ws = plan.workspace()
+    plan.bind(ws, None, None, None, None)
+    g = torch.Generator().manual_seed(7)
+    lat = torch.randn(B, len(scales), C, F, gh * patch, gw * patch, generator=g)
+    wt = {s: torch.randn(E, C * (patch * s) ** 2, generator=g) * (C * (patch * s) ** 2) ** -0.5 for s in set(scales)}
+    wo = {s: torch.randn(C * (patch * s) ** 2, E, generator=g) * E ** -0.5 for s in set(scales)}
+    N = plan.info.n_tokens
+    h = torch.randn(B, N, E, generator=g)
+    if edit:
+        edit(lat, wt, h, wo)
+    dev = {s: v.cuda() for s, v in wt.items()}
+    tok = torch.full((B, N, E), float("nan"), device="cuda")
+    plan.patchify(lat.cuda(), [dev[s] for s in scales], tok)
+    back, hd = [], h.cuda()
+    for l, s in enumerate(scales):
+        y = torch.full(lat[:, l].shape, float("nan"), device="cuda")
+        plan.unpatchify(l, hd, wo[s].cuda(), y)
+        back.append(y.cpu())
+    torch.cuda.synchronize()
+    assert plan.device_status() == m.MSF_OK
+    del ws
+    toks, lats, off = [], [], 0
+    for l, s in enumerate(scales):
+        P = patch * s
+        x = lat[:, l].double().reshape(B, C, F * gh // s, P, gw // s, P)
+        n = F * (gh // s) * (gw // s)
+        rows = x.permute(0, 2, 4, 1, 3, 5).reshape(B, n, C * P * P)
+        toks.append(rows @ wt[s].double().T)
+        y = (h[:, off:off + n].double() @ wo[s].double().T).reshape(B, F * gh // s, gw // s, C, P, P)
+        lats.append(y.permute(0, 3, 1, 4, 2, 5).reshape(lat[:, l].shape))
+        off += n
+    return tok.cpu(), torch.cat(toks, 1), back, lats
+
+
+@pytest.mark.parametrize("shape", SHAPES, ids=[f"{s[0]}-{s[1]}-E{s[2]}-C{s[3]}" for s in SHAPES])
+def test_f32_projections(shape):
+    tok, ref, back, lats = _run(shape)
+    assert (tok.double() - ref).abs().max() <= 5e-6
+    for y, r in zip(back, lats):
+        assert (y.double() - r).abs().max() <= 5e-6
+
+
+@pytest.mark.parametrize("value", [float("inf"), float("-inf"), float("nan"), torch.finfo(F32).min])
+def test_f32_projections_of_values_the_planes_cannot_hold(value):
+    def edit(lat, wt, h, wo):
+        lat[0, 1, 2, 0, 3, 5] = value
+        h[1, 7, 11] = value
+    tok, ref, back, lats = _run(SHAPES[1], edit)
+    ref32 = ref.float()  # fp64 sums of |value| up to fp32's range round to it or to infinity
+    for a, b in [(tok, ref32)] + list(zip(back, [x.float() for x in lats])):
+        assert torch.equal(torch.isnan(a), torch.isnan(b))
+        assert torch.equal(torch.isinf(a), torch.isinf(b)) and torch.equal(a[torch.isinf(a)], b[torch.isinf(b)])
+        f = torch.isfinite(b)
+        assert ((a[f] - b[f]).abs() <= 5e-6 * b[f].abs().clamp(min=1.0)).all()
