@@ -159,10 +159,19 @@ def _ptr(t) -> Optional[int]:
     return t.data_ptr()
 
 
+_torch_c = None  # torch's C module once CUDA is initialised
+
+
 def _stream(stream) -> Optional[int]:
     if stream is None:
-        import torch
-        return torch.cuda.current_stream().cuda_stream
+        # torch.cuda.current_stream() builds a Stream object: 2.9 us of a
+        # small call's 7 us on a Grace core; the handle alone takes 0.2 us.
+        global _torch_c
+        if _torch_c is None:
+            import torch
+            torch.cuda.current_stream()  # initialises CUDA, or raises
+            _torch_c = torch._C
+        return _torch_c._cuda_getCurrentRawStream(_torch_c._cuda_getDevice())
     return stream if isinstance(stream, int) else stream.cuda_stream
 
 
