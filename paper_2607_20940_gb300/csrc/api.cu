@@ -907,7 +907,7 @@ extern "C" msf_status msf_patchify_tiers(msf_plan_t plan, const void* latent,
     const Plan& p = *plan;
     if (p.d.latent_channels <= 0 || p.d.patch <= 0 || p.d.embed_dim <= 0 || p.elem != 2)
         return MSF_ERR_UNSUPPORTED;
-    if (!p.bound) return MSF_ERR_STATE;  // the LoRA codes go through the workspace
+    if (!p.bound) return MSF_ERR_STATE;
     if (!aligned16(latent) || !aligned16(tokens)) return MSF_ERR_INVALID_ARG;
     for (int l = 0; l < p.T; ++l) {
         const msf_tier_module* t = tiers[l];
@@ -917,11 +917,9 @@ extern "C" msf_status msf_patchify_tiers(msf_plan_t plan, const void* latent,
     const msf::MspShape sh = msp_shape(p);
     cudaStream_t s = (cudaStream_t)stream;
     const int E = p.d.embed_dim;
-    char* codes = msf::tier_codes(p);
-    const long long codes_bstride = (long long)p.N * msf::kTierCodeCols;
     // Runs of consecutive states that share a tier module.
-    msf::MspEmbedRun runs[MSF_MAX_STATES], code_runs[MSF_MAX_STATES];
-    int n_runs = 0, n_code = 0;
+    msf::MspEmbedRun runs[MSF_MAX_STATES];
+    int n_runs = 0;
     for (int l0 = 0; l0 < p.T;) {
         int l1 = l0 + 1;
         while (l1 < p.T && p.d.scales[l1] == p.d.scales[l0] && tiers[l1] == tiers[l0]) ++l1;
@@ -936,35 +934,16 @@ extern "C" msf_status msf_patchify_tiers(msf_plan_t plan, const void* latent,
         r.gw = sh.Wl / r.P;
         r.tok_off = p.st_off[l0];
         if (t->embed_down) {
-            // The rank-r codes gamma * x A^T of the run's tokens, by the same
-            // fused gather + GEMM kernel with A as its weight (rows past r and
-            // columns past 64 are zero), then the embedding with one more K
-            // chunk: codes x the up projection.
-            msf::MspEmbedRun& c = code_runs[n_code++];
-            c = r;
-            c.w = t->embed_down;
-            c.w_rows = t->lora_rank;
-            c.scale = t->lora_scale;
+            r.lora_down = t->embed_down;
             r.lora_up = t->embed_up;
             r.rank = t->lora_rank;
-            r.codes = codes + (size_t)r.tok_off * msf::kTierCodeCols * 2;
-            r.codes_bstride = codes_bstride;
+            r.lora_scale = t->lora_scale;
         }
         l0 = l1;
-    }
-    for (int r0 = 0; r0 < n_code; r0 += msf::kMaxGemmProblems) {
-        const int n = n_code - r0 < msf::kMaxGemmProblems ? n_code - r0 : msf::kMaxGemmProblems;
-        if (!msf::msp_embed_supported(code_runs + r0, n, msf::kTierCodeCols)) return MSF_ERR_UNSUPPORTED;
     }
     for (int r0 = 0; r0 < n_runs; r0 += msf::kMaxGemmProblems) {
         const int n = n_runs - r0 < msf::kMaxGemmProblems ? n_runs - r0 : msf::kMaxGemmProblems;
         if (!msf::msp_embed_supported(runs + r0, n, E)) return MSF_ERR_UNSUPPORTED;
-    }
-    for (int r0 = 0; r0 < n_code; r0 += msf::kMaxGemmProblems) {
-        const int n = n_code - r0 < msf::kMaxGemmProblems ? n_code - r0 : msf::kMaxGemmProblems;
-        cudaError_t e = msf::launch_msp_embed(code_runs + r0, n, sh, msf::kTierCodeCols, latent, codes,
-                                              codes_bstride, p.B, msf::status_word(p), s);
-        if (e != cudaSuccess) return cuda_status(e);
     }
     for (int r0 = 0; r0 < n_runs; r0 += msf::kMaxGemmProblems) {
         const int n = n_runs - r0 < msf::kMaxGemmProblems ? n_runs - r0 : msf::kMaxGemmProblems;
@@ -997,28 +976,16 @@ extern "C" msf_status msf_unpatchify_tier(msf_plan_t plan, int32_t position, con
     const int M = p.st_n[position];
     const long long per = (long long)sh.C * sh.Hl * sh.Wl;
     if (!msf::msp_deembed_supported(M, F, E)) return MSF_ERR_UNSUPPORTED;
-    char* codes = msf::tier_codes(p);
     msf::DeembedTier extra;
     if (tier->out_down) {
-        // codes = gamma * h A^T for the state's tokens (columns past r zero),
-        // by the de-embedding's cluster split-K kernel with a row output
-        cudaError_t e = msf::launch_msp_rows_splitk(
-            tokens, (long long)p.N * E, p.N, p.st_off[position], tier->out_down, tier->lora_rank, M, E,
-            codes + (size_t)p.st_off[position] * msf::kTierCodeCols * 2, (long long)p.N * msf::kTierCodeCols,
-            msf::kTierCodeCols, tier->lora_scale, p.B, msf::status_word(p), s);
-        if (e != cudaSuccess) return cuda_status(e);
-        extra.codes = codes;
-        extra.codes_bstride = (long long)p.N * msf::kTierCodeCols;
+        extra.down = tier->out_down;
         extra.up = tier->out_up;
         extra.rank = tier->lora_rank;
+        extra.scale = tier->lora_scale;
     }
     if (tier->residual) {
-        // the state's raw patch vectors (its block of the raw layout) feed the residual
-        char* raw = msf::msp_scratch(p);
-        cudaError_t e = msf::launch_patchify_raw(latent_in, raw, sh, p.B, true, s, position, 1);
-        if (e != cudaSuccess) return cuda_status(e);
-        extra.xraw = raw + (size_t)position * per * 2;
-        extra.xraw_bstride = (long long)p.T * per;
+        extra.latent = (const char*)latent_in + (size_t)position * per * 2;
+        extra.latent_bstride = (long long)p.T * per;
         extra.residual = tier->residual;
     }
     return cuda_status(msf::launch_msp_deembed(tokens, (long long)p.N * E, p.N, p.st_off[position], tier->w_out,

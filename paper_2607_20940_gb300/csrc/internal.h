@@ -62,7 +62,8 @@ namespace msf {
 using Plan = ::msf_plan;
 
 // Workspace layout: [status area | pyramid K | pyramid V | MSP scratch | attention
-// merge counters | attention partial slots | de-embedding split partials | tier codes]
+// merge counters | attention partial slots | de-embedding split partials | fp32 plans: operand
+// planes, unit partials and flags]
 constexpr size_t kStatusBytes = 256;
 inline size_t round256(size_t x) { return (x + 255) / 256 * 256; }
 inline size_t pyramid_bytes(const Plan& p) {
@@ -95,13 +96,7 @@ inline size_t msp_split_bytes(const Plan& p) {
     size_t per = (size_t)p.d.latent_channels * p.d.patch * p.gh * p.d.patch * p.d.grid_w;
     return round256((size_t)kMaxDeembedSplits * p.B * per * 4);
 }
-// LoRA codes of the tier modules (msf_patchify_tiers, msf_unpatchify_tier):
-// [B, N, 64] bf16, the rank-r code of every window token zero-padded to 64.
-constexpr int kTierCodeCols = 64;
-inline size_t tier_codes_bytes(const Plan& p) {
-    if (p.d.latent_channels <= 0 || p.d.patch <= 0 || p.elem != 2 || p.d.embed_dim <= 0) return 0;
-    return round256((size_t)p.B * p.N * kTierCodeCols * 2);
-}
+constexpr int kTierCodeCols = 64;  // largest LoRA rank of a tier module
 // fp32 plans: the tensor-core attention's operands as three bf16 planes,
 // [B, 3, rows, H, D] for q and for k, v of the sink, the ring, each group's
 // pyramid part and the window; the output units of split query tiles, each
@@ -155,7 +150,7 @@ inline size_t bwd_workspace_bytes(const Plan& p) {
 }
 inline size_t workspace_bytes(const Plan& p) {
     return kStatusBytes + 2 * pyramid_bytes(p) + msp_scratch_bytes(p) + attn_counter_bytes(p) +
-           attn_partial_bytes(p) + msp_split_bytes(p) + tier_codes_bytes(p) + f32_plane_bytes(p) +
+           attn_partial_bytes(p) + msp_split_bytes(p) + f32_plane_bytes(p) +
            f32_partial_bytes(p);
 }
 inline unsigned int* status_word(const Plan& p) { return (unsigned int*)p.ws; }
@@ -174,16 +169,15 @@ inline float* attn_partials(const Plan& p) {
 inline float* msp_split(const Plan& p) {
     return (float*)((char*)attn_partials(p) + attn_partial_bytes(p));
 }
-inline char* tier_codes(const Plan& p) { return (char*)msp_split(p) + msp_split_bytes(p); }
 inline char* f32_planes(const Plan& p, int part, int which) {  // which: 0 = q or k, 1 = v
-    char* base = tier_codes(p) + tier_codes_bytes(p);
+    char* base = (char*)msp_split(p) + msp_split_bytes(p);
     if (part == kF32Q) return base;
     base += f32_part_bytes(p, kF32Q);
     for (int i = kF32Sink; i < part; ++i) base += 2 * f32_part_bytes(p, i);
     return base + which * f32_part_bytes(p, part);
 }
 inline float* f32_partials(const Plan& p) {
-    return (float*)(tier_codes(p) + tier_codes_bytes(p) + f32_plane_bytes(p));
+    return (float*)(f32_planes(p, kF32Q, 0) + f32_plane_bytes(p));
 }
 inline unsigned int* f32_flags(const Plan& p) {
     return (unsigned int*)((char*)f32_partials(p) + round256((size_t)f32_max_slots(p) * 128 * (p.D + 2) * 4));

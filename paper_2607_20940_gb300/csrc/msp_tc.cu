@@ -34,6 +34,7 @@ constexpr int kThreads = 256;
 constexpr long long kWaitLimit = 2000000000LL;
 constexpr int kChunkA = 128 * 128;  // 128 rows x 64 bf16 (one K chunk), swizzled
 constexpr int kEmbedBN = 256;
+constexpr int kLoraBN = 192;  // columns of a tile with an adapter: 64 of the 256 hold the codes
 constexpr int kEmbedStages = 2;
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*,
@@ -135,14 +136,13 @@ struct EmbedRun {
     int P;          // patch edge in latent pixels
     int K;          // C * P * P
     int tok_off;    // first token row of the run in the output
-    int lora;       // 1: one more K chunk (LoRA codes x up projection)
-    float scale;    // accumulator scale
+    int lora;       // 1: one more K chunk (LoRA codes x up projection), 192-column tiles
+    float scale;    // LoRA scale
 };
 struct EmbedParams {
     int n_runs;
     EmbedRun run[kMaxGemmProblems];
     int T, C, Hl, Wl, E;
-    int n_tiles_n;  // 256-column tiles per 128-row tile: ceil(E / 256)
     int n_embed_tiles;  // CTAs [0, n_embed_tiles) of a stream embed; the rest pool
     int pool_ctas;      // CTAs per stream that run the pyramid jobs (0: none)
     int pool_tasks;     // vector-pair tasks per pyramid job
@@ -152,19 +152,30 @@ struct EmbedParams {
     unsigned int* status;
 };
 struct EmbedMaps {
-    CUtensorMap w[kMaxGemmProblems];      // [E, K] weight of each run: dims {K, E}
-    CUtensorMap out[kMaxGemmProblems];    // the run's tokens: dims {E, M, B}, rows past M clipped
-    CUtensorMap codes[kMaxGemmProblems];  // LoRA codes of the run's tokens: dims {64, M, B}
-    CUtensorMap up[kMaxGemmProblems];     // LoRA up projection [E, r]: dims {r, E}
+    CUtensorMap w[kMaxGemmProblems];    // [E, K] weight of each run: dims {K, E}
+    CUtensorMap out[kMaxGemmProblems];  // the run's tokens: dims {E, M, B}, rows past M clipped
 };
+struct LoraMaps {
+    CUtensorMap down[kMaxGemmProblems];  // LoRA down projection [r, K]: dims {K, r}
+    CUtensorMap up[kMaxGemmProblems];    // LoRA up projection [E, r]: dims {r, E}
+};
+struct NoLora {};
 
 // 128 tokens x 256 embedding columns per CTA (one N=256 MMA per K step, half
 // the gathers of 128-column tiles); two CTAs per SM (97 KB of shared memory
 // each), so the 480p window's 210 tiles run in one wave on 152 SMs.
+//
+// kLora (its own instantiation, with the adapters' maps): a run with an adapter
+// has 192-column tiles; each K chunk is also multiplied by the down projection
+// into the 64 accumulator columns left, the gathering warps round those codes
+// (scaled, once) into one more A chunk, and the last K chunk is codes x up
+// projection. Every column tile of a token tile computes the codes again, which
+// costs a 64-wide MMA per K step; a launch of their own cost 4.8 us (480p).
+template <bool kLora, class Lora>
 __global__ void __launch_bounds__(kThreads, 2)
     msp_embed_kernel(const __grid_constant__ EmbedMaps maps, const __grid_constant__ EmbedParams p,
-                     const __grid_constant__ PoolBatch pool) {
-    if ((int)blockIdx.x >= p.n_embed_tiles) {
+                     const __grid_constant__ PoolBatch pool, const __grid_constant__ Lora lmaps) {
+    if (!kLora && (int)blockIdx.x >= p.n_embed_tiles) {
         // ---- K/V pyramid jobs in the CTAs after the embedding tiles (the
         // longest tiles, those of the runs with the most K chunks, come
         // first): the same per-thread pooling as pool_kernel, one task per
@@ -185,7 +196,7 @@ __global__ void __launch_bounds__(kThreads, 2)
     unsigned char* sB = smem + kEmbedStages * kChunkA;          // [stage][BN rows x 128 B]
     constexpr int kBBytes = kEmbedBN * 128;
     __shared__ uint64_t a_full[kEmbedStages], a_empty[kEmbedStages];
-    __shared__ uint64_t b_full[kEmbedStages], b_empty[kEmbedStages], acc_full;
+    __shared__ uint64_t b_full[kEmbedStages], b_empty[kEmbedStages], acc_full, codes_full;
     __shared__ uint32_t tmem_base_sh;
     __shared__ int abort_flag;
 
@@ -198,7 +209,9 @@ __global__ void __launch_bounds__(kThreads, 2)
     const int mt = local % R.m_tiles, nt = local / R.m_tiles;
     const int b = blockIdx.z;
     const int nk_patch = R.K / 64;      // chunks gathered from the latent
-    const int nk = nk_patch + R.lora;   // plus the LoRA chunk
+    const bool lora = kLora && R.lora;
+    const int nk = nk_patch + (lora ? 1 : 0);   // plus the LoRA chunk
+    const int bn = lora ? kLoraBN : kEmbedBN;   // output columns of this tile
 
     if (threadIdx.x == 0) {
         abort_flag = 0;
@@ -209,6 +222,7 @@ __global__ void __launch_bounds__(kThreads, 2)
             ptx::mbar_init(&b_empty[s], 1);
         }
         ptx::mbar_init(&acc_full, 1);
+        ptx::mbar_init(&codes_full, 1);
         ptx::fence_mbar_init();
     }
     if (warp == 2) {
@@ -236,11 +250,19 @@ __global__ void __launch_bounds__(kThreads, 2)
                     ok = false;
                     break;
                 }
-                ptx::mbar_arrive_expect_tx(&b_full[st], kBBytes);
-                if (kc < nk_patch)
-                    ptx::tma_load_2d(sB + st * kBBytes, &maps.w[ri], &b_full[st], kc * 64, nt * kEmbedBN);
-                else
-                    ptx::tma_load_2d(sB + st * kBBytes, &maps.up[ri], &b_full[st], 0, nt * kEmbedBN);
+                // a LoRA run's patch chunk: 192 rows of the weight, then the 64
+                // (zero past the rank) of the down projection
+                ptx::mbar_arrive_expect_tx(&b_full[st], lora && kc == nk_patch ? kLoraBN * 128 : kBBytes);
+                if constexpr (kLora) {
+                    if (kc == nk_patch)
+                        ptx::tma_load_2d(sB + st * kBBytes, &lmaps.up[ri], &b_full[st], 0, nt * bn);
+                    else
+                        ptx::tma_load_2d(sB + st * kBBytes, &maps.w[ri], &b_full[st], kc * 64, nt * bn);
+                    if (lora && kc < nk_patch)
+                        ptx::tma_load_2d(sB + st * kBBytes + kLoraBN * 128, &lmaps.down[ri], &b_full[st], kc * 64, 0);
+                } else {
+                    ptx::tma_load_2d(sB + st * kBBytes, &maps.w[ri], &b_full[st], kc * 64, nt * bn);
+                }
                 ++issued;
             }
             if (!ok) {
@@ -251,7 +273,9 @@ __global__ void __launch_bounds__(kThreads, 2)
             }
         }
     } else if (warp == 1) {
-        constexpr uint32_t idesc = ptx::idesc_bf16(128, kEmbedBN, false, false);
+        const uint32_t idesc =
+            lora ? ptx::idesc_bf16(128, kLoraBN, false, false) : ptx::idesc_bf16(128, kEmbedBN, false, false);
+        constexpr uint32_t id_codes = ptx::idesc_bf16(128, 64, false, false);
         const uint64_t a_desc = ptx::sdesc_sw128(ptx::smem_u32(sA), 16, 1024);
         const uint64_t b_desc = ptx::sdesc_sw128(ptx::smem_u32(sB), 16, 1024);
         bool ok = true;
@@ -270,6 +294,14 @@ __global__ void __launch_bounds__(kThreads, 2)
                 for (int kk = 0; kk < 4; ++kk)
                     ptx::mma_ss(tbase, ad + (uint64_t)(kk * 2), bd + (uint64_t)(kk * 2), idesc,
                                 (kc > 0 || kk > 0) ? 1u : 0u);
+                if (lora && kc < nk_patch) {
+#pragma unroll
+                    for (int kk = 0; kk < 4; ++kk)
+                        ptx::mma_ss(tbase + kLoraBN, ad + (uint64_t)(kk * 2),
+                                    bd + (uint64_t)((kLoraBN * 128) >> 4) + (uint64_t)(kk * 2), id_codes,
+                                    (kc > 0 || kk > 0) ? 1u : 0u);
+                    if (kc + 1 == nk_patch) ptx::mma_commit(&codes_full);
+                }
                 ptx::mma_commit(&a_empty[st]);
                 ptx::mma_commit(&b_empty[st]);
             }
@@ -319,20 +351,33 @@ __global__ void __launch_bounds__(kThreads, 2)
             ptx::fence_proxy_async_smem();  // the tensor core reads through the async proxy
             ptx::mbar_arrive(&a_full[st]);
         }
-        if (ok && R.lora) {
-            // ---- LoRA chunk: the 128 rows' codes arrive by TMA into the A
-            // stage; one thread adds the bytes to the stage's barrier, the
-            // others arrive as for a gathered chunk.
+        if (ok && lora) {
+            // ---- LoRA chunk: this row's codes, scaled and rounded once
             const int st = nk_patch % kEmbedStages;
             const uint32_t ph = (uint32_t)((nk_patch / kEmbedStages) & 1);
-            ok = __all_sync(0xffffffffu, ptx::mbar_wait_bounded(&a_empty[st], ph ^ 1u, abort_p, kWaitLimit));
+            ok = __all_sync(0xffffffffu, ptx::mbar_wait_bounded(&codes_full, 0, abort_p, kWaitLimit) &&
+                                             ptx::mbar_wait_bounded(&a_empty[st], ph ^ 1u, abort_p, kWaitLimit));
             if (ok) {
-                if (r == 0) {
-                    ptx::mbar_arrive_expect_tx(&a_full[st], kChunkA);
-                    ptx::tma_load_3d(sA + st * kChunkA, &maps.codes[ri], &a_full[st], 0, mt * 128, b);
-                } else {
-                    ptx::mbar_arrive(&a_full[st]);
+                ptx::tc_fence_after();
+                const uint32_t taddr = tbase + kLoraBN + ((uint32_t)((warp - 4) * 32) << 16);
+                unsigned char* dst = sA + st * kChunkA;
+                const float sc = R.scale;
+#pragma unroll
+                for (int c = 0; c < 2; ++c) {
+                    uint32_t v[32];
+                    ptx::tmem_ld32(taddr + 32 * c, v);
+                    ptx::tmem_wait_ld();
+#pragma unroll
+                    for (int e = 0; e < 4; ++e)
+                        *reinterpret_cast<uint4*>(dst + swz_offset(r, 32 * c + 8 * e)) = make_uint4(
+                            ptx::pack_bf16(sc * __uint_as_float(v[8 * e]), sc * __uint_as_float(v[8 * e + 1])),
+                            ptx::pack_bf16(sc * __uint_as_float(v[8 * e + 2]), sc * __uint_as_float(v[8 * e + 3])),
+                            ptx::pack_bf16(sc * __uint_as_float(v[8 * e + 4]), sc * __uint_as_float(v[8 * e + 5])),
+                            ptx::pack_bf16(sc * __uint_as_float(v[8 * e + 6]), sc * __uint_as_float(v[8 * e + 7])));
                 }
+                ptx::tc_fence_before();
+                ptx::fence_proxy_async_smem();
+                ptx::mbar_arrive(&a_full[st]);
             }
         }
         // ---- epilogue: bf16 tile staged in the (now idle) A and B stages in
@@ -343,27 +388,26 @@ __global__ void __launch_bounds__(kThreads, 2)
             ptx::tc_fence_after();
             const uint32_t taddr = tbase + ((uint32_t)((warp - 4) * 32) << 16);
 #pragma unroll 1
-            for (int c = 0; c < kEmbedBN / 32; ++c) {
+            for (int c = 0; c < bn / 32; ++c) {
                 uint32_t v[32];
                 ptx::tmem_ld32(taddr + c * 32, v);
                 ptx::tmem_wait_ld();
                 unsigned char* stage = sA + (c / 2) * kChunkA;
-                const float sc = R.scale;
 #pragma unroll
                 for (int e = 0; e < 4; ++e)
-                    *reinterpret_cast<uint4*>(stage + swz_offset(r, (c % 2) * 32 + 8 * e)) = make_uint4(
-                        ptx::pack_bf16(sc * __uint_as_float(v[8 * e]), sc * __uint_as_float(v[8 * e + 1])),
-                        ptx::pack_bf16(sc * __uint_as_float(v[8 * e + 2]), sc * __uint_as_float(v[8 * e + 3])),
-                        ptx::pack_bf16(sc * __uint_as_float(v[8 * e + 4]), sc * __uint_as_float(v[8 * e + 5])),
-                        ptx::pack_bf16(sc * __uint_as_float(v[8 * e + 6]), sc * __uint_as_float(v[8 * e + 7])));
+                    *reinterpret_cast<uint4*>(stage + swz_offset(r, (c % 2) * 32 + 8 * e)) =
+                        make_uint4(ptx::pack_bf16(__uint_as_float(v[8 * e]), __uint_as_float(v[8 * e + 1])),
+                                   ptx::pack_bf16(__uint_as_float(v[8 * e + 2]), __uint_as_float(v[8 * e + 3])),
+                                   ptx::pack_bf16(__uint_as_float(v[8 * e + 4]), __uint_as_float(v[8 * e + 5])),
+                                   ptx::pack_bf16(__uint_as_float(v[8 * e + 6]), __uint_as_float(v[8 * e + 7])));
             }
             ptx::fence_proxy_async_smem();
         }
         // The four epilogue warps meet before one thread stores the tile.
         ok = ptx::named_bar_and(1, 128, ok);
         if (ok && warp == 4 && lane == 0) {
-            for (int h = 0; h < kEmbedBN / 64 && nt * kEmbedBN + h * 64 < p.E; ++h)
-                ptx::tma_store_3d(&maps.out[ri], sA + h * kChunkA, nt * kEmbedBN + h * 64, mt * 128, b);
+            for (int h = 0; h < bn / 64 && nt * bn + h * 64 < p.E; ++h)
+                ptx::tma_store_3d(&maps.out[ri], sA + h * kChunkA, nt * bn + h * 64, mt * 128, b);
             ptx::bulk_commit();
             ptx::bulk_wait_read_all();
         }
@@ -391,46 +435,79 @@ __global__ void __launch_bounds__(kThreads, 2)
 
 constexpr int kDeBN = 64;
 constexpr int kDeStages = 4;
+constexpr int kDeTierStages = 3;
 constexpr int kDeMaxSplits = 8;  // cluster size along the split (portable limit)
 constexpr int kDePartStride = kDeBN + 4;  // floats per staged row (padding spreads the banks)
 
 struct DeembedParams {
     int M;              // tokens of the position (per stream)
     int K;              // embedding width E
-    int nk_all;         // K chunks: E / 64 token chunks, then the tier's extras
-    int lora;           // 1: chunk E/64 is (LoRA codes, up projection)
-    int nk_res;         // then this many (raw patch vector, latent residual) chunks
+    int nk_all;         // K chunks: E / 64 token chunks, then the latent residual's
     int m_tiles;
     int splits;         // cluster size along y
     int P, gw, C, Hl, Wl;
     int tok_row0;       // first token row of the position
     __nv_bfloat16* latent;  // [B, C, Hl, Wl]
     unsigned int* status;
-    // Row output instead of the latent scatter (NULL: scatter): row m of
-    // stream b, columns [0, F), at rows_out + b * rows_bstride + m * rows_ld,
-    // each value scaled by rows_scale before the one rounding.
-    __nv_bfloat16* rows_out;
-    long long rows_bstride;
-    int rows_ld;
-    float rows_scale;
 };
+// The tier's extras of one position.
+struct DeembedTierParams {
+    int rank;                     // of the adapter, 0: none
+    float scale;                  // LoRA scale
+    const __nv_bfloat16* up;      // LoRA up projection [F, rank]
+    const __nv_bfloat16* latent;  // the position's input latent of stream 0 (residual)
+    long long latent_bstride;     // elements
+};
+struct NoTier {};
 struct DeembedMaps {
-    CUtensorMap a;      // tokens {E, rows, B}
-    CUtensorMap b;      // W_out {E, F}
-    CUtensorMap codes;  // LoRA codes of the tokens {64, rows, B}
-    CUtensorMap up;     // LoRA up projection [F, r]: {r, F}
-    CUtensorMap xraw;   // the state's raw patch vectors {F, M, B}
-    CUtensorMap res;    // latent residual [F, F]: {F, F}
+    CUtensorMap a;     // tokens {E, rows, B}
+    CUtensorMap b;     // W_out {E, F}
+    CUtensorMap down;  // LoRA down projection [r, E]: {E, r}
+    CUtensorMap res;   // latent residual [F, F]: {F, F}
 };
 
-__global__ void __launch_bounds__(kThreads, 1)
-    msp_deembed_kernel(const __grid_constant__ DeembedMaps maps, const __grid_constant__ DeembedParams p) {
+// One token row of the residual's K chunks c0, c0 + step, ... (n of them) into
+// the ring as chunk uses k0, k0 + 1, ...: each chunk's loads go out before the
+// wait for its stage (`go`: the producer, which follows every use of a stage,
+// says that it is free). Returns false if a wait gave up.
+template <int P, typename V, int kStages>
+__device__ __forceinline__ bool gather_residual(unsigned char* ring, int stage_bytes, uint64_t* a_full, uint64_t* go,
+                                                const __nv_bfloat16* base, size_t plane, int Wl, int r, int c0, int step,
+                                                int n, int k0, bool valid, volatile int* abort_p) {
+    V cur[64 / P];
+    for (int i = 0; i < n; ++i) {
+        load_chunk<P, V>(cur, base, plane, Wl, c0 + i * step, valid);
+        const int st = (k0 + i) % kStages;
+        if (!__all_sync(0xffffffffu, ptx::mbar_wait_bounded(&go[st], (uint32_t)((i / kStages) & 1), abort_p, kWaitLimit)))
+            return false;
+        store_chunk<P, V>(ring + st * stage_bytes, cur, r);
+        ptx::fence_proxy_async_smem();
+        ptx::mbar_arrive(&a_full[st]);
+    }
+    return true;
+}
+
+// kTier (its own instantiation): each token chunk is also multiplied by the
+// LoRA down projection into a second accumulator, the residual's K chunks are
+// gathered from the input latent, and the CTA that sums a row adds
+// up x bf16(scale * codes) to it in fp32. (The codes, the raw patch vectors and
+// the sum were three launches.)
+template <bool kTier, class Tier>
+__global__ void __launch_bounds__(kThreads, kTier ? 2 : 1)
+    msp_deembed_kernel(const __grid_constant__ DeembedMaps maps, const __grid_constant__ DeembedParams p,
+                       const __grid_constant__ Tier tier) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char* smem = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     constexpr int kBBytes = kDeBN * 128;
-    constexpr int kStageBytes = kChunkA + kBBytes;
+    constexpr int kStageBytes = kChunkA + (kTier ? 2 : 1) * kBBytes;  // tokens, W_out, down projection
     float* part = reinterpret_cast<float*>(smem);  // reuses the ring once every MMA is done
-    __shared__ uint64_t full[kDeStages], empty[kDeStages], acc_full;
+    float* cpart = part + 128 * kDePartStride;     // kTier: this split's codes
+    // kTier: then the up projection of the tile's features transposed
+    // [rank][kDePartStride], and the summed codes of this CTA's rows
+    float* up_s = cpart + 128 * kDePartStride;
+    float* code_s = up_s + 64 * kDePartStride;
+    constexpr int kStages = kTier ? kDeTierStages : kDeStages;
+    __shared__ uint64_t full[kStages], empty[kStages], go[kStages], a_full[kStages], acc_full;
     __shared__ uint32_t tmem_base_sh;
     __shared__ int abort_flag;
 
@@ -441,20 +518,29 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int b = blockIdx.z;
     const int nk_all = p.nk_all;
     const int nk_tok = p.K / 64;
-    const int kc0 = (int)((long long)split * nk_all / p.splits);
-    const int nk = (int)((long long)(split + 1) * nk_all / p.splits) - kc0;
+    // Chunks of this split: a contiguous run, or (kTier) every splits-th one, so
+    // that the gathered residual chunks, which come last, spread over the CTAs.
+    const int step = kTier ? p.splits : 1;
+    const int kc0 = kTier ? split : (int)((long long)split * nk_all / p.splits);
+    const int nk = kTier ? (nk_all - split + step - 1) / step
+                         : (int)((long long)(split + 1) * nk_all / p.splits) - kc0;
+    const int n_tok = kTier ? min(max((nk_tok - split + step - 1) / step, 0), nk) : nk;  // token chunks, then residual
+    bool lora = false;
+    if constexpr (kTier) lora = tier.rank > 0;
 
     if (threadIdx.x == 0) {
         abort_flag = 0;
-        for (int s = 0; s < kDeStages; ++s) {
+        for (int s = 0; s < kStages; ++s) {
             ptx::mbar_init(&full[s], 1);
             ptx::mbar_init(&empty[s], 1);
+            ptx::mbar_init(&go[s], 1);
+            ptx::mbar_init(&a_full[s], 128);  // residual chunks: one arrival per gathering thread
         }
         ptx::mbar_init(&acc_full, 1);
         ptx::fence_mbar_init();
     }
     if (warp == 2) {
-        ptx::tmem_alloc(&tmem_base_sh, kDeBN);
+        ptx::tmem_alloc(&tmem_base_sh, kTier ? 2 * kDeBN : kDeBN);
         ptx::tmem_relinquish();
     }
     ptx::tc_fence_before();
@@ -473,31 +559,29 @@ __global__ void __launch_bounds__(kThreads, 1)
             ptx::prefetch_tmap(&maps.b);
             int issued = 0;
             for (int kc = 0; kc < nk; ++kc) {
-                const int st = kc % kDeStages;
-                const uint32_t ph = (uint32_t)((kc / kDeStages) & 1);
+                const int st = kc % kStages;
+                const uint32_t ph = (uint32_t)((kc / kStages) & 1);
                 if (!ptx::mbar_wait_bounded(&empty[st], ph ^ 1u, abort_p, kWaitLimit)) {
                     ok = false;
                     break;
                 }
                 unsigned char* sa = smem + st * kStageBytes;
-                ptx::mbar_arrive_expect_tx(&full[st], kStageBytes);
-                const int g = kc0 + kc;
-                if (g < nk_tok) {
+                const int g = kc0 + kc * step;
+                if (!kTier || kc < n_tok) {
+                    ptx::mbar_arrive_expect_tx(&full[st], kChunkA + (lora ? 2 : 1) * kBBytes);
                     ptx::tma_load_3d(sa, &maps.a, &full[st], g * 64, p.tok_row0 + mt * 128, b);
                     ptx::tma_load_2d(sa + kChunkA, &maps.b, &full[st], g * 64, nt * kDeBN);
-                } else if (g == nk_tok && p.lora) {
-                    ptx::tma_load_3d(sa, &maps.codes, &full[st], 0, p.tok_row0 + mt * 128, b);
-                    ptx::tma_load_2d(sa + kChunkA, &maps.up, &full[st], 0, nt * kDeBN);
+                    if (lora) ptx::tma_load_2d(sa + kChunkA + kBBytes, &maps.down, &full[st], g * 64, 0);
                 } else {
-                    const int j = g - nk_tok - p.lora;
-                    ptx::tma_load_3d(sa, &maps.xraw, &full[st], j * 64, mt * 128, b);
-                    ptx::tma_load_2d(sa + kChunkA, &maps.res, &full[st], j * 64, nt * kDeBN);
+                    ptx::mbar_arrive(&go[st]);
+                    ptx::mbar_arrive_expect_tx(&full[st], kBBytes);
+                    ptx::tma_load_2d(sa + kChunkA, &maps.res, &full[st], (g - nk_tok) * 64, nt * kDeBN);
                 }
                 ++issued;
             }
             if (!ok) {
-                for (int kc = (issued > kDeStages ? issued - kDeStages : 0); kc < issued; ++kc)
-                    ptx::mbar_wait_bounded(&full[kc % kDeStages], (uint32_t)((kc / kDeStages) & 1), &never,
+                for (int kc = (issued > kStages ? issued - kStages : 0); kc < issued; ++kc)
+                    ptx::mbar_wait_bounded(&full[kc % kStages], (uint32_t)((kc / kStages) & 1), &never,
                                            kWaitLimit);
                 atomicOr(p.status, kDevTimeout);
             }
@@ -506,9 +590,13 @@ __global__ void __launch_bounds__(kThreads, 1)
         constexpr uint32_t idesc = ptx::idesc_bf16(128, kDeBN, false, false);
         const uint64_t desc0 = ptx::sdesc_sw128(ptx::smem_u32(smem), 16, 1024);
         for (int kc = 0; kc < nk && ok; ++kc) {
-            const int st = kc % kDeStages;
-            const uint32_t ph = (uint32_t)((kc / kDeStages) & 1);
-            ok = __all_sync(0xffffffffu, ptx::mbar_wait_bounded(&full[st], ph, abort_p, kWaitLimit));
+            const int st = kc % kStages;
+            const uint32_t ph = (uint32_t)((kc / kStages) & 1);
+            bool rf = ptx::mbar_wait_bounded(&full[st], ph, abort_p, kWaitLimit);
+            if (kTier && kc >= n_tok)  // the residual's use of this stage, counted from its first chunk
+                rf = rf && ptx::mbar_wait_bounded(&a_full[st], (uint32_t)(((kc - n_tok) / kStages) & 1), abort_p,
+                                                  kWaitLimit);
+            ok = __all_sync(0xffffffffu, rf);
             if (!ok) break;
             ptx::tc_fence_after();
             if (ptx::elect_one_sync()) {
@@ -518,6 +606,13 @@ __global__ void __launch_bounds__(kThreads, 1)
                 for (int kk = 0; kk < 4; ++kk)
                     ptx::mma_ss(tbase, ad + (uint64_t)(kk * 2), bd + (uint64_t)(kk * 2), idesc,
                                 (kc > 0 || kk > 0) ? 1u : 0u);
+                if (lora && kc < n_tok) {
+#pragma unroll
+                    for (int kk = 0; kk < 4; ++kk)
+                        ptx::mma_ss(tbase + kDeBN, ad + (uint64_t)(kk * 2),
+                                    bd + (uint64_t)(kBBytes >> 4) + (uint64_t)(kk * 2), idesc,
+                                    (kc > 0 || kk > 0) ? 1u : 0u);
+                }
                 ptx::mma_commit(&empty[st]);
             }
             __syncwarp();
@@ -526,67 +621,158 @@ __global__ void __launch_bounds__(kThreads, 1)
         __syncwarp();
         if (!ok && lane == 0) atomicOr(p.status, kDevTimeout);
     } else if (warp >= 4) {
-        // ---- this split's partial tile into shared memory (row-major, padded rows)
         const int r = (warp - 4) * 32 + lane;
-        ok = __all_sync(0xffffffffu, ptx::mbar_wait_bounded(&acc_full, 0, abort_p, kWaitLimit));
+        if constexpr (kTier) {
+            // ---- residual chunks: one token row of raw patch vectors per thread
+            if (n_tok < nk) {
+                const int m = mt * 128 + r;
+                const bool valid = m < p.M;
+                const __nv_bfloat16* base =
+                    tier.latent + b * tier.latent_bstride +
+                    (valid ? (size_t)(p.P * (m / p.gw)) * p.Wl + (size_t)p.P * (m % p.gw) : 0);
+                const size_t plane = (size_t)p.Hl * p.Wl;
+                const int c0 = kc0 + n_tok * step - nk_tok, n = nk - n_tok;
+                if (p.P == 2)
+                    ok = gather_residual<2, uint32_t, kStages>(smem, kStageBytes, a_full, go, base, plane, p.Wl, r, c0,
+                                                               step, n, n_tok, valid, abort_p);
+                else if (p.P == 4)
+                    ok = gather_residual<4, uint2, kStages>(smem, kStageBytes, a_full, go, base, plane, p.Wl, r, c0,
+                                                            step, n, n_tok, valid, abort_p);
+                else if (p.P == 8)
+                    ok = gather_residual<8, uint4, kStages>(smem, kStageBytes, a_full, go, base, plane, p.Wl, r, c0,
+                                                            step, n, n_tok, valid, abort_p);
+                else
+                    for (int i = 0; i < n && ok; ++i) {  // any other patch edge, pixel by pixel
+                        const int st = (n_tok + i) % kStages;
+                        ok = __all_sync(0xffffffffu,
+                                        ptx::mbar_wait_bounded(&go[st], (uint32_t)((i / kStages) & 1), abort_p, kWaitLimit));
+                        if (!ok) break;
+                        for (int x = 0; x < 64; ++x) {
+                            const int f = (c0 + i * step) * 64 + x, PP = p.P * p.P;
+                            *reinterpret_cast<__nv_bfloat16*>(smem + st * kStageBytes + swz_offset(r, x)) =
+                                valid ? base[f / PP * plane + (size_t)(f % PP / p.P) * p.Wl + f % p.P]
+                                      : __float2bfloat16(0.f);
+                        }
+                        ptx::fence_proxy_async_smem();
+                        ptx::mbar_arrive(&a_full[st]);
+                    }
+            }
+        }
+        // ---- this split's partial tile into shared memory (row-major, padded rows)
+        ok = ok && __all_sync(0xffffffffu, ptx::mbar_wait_bounded(&acc_full, 0, abort_p, kWaitLimit));
         if (ok) {
             ptx::tc_fence_after();
             const uint32_t taddr = tbase + ((uint32_t)((warp - 4) * 32) << 16);
-            uint32_t vb[kDeBN / 32][32];
+            auto stage = [&](uint32_t t, float* dst, bool any) {
+                uint32_t vb[kDeBN / 32][32];
+                if (any) {
 #pragma unroll
-            for (int c = 0; c < kDeBN / 32; ++c) ptx::tmem_ld32(taddr + c * 32, vb[c]);
-            ptx::tmem_wait_ld();
+                    for (int c = 0; c < kDeBN / 32; ++c) ptx::tmem_ld32(t + c * 32, vb[c]);
+                    ptx::tmem_wait_ld();
+                } else {
 #pragma unroll
-            for (int c = 0; c < kDeBN / 32; ++c) {
-                const uint32_t* v = vb[c];
-                float4* d4 = reinterpret_cast<float4*>(part + r * kDePartStride + c * 32);
+                    for (int c = 0; c < kDeBN / 32; ++c)
 #pragma unroll
-                for (int e = 0; e < 8; ++e)
-                    d4[e] = make_float4(__uint_as_float(v[4 * e]), __uint_as_float(v[4 * e + 1]),
-                                        __uint_as_float(v[4 * e + 2]), __uint_as_float(v[4 * e + 3]));
-            }
+                        for (int e = 0; e < 32; ++e) vb[c][e] = 0u;
+                }
+#pragma unroll
+                for (int c = 0; c < kDeBN / 32; ++c) {
+                    const uint32_t* v = vb[c];
+                    float4* d4 = reinterpret_cast<float4*>(dst + r * kDePartStride + c * 32);
+#pragma unroll
+                    for (int e = 0; e < 8; ++e)
+                        d4[e] = make_float4(__uint_as_float(v[4 * e]), __uint_as_float(v[4 * e + 1]),
+                                            __uint_as_float(v[4 * e + 2]), __uint_as_float(v[4 * e + 3]));
+                }
+            };
+            stage(taddr, part, true);
+            if (lora) stage(taddr + kDeBN, cpart, n_tok > 0);
         } else if (lane == 0) {
             atomicOr(p.status, kDevTimeout);
+        }
+    } else if constexpr (kTier) {
+        // ---- warps 2 and 3: the up projection's rows of the tile's 64
+        // features, loaded early and put into the ring's space at its end
+        if (lora) {
+            const int f = (warp - 2) * 32 + lane;
+            const uint4* src = reinterpret_cast<const uint4*>(tier.up + (size_t)(nt * kDeBN + f) * tier.rank);
+            uint4 u[8];
+#pragma unroll
+            for (int x = 0; x < 8; ++x) u[x] = 8 * x < tier.rank ? __ldg(src + x) : make_uint4(0u, 0u, 0u, 0u);
+            if (ptx::mbar_wait_bounded(&acc_full, 0, abort_p, kWaitLimit)) {
+#pragma unroll
+                for (int x = 0; x < 8; ++x) {
+                    const uint32_t w[4] = {u[x].x, u[x].y, u[x].z, u[x].w};
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        up_s[(8 * x + 2 * e) * kDePartStride + f] = __uint_as_float(w[e] << 16);
+                        up_s[(8 * x + 2 * e + 1) * kDePartStride + f] = __uint_as_float(w[e] & 0xffff0000u);
+                    }
+                }
+            }
         }
     }
     // Every thread of every CTA of the cluster: partials are staged.
     __syncwarp();
     ptx::tc_fence_before();
     ptx::cluster_sync();
+    const int R = 128 / p.splits;  // rows [split * R, split * R + R) of the tile are this CTA's
+    // All splits' partials requested before the first add (remote
+    // shared-memory loads are independent), summed in split order.
+    auto sum4 = [&](const float* src) {
+        float4 v[kDeMaxSplits];
+#pragma unroll
+        for (int sp = 0; sp < kDeMaxSplits; ++sp)
+            v[sp] = sp < p.splits ? ptx::ld_cluster_f4(src, (uint32_t)sp) : make_float4(0.f, 0.f, 0.f, 0.f);
+        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int sp = 0; sp < kDeMaxSplits; ++sp) {
+            acc.x += v[sp].x;
+            acc.y += v[sp].y;
+            acc.z += v[sp].z;
+            acc.w += v[sp].w;
+        }
+        return acc;
+    };
+    const int per_row = kDeBN / 4;  // float4 per row
+    if constexpr (kTier) {
+        if (lora) {
+            // the rows' codes: summed, scaled, rounded once to bf16
+            for (int q = threadIdx.x; q < R * per_row; q += kThreads) {
+                const int row = q / per_row, c4 = q % per_row;
+                const float4 a = sum4(cpart + (split * R + row) * kDePartStride + 4 * c4);
+                const uint32_t lo = ptx::pack_bf16(tier.scale * a.x, tier.scale * a.y);
+                const uint32_t hi = ptx::pack_bf16(tier.scale * a.z, tier.scale * a.w);
+                *reinterpret_cast<float4*>(code_s + row * kDePartStride + 4 * c4) =
+                    make_float4(__uint_as_float(lo << 16), __uint_as_float(lo & 0xffff0000u),
+                                __uint_as_float(hi << 16), __uint_as_float(hi & 0xffff0000u));
+            }
+            __syncthreads();
+        }
+    }
     {
-        // ---- rows [rank*R, rank*R + R) of the tile: sum the S partials in
-        // split order, round once, scatter into the latent.
-        const int R = 128 / p.splits;             // rows per CTA
-        const int per_row = kDeBN / 4;            // float4 per row
+        // ---- sum the S partials in split order, add the adapter, round once,
+        // scatter into the latent
         const int P = p.P, PP = P * P;
         const size_t plane = (size_t)p.Hl * p.Wl;
         for (int q = threadIdx.x; q < R * per_row; q += kThreads) {
             const int row = split * R + q / per_row;
             const int c4 = q % per_row;
             const int m = mt * 128 + row;
-            // All splits' partials requested before the first add (remote
-            // shared-memory loads are independent), summed in split order.
-            float4 v[kDeMaxSplits];
-#pragma unroll
-            for (int sp = 0; sp < kDeMaxSplits; ++sp)
-                v[sp] = sp < p.splits ? ptx::ld_cluster_f4(part + row * kDePartStride + 4 * c4, (uint32_t)sp)
-                                      : make_float4(0.f, 0.f, 0.f, 0.f);
-            float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-            for (int sp = 0; sp < kDeMaxSplits; ++sp) {
-                acc.x += v[sp].x;
-                acc.y += v[sp].y;
-                acc.z += v[sp].z;
-                acc.w += v[sp].w;
+            float4 acc = sum4(part + row * kDePartStride + 4 * c4);
+            if constexpr (kTier) {
+                const float* code = code_s + (q / per_row) * kDePartStride;
+#pragma unroll 8
+                for (int k = 0; k < tier.rank; ++k) {  // a multiple of 8
+                    const float4 u = *reinterpret_cast<const float4*>(up_s + k * kDePartStride + 4 * c4);
+                    const float c = code[k];
+                    acc.x = fmaf(c, u.x, acc.x);
+                    acc.y = fmaf(c, u.y, acc.y);
+                    acc.z = fmaf(c, u.z, acc.z);
+                    acc.w = fmaf(c, u.w, acc.w);
+                }
             }
-            if (m < p.M && p.rows_out) {
-                const float sc = p.rows_scale;
-                uint2 v2;
-                v2.x = ptx::pack_bf16(sc * acc.x, sc * acc.y);
-                v2.y = ptx::pack_bf16(sc * acc.z, sc * acc.w);
-                *reinterpret_cast<uint2*>(p.rows_out + (size_t)b * p.rows_bstride + (size_t)m * p.rows_ld +
-                                          nt * kDeBN + 4 * c4) = v2;
-            } else if (m < p.M) {
+            if (m < p.M) {
                 const int i = m / p.gw, jj = m % p.gw;
                 __nv_bfloat16* lat =
                     p.latent + (size_t)b * p.C * plane + (size_t)(P * i) * p.Wl + (size_t)P * jj;
@@ -605,12 +791,22 @@ __global__ void __launch_bounds__(kThreads, 1)
     __syncthreads();
     if (warp == 2) {
         ptx::tc_fence_after();
-        ptx::tmem_dealloc(tbase, kDeBN);
+        ptx::tmem_dealloc(tbase, kTier ? 2 * kDeBN : kDeBN);
     }
 }
 
 constexpr int kDeSmem = kDeStages * (kChunkA + kDeBN * 128) + 1024;
+// With an adapter or residual: three stages, then two partial tiles, the up
+// projection and 128 / splits rows of codes in their space, so that two CTAs
+// share an SM (a 480p coarse state has 16 clusters of eight CTAs, and with one
+// CTA per SM only 15 of them ran at once: 21.7 us).
+constexpr int de_tier_smem(int splits) {
+    const int ring = kDeTierStages * (kChunkA + 2 * kDeBN * 128);
+    const int sums = (128 + 128 + 64 + 128 / splits) * kDePartStride * 4;
+    return (ring > sums ? ring : sums) + 1024;
+}
 static_assert(128 * kDePartStride * 4 <= kDeStages * (kChunkA + kDeBN * 128), "partial tile fits the ring");
+
 
 constexpr int kEmbedSmem = kEmbedStages * (kChunkA + kEmbedBN * 128) + 1024;
 
@@ -621,9 +817,8 @@ bool msp_embed_supported(const MspEmbedRun* runs, int n, int E) {
     for (int i = 0; i < n; ++i) {
         const MspEmbedRun& r = runs[i];
         if (r.K % 64 != 0 || r.P < 1 || 64 % r.P != 0 || ((uintptr_t)r.w & 15) || r.M <= 0) return false;
-        if (r.w_rows < 0 || r.w_rows > E) return false;
-        if (r.lora_up && (r.rank < 8 || r.rank > 64 || r.rank % 8 != 0 || !r.codes ||
-                          ((uintptr_t)r.lora_up & 15) || ((uintptr_t)r.codes & 15) || r.codes_bstride % 8))
+        if (r.lora_up && (r.rank < 8 || r.rank > 64 || r.rank % 8 != 0 || !r.lora_down ||
+                          ((uintptr_t)r.lora_up & 15) || ((uintptr_t)r.lora_down & 15)))
             return false;
     }
     return true;
@@ -634,24 +829,19 @@ cudaError_t launch_msp_embed(const MspEmbedRun* runs, int n, const MspShape& sh,
                              cudaStream_t st, const PoolBatch* pool, int pool_ctas) {
     EmbedMaps maps;
     memset(&maps, 0, sizeof(maps));
+    LoraMaps lmaps;
+    bool lora = false;
     EmbedParams p;
     memset(&p, 0, sizeof(p));
     int tiles = 0;
     for (int i = 0; i < n; ++i) {
         const MspEmbedRun& r = runs[i];
-        if (!encode_2d(&maps.w[i], r.w, r.K, r.w_rows > 0 ? r.w_rows : E, (long long)r.K * 2, 64, kEmbedBN))
-            return cudaErrorInvalidValue;
+        const int bn = r.lora_up ? kLoraBN : kEmbedBN;
+        if (!encode_2d(&maps.w[i], r.w, r.K, E, (long long)r.K * 2, 64, bn)) return cudaErrorInvalidValue;
         if (r.lora_up) {
-            EncodeTiledFn enc = encoder();
-            if (!encode_2d(&maps.up[i], r.lora_up, r.rank, E, (long long)r.rank * 2, 64, kEmbedBN))
-                return cudaErrorInvalidValue;
-            cuuint64_t dims[3] = {64, (cuuint64_t)r.M, (cuuint64_t)batch};
-            cuuint64_t strides[2] = {128, (cuuint64_t)r.codes_bstride * 2};
-            cuuint32_t box[3] = {64, 128, 1};
-            cuuint32_t es[3] = {1, 1, 1};
-            if (!enc || enc(&maps.codes[i], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(r.codes), dims,
-                            strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-                            CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+            lora = true;
+            if (!encode_2d(&lmaps.up[i], r.lora_up, r.rank, E, (long long)r.rank * 2, 64, bn) ||
+                !encode_2d(&lmaps.down[i], r.lora_down, r.K, r.rank, (long long)r.K * 2, 64, 64))
                 return cudaErrorInvalidValue;
         }
         {
@@ -677,10 +867,9 @@ cudaError_t launch_msp_embed(const MspEmbedRun* runs, int n, const MspShape& sh,
         R.K = r.K;
         R.tok_off = r.tok_off;
         R.lora = r.lora_up ? 1 : 0;
-        R.scale = r.scale;
-        tiles += R.m_tiles * ((E + kEmbedBN - 1) / kEmbedBN);
+        R.scale = r.lora_scale;
+        tiles += R.m_tiles * ((E + bn - 1) / bn);
     }
-    p.n_tiles_n = (E + kEmbedBN - 1) / kEmbedBN;
     p.n_runs = n;
     p.T = sh.T;
     p.C = sh.C;
@@ -691,7 +880,9 @@ cudaError_t launch_msp_embed(const MspEmbedRun* runs, int n, const MspShape& sh,
     p.tokens = (__nv_bfloat16*)tokens;
     p.tok_bstride = tok_bstride;
     p.status = status;
-    cudaError_t e = set_smem_attr((const void*)msp_embed_kernel, kEmbedSmem, 100);
+    if (lora && pool && pool->n > 0) return cudaErrorInvalidValue;  // no caller pools beside adapters
+    const void* fn = lora ? (const void*)msp_embed_kernel<true, LoraMaps> : (const void*)msp_embed_kernel<false, NoLora>;
+    cudaError_t e = set_smem_attr(fn, kEmbedSmem, 100);
     if (e != cudaSuccess) return e;
     p.n_embed_tiles = tiles;
     PoolBatch pb;
@@ -704,8 +895,9 @@ cudaError_t launch_msp_embed(const MspEmbedRun* runs, int n, const MspShape& sh,
     } else {
         memset(&pb, 0, sizeof(pb));
     }
-    return launch_pdl(msp_embed_kernel, dim3((unsigned)(tiles + p.pool_ctas), 1, (unsigned)batch), dim3(kThreads),
-                      kEmbedSmem, st, maps, p, pb);
+    const dim3 grid((unsigned)(tiles + p.pool_ctas), 1, (unsigned)batch);
+    return lora ? launch_pdl(msp_embed_kernel<true, LoraMaps>, grid, dim3(kThreads), kEmbedSmem, st, maps, p, pb, lmaps)
+                : launch_pdl(msp_embed_kernel<false, NoLora>, grid, dim3(kThreads), kEmbedSmem, st, maps, p, pb, NoLora{});
 }
 
 
@@ -733,42 +925,25 @@ cudaError_t launch_msp_deembed(const void* tokens, long long tok_bstride_elems, 
     if (!encode_2d(&maps.b, w_out, E, F, (long long)E * 2, 64, kDeBN)) return cudaErrorInvalidValue;
     const bool lora = tier && tier->up;
     const bool res = tier && tier->residual;
-    if (lora) {
-        EncodeTiledFn enc = encoder();
-        cuuint64_t dims[3] = {64, (cuuint64_t)tok_rows, (cuuint64_t)batch};
-        cuuint64_t strides[2] = {128, (cuuint64_t)tier->codes_bstride * 2};
-        cuuint32_t box[3] = {64, 128, 1};
-        cuuint32_t es[3] = {1, 1, 1};
-        if (!enc || enc(&maps.codes, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(tier->codes), dims,
-                        strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-                        CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-            return cudaErrorInvalidValue;
-        if (!encode_2d(&maps.up, tier->up, tier->rank, F, (long long)tier->rank * 2, 64, kDeBN))
-            return cudaErrorInvalidValue;
-    }
-    if (res) {
-        EncodeTiledFn enc = encoder();
-        cuuint64_t dims[3] = {(cuuint64_t)F, (cuuint64_t)M, (cuuint64_t)batch};
-        cuuint64_t strides[2] = {(cuuint64_t)F * 2, (cuuint64_t)tier->xraw_bstride * 2};
-        cuuint32_t box[3] = {64, 128, 1};
-        cuuint32_t es[3] = {1, 1, 1};
-        if (!enc || enc(&maps.xraw, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(tier->xraw), dims,
-                        strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-                        CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-            return cudaErrorInvalidValue;
-        if (!encode_2d(&maps.res, tier->residual, F, F, (long long)F * 2, 64, kDeBN)) return cudaErrorInvalidValue;
-    }
-    const int nk_all = E / 64 + (lora ? 1 : 0) + (res ? F / 64 : 0);
-    // The largest power of two <= 8 that leaves each split at least one K chunk.
-    int splits = 8;
+    if (lora && !encode_2d(&maps.down, tier->down, E, tier->rank, (long long)E * 2, 64, kDeBN))
+        return cudaErrorInvalidValue;
+    if (res && !encode_2d(&maps.res, tier->residual, F, F, (long long)F * 2, 64, kDeBN)) return cudaErrorInvalidValue;
+    const int nk_all = E / 64 + (res ? F / 64 : 0);
+    // Splits (the cluster size) by the number of clusters: one wave. At most 15
+    // clusters of eight CTAs and about 36 of four run at once on 152 SMs (72
+    // without extras, two CTAs per SM); measured at E 1536, eight / four / two /
+    // one: 13 tiles 5.6 / 6.5 / 9.6 / 15.0 us, 26 8.0 / 6.7 / 9.8 / 15.1, 52 14.6 /
+    // 9.1 / 10.0 / 15.3, 111 27.3 / 17.8 / 13.7 / 15.5; with extras 16 tiles 10.5 /
+    // 10.2 / 14.8 / 24.8, 40 20.3 / 16.1 / 15.1 / 25.0, 120 45.0 / 29.5 / 24.9 / 25.6.
+    // Each split keeps at least one K chunk.
+    const int clusters = (M + 127) / 128 * (F / kDeBN) * batch;
+    int splits = clusters <= 15 ? 8 : clusters <= (lora || res ? 36 : 72) ? 4 : clusters <= 152 ? 2 : 1;
     while (splits > 1 && splits > nk_all) splits /= 2;
     DeembedParams p;
     memset(&p, 0, sizeof(p));
     p.M = M;
     p.K = E;
     p.nk_all = nk_all;
-    p.lora = lora ? 1 : 0;
-    p.nk_res = res ? F / 64 : 0;
     p.m_tiles = (M + 127) / 128;
     p.splits = splits;
     p.P = P;
@@ -779,52 +954,25 @@ cudaError_t launch_msp_deembed(const void* tokens, long long tok_bstride_elems, 
     p.tok_row0 = tok_row0;
     p.latent = (__nv_bfloat16*)latent;
     p.status = status;
-    cudaError_t e = set_smem_attr((const void*)msp_deembed_kernel, kDeSmem);
-    if (e != cudaSuccess) return e;
     const dim3 grid((unsigned)(p.m_tiles * (F / kDeBN)), (unsigned)splits, (unsigned)batch);
-    return launch_pdl_cluster(msp_deembed_kernel, grid, dim3(kThreads), kDeSmem, st, dim3(1, splits, 1), maps, p);
-}
-
-cudaError_t launch_msp_rows_splitk(const void* tokens, long long tok_bstride_elems, int tok_rows, int tok_row0,
-                                   const void* w, int w_rows, int M, int E, void* out, long long out_bstride,
-                                   int out_ld, float scale, int batch, unsigned int* status, cudaStream_t st) {
-    DeembedMaps maps;
-    memset(&maps, 0, sizeof(maps));
-    EncodeTiledFn enc = encoder();
-    if (!enc) return cudaErrorNotSupported;
-    {
-        cuuint64_t dims[3] = {(cuuint64_t)E, (cuuint64_t)tok_rows, (cuuint64_t)batch};
-        cuuint64_t strides[2] = {(cuuint64_t)E * 2, (cuuint64_t)tok_bstride_elems * 2};
-        cuuint32_t box[3] = {64, 128, 1};
-        cuuint32_t es[3] = {1, 1, 1};
-        if (enc(&maps.a, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(tokens), dims, strides, box, es,
-                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-            return cudaErrorInvalidValue;
+    const dim3 cluster(1, (unsigned)splits, 1);
+    if (lora || res) {
+        DeembedTierParams tp;
+        memset(&tp, 0, sizeof(tp));
+        tp.rank = lora ? tier->rank : 0;
+        tp.scale = tier->scale;
+        tp.up = (const __nv_bfloat16*)tier->up;
+        tp.latent = (const __nv_bfloat16*)tier->latent;
+        tp.latent_bstride = tier->latent_bstride;
+        cudaError_t e = set_smem_attr((const void*)msp_deembed_kernel<true, DeembedTierParams>, de_tier_smem(1), 100);
+        if (e != cudaSuccess) return e;
+        return launch_pdl_cluster(msp_deembed_kernel<true, DeembedTierParams>, grid, dim3(kThreads),
+                                  de_tier_smem(splits), st, cluster, maps, p, tp);
     }
-    if (!encode_2d(&maps.b, w, E, w_rows, (long long)E * 2, 64, kDeBN)) return cudaErrorInvalidValue;
-    const int nk_all = E / 64;
-    int splits = 8;
-    while (splits > 1 && splits > nk_all) splits /= 2;
-    DeembedParams p;
-    memset(&p, 0, sizeof(p));
-    p.M = M;
-    p.K = E;
-    p.nk_all = nk_all;
-    p.m_tiles = (M + 127) / 128;
-    p.splits = splits;
-    p.P = 1;
-    p.gw = 1;
-    p.tok_row0 = tok_row0;
-    p.status = status;
-    p.rows_out = (__nv_bfloat16*)out;
-    p.rows_bstride = out_bstride;
-    p.rows_ld = out_ld;
-    p.rows_scale = scale;
-    cudaError_t e = set_smem_attr((const void*)msp_deembed_kernel, kDeSmem);
+    cudaError_t e = set_smem_attr((const void*)msp_deembed_kernel<false, NoTier>, kDeSmem);
     if (e != cudaSuccess) return e;
-    const dim3 grid((unsigned)p.m_tiles, (unsigned)splits, (unsigned)batch);
-    return launch_pdl_cluster(msp_deembed_kernel, grid, dim3(kThreads), kDeSmem, st, dim3(1, splits, 1), maps, p);
+    return launch_pdl_cluster(msp_deembed_kernel<false, NoTier>, grid, dim3(kThreads), kDeSmem, st, cluster, maps, p,
+                              NoTier{});
 }
 
 }  // namespace msf
