@@ -141,7 +141,10 @@ __global__ void __launch_bounds__(kThreads, 1)
     unsigned char* smem = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     unsigned char* sQ = smem;                // [3] planes h, m, l
     unsigned char* sR = smem + 3 * C::kTile;  // [kRing]
-    __shared__ uint64_t q_full, full[kRing], empty[kRing], s_full, p_full, o_full, meet_bar, drain_bar;
+    __shared__ uint64_t q_full, full[kRing], empty[kRing], p_full, o_full, meet_bar, drain_bar;
+    // Scores ready, per S buffer: S of tile j + 1 may be ready before a softmax
+    // warp has looked for tile j's, so one barrier could run two phases ahead.
+    __shared__ uint64_t s_full[2];
     __shared__ float sx[2][kBM];  // row maxima, at the end row sums, of the two column halves
     __shared__ uint32_t tmem_base_sh;
     __shared__ int abort_flag;
@@ -167,7 +170,8 @@ __global__ void __launch_bounds__(kThreads, 1)
             ptx::mbar_init(&full[s], 1);
             ptx::mbar_init(&empty[s], 1);
         }
-        ptx::mbar_init(&s_full, 1);
+        ptx::mbar_init(&s_full[0], 1);
+        ptx::mbar_init(&s_full[1], 1);
         ptx::mbar_init(&p_full, 8);
         ptx::mbar_init(&o_full, 1);
         ptx::mbar_init(&meet_bar, 8);
@@ -276,7 +280,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                         }
                     }
                     ptx::mma_commit(&empty[st]);
-                    if (kp == 0) ptx::mma_commit(&s_full);
+                    if (kp == 0) ptx::mma_commit(&s_full[j & 1]);
                 }
                 __syncwarp();
             }
@@ -345,7 +349,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         for (int j = 0; j < n && ok; ++j) {
             int map, row, valid;
             tile_of(u0 + j, map, row, valid);
-            ok = __all_sync(0xffffffffu, ptx::mbar_wait_bounded(&s_full, (uint32_t)(j & 1), abort_p, p.wait_limit));
+            ok = __all_sync(0xffffffffu, ptx::mbar_wait_bounded(&s_full[j & 1], (uint32_t)((j >> 1) & 1), abort_p, p.wait_limit));
             if (!ok) break;
             ptx::tc_fence_after();
             const uint32_t tS = tbase + (uint32_t)((j & 1) * kSBuf) + 64 * half + lane_off;
