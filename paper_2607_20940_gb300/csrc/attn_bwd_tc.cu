@@ -111,7 +111,9 @@ struct BwdMaps {
 struct BwdBars {
     // dq items: Q and dO, the K and V rings, S + dP ready, dP read, dS written, dQ complete
     uint64_t qg_full, qg_empty, k_full[3], k_empty[3], v_full[2], v_empty[2];
-    uint64_t sdp_full, dp_free, ds_full, dq_full;
+    // (ds_full by tile parity: dP_{j+1} may be read by one warp before another
+    // has written dS_j)
+    uint64_t sdp_full, dp_free, ds_full[2], dq_full;
     // dk/dv items: K, V, the Q and dO rings, S^T ready, P^T written, dP^T
     // ready, dS^T written, dV and dK complete; the warps of a half meet
     uint64_t kst_full, kst_empty, vst_full, vst_empty, q_full[3], q_empty[3], g_full[2], g_empty[2];
@@ -274,7 +276,8 @@ __global__ void __launch_bounds__(kThreads, 1)
             ptx::mbar_init(&bar.meet[s], 4);
         }
         ptx::mbar_init(&bar.dp_free, 8);
-        ptx::mbar_init(&bar.ds_full, 8);
+        ptx::mbar_init(&bar.ds_full[0], 8);
+        ptx::mbar_init(&bar.ds_full[1], 8);
         ptx::mbar_init(&bar.p_full, 8);
         ptx::mbar_init(&bar.dst_full, 8);
         ptx::mbar_init(&bar.item_done, 8);
@@ -468,10 +471,11 @@ __global__ void __launch_bounds__(kThreads, 1)
                     // landed yet, dQ_j goes first and S_{j+2} after its own wait.
                     bool k_ready;
                     {
-                        const bool rs = ptx::mbar_try_wait(&bar.ds_full, par);
+                        const uint32_t dpar = (uint32_t)((tq >> 1) & 1);
+                        const bool rs = ptx::mbar_try_wait(&bar.ds_full[par], dpar);
                         k_ready = !next2 || ptx::mbar_try_wait(k_full(j + 2), k_par(j + 2));
                         k_ready = __all_sync(0xffffffffu, k_ready);
-                        if (!__all_sync(0xffffffffu, rs)) ok = wait_all(&bar.ds_full, par);
+                        if (!__all_sync(0xffffffffu, rs)) ok = wait_all(&bar.ds_full[par], dpar);
                     }
                     if (!ok) break;
                     ptx::tc_fence_after();
@@ -663,7 +667,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                     }
                     ptx::tmem_wait_st();
                     ptx::tc_fence_before();
-                    arrive(&bar.ds_full);
+                    arrive(&bar.ds_full[tq & 1]);
                 }
                 ok = ok && wait_all(&bar.dq_full, (uint32_t)(iq & 1));
                 if (!ok) break;
