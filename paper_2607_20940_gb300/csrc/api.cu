@@ -765,7 +765,7 @@ extern "C" msf_status msf_patchify_resample(msf_plan_t plan, const void* latent,
     const msf::MspShape sh = msp_shape(p);
     const int E = p.d.embed_dim;
     msf::MspEmbedRun runs[MSF_MAX_STATES];
-    int n_runs = 0, tiles = 0;
+    int n_runs = 0;
     for (int l0 = 0; l0 < p.T;) {
         int l1 = l0 + 1;
         while (l1 < p.T && p.d.scales[l1] == p.d.scales[l0] && w_tier[l1] == w_tier[l0]) ++l1;
@@ -778,7 +778,6 @@ extern "C" msf_status msf_patchify_resample(msf_plan_t plan, const void* latent,
         r.M = p.st_off[l1 - 1] + p.st_n[l1 - 1] - p.st_off[l0];
         r.gw = sh.Wl / r.P;
         r.tok_off = p.st_off[l0];
-        if (n_runs <= msf::kMaxGemmProblems) tiles += ((r.M + 127) / 128) * ((E + 255) / 256);
         l0 = l1;
     }
     // Runs with the widest patch vectors (most K chunks, the longest tiles)
@@ -798,20 +797,12 @@ extern "C" msf_status msf_patchify_resample(msf_plan_t plan, const void* latent,
     jb.row_vecs = (int)(row_bytes(p) / 16);
     jb.mode = p.d.resample;
     add_window_jobs(p, k_win, v_win, with_hist, jb);
-    // Pool CTAs per stream: one 256-thread block per 256 tasks, as the pool
-    // kernel launches them, after the embedding tiles in the grid (the
-    // longest tiles, those of the widest patch vectors, first).
-    int max_n = 0;
-    for (int k = 0; k < jb.n; ++k) max_n = jb.j[k].out_n > max_n ? jb.j[k].out_n : max_n;
-    long long pool_ctas = ((long long)jb.n * max_n * (jb.row_vecs / 2) + 255) / 256;
-    if (pool_ctas < 1) pool_ctas = 1;
-    (void)tiles;
     cudaError_t e = cudaSuccess;
     cudaStream_t s = (cudaStream_t)stream;
     for (int r0 = 0; r0 < n_runs; r0 += msf::kMaxGemmProblems) {
         const int n = n_runs - r0 < msf::kMaxGemmProblems ? n_runs - r0 : msf::kMaxGemmProblems;
         e = msf::launch_msp_embed(runs + r0, n, sh, E, latent, tokens, (long long)p.N * E, p.B, msf::status_word(p), s,
-                                  r0 == 0 && jb.n > 0 ? &jb : nullptr, (int)pool_ctas);
+                                  r0 == 0 && jb.n > 0 ? &jb : nullptr);
         if (e != cudaSuccess) return cuda_status(e);
     }
     return MSF_OK;

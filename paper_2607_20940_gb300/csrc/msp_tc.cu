@@ -138,6 +138,8 @@ struct EmbedRun {
     int tok_off;    // first token row of the run in the output
     int lora;       // 1: one more K chunk (LoRA codes x up projection), 192-column tiles
     float scale;    // LoRA scale
+    int pool_base;  // first pyramid task of this run's tiles, and tasks of each
+    int pool_per;   // thread of their two idle warps (0: none)
 };
 struct EmbedParams {
     int n_runs;
@@ -146,6 +148,7 @@ struct EmbedParams {
     int n_embed_tiles;  // CTAs [0, n_embed_tiles) of a stream embed; the rest pool
     int pool_ctas;      // CTAs per stream that run the pyramid jobs (0: none)
     int pool_tasks;     // vector-pair tasks per pyramid job
+    int pool_first;     // first task of those CTAs (the tiles' idle warps run the others)
     const __nv_bfloat16* latent;  // [B, T, C, Hl, Wl]
     __nv_bfloat16* tokens;        // [B, N, E]
     long long tok_bstride;        // elements
@@ -186,7 +189,8 @@ __global__ void __launch_bounds__(kThreads, 2)
         ptx::grid_dep_launch();
         const int stride = p.pool_ctas * kThreads;
         const int total = pool.n * p.pool_tasks;
-        for (int t = ((int)blockIdx.x - p.n_embed_tiles) * kThreads + (int)threadIdx.x; t < total; t += stride)
+        for (int t = p.pool_first + ((int)blockIdx.x - p.n_embed_tiles) * kThreads + (int)threadIdx.x; t < total;
+             t += stride)
             pool_task<__nv_bfloat16>(pool, t / p.pool_tasks, blockIdx.z, t % p.pool_tasks);
         return;
     }
@@ -310,7 +314,15 @@ __global__ void __launch_bounds__(kThreads, 2)
         if (ptx::elect_one_sync()) ptx::mma_commit(&acc_full);  // also after an abort: drains the MMAs
         __syncwarp();
         if (!ok && lane == 0) atomicOr(p.status, kDevTimeout);
-    } else if (warp >= 4) {
+    } else if (warp < 4) {
+        // ---- warps 2 and 3: this tile's share of the pyramid jobs
+        if constexpr (!kLora) {
+            const int total = pool.n * p.pool_tasks;
+            int t = R.pool_base + local * 64 * R.pool_per + (int)threadIdx.x - 64;
+            for (int k = 0; k < R.pool_per && t < total; ++k, t += 64)
+                pool_task<__nv_bfloat16>(pool, t / p.pool_tasks, blockIdx.z, t % p.pool_tasks);
+        }
+    } else {
         // ---- gather: one token row per thread
         const int r = (warp - 4) * 32 + lane;
         const int m = mt * 128 + r;
@@ -826,7 +838,7 @@ bool msp_embed_supported(const MspEmbedRun* runs, int n, int E) {
 
 cudaError_t launch_msp_embed(const MspEmbedRun* runs, int n, const MspShape& sh, int E, const void* latent,
                              void* tokens, long long tok_bstride, int batch, unsigned int* status,
-                             cudaStream_t st, const PoolBatch* pool, int pool_ctas) {
+                             cudaStream_t st, const PoolBatch* pool) {
     EmbedMaps maps;
     memset(&maps, 0, sizeof(maps));
     LoraMaps lmaps;
@@ -891,7 +903,35 @@ cudaError_t launch_msp_embed(const MspEmbedRun* runs, int n, const MspShape& sh,
         int max_n = 0;
         for (int k = 0; k < pb.n; ++k) max_n = pb.j[k].out_n > max_n ? pb.j[k].out_n : max_n;
         p.pool_tasks = max_n * (pb.row_vecs / 2);
-        p.pool_ctas = pool_ctas > 0 ? pool_ctas : 1;
+        const long long total = (long long)pb.n * p.pool_tasks;
+        // The tiles' idle warps take tasks while the pool CTAs do not all start
+        // at once (two CTAs per SM): one a thread on tiles of one K chunk and
+        // three on longer ones, or two and four, up to a third or a quarter of
+        // all tasks, so that no tile waits for them. Launch, us, none / one and
+        // three / two and four: 480p with the history 16.2 / 16.1 / 14.7, window
+        // only 11.5 / 10.9 / 11.7, four streams 79.8 / 74.4 / 72.5 and 51.8 / 46.8
+        // / 45.4; where every pool CTA starts at once they only cost (6.6 / 7.0 /
+        // 7.6).
+        auto share_of = [&](int one, int more) {
+            long long x = 0;
+            for (int i = 0; i < n; ++i)
+                x += 64ll * (p.run[i].K <= 64 ? one : more) * ((i + 1 < n ? p.run[i + 1].tile_base : tiles) - p.run[i].tile_base);
+            return x;
+        };
+        int one = 0, more = 0;
+        if (batch * (tiles + (total + kThreads - 1) / kThreads) > 2 * 152) {
+            if (4 * share_of(2, 4) <= total)
+                one = 2, more = 4;
+            else if (3 * share_of(1, 3) <= total)
+                one = 1, more = 3;
+        }
+        for (int i = 0; i < n && one > 0; ++i) {
+            EmbedRun& R = p.run[i];
+            R.pool_base = p.pool_first;
+            R.pool_per = R.K <= 64 ? one : more;
+            p.pool_first += 64 * R.pool_per * ((i + 1 < n ? p.run[i + 1].tile_base : tiles) - R.tile_base);
+        }
+        p.pool_ctas = (int)((total - p.pool_first + kThreads - 1) / kThreads);
     } else {
         memset(&pb, 0, sizeof(pb));
     }

@@ -29,12 +29,12 @@ struct MspEmbedRun {
 
 bool msp_embed_supported(const MspEmbedRun* runs, int n, int E);
 // Up to kMaxGemmProblems runs in one launch. With `pool` (bf16 jobs) the
-// same launch also runs those K/V pyramid jobs on `pool_ctas` more CTAs per
-// stream after the embedding tiles: they read and write buffers the
-// embedding does not touch, so the two share the SMs of one launch.
+// same launch also runs those K/V pyramid jobs, on more CTAs after the
+// embedding tiles and on the tiles' idle warps: they read and write buffers
+// the embedding does not touch, so the two share the SMs of one launch.
 cudaError_t launch_msp_embed(const MspEmbedRun* runs, int n, const MspShape& sh, int E, const void* latent,
                              void* tokens, long long tok_bstride, int batch, unsigned int* status,
-                             cudaStream_t st, const PoolBatch* pool = nullptr, int pool_ctas = 0);
+                             cudaStream_t st, const PoolBatch* pool = nullptr);
 
 // The coarse tier's extras of a de-embedding (Sec. 4.1), computed in the same
 // launch.
