@@ -75,7 +75,6 @@ struct FBClass {
     int slot_base;  // first partial slot (n_split > 1)
     int item_base;  // first own tile of the merge launch (n_split > 1)
 };
-constexpr int kMaxClasses = 3 * MSF_MAX_GROUPS;
 struct FBParams {
     int H, B, N, R;
     float scale, scale_log2;
@@ -91,7 +90,7 @@ struct FBParams {
     unsigned int* status;
     long long wait_limit;
     int n_classes;
-    FBClass c[kMaxClasses];  // longest units first
+    FBClass c[kMaxF32Classes];  // longest units first
     FBGroup g[MSF_MAX_GROUPS];
 };
 
@@ -651,30 +650,13 @@ msf_status launch_bwd_f32_tc(msf_plan_t plan, const BwdCommon& c, const AttnArgs
             fp.c[fp.n_classes++] = {kDv, gi, kt, n_qt};
         }
     }
-    // Units per own tile, as in the forward (a dV tile counts like the others).
+    // Units per own tile (a dV tile costs what a forward tile does).
     const int HB = P.H * P.B, max_slots = f32_max_slots(P);
-    {
-        long long total = 0;
-        int longest = 0;
-        for (int i = 0; i < fp.n_classes; ++i) {
-            total += (long long)fp.c[i].n_own * HB * fp.c[i].n_tiles;
-            longest = fp.c[i].n_tiles > longest ? fp.c[i].n_tiles : longest;
-        }
-        const double T = (double)total / sms;
-        int len = f32_unit_tiles(T);
-        const bool one_round = len >= T;
-        for (;; ++len) {
-            long long units = 0, slots = 0;
-            for (int i = 0; i < fp.n_classes; ++i) {
-                FBClass& cl = fp.c[i];
-                cl.n_split = (cl.n_tiles + len - 1) / len;
-                const long long u = (long long)cl.n_own * HB * cl.n_split;
-                units += u;
-                slots += cl.n_split > 1 ? u : 0;
-            }
-            if (len >= longest || (slots <= max_slots && (!one_round || units <= sms))) break;
-        }
-    }
+    F32Class cls[kMaxF32Classes];
+    for (int i = 0; i < fp.n_classes; ++i)
+        cls[i] = {(long long)fp.c[i].n_own * HB, fp.c[i].n_tiles, fp.c[i].kind == kDv ? 1.0 : 1.5};
+    const int len = f32_unit_tiles(cls, fp.n_classes, P.D, sms, max_slots);
+    for (int i = 0; i < fp.n_classes; ++i) fp.c[i].n_split = (fp.c[i].n_tiles + len - 1) / len;
     // Longest units first (a dV tile is two thirds of the others' MMAs).
     auto cost = [](const FBClass& x) { return (double)x.n_tiles / x.n_split * (x.kind == kDv ? 2 : 3); };
     for (int i = 0; i < fp.n_classes; ++i)

@@ -513,43 +513,108 @@ __global__ void __launch_bounds__(256) merge_f32_kernel(const __grid_constant__ 
 
 // ---------------------------------------------------------------- host side
 
-// Units per query tile (f32_unit_tiles), within the partial slots; with one
-// round of units per SM every unit has to start at once, so units grow until
-// they fit.
-void choose_splits(FParams& p, int sms, int max_slots) {
-    long long total = 0;
-    int longest = 0;
-    for (int i = 0; i < p.n_groups; ++i) {
-        total += (long long)p.g[i].n_qt * p.H * p.B * p.g[i].n_tiles;
-        longest = p.g[i].n_tiles > longest ? p.g[i].n_tiles : longest;
-    }
-    const double T = (double)total / sms;
-    int len = f32_unit_tiles(T);
-    const bool one_round = len >= T;
-    for (;; ++len) {
-        long long units = 0, slots = 0;
-        for (int i = 0; i < p.n_groups; ++i) {
-            FGroup& g = p.g[i];
-            g.n_split = (g.n_tiles + len - 1) / len;
-            const long long u = (long long)g.n_qt * p.H * p.B * g.n_split;
-            units += u;
-            slots += g.n_split > 1 ? u : 0;
-        }
-        if (len >= longest || (slots <= max_slots && (!one_round || units <= sms))) return;
-    }
-}
-
 }  // namespace
 
-// T tiles per SM in all: a unit costs about two tiles besides its own (the
-// resident planes, the pipeline's start, the read-out and merge), and the last
-// of k rounds of units leaves the SMs half a unit idle on average, T / 2k
-// tiles: k = sqrt(T / 4) rounds cost least.
-int f32_unit_tiles(double T) {
-    int k = (int)(sqrt(T / 4.0) + 0.5);
-    k = k < 1 ? 1 : k > kF32MaxRounds ? kF32MaxRounds : k;
-    const int len = (int)ceil(T / k);
-    return len < 2 ? 2 : len;
+
+// The limit with the earliest estimated end: the units placed longest first on
+// the least loaded SM, a unit costing 2 tiles besides its own (the resident
+// planes, the pipeline's start, the read-out; D = 64 tiles take half as long:
+// 4) and 0.7 more if it writes a partial result, and the merge. Tried: no
+// split, one to six units per SM, and the longest that starts all at once.
+// Against one split rule (as many rounds as sqrt(tiles per SM / 4)): 480p
+// forward 833 -> 775 us, gradient of a small window (1008 tokens) 127 -> 86.
+int f32_unit_tiles(const F32Class* c, int n, int D, int sms, int max_slots) {
+    double total = 0;
+    int longest = 1;
+    for (int i = 0; i < n; ++i) {
+        total += c[i].items * c[i].n_tiles * c[i].weight;
+        longest = c[i].n_tiles > longest ? c[i].n_tiles : longest;
+    }
+    const double own = D == 64 ? 4.0 : 2.0;
+    struct Level {
+        double load;
+        long long count;
+    };
+    auto estimate = [&](int len) -> double {
+        struct U {
+            double cost;
+            long long n;
+        } u[kMaxF32Classes];
+        long long slots = 0;
+        for (int i = 0; i < n; ++i) {
+            const int ns = (c[i].n_tiles + len - 1) / len;
+            u[i] = {(double)((c[i].n_tiles + ns - 1) / ns) * c[i].weight + own + (ns > 1 ? 0.7 : 0.0), c[i].items * ns};
+            if (ns > 1) slots += u[i].n;
+        }
+        if (slots > max_slots) return 1e30;
+        for (int i = 0; i < n; ++i)
+            for (int k = i + 1; k < n; ++k)
+                if (u[k].cost > u[i].cost) {
+                    const U t = u[i];
+                    u[i] = u[k];
+                    u[k] = t;
+                }
+        // SMs by load, equal loads together, lightest first
+        Level lv[64] = {{0.0, sms}};
+        int nl = 1;
+        double end = 0;
+        for (int i = 0; i < n; ++i)
+            while (u[i].n > 0) {
+                // many rounds: whole rounds over every SM do not change their order
+                if (u[i].n >= 4ll * sms) {
+                    const long long r = u[i].n / sms - 2;
+                    for (int k = 0; k < nl; ++k) lv[k].load += r * u[i].cost;
+                    u[i].n -= r * sms;
+                    continue;
+                }
+                const long long m = u[i].n < lv[0].count ? u[i].n : lv[0].count;
+                const double load = lv[0].load + u[i].cost;
+                u[i].n -= m;
+                lv[0].count -= m;
+                if (lv[0].count == 0) {
+                    for (int k = 1; k < nl; ++k) lv[k - 1] = lv[k];
+                    --nl;
+                }
+                int at = 0;
+                while (at < nl && lv[at].load < load) ++at;
+                if (at < nl && lv[at].load == load) {
+                    lv[at].count += m;
+                } else if (nl < 64) {
+                    for (int k = nl; k > at; --k) lv[k] = lv[k - 1];
+                    lv[at] = {load, m};
+                    ++nl;
+                } else {
+                    lv[at < nl ? at : nl - 1].count += m;
+                }
+                end = load > end ? load : end;
+            }
+        for (int k = 0; k < nl; ++k) end = lv[k].load > end ? lv[k].load : end;
+        return end + (slots > 0 ? 1.0 + 0.006 * (double)slots : 0.0);
+    };
+    int best = longest;
+    double least = estimate(longest);
+    auto try_len = [&](int len) {
+        len = len < 1 ? 1 : len;
+        if (len >= longest) return;
+        const double e = estimate(len);
+        if (e < least) {
+            least = e;
+            best = len;
+        }
+    };
+    for (int k = 1; k <= kF32MaxRounds; ++k) try_len((int)ceil(total / sms / k));
+    // all at once: the shortest limit whose units fit the SMs
+    for (int lo = 1, hi = longest; lo < hi;) {
+        const int mid = (lo + hi) / 2;
+        long long units = 0;
+        for (int i = 0; i < n; ++i) units += c[i].items * ((c[i].n_tiles + mid - 1) / mid);
+        if (units <= sms)
+            hi = mid;
+        else
+            lo = mid + 1;
+        if (lo >= hi) try_len(hi);
+    }
+    return best;
 }
 
 bool add_planes(const Plan& P, SplitParams& sp, const void* src, long long src_bstride_bytes, char* dst, int alloc,
@@ -646,7 +711,10 @@ msf_status launch_attn_f32_tc(msf_plan_t plan, const AttnArgs& a, cudaStream_t s
     fp.flags = sp.flags;
     fp.status = a.status;
     fp.wait_limit = kWaitLimit;
-    choose_splits(fp, sms, f32_max_slots(P));
+    F32Class cls[MSF_MAX_GROUPS];
+    for (int i = 0; i < fp.n_groups; ++i) cls[i] = {(long long)fp.g[i].n_qt * P.H * P.B, fp.g[i].n_tiles, 1.0};
+    const int len = f32_unit_tiles(cls, fp.n_groups, P.D, sms, f32_max_slots(P));
+    for (int i = 0; i < fp.n_groups; ++i) fp.g[i].n_split = (fp.g[i].n_tiles + len - 1) / len;
     // longest units first
     for (int i = 0; i < fp.n_groups; ++i)
         for (int k = i + 1; k < fp.n_groups; ++k)

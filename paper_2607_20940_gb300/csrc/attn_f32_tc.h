@@ -39,8 +39,17 @@ bool add_planes(const Plan& P, SplitParams& sp, const void* src, long long src_b
 bool add_context_planes(const Plan& P, const AttnArgs& a, SplitParams& sp, F32Maps& maps);
 // Write the planes and the flags; *n_flags is the number of flag words.
 cudaError_t launch_split_planes(const SplitParams& sp, int* n_flags, cudaStream_t st);
-// K/V tiles per unit of work: see the definition.
-int f32_unit_tiles(double tiles_per_sm);
+// A class of equal own tiles (query tiles of a group, gradient rows of one) and
+// the other tiles each walks; `weight`: the cost of one, K/V tile = 1.
+constexpr int kMaxF32Classes = 3 * MSF_MAX_GROUPS;
+struct F32Class {
+    long long items;
+    int n_tiles;
+    double weight;
+};
+// The most tiles a unit of work may have (a tile of more is split evenly over
+// several units, with a partial slot each): see the definition.
+int f32_unit_tiles(const F32Class* c, int n, int D, int sms, int max_slots);
 
 // The fp32 attention of `a` (a plan with fp32 tensors, workspace bound): the
 // operands split into bf16 planes, the tensor-core kernel, the merge of split

@@ -118,8 +118,8 @@ inline size_t f32_plane_bytes(const Plan& p) {
     for (int i = kF32Sink; i <= kF32Win; ++i) n += 2 * f32_part_bytes(p, i);
     return n;
 }
-// Units are at least half as long as the rounds ask for, so kF32MaxRounds
-// rounds make at most twice as many per SM, and never more than K/V tiles.
+// Partial slots: twice kF32MaxRounds units per SM, and never more than K/V
+// tiles; the choice of the units stays within them.
 inline int f32_max_slots(const Plan& p) {
     const long long n = 2ll * kF32MaxRounds * kF32MaxSms;
     return (int)(p.f32_tiles < n ? p.f32_tiles : n);
