@@ -549,6 +549,7 @@ __global__ void __launch_bounds__(256) bwd_f32_merge_kernel(const __grid_constan
         float acc[E];
 #pragma unroll
         for (int e = 0; e < E; ++e) acc[e] = 0.f;
+#pragma unroll 4
         for (int i = 0; i < cl.n_split; ++i) {
             const float* s = first + i * step + r * D + E * lane;
             if (E == 4) {

@@ -479,25 +479,38 @@ __global__ void __launch_bounds__(256) merge_f32_kernel(const __grid_constant__ 
     for (int r = threadIdx.x / 32 + 16 * blockIdx.y; r < 16 * (blockIdx.y + 1); r += 8) {
         const int q = G.q_begin + qt * kBM + r;
         if (q >= G.q_end) break;
+        // The units' maxima and sums by lanes, 32 at a time, so that a row costs
+        // two round trips to L2 and not two per unit.
         float M = -INFINITY;
-        for (int i = 0; i < G.n_split; ++i) M = fmaxf(M, __ldcg(first + i * step + kBM * D + r));
+        for (int i0 = 0; i0 < G.n_split; i0 += 32) {
+            const int i = i0 + lane;
+            M = fmaxf(M, i < G.n_split ? __ldcg(first + i * step + kBM * D + r) : -INFINITY);
+        }
+#pragma unroll
+        for (int x = 16; x > 0; x >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, x));
         float L = 0.f, acc[E];
 #pragma unroll
         for (int e = 0; e < E; ++e) acc[e] = 0.f;
-        for (int i = 0; i < G.n_split; ++i) {
-            const float* s = first + i * step;
-            const float w = ex2(__ldcg(s + kBM * D + r) - M);
-            L = fmaf(w, __ldcg(s + kBM * D + kBM + r), L);
-            if (E == 4) {
-                const float4 v = __ldcg(reinterpret_cast<const float4*>(s + r * D) + lane);
-                acc[0] = fmaf(w, v.x, acc[0]);
-                acc[1] = fmaf(w, v.y, acc[1]);
-                acc[2] = fmaf(w, v.z, acc[E - 2]);
-                acc[E - 1] = fmaf(w, v.w, acc[E - 1]);
-            } else {
-                const float2 v = __ldcg(reinterpret_cast<const float2*>(s + r * D) + lane);
-                acc[0] = fmaf(w, v.x, acc[0]);
-                acc[1] = fmaf(w, v.y, acc[1]);
+        for (int i0 = 0; i0 < G.n_split; i0 += 32) {
+            const int i = i0 + lane, n = min(32, G.n_split - i0);
+            const float w_own = i < G.n_split ? ex2(__ldcg(first + i * step + kBM * D + r) - M) : 0.f;
+            const float l_own = i < G.n_split ? __ldcg(first + i * step + kBM * D + kBM + r) : 0.f;
+#pragma unroll 4
+            for (int k = 0; k < n; ++k) {
+                const float* s = first + (size_t)(i0 + k) * step + r * D;
+                const float w = __shfl_sync(0xffffffffu, w_own, k);
+                L = fmaf(w, __shfl_sync(0xffffffffu, l_own, k), L);
+                if (E == 4) {
+                    const float4 v = __ldcg(reinterpret_cast<const float4*>(s) + lane);
+                    acc[0] = fmaf(w, v.x, acc[0]);
+                    acc[1] = fmaf(w, v.y, acc[1]);
+                    acc[E - 2] = fmaf(w, v.z, acc[E - 2]);
+                    acc[E - 1] = fmaf(w, v.w, acc[E - 1]);
+                } else {
+                    const float2 v = __ldcg(reinterpret_cast<const float2*>(s) + lane);
+                    acc[0] = fmaf(w, v.x, acc[0]);
+                    acc[1] = fmaf(w, v.y, acc[1]);
+                }
             }
         }
         const float inv = 1.0f / L;
