@@ -41,6 +41,7 @@
 #include "attn_f32_tc.h"
 #include "attn_tc.h"
 #include "ptx.cuh"
+#include "sched.h"
 
 namespace msf {
 namespace {
@@ -544,15 +545,8 @@ int f32_unit_tiles(const F32Class* c, int n, int D, int sms, int max_slots) {
         longest = c[i].n_tiles > longest ? c[i].n_tiles : longest;
     }
     const double own = D == 64 ? 4.0 : 2.0;
-    struct Level {
-        double load;
-        long long count;
-    };
     auto estimate = [&](int len) -> double {
-        struct U {
-            double cost;
-            long long n;
-        } u[kMaxF32Classes];
+        WorkUnits u[kMaxF32Classes];
         long long slots = 0;
         for (int i = 0; i < n; ++i) {
             const int ns = (c[i].n_tiles + len - 1) / len;
@@ -560,49 +554,7 @@ int f32_unit_tiles(const F32Class* c, int n, int D, int sms, int max_slots) {
             if (ns > 1) slots += u[i].n;
         }
         if (slots > max_slots) return 1e30;
-        for (int i = 0; i < n; ++i)
-            for (int k = i + 1; k < n; ++k)
-                if (u[k].cost > u[i].cost) {
-                    const U t = u[i];
-                    u[i] = u[k];
-                    u[k] = t;
-                }
-        // SMs by load, equal loads together, lightest first
-        Level lv[64] = {{0.0, sms}};
-        int nl = 1;
-        double end = 0;
-        for (int i = 0; i < n; ++i)
-            while (u[i].n > 0) {
-                // many rounds: whole rounds over every SM do not change their order
-                if (u[i].n >= 4ll * sms) {
-                    const long long r = u[i].n / sms - 2;
-                    for (int k = 0; k < nl; ++k) lv[k].load += r * u[i].cost;
-                    u[i].n -= r * sms;
-                    continue;
-                }
-                const long long m = u[i].n < lv[0].count ? u[i].n : lv[0].count;
-                const double load = lv[0].load + u[i].cost;
-                u[i].n -= m;
-                lv[0].count -= m;
-                if (lv[0].count == 0) {
-                    for (int k = 1; k < nl; ++k) lv[k - 1] = lv[k];
-                    --nl;
-                }
-                int at = 0;
-                while (at < nl && lv[at].load < load) ++at;
-                if (at < nl && lv[at].load == load) {
-                    lv[at].count += m;
-                } else if (nl < 64) {
-                    for (int k = nl; k > at; --k) lv[k] = lv[k - 1];
-                    lv[at] = {load, m};
-                    ++nl;
-                } else {
-                    lv[at < nl ? at : nl - 1].count += m;
-                }
-                end = load > end ? load : end;
-            }
-        for (int k = 0; k < nl; ++k) end = lv[k].load > end ? lv[k].load : end;
-        return end + (slots > 0 ? 1.0 + 0.006 * (double)slots : 0.0);
+        return lpt_end(u, n, sms) + (slots > 0 ? 1.0 + 0.006 * (double)slots : 0.0);
     };
     int best = longest;
     double least = estimate(longest);

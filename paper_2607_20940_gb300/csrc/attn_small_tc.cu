@@ -23,8 +23,11 @@
 #include <math.h>
 #include <string.h>
 
+#include <type_traits>
+
 #include "attn_small_tc.h"
 #include "ptx.cuh"
+#include "sched.h"
 
 namespace msf {
 namespace {
@@ -34,9 +37,9 @@ constexpr int kThreads = 384;  // 12 warps
 constexpr int kRing = 3;       // K and V tiles in flight
 constexpr int kMaxCluster = 8;
 constexpr long long kWaitLimit = 2000000000LL;  // ~1 s of SM clock
-// 168 registers per thread at launch; the control warpgroup drops to 104 and
-// the two softmax warpgroups rise to 192: 4 x 104 + 8 x 192 <= 12 x 168.
-constexpr int kLaunchRegs = 168, kCtrlRegs = 104, kSoftmaxRegs = 192;
+// 168 registers per thread at launch; the control warpgroup drops to 120 and
+// the two softmax warpgroups rise to 192: 4 x 120 + 8 x 192 <= 12 x 168.
+constexpr int kLaunchRegs = 168, kCtrlRegs = 120, kSoftmaxRegs = 192;
 static_assert(4 * kCtrlRegs + 8 * kSoftmaxRegs <= 12 * kLaunchRegs, "register split");
 
 struct SmallParams {
@@ -232,6 +235,8 @@ __global__ void __launch_bounds__(kThreads, 1)
             __syncwarp();
             if (!ok && lane == 0) atomicOr(p.status, kDevTimeout);
         }
+        __syncwarp();
+        ptx::cluster_sync();  // the partial results are staged (below)
     } else {
         ptx::setmaxnreg_inc<kSoftmaxRegs>();
         // =================== softmax: one thread per query row ===================
@@ -357,12 +362,11 @@ __global__ void __launch_bounds__(kThreads, 1)
         } else if (lane == 0) {
             atomicOr(p.status, kDevTimeout);
         }
-    }
-    // Every thread of every CTA of the cluster: the partial results are staged.
-    __syncwarp();
-    ptx::tc_fence_before();
-    ptx::cluster_sync();
-    if (warp >= 4) {
+        // Every thread of every CTA of the cluster: the partial results are
+        // staged. (The sums stay in this branch, whose registers they need.)
+        __syncwarp();
+        ptx::tc_fence_before();
+        ptx::cluster_sync();
         // ---- rows [rank * R, rank * R + R): the 2 * cluster partial results in
         // order of CTA and warpgroup
         const int R = kBM / cluster;
@@ -371,32 +375,45 @@ __global__ void __launch_bounds__(kThreads, 1)
             const int row = rank * R + x / kVec, c4 = x % kVec;
             const int q = q_row0 + row;
             if (q >= G.q_end) continue;
-            float4 w[kMaxCluster];  // max, sum, max, sum of each CTA; then the weights
-#pragma unroll
-            for (int k = 0; k < kMaxCluster; ++k)
-                w[k] = k < cluster ? ptx::ld_cluster_f4(&ml[row][0], (uint32_t)k) : make_float4(-INFINITY, 0.f, -INFINITY, 0.f);
-            float M = -INFINITY;
-#pragma unroll
-            for (int k = 0; k < kMaxCluster; ++k) M = ptx::fmax3(M, w[k].x, w[k].z);
-            float L = 0.f;
-#pragma unroll
-            for (int k = 0; k < kMaxCluster; ++k) {
-                if (k >= cluster) break;
-                w[k].x = ex2(w[k].x - M);
-                w[k].z = ex2(w[k].z - M);
-                L = fmaf(w[k].x, w[k].y, L);
-                L = fmaf(w[k].z, w[k].w, L);
-            }
+            float M, L = 0.f;
             float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+            auto add = [&](const float4& w, const float4& o0, const float4& o1) {  // w: max, sum, max, sum
+                const float a = ex2(w.x - M), c = ex2(w.z - M);
+                L = fmaf(c, w.w, fmaf(a, w.y, L));
+                acc.x = fmaf(c, o1.x, fmaf(a, o0.x, acc.x));
+                acc.y = fmaf(c, o1.y, fmaf(a, o0.y, acc.y));
+                acc.z = fmaf(c, o1.z, fmaf(a, o0.z, acc.z));
+                acc.w = fmaf(c, o1.w, fmaf(a, o0.w, acc.w));
+            };
+            const float* p0 = part + row * C::kRow + 4 * c4;
+            const float* p1 = p0 + kBM * C::kRow;
+            if (cluster == 1) {
+                const float4 w = *reinterpret_cast<const float4*>(&ml[row][0]);
+                M = fmaxf(w.x, w.z);
+                add(w, *reinterpret_cast<const float4*>(p0), *reinterpret_cast<const float4*>(p1));
+            } else {
+                // Everything this thread needs of every CTA is asked for at once.
+                auto sum = [&](auto size) {
+                    constexpr int kC = decltype(size)::value;
+                    float4 w[kC], o0[kC], o1[kC];
 #pragma unroll
-            for (int k = 0; k < kMaxCluster; ++k) {
-                if (k >= cluster) break;
-                const float4 o0 = ptx::ld_cluster_f4(part + row * C::kRow + 4 * c4, (uint32_t)k);
-                const float4 o1 = ptx::ld_cluster_f4(part + (kBM + row) * C::kRow + 4 * c4, (uint32_t)k);
-                acc.x = fmaf(w[k].z, o1.x, fmaf(w[k].x, o0.x, acc.x));
-                acc.y = fmaf(w[k].z, o1.y, fmaf(w[k].x, o0.y, acc.y));
-                acc.z = fmaf(w[k].z, o1.z, fmaf(w[k].x, o0.z, acc.z));
-                acc.w = fmaf(w[k].z, o1.w, fmaf(w[k].x, o0.w, acc.w));
+                    for (int k = 0; k < kC; ++k) {
+                        w[k] = ptx::ld_cluster_f4(&ml[row][0], (uint32_t)k);
+                        o0[k] = ptx::ld_cluster_f4(p0, (uint32_t)k);
+                        o1[k] = ptx::ld_cluster_f4(p1, (uint32_t)k);
+                    }
+                    M = -INFINITY;
+#pragma unroll
+                    for (int k = 0; k < kC; ++k) M = ptx::fmax3(M, w[k].x, w[k].z);
+#pragma unroll
+                    for (int k = 0; k < kC; ++k) add(w[k], o0[k], o1[k]);
+                };
+                if (cluster == 2)
+                    sum(std::integral_constant<int, 2>{});
+                else if (cluster == 4)
+                    sum(std::integral_constant<int, 4>{});
+                else
+                    sum(std::integral_constant<int, kMaxCluster>{});
             }
             const float inv = 1.0f / L;
             *reinterpret_cast<uint2*>(p.out + (((size_t)b * p.N + q) * p.H + h) * D + 4 * c4) =
@@ -415,14 +432,14 @@ __global__ void __launch_bounds__(kThreads, 1)
 
 }  // namespace
 
-// The rule: every query tile's cluster has to start at once (one CTA per SM;
-// clusters of four and eight leave some SMs of a GPC over), and the estimate
-// has to be below the persistent kernel's. Microseconds fitted on a GB300 over
-// 34 windows of 0.02 to 203 GFLOP (cold start, steps of two K/V tiles, cluster
-// merge; for the persistent kernel start, two-tile steps over the SMs, merge):
-// 8 heads x 64, 24 tiles, cluster 2: 15.4 us against 20.1; one query block a
-// head, 32 tiles, cluster 8: 14.3 against 58.2; 96 query tiles of 49 tiles,
-// cluster 1: 50.7 against 38.4, which the estimates tell apart.
+// The rule: the estimate of this kernel's end (its clusters placed longest
+// first; clusters of four and eight leave some SMs of a GPC over) against the
+// persistent kernel's. Microseconds fitted on a GB300 over 34 windows of 0.02 to
+// 203 GFLOP: here 6.5 and a step of two K/V tiles, for the persistent kernel
+// its start and merges and two-tile steps over the SMs. 8 heads x 64, 24 tiles,
+// cluster 2: 14.2 us against 20.1; one query tile a head, 32 tiles, cluster 8:
+// 13.3 against 58.2; 96 query tiles of 49 K/V tiles: 50 against 38.4, which the
+// estimates tell apart. More than one round has to win by a tenth.
 int attn_small_cluster(const TcGroup* g, int n_groups, int H, int B, int D, int sms) {
     long long items = 0, blocks = 0;  // 128-row query tiles; 256-row x 128 block tiles of the persistent kernel
     int longest = 0;
@@ -432,12 +449,18 @@ int attn_small_cluster(const TcGroup* g, int n_groups, int H, int B, int D, int 
         blocks += (long long)((nq + 2 * kBM - 1) / (2 * kBM)) * H * B * g[i].n_tiles;
         longest = g[i].n_tiles > longest ? g[i].n_tiles : longest;
     }
+    if (items > 2 * sms) return 0;
     const double step = D == 64 ? 1.2 : 1.75;
     double best = 16.0 + (D == 64 ? 0.9 : 1.3) * (double)blocks / sms;
     int cluster = 0;
-    for (int c = 1; c <= kMaxCluster; c *= 2) {
-        if (items * c > (c <= 2 ? sms : sms * 5 / 6) || c > longest) break;
-        const double t = 8.0 + step * ((longest + 2 * c - 1) / (2 * c)) + (c > 1 ? 0.8 : 0.0);
+    for (int c = 1; c <= kMaxCluster && (c == 1 || c <= longest); c *= 2) {
+        const int places = (c <= 2 ? sms : sms * 5 / 6) / c;
+        if (c > 1 && items > places) break;
+        WorkUnits u[MSF_MAX_GROUPS];
+        for (int i = 0; i < n_groups; ++i)
+            u[i] = {6.5 + step * ((g[i].n_tiles + 2 * c - 1) / (2 * c)) + (c > 1 ? 0.5 : 0.0),
+                    (long long)((g[i].q_end - g[i].q_begin + kBM - 1) / kBM) * H * B};
+        const double t = lpt_end(u, n_groups, places) * (items > places ? 1.1 : 1.0);
         if (t < best) {
             best = t;
             cluster = c;
