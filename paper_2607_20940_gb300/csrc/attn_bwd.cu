@@ -97,6 +97,9 @@ __device__ __forceinline__ bool wanted(const BwdRunIf& c) {
     return __syncthreads_or(f);
 }
 
+// (The tensor-core backward, launched next, starts its loads of q, k, v and
+// dout without a wait of its own: the launch_dependents here comes after this
+// kernel's wait, when everything before it is complete.)
 // delta[b, h, t] = sum_d dout * out: a row of D elements is shared by D/8
 // consecutive threads, each loading 8 elements of both tensors (one 16-byte
 // vector each for bf16). One row per thread group: giving a warp several

@@ -293,7 +293,10 @@ __global__ void __launch_bounds__(kThreads, 1)
     const uint32_t tbase = bar.tmem_base;
     volatile int* abort_p = &bar.abort_flag;
     volatile int never = 0;
-    ptx::grid_dep_wait();
+    // Only delta comes from the launch right before this one (bwd_delta_kernel,
+    // on every path), and that launch let this one start after its own wait,
+    // when q, k, v, dO and lse were complete: the softmax warps wait, the first
+    // loads and MMAs need not.
     ptx::grid_dep_launch();
 
     if (warp == 0) {
@@ -607,6 +610,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             if (lane == 0) ptx::mbar_arrive(b);
         };
         int tq = 0, tk = 0, iq = 0, ik = 0;
+        ptx::grid_dep_wait();
         for (int k = 0; ok; ++k) {
             const int idx = round_item(k);
             if (idx >= p.n_items) break;
