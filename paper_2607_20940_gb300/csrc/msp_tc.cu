@@ -228,6 +228,7 @@ __global__ void __launch_bounds__(kThreads, 2)
         ptx::mbar_init(&acc_full, 1);
         ptx::mbar_init(&codes_full, 1);
         ptx::fence_mbar_init();
+        ptx::prefetch_tmap(&maps.w[ri]);
     }
     if (warp == 2) {
         ptx::tmem_alloc(&tmem_base_sh, kEmbedBN);
@@ -244,7 +245,6 @@ __global__ void __launch_bounds__(kThreads, 2)
 
     if (warp == 0) {
         if (lane == 0) {
-            ptx::prefetch_tmap(&maps.w[ri]);
             int issued = 0;
             bool ok = true;
             for (int kc = 0; kc < nk; ++kc) {
@@ -545,11 +545,15 @@ __global__ void __launch_bounds__(kThreads, kTier ? 2 : 1)
         for (int s = 0; s < kStages; ++s) {
             ptx::mbar_init(&full[s], 1);
             ptx::mbar_init(&empty[s], 1);
-            ptx::mbar_init(&go[s], 1);
-            ptx::mbar_init(&a_full[s], 128);  // residual chunks: one arrival per gathering thread
+            if constexpr (kTier) {
+                ptx::mbar_init(&go[s], 1);
+                ptx::mbar_init(&a_full[s], 128);  // residual chunks: one arrival per gathering thread
+            }
         }
         ptx::mbar_init(&acc_full, 1);
         ptx::fence_mbar_init();
+        ptx::prefetch_tmap(&maps.a);  // before the wait for the previous launch: 0.2 us behind an attention
+        ptx::prefetch_tmap(&maps.b);
     }
     if (warp == 2) {
         ptx::tmem_alloc(&tmem_base_sh, kTier ? 2 * kDeBN : kDeBN);
@@ -567,8 +571,6 @@ __global__ void __launch_bounds__(kThreads, kTier ? 2 : 1)
     bool ok = true;
     if (warp == 0) {
         if (lane == 0) {
-            ptx::prefetch_tmap(&maps.a);
-            ptx::prefetch_tmap(&maps.b);
             int issued = 0;
             for (int kc = 0; kc < nk; ++kc) {
                 const int st = kc % kStages;
@@ -969,15 +971,20 @@ cudaError_t launch_msp_deembed(const void* tokens, long long tok_bstride_elems, 
         return cudaErrorInvalidValue;
     if (res && !encode_2d(&maps.res, tier->residual, F, F, (long long)F * 2, 64, kDeBN)) return cudaErrorInvalidValue;
     const int nk_all = E / 64 + (res ? F / 64 : 0);
-    // Splits (the cluster size) by the number of clusters: one wave. At most 15
-    // clusters of eight CTAs and about 36 of four run at once on 152 SMs (72
-    // without extras, two CTAs per SM); measured at E 1536, eight / four / two /
-    // one: 13 tiles 5.6 / 6.5 / 9.6 / 15.0 us, 26 8.0 / 6.7 / 9.8 / 15.1, 52 14.6 /
-    // 9.1 / 10.0 / 15.3, 111 27.3 / 17.8 / 13.7 / 15.5; with extras 16 tiles 10.5 /
-    // 10.2 / 14.8 / 24.8, 40 20.3 / 16.1 / 15.1 / 25.0, 120 45.0 / 29.5 / 24.9 / 25.6.
-    // Each split keeps at least one K chunk.
+    // Splits (the cluster size) by the number of clusters. At most 15 clusters of
+    // eight CTAs and about 36 of four run at once on 152 SMs (72 without extras,
+    // two CTAs per SM), so launches in a row favour one wave: E 1536, eight /
+    // four / two / one: 13 tiles 5.6 / 6.5 / 9.6 / 15.0 us, 26 8.0 / 6.7 / 9.8 /
+    // 15.1, 52 14.6 / 9.1 / 10.0 / 15.3, 111 27.3 / 17.8 / 13.7 / 15.5. Behind an
+    // attention launch, whose CTAs do not end together, the shorter chain of
+    // eight is still ahead at two waves (whole step, eight / four / two): 18
+    // tiles 42.5 / 44.2 / 48.0 us, 26 161.8 / 163.2 / 168.0, 39 118.7 / 116.7 /
+    // 119.6, 52 113.9 / 109.6 / 113.2, 78 161.5 / 155.6 / 153.9. With extras, alone:
+    // 16 tiles 10.5 / 10.2 / 14.8 / 24.8, 40 20.3 / 16.1 / 15.1 / 25.0, 120 45.0 /
+    // 29.5 / 24.9 / 25.6. Each split keeps at least one K chunk.
     const int clusters = (M + 127) / 128 * (F / kDeBN) * batch;
-    int splits = clusters <= 15 ? 8 : clusters <= (lora || res ? 36 : 72) ? 4 : clusters <= 152 ? 2 : 1;
+    const bool extras = lora || res;
+    int splits = clusters <= (extras ? 15 : 30) ? 8 : clusters <= (extras ? 36 : 72) ? 4 : clusters <= 152 ? 2 : 1;
     while (splits > 1 && splits > nk_all) splits /= 2;
     DeembedParams p;
     memset(&p, 0, sizeof(p));
