@@ -697,16 +697,15 @@ def other_configs(msf, synth, dev, flush, peaks, rank):
         de_tier = _timed(lambda: plan_t.unpatchify_tier(pos, tok_t, lat_t, mods[2], lat_o), flush)
         if plan_t.device_status() != msf.MSF_OK:
             raise RuntimeError("device status error (tier modules)")
-        n_coarse = sum(plan_t.info.state_tokens[l] for l, sc in enumerate(w.scales) if sc > 1)
         M = plan_t.info.state_tokens[pos]
-        emb_bytes = lat_t.numel() * 2 + tok_t.numel() * 2 + 2 * B * n_coarse * 64 * 2
-        de_bytes = B * M * E * 2 + 2 * B * C * Hl * Wl * 2 + B * M * 64 * 2 * 2
+        emb_bytes = lat_t.numel() * 2 + tok_t.numel() * 2
+        de_bytes = B * M * E * 2 + 2 * B * C * Hl * Wl * 2
         tier[w.name] = {
             "lora_rank": rank, "embed_plain_us": emb_base * 1e3, "embed_tier_us": emb_tier * 1e3,
             "embed_tier_gbs": emb_bytes / (emb_tier * 1e-3) / 1e9,
             "deembed_position": pos, "deembed_plain_us": de_base * 1e3, "deembed_tier_us": de_tier * 1e3,
             "deembed_tier_gbs": de_bytes / (de_tier * 1e-3) / 1e9,
-            "launches": {"embed_tier": 2, "deembed_tier": 3},
+            "launches": {"embed_tier": 1, "deembed_tier": 1},
         }
         del keep
         plan_t.close()

@@ -266,11 +266,10 @@ typedef struct msf_tier_module {
  * latent [B, T, C, Hl, Wl] (as msf_patchify), state l embedded by
  * tiers[l] (an array of T pointers; consecutive states with the same pointer
  * and scale share one run). With an embedding adapter the tokens get
- * g * U (A x): the codes g * A x (fp32 sums, rounded once to bf16) are
- * computed by one launch of the fused gather + GEMM kernel into the
- * workspace, and the embedding launch adds one K chunk (codes x U) to the
- * same fp32 accumulation. bf16 plans with an embedding, bound (the codes
- * live in the workspace). Errors: INVALID_ARG (NULL or misaligned pointers,
+ * g * U (A x), all in one launch: a tile computes its rows' codes g * A x
+ * (fp32 sums, rounded once to bf16) beside W x and adds one K chunk
+ * (codes x U) to the same fp32 accumulation. bf16 plans with an embedding,
+ * bound. Errors: INVALID_ARG (NULL or misaligned pointers,
  * rank outside 8..64 or not a multiple of 8), UNSUPPORTED (fp32 plan, no
  * embedding, E not a multiple of 64, a patch edge that does not divide 64),
  * STATE (not bound), CUDA. */
@@ -281,11 +280,11 @@ msf_status msf_patchify_tiers(msf_plan_t plan, const void* latent, const msf_tie
  * module: tokens [B, N, E] (for example the attention output viewed as
  * [B, N, H*D]), latent_in the window latent [B, T, C, Hl, Wl] the pass
  * started from (read only when tier->residual is set), latent_out
- * [B, C, Hl, Wl]. The adapter's codes g * Ao h come from a tensor-core GEMM
- * into the workspace; the residual's raw patch vectors from the raw
- * patchify kernel into the workspace; the de-embedding kernel then sums the
- * E/64 token chunks, the code chunk and the K/64 residual chunks in one fp32
- * accumulation (split over a cluster) and rounds once. Errors: INVALID_ARG,
+ * [B, C, Hl, Wl]. One launch: the E/64 token chunks and the K/64 residual
+ * chunks (patch vectors gathered from latent_in) are summed in one fp32
+ * accumulation, the codes g * Ao h in a second beside it (both split over a
+ * cluster); the codes, rounded once to bf16, times Uo are added in fp32 and
+ * the sum is rounded once. Errors: INVALID_ARG,
  * UNSUPPORTED (fp32 plan, no embedding, K or E not a multiple of 64), STATE,
  * CUDA. */
 msf_status msf_unpatchify_tier(msf_plan_t plan, int32_t position, const void* tokens,

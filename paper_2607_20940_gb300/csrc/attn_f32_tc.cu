@@ -11,7 +11,7 @@
 // S is one tile's scores, and each tile's P V is read out and added to the
 // running output in fp32 registers. Against 64 bits the result is closer than
 // the CUDA-core kernel's on every size tried (480p layer: relative error
-// 5.5e-7 against 2.0e-6), and the 480p layer (202.8 GFLOP) takes 0.85 ms
+// 5.5e-7 against 2.0e-6), and the 480p layer (202.8 GFLOP) takes 0.78 ms
 // against 13.9 ms.
 //
 // split_planes_kernel  reads q and the context's k, v once and writes the
