@@ -22,8 +22,9 @@
 //   buffers. A gather kernel applies the adjoint of Subsample afterwards.
 //
 // CTA c takes items c, 2G-1-c, 2G+c, ... of the list sorted by cost (G CTAs,
-// back and forth so that no CTA always gets a round's longest), and its roles
-// run on from item to item: the next item's loads and first MMAs overlap the
+// back and forth so that no CTA always gets a round's longest), or a list of its
+// own where that ends earlier (place_items), and its roles run on from item to
+// item: the next item's loads and first MMAs overlap the
 // output of the one before, and tensor memory and barriers are set up once.
 // On the 480p layer an item used to cost 5-9 us besides its tiles.
 //
@@ -40,6 +41,7 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <math.h>
+#include <stdint.h>
 #include <string.h>
 
 #include "attn_bwd_tc.h"
@@ -100,6 +102,13 @@ struct BwdTcParams {
     struct Range {
         int kind, group, base, count;
     } range[2 * MSF_MAX_GROUPS];
+};
+// The items of every CTA: CTA c takes item[first[c]], ..., item[first[c + 1] - 1].
+constexpr int kMaxOrderCtas = 160, kMaxOrderItems = 2048;
+struct BwdOrder {
+    int on;  // 0: rounds of alternating direction
+    uint16_t first[kMaxOrderCtas + 1];
+    uint16_t item[kMaxOrderItems];
 };
 struct BwdMaps {
     CUtensorMap q, dout;
@@ -214,10 +223,12 @@ __device__ __forceinline__ void kv_tile(const BGroupQ& G, int u, int& map, int& 
     valid = min(kBM, G.seg[s].len - kt * kBM);
 }
 
-// Item of round k of this CTA: rounds alternate direction.
-__device__ __forceinline__ int round_item(int k) {
+// k-th item of this CTA (n_items or more: none left).
+__device__ __forceinline__ int next_item(const BwdTcParams& p, const BwdOrder& o, int k) {
     const int g = (int)gridDim.x, c = (int)blockIdx.x;
-    return k * g + ((k & 1) ? g - 1 - c : c);
+    if (!o.on) return k * g + ((k & 1) ? g - 1 - c : c);
+    const int at = o.first[c] + k;
+    return at < o.first[c + 1] ? o.item[at] : p.n_items;
 }
 
 // 64 fp32 columns of a row scaled by mul: 32-byte stores when aligned.
@@ -248,7 +259,8 @@ __device__ __forceinline__ void store_f32(float* dst, const uint32_t (&o)[32], f
 // cycles per 64-wide MMA (shared-memory reads bound it) against 82 per 128.
 template <int D>
 __global__ void __launch_bounds__(kThreads, 1)
-    bwd_tc_kernel(const __grid_constant__ BwdMaps maps, const __grid_constant__ BwdTcParams p) {
+    bwd_tc_kernel(const __grid_constant__ BwdMaps maps, const __grid_constant__ BwdTcParams p,
+                  const __grid_constant__ BwdOrder order) {
     using C = BCfg<D>;
     extern __shared__ __align__(1024) unsigned char smem[];
     BwdBars& bar = *reinterpret_cast<BwdBars*>(smem + C::kBars);
@@ -311,7 +323,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             };
             int prev_kind = -1;
             for (int k = 0; ok; ++k) {
-                const int idx = round_item(k);
+                const int idx = next_item(p, order, k);
                 if (idx >= p.n_items) break;
                 const BItem it = item_of(p, idx);
                 // The item before the last is done (so that the phases of
@@ -420,7 +432,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         int tq = 0, tk = 0;                  // tiles done of each kind
         int iq = 0, ik = 0;                  // items done of each kind
         for (int k = 0; ok; ++k) {
-            const int idx = round_item(k);
+            const int idx = next_item(p, order, k);
             if (idx >= p.n_items) break;
             const BItem it = item_of(p, idx);
             const int n = it.n;
@@ -612,7 +624,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         int tq = 0, tk = 0, iq = 0, ik = 0;
         ptx::grid_dep_wait();
         for (int k = 0; ok; ++k) {
-            const int idx = round_item(k);
+            const int idx = next_item(p, order, k);
             if (idx >= p.n_items) break;
             const BItem it = item_of(p, idx);
             const int n = it.n;
@@ -838,6 +850,78 @@ bool encode_all(BwdMaps& m, const Plan& P, const BwdTcInput& in) {
     return true;
 }
 
+// Equal items of a launch.
+struct ItemClass {
+    int kind, group, count;
+    int blocks;  // MMA blocks of 128x128xD: 3 per K/V tile of a dq item, 4 per query tile of a dK/dV item
+    int ns;      // what an item takes, as measured
+    int base;    // its first item
+};
+
+// Gives every item, longest first, to the CTA that would be free first, where
+// that ends the launch at least a hundredth and a microsecond earlier than the
+// rounds of alternating direction: those keep neighbouring tiles of a head and
+// items of one kind together, and are near enough once a CTA has a dozen items.
+// New loads of a class only grow, so two sorted queues hold the CTAs and an item
+// costs the host a few nanoseconds. Forward and backward, rounds / placed: a fine
+// and a coarse state of 40 x 36 tokens, 16 heads x 128, 278.6 / 238.0 us (576
+// items); 46 x 26, three frames a state, 3 heads x 64, 239.7 / 220.0; 8 x 39, four
+// streams, 113.4 / 107.7 (480); 480p 508.0 / 506.4 (1032).
+void place_items(BwdOrder& o, const ItemClass* cl, int n, int total, int ctas) {
+    o.on = 0;
+    if (total <= ctas || total > kMaxOrderItems || ctas > kMaxOrderCtas) return;
+    struct Cta {
+        long long load;
+        int c;
+    };
+    Cta old[kMaxOrderCtas], grown[kMaxOrderItems], rest[kMaxOrderCtas];
+    long long rounds[kMaxOrderCtas];
+    uint8_t cta_of[kMaxOrderItems];  // by item
+    uint16_t taken[kMaxOrderItems];  // items, longest first
+    for (int c = 0; c < ctas; ++c) {
+        old[c] = {0, c};
+        rounds[c] = 0;
+    }
+    int by_ns[2 * MSF_MAX_GROUPS];
+    for (int k = 0; k < n; ++k) {
+        int at = k;
+        for (; at > 0 && cl[by_ns[at - 1]].ns < cl[k].ns; --at) by_ns[at] = by_ns[at - 1];
+        by_ns[at] = k;
+        for (int x = 0; x < cl[k].count; ++x) {
+            const int r = (cl[k].base + x) / ctas, c = (cl[k].base + x) % ctas;
+            rounds[r & 1 ? ctas - 1 - c : c] += cl[k].ns;
+        }
+    }
+    memset(o.first, 0, sizeof(o.first));
+    int done = 0;
+    for (int k = 0; k < n; ++k) {
+        const ItemClass& ic = cl[by_ns[k]];
+        int i = 0, head = 0, tail = 0;
+        auto lightest = [&] {
+            return head == tail || (i < ctas && old[i].load <= grown[head].load) ? old[i++] : grown[head++];
+        };
+        for (int x = 0; x < ic.count; ++x) {
+            Cta t = lightest();
+            t.load += ic.ns;
+            grown[tail++] = t;
+            cta_of[ic.base + x] = (uint8_t)t.c;
+            taken[done++] = (uint16_t)(ic.base + x);
+            ++o.first[t.c + 1];
+        }
+        for (int m = 0; m < ctas; ++m) rest[m] = lightest();
+        memcpy(old, rest, sizeof(old));
+    }
+    long long end = 0;
+    for (int c = 0; c < ctas; ++c) end = rounds[c] > end ? rounds[c] : end;
+    const long long gain = end - old[ctas - 1].load;
+    if (gain < 1000 || 100 * gain < end) return;
+    o.on = 1;
+    for (int c = 0; c < ctas; ++c) o.first[c + 1] = (uint16_t)(o.first[c + 1] + o.first[c]);
+    uint16_t at[kMaxOrderCtas];
+    memcpy(at, o.first, sizeof(at));
+    for (int x = 0; x < total; ++x) o.item[at[cta_of[taken[x]]]++] = taken[x];
+}
+
 }  // namespace
 
 msf_status launch_bwd_tc(msf_plan_t plan, const BwdTcInput& in, cudaStream_t st) {
@@ -944,23 +1028,26 @@ msf_status launch_bwd_tc(msf_plan_t plan, const BwdTcInput& in, cudaStream_t st)
         kitems += kt0 * P.H * P.B;
     }
     tp.n_kgroups = nk;
-    // Ranges in decreasing cost per item (MMA blocks of 128x128xD: 3 per
-    // K/V tile of a dq item, 4 per query tile of a dK/dV item).
-    struct R {
-        int kind, group, count;
-        long long cost;
-    } rs[2 * MSF_MAX_GROUPS];
+    // Ranges with the most MMA blocks per item first; the times are from
+    // globaltimer stamps over eight windows of 1 to 175 tiles an item (within
+    // 8 % from two tiles on).
+    const bool d128 = P.D == 128;
+    ItemClass rs[2 * MSF_MAX_GROUPS];
     int nr = 0;
-    for (int oi = 0; oi < a.n_groups; ++oi)
+    for (int oi = 0; oi < a.n_groups; ++oi) {
+        const int n = tp.g[oi].n_tiles;
         if (tp.g[oi].n_qt > 0)
-            rs[nr++] = {0, oi, tp.g[oi].n_qt * P.H * P.B, 3LL * tp.g[oi].n_tiles};
-    for (int oi = 0; oi < nk; ++oi)
+            rs[nr++] = {0, oi, tp.g[oi].n_qt * P.H * P.B, 3 * n, d128 ? 1200 + 1085 * n : 1500 + 710 * n, 0};
+    }
+    for (int oi = 0; oi < nk; ++oi) {
+        const int n = tp.kg[oi].n_qt;
         if (tp.kg[oi].n_kt > 0)
-            rs[nr++] = {1, oi, tp.kg[oi].n_kt * P.H * P.B, 4LL * tp.kg[oi].n_qt};
+            rs[nr++] = {1, oi, tp.kg[oi].n_kt * P.H * P.B, 4 * n, d128 ? 4500 + 1355 * n : 2600 + 1110 * n, 0};
+    }
     for (int i = 0; i < nr; ++i)
         for (int k = i + 1; k < nr; ++k)
-            if (rs[k].cost > rs[i].cost) {
-                const R t = rs[i];
+            if (rs[k].blocks > rs[i].blocks) {
+                const ItemClass t = rs[i];
                 rs[i] = rs[k];
                 rs[k] = t;
             }
@@ -968,7 +1055,7 @@ msf_status launch_bwd_tc(msf_plan_t plan, const BwdTcInput& in, cudaStream_t st)
     for (int i = 0; i < nr; ++i) {
         tp.range[i].kind = rs[i].kind;
         tp.range[i].group = rs[i].group;
-        tp.range[i].base = total;
+        tp.range[i].base = rs[i].base = total;
         tp.range[i].count = rs[i].count;
         total += rs[i].count;
     }
@@ -988,7 +1075,8 @@ msf_status launch_bwd_tc(msf_plan_t plan, const BwdTcInput& in, cudaStream_t st)
         return MSF_ERR_CUDA;
     }
     const int grid = total < sms ? total : sms;
-    const bool d128 = P.D == 128;
+    BwdOrder placed;
+    place_items(placed, rs, nr, total, grid);
     const int smem = d128 ? BCfg<128>::kSmem : BCfg<64>::kSmem;
     e = d128 ? set_smem_attr((const void*)bwd_tc_kernel<128>, BCfg<128>::kSmem)
              : set_smem_attr((const void*)bwd_tc_kernel<64>, BCfg<64>::kSmem);
@@ -996,8 +1084,8 @@ msf_status launch_bwd_tc(msf_plan_t plan, const BwdTcInput& in, cudaStream_t st)
         set_cuda_error((int)e);
         return MSF_ERR_CUDA;
     }
-    e = d128 ? launch_pdl(bwd_tc_kernel<128>, dim3((unsigned)grid), dim3(kThreads), smem, st, maps, tp)
-             : launch_pdl(bwd_tc_kernel<64>, dim3((unsigned)grid), dim3(kThreads), smem, st, maps, tp);
+    e = d128 ? launch_pdl(bwd_tc_kernel<128>, dim3((unsigned)grid), dim3(kThreads), smem, st, maps, tp, placed)
+             : launch_pdl(bwd_tc_kernel<64>, dim3((unsigned)grid), dim3(kThreads), smem, st, maps, tp, placed);
     if (e != cudaSuccess) {
         set_cuda_error((int)e);
         return MSF_ERR_CUDA;
