@@ -1289,6 +1289,12 @@ msf_status launch_attn_tc(msf_plan_t plan, const AttnArgs& a, cudaStream_t st, c
     if (tp.n_groups > 0) tp.dp_rounds = (int)(tp.g[0].n_items / ncta);
     tp.dp_stride = tp.g[0].n_virt;
     tp.t_sk = (long long)tp.dp_rounds * ncta * tp.dp_stride;
+    // The split counts a piece for every CTA between an item's first and last:
+    // each must hold a tile, so a rest of fewer tiles than CTAs takes a round in.
+    if (tp.dp_rounds > 0 && total_tiles > tp.t_sk && total_tiles - tp.t_sk < ncta) {
+        --tp.dp_rounds;
+        tp.t_sk -= ncta * tp.dp_stride;
+    }
     // The launch's own pyramid (D = 128): vector-pair tasks of every job and
     // stream. Other head sizes run the pool kernel first.
     const bool own_pool = pool && pool->n > 0 && P.D == 128;
