@@ -350,8 +350,8 @@ msf_status msf_mssa_forward_lse(msf_plan_t plan, const void* q, const void* k_wi
  * (the last msf_kv_resample on the stream) and the same history state (no
  * commit or append in between). bwd_workspace: >= info.backward_workspace_bytes
  * bytes, 16-byte aligned, overwritten. Output buffers may not alias inputs.
- * bf16 plans run tcgen05 tensor-core kernels (one for dq over each query
- * tile's whole context, one per query group for the window rows' dk/dv);
+ * bf16 plans run one persistent tcgen05 tensor-core kernel (dq of each query
+ * tile over its whole context, dk/dv of each tile of window-derived rows);
  * fp32 plans run them on three bf16 planes per value (as the forward does),
  * or CUDA-core kernels where the planes cannot hold a value.
  * Errors: INVALID_ARG, STATE (not bound), WORKSPACE, CUDA. */
