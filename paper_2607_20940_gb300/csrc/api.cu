@@ -589,8 +589,7 @@ static msf_status mssa_backward(msf_plan_t plan, const void* q, const void* k_wi
             msf_status st = msf::launch_bwd_f32_tc(plan, c, a, bg, (float*)dq, planes, &run_if, s);
             if (st != MSF_OK) return st;
         }
-        e = msf::launch_bwd_dq_simt(c, a, dq, bf16, run_if, s);
-        if (e == cudaSuccess) e = msf::launch_bwd_dkdv_simt(c, bg, p.n_groups, bf16, run_if, s);
+        e = msf::launch_bwd_simt(c, a, bg, dq, bf16, run_if, s);
         if (e != cudaSuccess) return cuda_status(e);
     }
     return cuda_status(msf::launch_bwd_gather(c, ga, dk_win, dv_win, bf16, s));

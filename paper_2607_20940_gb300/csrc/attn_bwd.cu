@@ -134,16 +134,11 @@ __global__ void __launch_bounds__(256) bwd_delta_kernel(const BwdCommon c) {
 // dq: a block owns 32 queries of one (stream, head, group); four threads share
 // a query and hold every fourth element of q, dO and dq.
 template <typename T, int D>
-__global__ void __launch_bounds__(128) bwd_dq_kernel(const BwdCommon c, const AttnArgs a, T* dq,
-                                                     const BwdRunIf run_if) {
-    ptx::grid_dep_wait();
-    ptx::grid_dep_launch();
-    if (!wanted(run_if)) return;
+__device__ __forceinline__ void bwd_dq_rows(const BwdCommon& c, const AttnArgs& a, T* dq, int tile, float (&Ks)[32][D],
+                                            float (&Vs)[32][D]) {
     constexpr int DP = D / 4;
     constexpr int KT = 32;
-    __shared__ float Ks[KT][D];
-    __shared__ float Vs[KT][D];
-    int tile = blockIdx.x, gi = 0;
+    int gi = 0;
     while (gi < a.n_groups) {
         int nt = (a.g[gi].q_end - a.g[gi].q_begin + 31) / 32;
         if (tile < nt) break;
@@ -222,17 +217,11 @@ __host__ __device__ inline int grad_tiles(const BwdGroup& g) {
     return n;
 }
 template <typename T, int D>
-__global__ void __launch_bounds__(128)
-    bwd_dkdv_kernel(const BwdCommon c, const __grid_constant__ BwdGroups groups, const BwdRunIf run_if) {
-    ptx::grid_dep_wait();
-    ptx::grid_dep_launch();
-    if (!wanted(run_if)) return;
+__device__ __forceinline__ void bwd_dkdv_rows(const BwdCommon& c, const BwdGroups& groups, int tile, float (&Qs)[32][D],
+                                              float (&Gs)[32][D], float (&Ls)[32], float (&Ds)[32]) {
     constexpr int DP = D / 4;
     constexpr int QT = 32;
-    __shared__ float Qs[QT][D];
-    __shared__ float Gs[QT][D];
-    __shared__ float Ls[QT], Ds[QT];
-    int tile = blockIdx.x, si = 0, gi = 0;
+    int si = 0, gi = 0;
     for (int nt; gi + 1 < groups.n && tile >= (nt = grad_tiles(groups.g[gi])); ++gi) tile -= nt;
     const BwdGroup& G = groups.g[gi];
     while (si < G.n_gseg) {
@@ -301,6 +290,28 @@ __global__ void __launch_bounds__(128)
         c.dk_ctx[o + 4 * e + cc] = dk[e] * c.scale;
         c.dv_ctx[o + 4 * e + cc] = dv[e];
     }
+}
+
+// Both in one launch, dq's tiles first. As two, an fp32 training pass whose
+// operands the planes hold paid for a second idle launch (1008 tokens, 4 heads x
+// 128: 127.6 -> 124.8 us), and where they run, dk/dv waited for the last dq block
+// (the same window 1316 -> 967 us; 480p 32.4 -> 30.6 ms). Three blocks an SM: the
+// 168 registers spill 24 bytes at D = 128, but with 210 and two blocks the 480p
+// layer takes 34.7 ms.
+template <typename T, int D>
+__global__ void __launch_bounds__(128, 3)
+    bwd_simt_kernel(const BwdCommon c, const __grid_constant__ AttnArgs a, const __grid_constant__ BwdGroups groups,
+                    T* dq, int dq_tiles, const BwdRunIf run_if) {
+    ptx::grid_dep_wait();
+    ptx::grid_dep_launch();
+    if (!wanted(run_if)) return;
+    __shared__ float s0[32][D];
+    __shared__ float s1[32][D];
+    __shared__ float l[32], d[32];
+    if ((int)blockIdx.x < dq_tiles)
+        bwd_dq_rows<T, D>(c, a, dq, (int)blockIdx.x, s0, s1);
+    else
+        bwd_dkdv_rows<T, D>(c, groups, (int)blockIdx.x - dq_tiles, s0, s1, l, d);
 }
 
 // dk_win, dv_win: one block per (stream, token); the token's rows of every
@@ -392,37 +403,27 @@ cudaError_t launch_bwd_delta(const BwdCommon& c, bool bf16, cudaStream_t st) {
                 : launch_pdl(bwd_delta_kernel<float, 64>, grid, dim3(256), 0, st, c);
 }
 
-cudaError_t launch_bwd_dq_simt(const BwdCommon& c, const AttnArgs& a, void* dq, bool bf16, BwdRunIf run_if,
-                               cudaStream_t st) {
-    int tiles = 0;
-    for (int gi = 0; gi < a.n_groups; ++gi) tiles += (a.g[gi].q_end - a.g[gi].q_begin + 31) / 32;
-    if (tiles == 0) return cudaSuccess;
-    dim3 grid((unsigned)tiles, (unsigned)c.H, (unsigned)c.B);
-    if (c.D == 128)
-        return bf16 ? launch_pdl(bwd_dq_kernel<__nv_bfloat16, 128>, grid, dim3(128), 0, st, c, a,
-                                 (__nv_bfloat16*)dq, run_if)
-                    : launch_pdl(bwd_dq_kernel<float, 128>, grid, dim3(128), 0, st, c, a, (float*)dq, run_if);
-    return bf16 ? launch_pdl(bwd_dq_kernel<__nv_bfloat16, 64>, grid, dim3(128), 0, st, c, a,
-                             (__nv_bfloat16*)dq, run_if)
-                : launch_pdl(bwd_dq_kernel<float, 64>, grid, dim3(128), 0, st, c, a, (float*)dq, run_if);
-}
-
-cudaError_t launch_bwd_dkdv_simt(const BwdCommon& c, const BwdGroup* g, int n_groups, bool bf16, BwdRunIf run_if,
-                                 cudaStream_t st) {
+cudaError_t launch_bwd_simt(const BwdCommon& c, const AttnArgs& a, const BwdGroup* g, void* dq, bool bf16,
+                            BwdRunIf run_if, cudaStream_t st) {
     BwdGroups gs;
-    gs.n = n_groups;
-    int tiles = 0;
-    for (int i = 0; i < n_groups; ++i) {
+    gs.n = a.n_groups;
+    int dq_tiles = 0, tiles = 0;
+    for (int i = 0; i < a.n_groups; ++i) {
         gs.g[i] = g[i];
+        dq_tiles += (a.g[i].q_end - a.g[i].q_begin + 31) / 32;
         tiles += grad_tiles(g[i]);
     }
+    tiles += dq_tiles;
     if (tiles == 0) return cudaSuccess;
     dim3 grid((unsigned)tiles, (unsigned)c.H, (unsigned)c.B);
+    auto run = [&](auto* kernel, auto* out) {
+        return launch_pdl(kernel, grid, dim3(128), 0, st, c, a, gs, out, dq_tiles, run_if);
+    };
     if (c.D == 128)
-        return bf16 ? launch_pdl(bwd_dkdv_kernel<__nv_bfloat16, 128>, grid, dim3(128), 0, st, c, gs, run_if)
-                    : launch_pdl(bwd_dkdv_kernel<float, 128>, grid, dim3(128), 0, st, c, gs, run_if);
-    return bf16 ? launch_pdl(bwd_dkdv_kernel<__nv_bfloat16, 64>, grid, dim3(128), 0, st, c, gs, run_if)
-                : launch_pdl(bwd_dkdv_kernel<float, 64>, grid, dim3(128), 0, st, c, gs, run_if);
+        return bf16 ? run(bwd_simt_kernel<__nv_bfloat16, 128>, (__nv_bfloat16*)dq)
+                    : run(bwd_simt_kernel<float, 128>, (float*)dq);
+    return bf16 ? run(bwd_simt_kernel<__nv_bfloat16, 64>, (__nv_bfloat16*)dq)
+                : run(bwd_simt_kernel<float, 64>, (float*)dq);
 }
 
 cudaError_t launch_bwd_gather(const BwdCommon& c, const GatherArgs& g, void* dk, void* dv,

@@ -212,12 +212,10 @@ struct BwdRunIf {
     const unsigned int* flags = nullptr;
     int n = 0;
 };
-// dq for every query of every group (context of each group as in the forward).
-cudaError_t launch_bwd_dq_simt(const BwdCommon& c, const AttnArgs& a, void* dq, bool bf16, BwdRunIf run_if,
-                               cudaStream_t st);
-// Context-row gradients of every group's window-derived rows.
-cudaError_t launch_bwd_dkdv_simt(const BwdCommon& c, const BwdGroup* g, int n_groups, bool bf16, BwdRunIf run_if,
-                                 cudaStream_t st);
+// On CUDA cores: dq for every query of every group (context of each group as in
+// the forward) and the context-row gradients of every group's window-derived rows.
+cudaError_t launch_bwd_simt(const BwdCommon& c, const AttnArgs& a, const BwdGroup* g, void* dq, bool bf16,
+                            BwdRunIf run_if, cudaStream_t st);
 // dk_win, dv_win from the context-row gradients (adjoint of Subsample, sum
 // over groups, one rounding to the dtype).
 cudaError_t launch_bwd_gather(const BwdCommon& c, const GatherArgs& g, void* dk, void* dv,
