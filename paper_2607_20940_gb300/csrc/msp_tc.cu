@@ -971,20 +971,22 @@ cudaError_t launch_msp_deembed(const void* tokens, long long tok_bstride_elems, 
         return cudaErrorInvalidValue;
     if (res && !encode_2d(&maps.res, tier->residual, F, F, (long long)F * 2, 64, kDeBN)) return cudaErrorInvalidValue;
     const int nk_all = E / 64 + (res ? F / 64 : 0);
-    // Splits (the cluster size) by the number of clusters. At most 15 clusters of
-    // eight CTAs and about 36 of four run at once on 152 SMs (72 without extras,
-    // two CTAs per SM), so launches in a row favour one wave: E 1536, eight /
-    // four / two / one: 13 tiles 5.6 / 6.5 / 9.6 / 15.0 us, 26 8.0 / 6.7 / 9.8 /
-    // 15.1, 52 14.6 / 9.1 / 10.0 / 15.3, 111 27.3 / 17.8 / 13.7 / 15.5. Behind an
-    // attention launch, whose CTAs do not end together, the shorter chain of
-    // eight is still ahead at two waves (whole step, eight / four / two): 18
-    // tiles 42.5 / 44.2 / 48.0 us, 26 161.8 / 163.2 / 168.0, 39 118.7 / 116.7 /
-    // 119.6, 52 113.9 / 109.6 / 113.2, 78 161.5 / 155.6 / 153.9. With extras, alone:
-    // 16 tiles 10.5 / 10.2 / 14.8 / 24.8, 40 20.3 / 16.1 / 15.1 / 25.0, 120 45.0 /
-    // 29.5 / 24.9 / 25.6. Each split keeps at least one K chunk.
+    // Splits (the cluster size) by the number of clusters, as measured. Launches
+    // in a row favour one wave: E 1536, eight / four / two / one: 13 tiles 5.6 /
+    // 6.5 / 9.6 / 15.0 us, 26 8.0 / 6.7 / 9.8 / 15.1, 52 14.6 / 9.1 / 10.0 / 15.3, 111
+    // 27.3 / 17.8 / 13.7 / 15.5. Behind an attention launch, whose CTAs do not end
+    // together, the shorter chain of eight is still ahead at two waves (whole
+    // step, eight / four / two): 18 tiles 42.5 / 44.2 / 48.0 us, 26 161.8 / 163.2 /
+    // 168.0, 39 118.7 / 116.7 / 119.6, 52 113.9 / 109.6 / 113.2, 78 161.5 / 155.6 /
+    // 153.9, two and one from 156 on within 1 %. With extras, the tiers of a window
+    // in turn (eight / four / two / one): 16 tiles 61.3 / 57.2 / 69.9 / 100.4 us, 32
+    // 75.8 / 77.6 / 83.0 / 113.9, 48 111.8 / 90.2 / 91.6 / 123.3, 64 124.2 / 97.6 /
+    // 109.1 / 131.5, 80 155.3 / 129.5 / 122.7 / 139.8, and from there on two (160
+    // 266.8 / 213.7 / 200.1 / 238.1: one CTA's gather and sums are too long a
+    // chain). Each split keeps at least one K chunk.
     const int clusters = (M + 127) / 128 * (F / kDeBN) * batch;
     const bool extras = lora || res;
-    int splits = clusters <= (extras ? 15 : 30) ? 8 : clusters <= (extras ? 36 : 72) ? 4 : clusters <= 152 ? 2 : 1;
+    int splits = clusters <= (extras ? 15 : 30) ? 8 : clusters <= 72 ? 4 : extras || clusters <= 152 ? 2 : 1;
     while (splits > 1 && splits > nk_all) splits /= 2;
     DeembedParams p;
     memset(&p, 0, sizeof(p));

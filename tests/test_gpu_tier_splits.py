@@ -16,12 +16,12 @@ pytestmark = pytest.mark.gpu
 CASES = {
     # clusters of eight (one 128-token tile), many chunks per CTA
     "e4096_one_tile": dataclasses.replace(SMALL, embed_dim=4096, batch=1),
-    # sixteen to 36 clusters: four CTAs, six token chunks before the residual's
+    # sixteen to 72 clusters: four CTAs, six token chunks before the residual's
     "four": dataclasses.replace(synth.LAYER_480P, heads=2, batch=2),
-    # 40 to 152 clusters: two CTAs
-    "two": dataclasses.replace(synth.LAYER_480P, heads=2, batch=3, embed_dim=512),
-    # more: one CTA per tile, every chunk of the contraction in one ring
-    "one": dataclasses.replace(synth.LAYER_480P, heads=1, batch=10, embed_dim=256),
+    # four with a short contraction, two (73 clusters and more)
+    "four_short": dataclasses.replace(synth.LAYER_480P, heads=2, batch=3, embed_dim=512),
+    "two": dataclasses.replace(synth.LAYER_480P, heads=2, batch=5, embed_dim=512),
+    "two_many": dataclasses.replace(synth.LAYER_480P, heads=1, batch=10, embed_dim=256),
     # one token chunk: no split, a tile column of 64 and no whole 192
     "e64": dataclasses.replace(SMALL, embed_dim=64),
     # patch edges 8 (16-byte gathers) and 16 (pixel by pixel)
@@ -35,6 +35,7 @@ def test_tier_cluster_sizes(name):
     _check_window(CASES[name], 24)
 
 
-def test_adapter_alone_at_one_cta_per_tile():
-    _check_window(CASES["one"], 64, lora=True, residual=False)
-    _check_window(CASES["one"], 64, lora=False, residual=True)
+def test_adapter_or_residual_alone():
+    _check_window(CASES["two_many"], 64, lora=True, residual=False)
+    _check_window(CASES["two_many"], 64, lora=False, residual=True)
+    _check_window(CASES["e64"], 64, lora=True, residual=False)  # one CTA per tile
