@@ -435,23 +435,21 @@ __global__ void __launch_bounds__(kThreads, 1)
 // The rule: the estimate of this kernel's end (its clusters placed longest
 // first; clusters of four and eight leave some SMs of a GPC over) against the
 // persistent kernel's. Microseconds fitted on a GB300 over 34 windows of 0.02 to
-// 203 GFLOP: here 6.5 and a step of two K/V tiles, for the persistent kernel
-// its start and merges and two-tile steps over the SMs. 8 heads x 64, 24 tiles,
+// 203 GFLOP: here 6.5 and a step of two K/V tiles. 8 heads x 64, 24 tiles,
 // cluster 2: 14.2 us against 20.1; one query tile a head, 32 tiles, cluster 8:
 // 13.3 against 58.2; 96 query tiles of 49 K/V tiles: 50 against 38.4, which the
 // estimates tell apart. More than one round has to win by a tenth.
-int attn_small_cluster(const TcGroup* g, int n_groups, int H, int B, int D, int sms) {
-    long long items = 0, blocks = 0;  // 128-row query tiles; 256-row x 128 block tiles of the persistent kernel
+int attn_small_cluster(const TcGroup* g, int n_groups, int H, int B, int D, int sms, double persistent_us) {
+    long long items = 0;  // 128-row query tiles
     int longest = 0;
     for (int i = 0; i < n_groups; ++i) {
         const int nq = g[i].q_end - g[i].q_begin;
         items += (long long)((nq + kBM - 1) / kBM) * H * B;
-        blocks += (long long)((nq + 2 * kBM - 1) / (2 * kBM)) * H * B * g[i].n_tiles;
         longest = g[i].n_tiles > longest ? g[i].n_tiles : longest;
     }
     if (items > 2 * sms) return 0;
     const double step = D == 64 ? 1.2 : 1.75;
-    double best = 16.0 + (D == 64 ? 0.9 : 1.3) * (double)blocks / sms;
+    double best = persistent_us;
     int cluster = 0;
     for (int c = 1; c <= kMaxCluster && (c == 1 || c <= longest); c *= 2) {
         const int places = (c <= 2 ? sms : sms * 5 / 6) / c;

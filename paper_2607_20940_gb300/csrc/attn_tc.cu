@@ -107,6 +107,11 @@ struct TcParams {
     int pool_ring;  // the batch also writes the history ring (the staged head)
     unsigned int* pyr_sync;
 };
+// Whole items only: CTA c's range is [at[c], at[c + 1]).
+constexpr int kMaxBoundCtas = 160;
+struct TcBounds {
+    int at[kMaxBoundCtas + 1];
+};
 template <int D>
 struct Cfg {
     static constexpr int kChunks = D / 64;                    // 128-byte swizzle chunks per row
@@ -201,8 +206,9 @@ __device__ __forceinline__ int slot_of(long long c, long long c1, long long item
 
 // The kernel body; kPool: the launch also builds its K/V pyramid (`pool`),
 // compiled as its own kernel so that the plain attention carries none of it.
-template <int D, bool kPool>
-__device__ __forceinline__ void mssa_tc_body(const TcMaps& maps, const TcParams& p, const PoolBatch* pool) {
+template <int D, bool kPool, bool kWhole>
+__device__ __forceinline__ void mssa_tc_body(const TcMaps& maps, const TcParams& p, const PoolBatch* pool,
+                                             const TcBounds* bounds) {
     using C = Cfg<D>;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char* smem = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -228,8 +234,8 @@ __device__ __forceinline__ void mssa_tc_body(const TcMaps& maps, const TcParams&
     // group (items blockIdx.x, blockIdx.x + ncta, ...). Split items thus end
     // early, and their merges run on the helper warps beside the whole items.
     const long long Tsk = T - p.t_sk;
-    const long long r0 = p.t_sk + cta_begin(blockIdx.x, Tsk, ncta);
-    const long long r1 = p.t_sk + cta_begin(blockIdx.x + 1, Tsk, ncta);
+    const long long r0 = kWhole ? bounds->at[blockIdx.x] : p.t_sk + cta_begin(blockIdx.x, Tsk, ncta);
+    const long long r1 = kWhole ? bounds->at[blockIdx.x + 1] : p.t_sk + cta_begin(blockIdx.x + 1, Tsk, ncta);
     auto phase_range = [&](int ph, long long& a0, long long& a1) {
         if (ph == 0) {
             a0 = r0;
@@ -240,7 +246,7 @@ __device__ __forceinline__ void mssa_tc_body(const TcMaps& maps, const TcParams&
         }
     };
     // Merges of split items go to the helper warps while whole items follow.
-    const bool helper_merges = p.dp_rounds > 0;
+    const bool helper_merges = !kWhole && p.dp_rounds > 0;
 
 
     if (threadIdx.x == 0) {
@@ -676,7 +682,7 @@ __device__ __forceinline__ void mssa_tc_body(const TcMaps& maps, const TcParams&
             for (int u = pc.u0; u < pc.u1; ++u, ++js) {
                 int seg, row, valid;
                 tile_info(G, u, seg, row, valid);
-                if (!pc.whole && u == pc.u1 - 1 && warp == 4 && lane == 0) fin_old = atomicAdd(cnt, 1u);
+                if (!kWhole && !pc.whole && u == pc.u1 - 1 && warp == 4 && lane == 0) fin_old = atomicAdd(cnt, 1u);
                 ok = ptx::mbar_wait_bounded(&s_full[t], (uint32_t)(js & 1), abort_p, p.wait_limit);
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) break;
@@ -774,7 +780,7 @@ __device__ __forceinline__ void mssa_tc_body(const TcMaps& maps, const TcParams&
             const bool store = qrow < G.q_end;
             __nv_bfloat16* dst =
                 p.out + (size_t)pc.b * p.out_bstride + ((size_t)qrow * p.H + pc.h) * D;
-            if (pc.whole) {
+            if (kWhole || pc.whole) {
                 const float inv = 1.0f / l;
                 // P, O and l share the scale 2^-m_used: ln sum exp = (m_used + log2 l) ln 2
                 if (store && p.lse)
@@ -1074,14 +1080,23 @@ __device__ __forceinline__ void mssa_tc_body(const TcMaps& maps, const TcParams&
 template <int D>
 __global__ void __launch_bounds__(kThreads, 1)
     mssa_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcParams p) {
-    mssa_tc_body<D, false>(maps, p, nullptr);
+    mssa_tc_body<D, false, false>(maps, p, nullptr, nullptr);
+}
+
+// Whole items only: no partial results and no merge (its own kernel, so that
+// the split's carries none of it).
+template <int D>
+__global__ void __launch_bounds__(kThreads, 1)
+    mssa_tc_whole_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcParams p,
+                         const __grid_constant__ TcBounds bounds) {
+    mssa_tc_body<D, false, true>(maps, p, nullptr, &bounds);
 }
 
 // The same attention with the launch's own pyramid (bf16 D = 128 plans).
 __global__ void __launch_bounds__(kThreads, 1)
     mssa_tc_pool_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcParams p,
                         const __grid_constant__ PoolBatch pool) {
-    mssa_tc_body<128, true>(maps, p, &pool);
+    mssa_tc_body<128, true, false>(maps, p, &pool, nullptr);
 }
 
 // ---------------------------------------------------------------- host side
@@ -1150,6 +1165,64 @@ void tc_cache_invalidate(msf_plan_t plan) {
         for (int i = 0; i < 2 * kNumMaps + 1; ++i) c->valid[i] = false;
         c->num_sms = 0;
     }
+}
+
+// Estimated end in us of the even (stream-K) split: the start and the merges, and
+// the SMs' equal shares of the 256 x 128 tiles (fitted over 34 windows of 0.02 to
+// 203 GFLOP).
+static double split_us(const TcGroup* g, int n, int D, int sms) {
+    double tiles = 0;
+    for (int i = 0; i < n; ++i) tiles += (double)g[i].n_items * g[i].n_tiles;
+    return 16.0 + (D == 64 ? 0.9 : 1.3) * tiles / sms;
+}
+
+// Whole blocks instead: CTA c takes the blocks of the sequence positions
+// [bound[c], bound[c + 1]), cut so that the longest share is shortest. Returns
+// the estimated end in us, 1e9 where there are too many blocks to count.
+static double whole_us(const TcGroup* g, int n, int D, int sms, int* bound, int* ctas) {
+    long long items = 0;
+    double longest = 0, sum = 0, cost[MSF_MAX_GROUPS];
+    for (int i = 0; i < n; ++i) {
+        cost[i] = 3.3 + (D == 64 ? 0.95 : 1.25) * g[i].n_tiles;
+        items += g[i].n_items;
+        sum += cost[i] * g[i].n_items;
+        longest = g[i].n_items > 0 && cost[i] > longest ? cost[i] : longest;
+    }
+    if (items == 0 || items > 4ll * sms || sms > kMaxBoundCtas ||
+        g[n - 1].tile_base + (long long)g[n - 1].n_items * g[n - 1].n_virt > 0x7fffffff)
+        return 1e9;
+    auto cut = [&](double most) {
+        int c = 0;
+        double load = 0;
+        bound[0] = 0;
+        for (int i = 0; i < n; ++i)
+            for (long long at = 0; at < g[i].n_items;) {
+                long long k = (long long)((most - load) / cost[i] + 1e-9);
+                if (k <= 0) {
+                    if (++c == sms) return false;
+                    bound[c] = (int)(g[i].tile_base + at * g[i].n_virt);
+                    load = 0;
+                    continue;
+                }
+                k = k < g[i].n_items - at ? k : g[i].n_items - at;
+                load += k * cost[i];
+                at += k;
+            }
+        *ctas = c + 1;
+        bound[c + 1] = (int)(g[n - 1].tile_base + (long long)g[n - 1].n_items * g[n - 1].n_virt);
+        return true;
+    };
+    double lo = longest, hi = sum / sms + longest;
+    if (sum / sms > lo) lo = sum / sms;
+    if (!cut(lo)) {
+        for (int it = 0; it < 8; ++it) {
+            const double mid = 0.5 * (lo + hi);
+            (cut(mid) ? hi : lo) = mid;
+        }
+        if (!cut(hi)) return 1e9;
+        lo = hi;
+    }
+    return 5.5 + lo;
 }
 
 msf_status launch_attn_tc(msf_plan_t plan, const AttnArgs& a, cudaStream_t st, const PoolBatch* pool) {
@@ -1270,7 +1343,20 @@ msf_status launch_attn_tc(msf_plan_t plan, const AttnArgs& a, cudaStream_t st, c
     if (item_base > P.attn_items) return MSF_ERR_STATE;
     // Small calls: one 128-row query tile per cluster (after the pyramid, if
     // the launch was to build it).
-    const int cluster = attn_small_cluster(tp.g, tp.n_groups, P.H, P.B, P.D, cache.num_sms);
+    long long ncta = cache.num_sms;
+    if (ncta > P.attn_max_ctas) ncta = P.attn_max_ctas;
+    const double split = split_us(tp.g, tp.n_groups, P.D, cache.num_sms);
+    TcBounds bounds;
+    int ctas = 0;
+    const double whole = whole_us(tp.g, tp.n_groups, P.D, (int)ncta, bounds.at, &ctas);
+    // Whole blocks where they end first: the partial results and merges of the
+    // even split cost about 10 us. Even / whole, us: 108 blocks of 12 tiles 30.1 /
+    // 23.3, 208 of 5 to 14 38.5 / 26.5, 132 of up to 20 (D 64) 19.7 / 14.3, 22 of 40
+    // 42.7 / 117.5; over 220 windows the choice was never slower than the even
+    // split beyond what two runs of it differ, and up to 1.56 times faster.
+    const bool by_item = whole < 0.97 * split;
+    const int cluster =
+        attn_small_cluster(tp.g, tp.n_groups, P.H, P.B, P.D, cache.num_sms, by_item ? whole : split);
     if (cluster > 0) {
         e = pool ? launch_pool(*pool, P.B, true, st) : cudaSuccess;
         if (e == cudaSuccess) e = launch_attn_small(cache.maps, tp.g, tp.n_groups, P, a, cluster, st);
@@ -1278,8 +1364,6 @@ msf_status launch_attn_tc(msf_plan_t plan, const AttnArgs& a, cudaStream_t st, c
         set_cuda_error((int)e);
         return MSF_ERR_CUDA;
     }
-    long long ncta = cache.num_sms;
-    if (ncta > P.attn_max_ctas) ncta = P.attn_max_ctas;
     if (ncta > total_tiles) ncta = total_tiles;
     if (ncta < 1) ncta = 1;
     // Data-parallel rounds: while the longest group has at least one item per
@@ -1295,9 +1379,13 @@ msf_status launch_attn_tc(msf_plan_t plan, const AttnArgs& a, cudaStream_t st, c
         --tp.dp_rounds;
         tp.t_sk -= ncta * tp.dp_stride;
     }
+    if (by_item) {
+        tp.dp_rounds = 0;
+        tp.t_sk = 0;
+    }
     // The launch's own pyramid (D = 128): vector-pair tasks of every job and
     // stream. Other head sizes run the pool kernel first.
-    const bool own_pool = pool && pool->n > 0 && P.D == 128;
+    const bool own_pool = pool && pool->n > 0 && P.D == 128 && !by_item;
     if (pool && pool->n > 0 && !own_pool) {
         e = launch_pool(*pool, P.B, true, st);
         if (e != cudaSuccess) {
@@ -1316,7 +1404,17 @@ msf_status launch_attn_tc(msf_plan_t plan, const AttnArgs& a, cudaStream_t st, c
             if (pool->j[k].copy_k || pool->j[k].dst_k == P.k_hist) tp.pool_ring = 1;
     }
 
-    if (own_pool) {
+    if (by_item) {
+        const bool d128 = P.D == 128;
+        const int smem = d128 ? Cfg<128>::kSmem : Cfg<64>::kSmem;
+        const void* fn = d128 ? (const void*)mssa_tc_whole_kernel<128> : (const void*)mssa_tc_whole_kernel<64>;
+        e = set_smem_attr(fn, smem, -1, kLaunchRegs);
+        if (e == cudaSuccess)
+            e = d128 ? launch_pdl(mssa_tc_whole_kernel<128>, dim3((unsigned)ctas), dim3(kThreads), smem, st, cache.maps,
+                                  tp, bounds)
+                     : launch_pdl(mssa_tc_whole_kernel<64>, dim3((unsigned)ctas), dim3(kThreads), smem, st, cache.maps,
+                                  tp, bounds);
+    } else if (own_pool) {
         if (!cache.attr_set[2]) {
             cudaFuncAttributes fa;
             e = cudaFuncGetAttributes(&fa, mssa_tc_pool_kernel);
