@@ -174,7 +174,11 @@ struct NoLora {};
 // (scaled, once) into one more A chunk, and the last K chunk is codes x up
 // projection. Every column tile of a token tile computes the codes again, which
 // costs a 64-wide MMA per K step; a launch of their own cost 4.8 us (480p).
-template <bool kLora, class Lora>
+//
+// kShare (its own instantiation): the tiles' idle warps pool. Compiled into the
+// plain kernel, that code alone made an attention behind a launch without
+// pyramid jobs end 1.5 us later (117.8 -> 119.3 us).
+template <bool kLora, bool kShare, class Lora>
 __global__ void __launch_bounds__(kThreads, 2)
     msp_embed_kernel(const __grid_constant__ EmbedMaps maps, const __grid_constant__ EmbedParams p,
                      const __grid_constant__ PoolBatch pool, const __grid_constant__ Lora lmaps) {
@@ -316,7 +320,7 @@ __global__ void __launch_bounds__(kThreads, 2)
         if (!ok && lane == 0) atomicOr(p.status, kDevTimeout);
     } else if (warp < 4) {
         // ---- warps 2 and 3: this tile's share of the pyramid jobs
-        if constexpr (!kLora) {
+        if constexpr (kShare) {
             const int total = pool.n * p.pool_tasks;
             int t = R.pool_base + local * 64 * R.pool_per + (int)threadIdx.x - 64;
             for (int k = 0; k < R.pool_per && t < total; ++k, t += 64)
@@ -895,9 +899,6 @@ cudaError_t launch_msp_embed(const MspEmbedRun* runs, int n, const MspShape& sh,
     p.tok_bstride = tok_bstride;
     p.status = status;
     if (lora && pool && pool->n > 0) return cudaErrorInvalidValue;  // no caller pools beside adapters
-    const void* fn = lora ? (const void*)msp_embed_kernel<true, LoraMaps> : (const void*)msp_embed_kernel<false, NoLora>;
-    cudaError_t e = set_smem_attr(fn, kEmbedSmem, 100);
-    if (e != cudaSuccess) return e;
     p.n_embed_tiles = tiles;
     PoolBatch pb;
     if (pool && pool->n > 0) {
@@ -913,7 +914,7 @@ cudaError_t launch_msp_embed(const MspEmbedRun* runs, int n, const MspShape& sh,
         // three / two and four: 480p with the history 16.2 / 16.1 / 14.7, window
         // only 11.5 / 10.9 / 11.7, four streams 79.8 / 74.4 / 72.5 and 51.8 / 46.8
         // / 45.4; where every pool CTA starts at once they only cost (6.6 / 7.0 /
-        // 7.6).
+        // 7.6), and at 410 CTAs still (5.65 / - / 5.8).
         auto share_of = [&](int one, int more) {
             long long x = 0;
             for (int i = 0; i < n; ++i)
@@ -921,7 +922,7 @@ cudaError_t launch_msp_embed(const MspEmbedRun* runs, int n, const MspShape& sh,
             return x;
         };
         int one = 0, more = 0;
-        if (batch * (tiles + (total + kThreads - 1) / kThreads) > 2 * 152) {
+        if (batch * (tiles + (total + kThreads - 1) / kThreads) > 3 * 152) {
             if (4 * share_of(2, 4) <= total)
                 one = 2, more = 4;
             else if (3 * share_of(1, 3) <= total)
@@ -937,9 +938,20 @@ cudaError_t launch_msp_embed(const MspEmbedRun* runs, int n, const MspShape& sh,
     } else {
         memset(&pb, 0, sizeof(pb));
     }
+    const bool share = p.pool_first > 0;
+    const void* fn = lora    ? (const void*)msp_embed_kernel<true, false, LoraMaps>
+                     : share ? (const void*)msp_embed_kernel<false, true, NoLora>
+                             : (const void*)msp_embed_kernel<false, false, NoLora>;
+    cudaError_t e = set_smem_attr(fn, kEmbedSmem, 100);
+    if (e != cudaSuccess) return e;
     const dim3 grid((unsigned)(tiles + p.pool_ctas), 1, (unsigned)batch);
-    return lora ? launch_pdl(msp_embed_kernel<true, LoraMaps>, grid, dim3(kThreads), kEmbedSmem, st, maps, p, pb, lmaps)
-                : launch_pdl(msp_embed_kernel<false, NoLora>, grid, dim3(kThreads), kEmbedSmem, st, maps, p, pb, NoLora{});
+    if (lora)
+        return launch_pdl(msp_embed_kernel<true, false, LoraMaps>, grid, dim3(kThreads), kEmbedSmem, st, maps, p, pb,
+                          lmaps);
+    return share ? launch_pdl(msp_embed_kernel<false, true, NoLora>, grid, dim3(kThreads), kEmbedSmem, st, maps, p, pb,
+                              NoLora{})
+                 : launch_pdl(msp_embed_kernel<false, false, NoLora>, grid, dim3(kThreads), kEmbedSmem, st, maps, p,
+                              pb, NoLora{});
 }
 
 
