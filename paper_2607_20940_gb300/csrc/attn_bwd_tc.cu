@@ -46,6 +46,7 @@
 
 #include "attn_bwd_tc.h"
 #include "attn_tc.h"
+#include "bwd_items.h"
 #include "ptx.cuh"
 
 namespace msf {
@@ -127,7 +128,7 @@ struct BwdBars {
     // ready, dS^T written, dV and dK complete; the warps of a half meet
     uint64_t kst_full, kst_empty, vst_full, vst_empty, q_full[3], q_empty[3], g_full[2], g_empty[2];
     uint64_t st_full, p_full, dpt_full, dst_full, kv_full, meet[2];
-    uint64_t item_done, drain;
+    uint64_t item_done[kDoneBars], drain;
     uint32_t tmem_base;
     int abort_flag;
 };
@@ -292,7 +293,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         ptx::mbar_init(&bar.ds_full[1], 8);
         ptx::mbar_init(&bar.p_full, 8);
         ptx::mbar_init(&bar.dst_full, 8);
-        ptx::mbar_init(&bar.item_done, 8);
+        for (int s = 0; s < kDoneBars; ++s) ptx::mbar_init(&bar.item_done[s], 8);
         ptx::fence_mbar_init();
     }
     if (warp == 2) {
@@ -326,11 +327,12 @@ __global__ void __launch_bounds__(kThreads, 1)
                 const int idx = next_item(p, order, k);
                 if (idx >= p.n_items) break;
                 const BItem it = item_of(p, idx);
-                // The item before the last is done (so that the phases of
-                // item_done are seen one by one); on a change of kind the last
-                // one too, whose tiles this one's overwrite.
-                if (k >= 2 && !take(&bar.item_done, (uint32_t)(k & 1))) break;
-                if (k >= 1 && it.kind != prev_kind && !take(&bar.item_done, (uint32_t)((k - 1) & 1))) break;
+                // The item before the last is done (so that every phase of
+                // item_done is seen); on a change of kind the last one too,
+                // whose tiles this one's overwrite.
+                auto done = [&](int i) { return take(&bar.item_done[done_bar(i)], done_parity(i)); };
+                if (k >= 2 && !done(k - 2)) break;
+                if (k >= 1 && it.kind != prev_kind && !done(k - 1)) break;
                 prev_kind = it.kind;
                 if (it.kind == 0) {
                     const BGroupQ& G = p.g[it.gi];
@@ -807,7 +809,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             // the item's accumulators are read: the next item's MMAs may
             // overwrite them (its first P or dS is written after this)
             ptx::tc_fence_before();
-            arrive(&bar.item_done);
+            arrive(&bar.item_done[done_bar(k)]);
         }
         if (!ok && lane == 0) atomicOr(p.status, kDevTimeout);
     }
