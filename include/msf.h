@@ -284,7 +284,9 @@ msf_status msf_patchify_tiers(msf_plan_t plan, const void* latent, const msf_tie
  * chunks (patch vectors gathered from latent_in) are summed in one fp32
  * accumulation, the codes g * Ao h in a second beside it (both split over a
  * cluster); the codes, rounded once to bf16, times Uo are added in fp32 and
- * the sum is rounded once. Errors: INVALID_ARG,
+ * the sum is rounded once. latent_out may lie over latent_in (the state's new
+ * latent over its old one): the input is then copied to the workspace by a
+ * launch of its own first. Errors: INVALID_ARG,
  * UNSUPPORTED (fp32 plan, no embedding, K or E not a multiple of 64), STATE,
  * CUDA. */
 msf_status msf_unpatchify_tier(msf_plan_t plan, int32_t position, const void* tokens,

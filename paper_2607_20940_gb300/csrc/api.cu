@@ -49,6 +49,10 @@ namespace {
 
 bool aligned16(const void* p) { return ((uintptr_t)p & 15u) == 0; }
 
+bool overlap(const void* a, size_t a_bytes, const void* b, size_t b_bytes) {
+    return (uintptr_t)a < (uintptr_t)b + b_bytes && (uintptr_t)b < (uintptr_t)a + a_bytes;
+}
+
 msf_status cuda_status(cudaError_t e) {
     if (e == cudaSuccess) return MSF_OK;
     msf::set_cuda_error((int)e);
@@ -974,9 +978,21 @@ extern "C" msf_status msf_unpatchify_tier(msf_plan_t plan, int32_t position, con
         extra.scale = tier->lora_scale;
     }
     if (tier->residual) {
-        extra.latent = (const char*)latent_in + (size_t)position * per * 2;
+        const char* in = (const char*)latent_in + (size_t)position * per * 2;
+        extra.latent = in;
         extra.latent_bstride = (long long)p.T * per;
         extra.residual = tier->residual;
+        // Every tile of a row reads the row's whole patch vectors and writes some
+        // of its features, so an output over the input is computed from a copy.
+        // (A state is a multiple of 64 elements: F is, see msp_deembed_supported.)
+        const size_t span = ((size_t)(p.B - 1) * p.T + 1) * per * 2;
+        if (overlap(latent_out, (size_t)p.B * per * 2, in, span)) {
+            char* raw = msf::msp_scratch(p);
+            cudaError_t e = msf::launch_copy_state(in, (long long)p.T * per / 8, raw, (int)(per / 8), p.B, s);
+            if (e != cudaSuccess) return cuda_status(e);
+            extra.latent = raw;
+            extra.latent_bstride = per;
+        }
     }
     return cuda_status(msf::launch_msp_deembed(tokens, (long long)p.N * E, p.N, p.st_off[position], tier->w_out,
                                                M, F, E, sh, P, latent_out, p.B, msf::status_word(p), s,

@@ -99,6 +99,9 @@ struct MspShape {
 // Raw patchify of every state into the [B, T, C*Hl*Wl] raw layout.
 cudaError_t launch_patchify_raw(const void* latent, void* raw, const MspShape& sh, int batch,
                                 bool bf16, cudaStream_t st);
+// `vecs` 16-byte vectors of every stream (streams src_bstride vectors apart),
+// to dst one stream after the other.
+cudaError_t launch_copy_state(const void* src, long long src_bstride, void* dst, int vecs, int batch, cudaStream_t st);
 cudaError_t launch_unpatchify_raw(const void* raw, void* latent, const MspShape& sh, int position,
                                   long long raw_bstride, int raw_offset, int batch, bool bf16,
                                   cudaStream_t st);

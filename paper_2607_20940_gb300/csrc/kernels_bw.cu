@@ -58,6 +58,18 @@ __global__ void __launch_bounds__(256) patchify_raw_kernel(const T* __restrict__
     raw[base + o] = latent[base + (size_t)c * sh.Hl * sh.Wl + (size_t)(P * i + dy) * sh.Wl + P * j + dx];
 }
 
+__global__ void __launch_bounds__(256) copy_state_kernel(const uint4* src, uint4* dst, long long src_bstride, int vecs) {
+    ptx::grid_dep_wait();
+    ptx::grid_dep_launch();
+    const int i = blockIdx.x * 256 + threadIdx.x;
+    if (i < vecs) dst[(long long)blockIdx.y * vecs + i] = src[blockIdx.y * src_bstride + i];
+}
+
+cudaError_t launch_copy_state(const void* src, long long src_bstride, void* dst, int vecs, int batch, cudaStream_t st) {
+    return launch_pdl(copy_state_kernel, dim3((unsigned)((vecs + 255) / 256), (unsigned)batch), dim3(256), 0, st,
+                      (const uint4*)src, (uint4*)dst, src_bstride, vecs);
+}
+
 template <typename T>
 __global__ void __launch_bounds__(256) unpatchify_raw_kernel(const T* __restrict__ raw,
                                                              T* __restrict__ latent, MspShape sh,
