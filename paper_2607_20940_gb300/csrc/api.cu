@@ -876,12 +876,16 @@ extern "C" msf_status msf_unpatchify(msf_plan_t plan, int32_t position, const vo
     g.ldc = F;
     g.a_bstride = (long long)p.N * E;
     g.c_bstride = per;
-    if (!bf16 && msf::gemm_f32_tc_supported(g)) {
-        // straight into the latent
+    const bool f32_tc = !bf16 && msf::gemm_f32_tc_supported(g);
+    // Straight into the latent, unless that lies over what the tiles still read.
+    const size_t out_bytes = (size_t)p.B * per * 4;
+    if (f32_tc && !overlap(latent_out, out_bytes, tokens, (size_t)p.B * p.N * E * 4) &&
+        !overlap(latent_out, out_bytes, w_out, (size_t)F * E * 4)) {
         g.C = latent_out;
         return cuda_status(msf::launch_gemm_f32_tc(&g, 1, p.B, msf::status_word(p), s, &sh, P));
     }
-    cudaError_t e = msf::launch_gemm_nt_simt(g, p.B, bf16, s);
+    cudaError_t e = f32_tc ? msf::launch_gemm_f32_tc(&g, 1, p.B, msf::status_word(p), s)
+                           : msf::launch_gemm_nt_simt(g, p.B, bf16, s);
     if (e != cudaSuccess) return cuda_status(e);
     return cuda_status(msf::launch_unpatchify_raw(raw, latent_out, sh, position, per, 0, p.B, bf16, s));
 }

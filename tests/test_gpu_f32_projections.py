@@ -86,3 +86,33 @@ def test_f32_projections_of_values_the_planes_cannot_hold(value):
         assert torch.equal(torch.isinf(a), torch.isinf(b)) and torch.equal(a[torch.isinf(a)], b[torch.isinf(b)])
         f = torch.isfinite(b)
         assert ((a[f] - b[f]).abs() <= 5e-6 * b[f].abs().clamp(min=1.0)).all()
+
+
+@pytest.mark.parametrize("shape", [SHAPES[2], SHAPES[4]], ids=["runs", "two_streams"])
+def test_f32_unpatchify_over_its_tokens(shape):
+    """A latent written over the tokens (or the weight) that it is computed from
+    has the bits of one written elsewhere."""
+    scales, (gh, gw), E, C, patch, B, F = shape
+    m = msf()
+    plan = m.Plan(m.make_desc(scales, gh, gw, 1, 64, 0, 0, batch=B, dtype=m.MSF_DTYPE_F32, latent_channels=C,
+                              patch=patch, embed_dim=E, frames_per_state=F))
+    ws = plan.workspace()
+    plan.bind(ws, None, None, None, None)
+    g = torch.Generator(device="cuda").manual_seed(3)
+    n = C * F * gh * gw * patch * patch
+    for pos in (0, len(scales) - 1):
+        h = torch.randn(B, plan.info.n_tokens, E, generator=g, device="cuda")
+        w = torch.randn(C * (patch * scales[pos]) ** 2, E, generator=g, device="cuda")
+        apart = torch.full((B * n,), float("nan"), device="cuda")
+        plan.unpatchify(pos, h, w, apart)
+        for over_tokens in (True, False):
+            src = h if over_tokens else w
+            room = torch.zeros(max(src.numel(), B * n) + 64, device="cuda")
+            room[32:32 + src.numel()] = src.flatten()
+            x = room[32:32 + src.numel()].view_as(src)
+            y = room[:B * n]
+            plan.unpatchify(pos, x if over_tokens else h, w if over_tokens else x, y)
+            torch.cuda.synchronize()
+            assert plan.device_status() == m.MSF_OK
+            assert torch.equal(y, apart)
+    del ws
