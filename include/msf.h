@@ -310,9 +310,12 @@ msf_status msf_kv_resample(msf_plan_t plan, const void* k_win, const void* v_win
  * pyramid the last msf_kv_resample on the same stream produced. bf16 plans
  * run the tcgen05 tensor-core kernel (bf16 operands, fp32 softmax and
  * accumulation); fp32 plans run the tensor cores on three bf16 planes per
- * value (24 bits), or, for a call with a value that is not finite or not below
- * 2^127 in magnitude, an fp32 CUDA-core kernel. Errors: INVALID_ARG, STATE,
- * CUDA. */
+ * value (each to 24 bits, or to 2^-30 of the largest of the eight neighbours
+ * along the head that it is split with), or, for a call whose operands they
+ * cannot hold (decided on the device), an fp32 CUDA-core kernel: a value that is not finite or not below 2^127, eight
+ * neighbours that are not all zero and all below 2^-96, or largest values
+ * between which a product leaves fp32's range (q k outside 2^-100 to 2^116,
+ * before or after the scale; v above 2^97). Errors: INVALID_ARG, STATE, CUDA. */
 msf_status msf_mssa_forward(msf_plan_t plan, const void* q, const void* k_win, const void* v_win,
                             void* out, void* stream);
 
@@ -355,7 +358,9 @@ msf_status msf_mssa_forward_lse(msf_plan_t plan, const void* q, const void* k_wi
  * bf16 plans run one persistent tcgen05 tensor-core kernel (dq of each query
  * tile over its whole context, dk/dv of each tile of window-derived rows);
  * fp32 plans run them on three bf16 planes per value (as the forward does),
- * or CUDA-core kernels where the planes cannot hold a value.
+ * or CUDA-core kernels where the planes cannot hold the operands (as there, and
+ * dout above 2^97, dout v outside 2^-70 to 2^80, or dout v q or dout v k outside
+ * 2^-80 to 2^80, of the largest values).
  * Errors: INVALID_ARG, STATE (not bound), WORKSPACE, CUDA. */
 msf_status msf_mssa_backward(msf_plan_t plan, const void* q, const void* k_win, const void* v_win,
                              const void* out, const void* dout, const float* lse, void* dq,

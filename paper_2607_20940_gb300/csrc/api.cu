@@ -587,13 +587,13 @@ static msf_status mssa_backward(msf_plan_t plan, const void* q, const void* k_wi
         msf_status st = msf::launch_bwd_tc(plan, in, s);
         if (st != MSF_OK) return st;
     } else {
-        msf::BwdRunIf run_if;  // the CUDA-core kernels: always, or where the planes cannot hold an operand
+        msf::F32Range unless = {};  // the CUDA-core kernels: always, or where the planes cannot hold the operands
         if (tc) {
             char* planes = (char*)bwd_ws + msf::bwd_delta_bytes(p) + 2 * msf::bwd_ctx_bytes(p);
-            msf_status st = msf::launch_bwd_f32_tc(plan, c, a, bg, (float*)dq, planes, &run_if, s);
+            msf_status st = msf::launch_bwd_f32_tc(plan, c, a, bg, (float*)dq, planes, &unless, s);
             if (st != MSF_OK) return st;
         }
-        e = msf::launch_bwd_simt(c, a, bg, dq, bf16, run_if, s);
+        e = msf::launch_bwd_simt(c, a, bg, dq, bf16, unless, s);
         if (e != cudaSuccess) return cuda_status(e);
     }
     return cuda_status(msf::launch_bwd_gather(c, ga, dk_win, dv_win, bf16, s));

@@ -19,6 +19,7 @@
 #include <cuda_runtime.h>
 #include <math.h>
 
+#include "f32_range.cuh"
 #include "kernels.h"
 #include "ptx.cuh"
 
@@ -88,14 +89,6 @@ __device__ __forceinline__ void stE(__nv_bfloat16* p, const float* x) {
 }
 
 constexpr float kLog2e = 1.4426950408889634f;
-
-// Whether a conditional kernel has to run (every thread of the block).
-__device__ __forceinline__ bool wanted(const BwdRunIf& c) {
-    if (!c.flags) return true;
-    bool f = false;
-    for (int i = threadIdx.x; i < c.n; i += blockDim.x) f |= __ldg(c.flags + i) != 0;
-    return __syncthreads_or(f);
-}
 
 // (The tensor-core backward, launched next, starts its loads of q, k, v and
 // dout without a wait of its own: the launch_dependents here comes after this
@@ -301,10 +294,10 @@ __device__ __forceinline__ void bwd_dkdv_rows(const BwdCommon& c, const BwdGroup
 template <typename T, int D>
 __global__ void __launch_bounds__(128, 3)
     bwd_simt_kernel(const BwdCommon c, const __grid_constant__ AttnArgs a, const __grid_constant__ BwdGroups groups,
-                    T* dq, int dq_tiles, const BwdRunIf run_if) {
+                    T* dq, int dq_tiles, const F32Range unless) {
     ptx::grid_dep_wait();
     ptx::grid_dep_launch();
-    if (!wanted(run_if)) return;
+    if (unless.words && planes_hold(unless)) return;
     __shared__ float s0[32][D];
     __shared__ float s1[32][D];
     __shared__ float l[32], d[32];
@@ -404,7 +397,7 @@ cudaError_t launch_bwd_delta(const BwdCommon& c, bool bf16, cudaStream_t st) {
 }
 
 cudaError_t launch_bwd_simt(const BwdCommon& c, const AttnArgs& a, const BwdGroup* g, void* dq, bool bf16,
-                            BwdRunIf run_if, cudaStream_t st) {
+                            const F32Range& unless, cudaStream_t st) {
     BwdGroups gs;
     gs.n = a.n_groups;
     int dq_tiles = 0, tiles = 0;
@@ -417,7 +410,7 @@ cudaError_t launch_bwd_simt(const BwdCommon& c, const AttnArgs& a, const BwdGrou
     if (tiles == 0) return cudaSuccess;
     dim3 grid((unsigned)tiles, (unsigned)c.H, (unsigned)c.B);
     auto run = [&](auto* kernel, auto* out) {
-        return launch_pdl(kernel, grid, dim3(128), 0, st, c, a, gs, out, dq_tiles, run_if);
+        return launch_pdl(kernel, grid, dim3(128), 0, st, c, a, gs, out, dq_tiles, unless);
     };
     if (c.D == 128)
         return bf16 ? run(bwd_simt_kernel<__nv_bfloat16, 128>, (__nv_bfloat16*)dq)

@@ -33,6 +33,7 @@
 
 #include "attn_bwd_tc.h"
 #include "attn_f32_tc.h"
+#include "f32_range.cuh"
 #include "ptx.cuh"
 
 namespace msf {
@@ -85,8 +86,7 @@ struct FBParams {
     float* dk_ctx;
     float* dv_ctx;
     float* partials;  // [slot][128][D]
-    const unsigned int* flags;
-    int n_flags;
+    F32Range range;
     unsigned int* status;
     long long wait_limit;
     int n_classes;
@@ -106,12 +106,6 @@ __device__ __forceinline__ float ex2(float x) {
     float y;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
-}
-
-__device__ __forceinline__ bool any_flag(const unsigned int* flags, int n) {
-    bool f = false;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) f |= __ldg(flags + i) != 0;
-    return __syncthreads_or(f);
 }
 
 // Own tile `own` of class c: the run it belongs to (dK, dV) and its tile there.
@@ -195,7 +189,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     volatile int never = 0;
     ptx::grid_dep_wait();
     ptx::grid_dep_launch();
-    const bool skip = any_flag(p.flags, p.n_flags);  // the CUDA-core kernels answer instead
+    const bool skip = !planes_hold(p.range);  // the CUDA-core kernels answer instead
 
     // other tile u: map of K/V (dQ), first row, valid rows
     auto tile_of = [&](int u, int& map, int& row, int& valid) {
@@ -531,7 +525,7 @@ __global__ void __launch_bounds__(256) bwd_f32_merge_kernel(const __grid_constan
     using C = FBCfg<D>;
     ptx::grid_dep_wait();
     ptx::grid_dep_launch();
-    if (any_flag(p.flags, p.n_flags)) return;
+    if (!planes_hold(p.range)) return;
     int ci = 0;
     while (ci + 1 < p.n_classes && (p.c[ci].n_split == 1 || (int)blockIdx.x >= p.c[ci + 1].item_base)) ++ci;
     const FBClass& cl = p.c[ci];
@@ -575,7 +569,7 @@ __global__ void __launch_bounds__(256) bwd_f32_merge_kernel(const __grid_constan
 }  // namespace
 
 msf_status launch_bwd_f32_tc(msf_plan_t plan, const BwdCommon& c, const AttnArgs& a, const BwdGroup* bg, float* dq,
-                             char* dout_planes, BwdRunIf* run_if, cudaStream_t st) {
+                             char* dout_planes, F32Range* range, cudaStream_t st) {
     const Plan& P = *plan;
     auto fail = [](cudaError_t e) {
         set_cuda_error((int)e);
@@ -591,8 +585,8 @@ msf_status launch_bwd_f32_tc(msf_plan_t plan, const BwdCommon& c, const AttnArgs
     memset(&sp, 0, sizeof(sp));
     F32Maps maps;
     memset(&maps, 0, sizeof(maps));
-    sp.flags = f32_flags(P);
-    if (!add_context_planes(P, a, sp, maps) || !add_planes(P, sp, c.dout, c.bstride, dout_planes, P.N, P.N, &maps.dout))
+    sp.words = f32_range_words(P);
+    if (!add_context_planes(P, a, sp, maps) || !add_planes(P, sp, kRangeDout, c.dout, c.bstride, dout_planes, P.N, P.N, &maps.dout))
         return fail(cudaErrorInvalidValue);
     FBParams fp;
     memset(&fp, 0, sizeof(fp));
@@ -609,7 +603,6 @@ msf_status launch_bwd_f32_tc(msf_plan_t plan, const BwdCommon& c, const AttnArgs
     fp.dk_ctx = c.dk_ctx;
     fp.dv_ctx = c.dv_ctx;
     fp.partials = f32_partials(P);
-    fp.flags = sp.flags;
     fp.status = a.status;
     fp.wait_limit = kWaitLimit;
     const size_t row = (size_t)P.H * P.D * 4;
@@ -680,10 +673,9 @@ msf_status launch_bwd_f32_tc(msf_plan_t plan, const BwdCommon& c, const AttnArgs
         }
     }
     if (slots > max_slots) return MSF_ERR_STATE;
-    e = launch_split_planes(sp, &fp.n_flags, st);
+    e = launch_split_planes(sp, c.scale_log2, &fp.range, st);
     if (e != cudaSuccess) return fail(e);
-    run_if->flags = sp.flags;
-    run_if->n = fp.n_flags;
+    *range = fp.range;
     if (units == 0) return MSF_OK;
     const bool d128 = P.D == 128;
     const int smem = d128 ? FBCfg<128>::kSmem : FBCfg<64>::kSmem;

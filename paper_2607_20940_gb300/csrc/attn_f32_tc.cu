@@ -40,6 +40,7 @@
 
 #include "attn_f32_tc.h"
 #include "attn_tc.h"
+#include "f32_range.cuh"
 #include "ptx.cuh"
 #include "sched.h"
 
@@ -61,7 +62,7 @@ constexpr long long kWaitLimit = 2000000000LL;  // ~1 s of SM clock
 __global__ void __launch_bounds__(256) split_planes_kernel(const __grid_constant__ SplitParams p) {
     ptx::grid_dep_wait();
     ptx::grid_dep_launch();
-    bool bad = false;
+    uint32_t codes = 0;
     for (long long i = blockIdx.x * 256 + threadIdx.x; i < p.total; i += gridDim.x * 256) {
         int k = 0;
         while (k + 1 < p.n && i >= p.j[k + 1].base) ++k;
@@ -71,20 +72,17 @@ __global__ void __launch_bounds__(256) split_planes_kernel(const __grid_constant
         const float4* s = reinterpret_cast<const float4*>(J.src + b * J.src_bstride + 8ll * v);
         const float4 x0 = __ldg(s), x1 = __ldg(s + 1);
         const float x[8] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w};
+        codes = __vmaxu4(codes, range_code(max(abs_bits4(x0), abs_bits4(x1))) << (8 * J.operand));
         uint32_t h[4], m[4], l[4];
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            ptx::split_bf16(x[2 * e], x[2 * e + 1], h[e], m[e], l[e]);
-            bad |= ((__float_as_uint(x[2 * e]) >> 23) & 255u) >= 254u ||
-                   ((__float_as_uint(x[2 * e + 1]) >> 23) & 255u) >= 254u;
-        }
+        for (int e = 0; e < 4; ++e) ptx::split_bf16(x[2 * e], x[2 * e + 1], h[e], m[e], l[e]);
         __nv_bfloat16* d = J.dst + b * J.dst_bstride + 8ll * v;
         *reinterpret_cast<uint4*>(d) = make_uint4(h[0], h[1], h[2], h[3]);
         *reinterpret_cast<uint4*>(d + J.dst_plane) = make_uint4(m[0], m[1], m[2], m[3]);
         *reinterpret_cast<uint4*>(d + 2 * J.dst_plane) = make_uint4(l[0], l[1], l[2], l[3]);
     }
-    bad = __syncthreads_or(bad);
-    if (threadIdx.x == 0) p.flags[blockIdx.x] = bad ? 1u : 0u;
+    codes = block_codes(codes);
+    if (threadIdx.x == 0) p.words[blockIdx.x] = codes;
 }
 
 // --------------------------------------------------------------- attention
@@ -108,8 +106,7 @@ struct FParams {
     float* out;
     float* lse;       // optional [B, H, N]
     float* partials;  // [slot]([128][D] output, [128] running max, [128] sum)
-    const unsigned int* flags;
-    int n_flags;
+    F32Range range;
     unsigned int* status;
     long long wait_limit;
 };
@@ -125,13 +122,6 @@ __device__ __forceinline__ float ex2(float x) {
     float y;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
-}
-
-// Whether a block of the split saw a value the planes cannot hold (all threads).
-__device__ __forceinline__ bool any_flag(const unsigned int* flags, int n) {
-    bool f = false;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) f |= __ldg(flags + i) != 0;
-    return __syncthreads_or(f);
 }
 
 template <int D>
@@ -191,7 +181,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     volatile int never = 0;
     ptx::grid_dep_wait();
     ptx::grid_dep_launch();
-    const bool skip = any_flag(p.flags, p.n_flags);  // the CUDA-core kernel answers instead
+    const bool skip = !planes_hold(p.range);  // the CUDA-core kernel answers instead
 
     auto tile_of = [&](int u, int& map, int& row, int& valid) {
         int s = 0;
@@ -462,7 +452,7 @@ __global__ void __launch_bounds__(256) merge_f32_kernel(const __grid_constant__ 
     using C = FCfg<D>;
     ptx::grid_dep_wait();
     ptx::grid_dep_launch();
-    if (any_flag(p.flags, p.n_flags)) return;
+    if (!planes_hold(p.range)) return;
     int tile = blockIdx.x, gi = 0;
     for (; gi < p.n_groups; ++gi) {
         const int nt = p.g[gi].n_split > 1 ? p.g[gi].n_qt * p.H * p.B : 0;
@@ -582,8 +572,8 @@ int f32_unit_tiles(const F32Class* c, int n, int D, int sms, int max_slots) {
     return best;
 }
 
-bool add_planes(const Plan& P, SplitParams& sp, const void* src, long long src_bstride_bytes, char* dst, int alloc,
-                int rows, CUtensorMap* m) {
+bool add_planes(const Plan& P, SplitParams& sp, int operand, const void* src, long long src_bstride_bytes, char* dst,
+                int alloc, int rows, CUtensorMap* m) {
     const long long rowe = (long long)P.H * P.D;
     SplitJob& j = sp.j[sp.n++];
     j.src = (const float*)src;
@@ -592,6 +582,7 @@ bool add_planes(const Plan& P, SplitParams& sp, const void* src, long long src_b
     j.dst_plane = alloc * rowe;
     j.dst_bstride = 3 * j.dst_plane;
     j.vecs = (int)(rows * rowe / 8);
+    j.operand = operand;
     j.base = sp.total;
     sp.total += (long long)j.vecs * P.B;
     return encode_rows(m, dst, P.D, P.H, rows, 3 * P.B, j.dst_plane * 2);
@@ -599,7 +590,7 @@ bool add_planes(const Plan& P, SplitParams& sp, const void* src, long long src_b
 
 bool add_context_planes(const Plan& P, const AttnArgs& a, SplitParams& sp, F32Maps& maps) {
     const size_t rowe = (size_t)P.H * P.D;
-    if (!add_planes(P, sp, a.q, a.q_bstride, f32_planes(P, kF32Q, 0), P.N, P.N, &maps.q)) return false;
+    if (!add_planes(P, sp, kRangeQ, a.q, a.q_bstride, f32_planes(P, kF32Q, 0), P.N, P.N, &maps.q)) return false;
     bool done[kNumMaps] = {false};
     for (int gi = 0; gi < a.n_groups; ++gi)
         for (int s = 0; s < a.g[gi].n_seg; ++s) {
@@ -615,17 +606,21 @@ bool add_context_planes(const Plan& P, const AttnArgs& a, SplitParams& sp, F32Ma
             const size_t off = pyr ? (size_t)3 * P.B * P.groups[gi].pyr_offset * rowe * 2 : 0;
             const int alloc = pyr ? P.groups[gi].pyr_cap : f32_part_rows(P, part);
             const size_t so = pyr ? (size_t)sg.row0 * rowe * 4 : 0;
-            if (!add_planes(P, sp, sg.k + so, sg.bstride, f32_planes(P, part, 0) + off, alloc, rows, &maps.k[map]) ||
-                !add_planes(P, sp, sg.v + so, sg.bstride, f32_planes(P, part, 1) + off, alloc, rows, &maps.v[map]))
+            if (!add_planes(P, sp, kRangeK, sg.k + so, sg.bstride, f32_planes(P, part, 0) + off, alloc, rows,
+                            &maps.k[map]) ||
+                !add_planes(P, sp, kRangeV, sg.v + so, sg.bstride, f32_planes(P, part, 1) + off, alloc, rows,
+                            &maps.v[map]))
                 return false;
         }
     return true;
 }
 
-cudaError_t launch_split_planes(const SplitParams& sp, int* n_flags, cudaStream_t st) {
+cudaError_t launch_split_planes(const SplitParams& sp, float scale_log2, F32Range* range, cudaStream_t st) {
     const long long want = (sp.total + 255) / 256;
-    *n_flags = want < kF32SplitBlocks ? (int)want : kF32SplitBlocks;
-    return launch_pdl(split_planes_kernel, dim3((unsigned)*n_flags), dim3(256), 0, st, sp);
+    range->words = sp.words;
+    range->n = want < kF32SplitBlocks ? (int)want : kF32SplitBlocks;
+    frexpf(scale_log2, &range->scale_exp);
+    return launch_pdl(split_planes_kernel, dim3((unsigned)range->n), dim3(256), 0, st, sp);
 }
 
 msf_status launch_attn_f32_tc(msf_plan_t plan, const AttnArgs& a, cudaStream_t st) {
@@ -645,7 +640,7 @@ msf_status launch_attn_f32_tc(msf_plan_t plan, const AttnArgs& a, cudaStream_t s
     memset(&maps, 0, sizeof(maps));
     FParams fp;
     memset(&fp, 0, sizeof(fp));
-    sp.flags = f32_flags(P);
+    sp.words = f32_range_words(P);
     if (!add_context_planes(P, a, sp, maps)) return fail(cudaErrorInvalidValue);
     fp.n_groups = a.n_groups;
     for (int gi = 0; gi < a.n_groups; ++gi) {
@@ -673,7 +668,6 @@ msf_status launch_attn_f32_tc(msf_plan_t plan, const AttnArgs& a, cudaStream_t s
     fp.out = (float*)a.out;
     fp.lse = a.lse;
     fp.partials = f32_partials(P);
-    fp.flags = sp.flags;
     fp.status = a.status;
     fp.wait_limit = kWaitLimit;
     F32Class cls[MSF_MAX_GROUPS];
@@ -702,7 +696,7 @@ msf_status launch_attn_f32_tc(msf_plan_t plan, const AttnArgs& a, cudaStream_t s
     }
     if (units == 0) return MSF_OK;
     if (slots > f32_max_slots(P)) return MSF_ERR_STATE;
-    e = launch_split_planes(sp, &fp.n_flags, st);
+    e = launch_split_planes(sp, a.scale_log2, &fp.range, st);
     if (e != cudaSuccess) return fail(e);
     const bool d128 = P.D == 128;
     const int smem = d128 ? FCfg<128>::kSmem : FCfg<64>::kSmem < 120 * 1024 ? 120 * 1024 : FCfg<64>::kSmem;
@@ -717,8 +711,7 @@ msf_status launch_attn_f32_tc(msf_plan_t plan, const AttnArgs& a, cudaStream_t s
                  : launch_pdl(merge_f32_kernel<64>, dim3((unsigned)merges, 8), dim3(256), 0, st, fp);
     if (e != cudaSuccess) return fail(e);
     AttnArgs fallback = a;
-    fallback.run_if = sp.flags;
-    fallback.n_run_if = fp.n_flags;
+    fallback.unless = fp.range;
     e = launch_attn_simt(fallback, false, st);
     return e == cudaSuccess ? MSF_OK : fail(e);
 }

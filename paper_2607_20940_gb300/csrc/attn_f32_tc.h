@@ -6,6 +6,7 @@
 #include <cuda_runtime.h>
 
 #include "attn_tc.h"
+#include "f32_range.h"
 #include "internal.h"
 #include "kernels.h"
 
@@ -17,6 +18,7 @@ struct SplitJob {
     __nv_bfloat16* dst;  // stream 0, plane 0
     long long src_bstride, dst_bstride, dst_plane;  // elements
     int vecs;            // 8-element vectors per stream
+    int operand;         // kRangeQ, ..
     long long base;      // first vector of the job (all streams) in the launch
 };
 constexpr int kMaxSplitJobs = 2 + 2 * (3 + MSF_MAX_GROUPS);
@@ -24,7 +26,7 @@ struct SplitParams {
     SplitJob j[kMaxSplitJobs];
     int n;
     long long total;
-    unsigned int* flags;  // one word per block: 1 = a value the planes cannot hold
+    unsigned int* words;  // one word of range codes per block (f32_range.h)
 };
 struct F32Maps {
     CUtensorMap q, dout;
@@ -33,12 +35,12 @@ struct F32Maps {
 };
 // Add the first `rows` rows per stream of a [B, .., H, D] fp32 tensor as planes
 // [B, 3, alloc, H, D] at `dst` to the split, and encode their tensor map.
-bool add_planes(const Plan& P, SplitParams& sp, const void* src, long long src_bstride_bytes, char* dst, int alloc,
-                int rows, CUtensorMap* m);
+bool add_planes(const Plan& P, SplitParams& sp, int operand, const void* src, long long src_bstride_bytes, char* dst,
+                int alloc, int rows, CUtensorMap* m);
 // q and the k, v of every context segment of `a`, in the workspace's planes.
 bool add_context_planes(const Plan& P, const AttnArgs& a, SplitParams& sp, F32Maps& maps);
-// Write the planes and the flags; *n_flags is the number of flag words.
-cudaError_t launch_split_planes(const SplitParams& sp, int* n_flags, cudaStream_t st);
+// Write the planes and the range words, which *range then names.
+cudaError_t launch_split_planes(const SplitParams& sp, float scale_log2, F32Range* range, cudaStream_t st);
 // A class of equal own tiles (query tiles of a group, gradient rows of one) and
 // the other tiles each walks; `weight`: the cost of one, K/V tile = 1.
 constexpr int kMaxF32Classes = 3 * MSF_MAX_GROUPS;

@@ -2,7 +2,7 @@
 //
 // The cross-check of the tensor-core kernels (max |err| <= 1e-4 against the
 // fp64 definition), and the fp32 path of operands that three bf16 planes
-// cannot hold (run_if: the plane split's flags). A block owns 32
+// cannot hold (`unless`: what the plane split found). A block owns 32
 // queries of one (stream, head, group); four threads share a query, each
 // holding every fourth element of q and of the running output, so that a
 // warp reads four consecutive shared-memory words per key (no bank
@@ -12,6 +12,7 @@
 #include <cuda_runtime.h>
 #include <math.h>
 
+#include "f32_range.cuh"
 #include "kernels.h"
 #include "ptx.cuh"
 
@@ -34,11 +35,7 @@ template <typename T, int D>
 __global__ void __launch_bounds__(128) attn_simt_kernel(const AttnArgs a) {
     ptx::grid_dep_wait();
     ptx::grid_dep_launch();
-    if (a.run_if) {
-        bool f = false;
-        for (int i = threadIdx.x; i < a.n_run_if; i += 128) f |= __ldg(a.run_if + i) != 0;
-        if (!__syncthreads_or(f)) return;
-    }
+    if (a.unless.words && planes_hold(a.unless)) return;
     constexpr int DP = D / 4;
     constexpr int KT = 32;
     __shared__ float Ks[KT][D];

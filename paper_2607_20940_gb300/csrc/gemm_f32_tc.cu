@@ -7,8 +7,8 @@
 // so that rounding at full size happens only in the four hh steps of each
 // 64-wide K chunk. A 128 x BN tile's K chunks are split over a thread-block
 // cluster; the CTAs' sums meet in distributed shared memory in a fixed order.
-// A CTA that reads a value that the planes cannot hold (not finite, or not
-// below 2^127) redoes its share with fp32 FMAs.
+// A CTA that reads operands that the planes cannot hold (f32_range.h) redoes its
+// share with fp32 FMAs.
 //
 // Bound: at K = 64 (the fine tier) the fp32 output's writes, at the
 // de-embedding's K = E latency, with the split's integer and FMA work (about
@@ -21,6 +21,7 @@
 #include <cuda_runtime.h>
 #include <string.h>
 
+#include "f32_range.cuh"
 #include "gemm_f32_tc.h"
 #include "ptx.cuh"
 
@@ -121,14 +122,13 @@ __global__ void __launch_bounds__(kThreads, 2) gemm_f32_kernel(const __grid_cons
                                        : make_float4(0.f, 0.f, 0.f, 0.f);
         }
     };
-    bool bad = false, ok = true;
-    auto put = [&](unsigned char* dst, int plane_bytes, int row, const float4& x) {
+    bool ok = true;
+    uint32_t code_a = 0, code_b = 0;
+    auto put = [&](unsigned char* dst, int plane_bytes, int row, const float4& x, uint32_t& code) {
         uint2 h, m, l;
         ptx::split_bf16(x.x, x.y, h.x, m.x, l.x);
         ptx::split_bf16(x.z, x.w, h.y, m.y, l.y);
-        const uint32_t big = 254u << 23;
-        bad |= (__float_as_uint(x.x) & 0x7f800000u) >= big || (__float_as_uint(x.y) & 0x7f800000u) >= big ||
-               (__float_as_uint(x.z) & 0x7f800000u) >= big || (__float_as_uint(x.w) & 0x7f800000u) >= big;
+        code = max(code, range_code(abs_bits4(x)));
         const uint32_t o = swz4(row, k4);
         *reinterpret_cast<uint2*>(dst + o) = h;
         *reinterpret_cast<uint2*>(dst + plane_bytes + o) = m;
@@ -139,9 +139,9 @@ __global__ void __launch_bounds__(kThreads, 2) gemm_f32_kernel(const __grid_cons
         // the chunk before has been multiplied: its space is free
         if (c > c0) ok = ok && ptx::mbar_wait_bounded(&mma_bar, (uint32_t)((c - c0 - 1) & 1), &abort_flag, kWaitLimit);
 #pragma unroll
-        for (int i = 0; i < RA; ++i) put(sA, kPlane, r0 + 16 * i, xa[i]);
+        for (int i = 0; i < RA; ++i) put(sA, kPlane, r0 + 16 * i, xa[i], code_a);
 #pragma unroll
-        for (int i = 0; i < RB; ++i) put(sB, C::kB, r0 + 16 * i, xb[i]);
+        for (int i = 0; i < RB; ++i) put(sB, C::kB, r0 + 16 * i, xb[i], code_b);
         ptx::fence_proxy_async_smem();
         __syncthreads();
         if (warp == 0) {
@@ -168,7 +168,8 @@ __global__ void __launch_bounds__(kThreads, 2) gemm_f32_kernel(const __grid_cons
     }
     if (c0 < c1) ok = ok && ptx::mbar_wait_bounded(&mma_bar, (uint32_t)((c1 - c0 - 1) & 1), &abort_flag, kWaitLimit);
     if (!ok && lane == 0) atomicOr(p.status, kDevTimeout);
-    const bool redo = __syncthreads_or(bad);
+    const uint32_t codes = block_codes(code_a | code_b << 8);
+    const bool redo = !range_holds_gemm(codes & 255u, codes >> 8);
     ptx::tc_fence_after();
     // ---- this CTA's share of the sums into shared memory
     if (redo) {

@@ -63,7 +63,7 @@ using Plan = ::msf_plan;
 
 // Workspace layout: [status area | pyramid K | pyramid V | MSP scratch | attention
 // merge counters | attention partial slots | de-embedding split partials | fp32 plans: operand
-// planes, unit partials and flags]
+// planes, unit partials and range words]
 constexpr size_t kStatusBytes = 256;
 inline size_t round256(size_t x) { return (x + 255) / 256 * 256; }
 inline size_t pyramid_bytes(const Plan& p) {
@@ -100,8 +100,8 @@ constexpr int kTierCodeCols = 64;  // largest LoRA rank of a tier module
 // fp32 plans: the tensor-core attention's operands as three bf16 planes,
 // [B, 3, rows, H, D] for q and for k, v of the sink, the ring, each group's
 // pyramid part and the window; the output units of split query tiles, each
-// [128 rows][D] fp32 and the rows' running max and sum; and one flag word per
-// block of the kernel that writes the planes.
+// [128 rows][D] fp32 and the rows' running max and sum; and one word of range
+// codes per block of the kernel that writes the planes.
 enum : int { kF32Q = 0, kF32Sink = 1, kF32Ring = 2, kF32Pyr = 3, kF32Win = 4 };
 constexpr int kF32MaxSms = 160;
 constexpr int kF32MaxRounds = 6;       // rounds of units per SM when tiles are split
@@ -179,7 +179,7 @@ inline char* f32_planes(const Plan& p, int part, int which) {  // which: 0 = q o
 inline float* f32_partials(const Plan& p) {
     return (float*)(f32_planes(p, kF32Q, 0) + f32_plane_bytes(p));
 }
-inline unsigned int* f32_flags(const Plan& p) {
+inline unsigned int* f32_range_words(const Plan& p) {
     return (unsigned int*)((char*)f32_partials(p) + round256((size_t)f32_max_slots(p) * 128 * (p.D + 2) * 4));
 }
 

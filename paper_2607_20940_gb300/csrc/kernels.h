@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "f32_range.h"
 #include "internal.h"
 
 namespace msf {
@@ -150,9 +151,7 @@ struct AttnArgs {
     unsigned int* status;
     float* lse;           // optional [B, H, N] row log-sum-exp (natural log); NULL = none
     int N;                // query rows per stream
-    // CUDA-core kernel only: run only if one of these words is set (NULL = run).
-    const unsigned int* run_if;
-    int n_run_if;
+    F32Range unless;      // CUDA-core kernel only: do nothing if the planes hold the operands
 };
 cudaError_t launch_attn_simt(const AttnArgs& a, bool bf16, cudaStream_t st);
 
@@ -210,15 +209,11 @@ struct GatherArgs {
     int mode;  // msf_resample_mode
 };
 cudaError_t launch_bwd_delta(const BwdCommon& c, bool bf16, cudaStream_t st);
-// Run a kernel only if one of these n words is set (NULL = run).
-struct BwdRunIf {
-    const unsigned int* flags = nullptr;
-    int n = 0;
-};
 // On CUDA cores: dq for every query of every group (context of each group as in
-// the forward) and the context-row gradients of every group's window-derived rows.
+// the forward) and the context-row gradients of every group's window-derived
+// rows; nothing if the planes hold the operands.
 cudaError_t launch_bwd_simt(const BwdCommon& c, const AttnArgs& a, const BwdGroup* g, void* dq, bool bf16,
-                            BwdRunIf run_if, cudaStream_t st);
+                            const F32Range& unless, cudaStream_t st);
 // dk_win, dv_win from the context-row gradients (adjoint of Subsample, sum
 // over groups, one rounding to the dtype).
 cudaError_t launch_bwd_gather(const BwdCommon& c, const GatherArgs& g, void* dk, void* dv,

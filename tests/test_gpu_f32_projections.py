@@ -88,6 +88,22 @@ def test_f32_projections_of_values_the_planes_cannot_hold(value):
         assert ((a[f] - b[f]).abs() <= 5e-6 * b[f].abs().clamp(min=1.0)).all()
 
 
+@pytest.mark.parametrize("ua,ub", [(-40, 40), (-112, 112), (112, -112), (-112, 0), (0, -105), (-60, -55), (60, 60)])
+def test_f32_projections_magnitudes(ua, ub):
+    """fp32's precision on both sides of csrc/f32_range.h (powers of two change no rounding)."""
+    def edit(lat, wt, h, wo):
+        lat *= 2.0 ** ua
+        h *= 2.0 ** ua
+        for x in (wt, wo):
+            for s in x:
+                x[s] *= 2.0 ** ub
+    tok, ref, back, lats = _run(SHAPES[1], edit)
+    u = 2.0 ** -(ua + ub)
+    assert ((tok.double() - ref) * u).abs().max() <= 5e-6
+    for y, r in zip(back, lats):
+        assert ((y.double() - r) * u).abs().max() <= 5e-6
+
+
 @pytest.mark.parametrize("shape", [SHAPES[2], SHAPES[4]], ids=["runs", "two_streams"])
 def test_f32_unpatchify_over_its_tokens(shape):
     """A latent written over the tokens (or the weight) that it is computed from

@@ -38,8 +38,8 @@ CASES = [
 ]
 
 
-def _forward(w, x):
-    plan = make_plan(w, F32)
+def _forward(w, x, plan=None):
+    plan = plan or make_plan(w, F32)
     d = device_inputs(x, w.history_capacity)
     ws = bind(plan, d)
     out = torch.full_like(d["q"], float("nan"))
@@ -101,7 +101,82 @@ def test_f32_tensor_attention_small_and_large_values():
     assert mx <= 1.5e-5, mx
 
 
-def _backward(w, x, seed=9):
+# ---- magnitudes on both sides of csrc/f32_range.h. Outside, the call gives exactly
+# what the CUDA-core kernel gives; on both sides fp32's precision is kept (the same
+# bounds as above, of results scaled back: powers of two change no rounding).
+def _scaled(w, uq=0, uk=0, uv=0):
+    x = synth.attention_inputs(w, F32)
+    u = {"q": uq, "k": uk, "v": uv}
+    return {k: t * 2.0 ** u[k[0]] for k, t in x.items()}
+
+
+@pytest.mark.parametrize("uq,uk,uv", [(40, -40, -90), (-40, 40, 90), (0, 0, -112), (0, 0, -118), (55, -55, 99),
+                                      (-112, 112, 0), (112, -112, 0), (-105, 105, -105)])
+@pytest.mark.parametrize("w", [CASES[3], CASES[4]], ids=["one_group", "groups"])
+def test_f32_attention_magnitudes(w, uq, uk, uv):
+    out, _, simt = _forward(w, _scaled(w, uq, uk, uv))
+    if max(abs(uq), abs(uk), abs(uv)) > 97:
+        assert torch.equal(out, simt)
+    mx, _ = err_stats(out.double() * 2.0 ** -uv, oracle_mssa(_scaled(w), w))
+    assert mx <= 1.5e-5, mx
+
+
+@pytest.mark.parametrize("u", [-97, -112])
+def test_f32_attention_one_small_head(u):
+    """One head's values far below the others': it keeps its own precision."""
+    w = CASES[4]
+    x = synth.attention_inputs(w, F32)
+    ref = oracle_mssa(x, w)
+    for k in ("v_win", "v_sink", "v_hist"):
+        x[k][..., 1, :] *= 2.0 ** u
+    out, _, _ = _forward(w, x)
+    out = out.double()
+    out[..., 1, :] *= 2.0 ** -u
+    mx, _ = err_stats(out, ref)
+    assert mx <= 1.5e-5, mx
+
+
+def test_f32_attention_scores_past_fp32_before_the_scale():
+    """q k reaches 2^130, the scaled scores 2^5."""
+    w = CASES[3]
+    m = msf()
+    plan = m.Plan(m.make_desc(w.scales, w.grid_h, w.grid_w, w.heads, w.head_dim, w.sink_tokens, 0, dtype=m.MSF_DTYPE_F32,
+                              softmax_scale=2.0 ** -126 * w.head_dim ** -0.5 * 4))
+    out, lse, simt = _forward(w, _scaled(w, 62, 62), plan)
+    assert torch.equal(out, simt)
+    mx, _ = err_stats(out, oracle_mssa(_scaled(w), w))
+    assert mx <= 1.5e-5 and torch.isfinite(lse).all(), mx
+
+
+def test_f32_attention_score_below_fp32():
+    """A key whose score is minus infinity has no weight (after a first key that has)."""
+    w = dataclasses.replace(CASES[0], sink_tokens=300)
+    x = synth.attention_inputs(w, F32)
+    x["q"] *= 2.0 ** 40
+    x["k_sink"] *= 2.0 ** -40
+    x["k_win"] *= 2.0 ** -40
+    x["k_sink"][:, 130:290] = -2.0 ** 100 * torch.sign(x["q"])
+    out, _, simt = _forward(w, x)
+    assert torch.isfinite(out).all() and torch.equal(out, simt)
+
+
+@pytest.mark.parametrize("uv,ug", [(0, -30), (-30, -30), (0, -112), (-45, -45), (-40, -60), (45, 45), (99, -40)])
+def test_f32_backward_magnitudes(uv, ug):
+    from oracle import mssa_bwd as obwd
+    w = CASES[4]
+    dout, (got, _, simt) = _backward(w, _scaled(w, uv=uv), scale=2.0 ** ug)
+    if uv + ug < -70 or uv + ug > 80 or max(abs(uv), abs(ug)) > 97:
+        assert all(torch.equal(a, b) for a, b in zip(got, simt))
+    f = synth.to_f64
+    x = synth.attention_inputs(w, F32)
+    ref = obwd.mssa_backward(f(x["q"]), f(x["k_win"]), f(x["v_win"]), f(x["k_sink"]), f(x["v_sink"]), f(x["k_hist"]),
+                             f(x["v_hist"]), f(dout), w.scales, w.grid_h, w.grid_w)
+    for g, key, u in zip(got, ("dq", "dk_win", "dv_win"), (uv + ug, uv + ug, ug)):
+        e = abs(g.double().cpu().numpy() * 2.0 ** -u - ref[key]).max() / abs(ref[key]).max()
+        assert e <= 1e-5, (key, e)
+
+
+def _backward(w, x, seed=9, scale=1.0):
     plan = make_plan(w, F32)
     d = device_inputs(x, w.history_capacity)
     ws = bind(plan, d)
@@ -114,7 +189,7 @@ def _backward(w, x, seed=9):
     got = []
     for fn in (plan.mssa_backward, plan.mssa_backward, plan.mssa_backward_simt):
         g = [torch.full_like(d["q"], float("nan")) for _ in range(3)]
-        fn(d["q"], d["k_win"], d["v_win"], out, dout.cuda(), lse, *g, bws)
+        fn(d["q"], d["k_win"], d["v_win"], out, (dout * scale).cuda(), lse, *g, bws)
         got.append(g)
     torch.cuda.synchronize()
     assert plan.device_status() == msf().MSF_OK
