@@ -22,6 +22,12 @@
  *   - `stream` is a cudaStream_t passed as void* (NULL = legacy default
  *     stream). Kernels run asynchronously on it; outputs are valid once the
  *     stream has reached the call.
+ *   - Calls of one plan share its workspace, so the caller orders them (one
+ *     stream, or events between streams). Attention and gradient calls of an
+ *     fp32 plan that only read the plan's tensors may be made on several
+ *     streams and threads: the library runs them one after the other on the
+ *     device (also among the calls of one capture; replays of different graphs
+ *     are the caller's to order).
  *   - Element type is the plan's dtype (bf16 or fp32) for every tensor.
  *   - Notation: B streams, T window states, fine token grid Gh x Gw
  *     (G = Gh*Gw tokens per fine frame), H heads, D head_dim, Ns sink tokens,
@@ -312,10 +318,11 @@ msf_status msf_kv_resample(msf_plan_t plan, const void* k_win, const void* v_win
  * accumulation); fp32 plans run the tensor cores on three bf16 planes per
  * value (each to 24 bits, or to 2^-30 of the largest of the eight neighbours
  * along the head that it is split with), or, for a call whose operands they
- * cannot hold (decided on the device), an fp32 CUDA-core kernel: a value that is not finite or not below 2^127, eight
- * neighbours that are not all zero and all below 2^-96, or largest values
- * between which a product leaves fp32's range (q k outside 2^-100 to 2^116,
- * before or after the scale; v above 2^97). Errors: INVALID_ARG, STATE, CUDA. */
+ * cannot hold (decided on the device), an fp32 CUDA-core kernel: a value that
+ * is not finite or not below 2^127, eight neighbours that are not all zero and
+ * all below 2^-96, or largest values between which a product leaves fp32's
+ * range (q k outside 2^-100 to 2^116, before or after the scale; v above
+ * 2^97). Errors: INVALID_ARG, STATE, CUDA. */
 msf_status msf_mssa_forward(msf_plan_t plan, const void* q, const void* k_win, const void* v_win,
                             void* out, void* stream);
 

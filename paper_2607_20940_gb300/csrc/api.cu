@@ -4,12 +4,14 @@
 #include <string.h>
 
 #include <mutex>
+#include <optional>
 #include <utility>
 #include <vector>
 
 #include "attn_bwd_tc.h"
 #include "attn_f32_tc.h"
 #include "attn_tc.h"
+#include "call_order.h"
 #include "gemm_f32_tc.h"
 #include "gemm_tc.h"
 #include "msp_tc.h"
@@ -217,6 +219,14 @@ void build_attn_args(const Plan& p, const void* q, const void* k_win, const void
     }
 }
 
+// An fp32 attention, after the plan's calls before it.
+msf_status attn_f32(Plan& p, const msf::AttnArgs& a, void* stream) {
+    msf::CallTurn turn(*p.order, (cudaStream_t)stream);
+    if (turn.error() != cudaSuccess) return cuda_status(turn.error());
+    const msf_status st = msf::launch_attn_f32_tc(&p, a, (cudaStream_t)stream);
+    return st == MSF_OK ? cuda_status(turn.end()) : st;
+}
+
 }  // namespace
 
 extern "C" void msf_plan_destroy_caches(msf_plan_t plan) { msf::tc_cache_free(plan); }
@@ -403,7 +413,7 @@ extern "C" msf_status msf_mssa_forward_lse(msf_plan_t plan, const void* q, const
     build_attn_args(p, q, k_win, v_win, out, a);
     a.lse = lse;
     if (p.elem == 2) return msf::launch_attn_tc(plan, a, (cudaStream_t)stream);
-    return msf::launch_attn_f32_tc(plan, a, (cudaStream_t)stream);
+    return attn_f32(p, a, stream);
 }
 
 extern "C" msf_status msf_mssa_forward(msf_plan_t plan, const void* q, const void* k_win,
@@ -415,7 +425,7 @@ extern "C" msf_status msf_mssa_forward(msf_plan_t plan, const void* q, const voi
     msf::AttnArgs a;
     build_attn_args(p, q, k_win, v_win, out, a);
     if (p.elem == 2) return msf::launch_attn_tc(plan, a, (cudaStream_t)stream);
-    return msf::launch_attn_f32_tc(plan, a, (cudaStream_t)stream);
+    return attn_f32(p, a, stream);
 }
 
 extern "C" msf_status msf_mssa_forward_resample(msf_plan_t plan, const void* q, const void* k_win,
@@ -440,7 +450,7 @@ extern "C" msf_status msf_mssa_forward_resample(msf_plan_t plan, const void* q, 
         st = cuda_status(msf::launch_pool(jb, p.B, false, s));
         if (st != MSF_OK) return st;
     }
-    return msf::launch_attn_f32_tc(plan, a, s);
+    return attn_f32(p, a, stream);
 }
 
 // Gradient rows of group gi: the context rows that come from the window,
@@ -588,12 +598,16 @@ static msf_status mssa_backward(msf_plan_t plan, const void* q, const void* k_wi
         if (st != MSF_OK) return st;
     } else {
         msf::F32Range unless = {};  // the CUDA-core kernels: always, or where the planes cannot hold the operands
+        std::optional<msf::CallTurn> turn;
         if (tc) {
+            turn.emplace(*p.order, s);
+            if (turn->error() != cudaSuccess) return cuda_status(turn->error());
             char* planes = (char*)bwd_ws + msf::bwd_delta_bytes(p) + 2 * msf::bwd_ctx_bytes(p);
             msf_status st = msf::launch_bwd_f32_tc(plan, c, a, bg, (float*)dq, planes, &unless, s);
             if (st != MSF_OK) return st;
         }
         e = msf::launch_bwd_simt(c, a, bg, dq, bf16, unless, s);
+        if (turn && e == cudaSuccess) e = turn->end();
         if (e != cudaSuccess) return cuda_status(e);
     }
     return cuda_status(msf::launch_bwd_gather(c, ga, dk_win, dv_win, bf16, s));

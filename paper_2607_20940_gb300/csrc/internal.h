@@ -19,6 +19,10 @@ struct Group {
 
 }  // namespace msf
 
+namespace msf {
+struct CallOrder;
+}
+
 // The opaque plan of the C ABI.
 struct msf_plan {
     msf_plan_desc d;
@@ -56,6 +60,9 @@ struct msf_plan {
 
     // opaque per-kernel caches (tensor maps etc.)
     void* tc_cache;
+
+    // fp32 plans: the order of the calls that write the operands' planes
+    msf::CallOrder* order;
 };
 
 namespace msf {

@@ -7,6 +7,7 @@
 #include <atomic>
 #include <new>
 
+#include "call_order.h"
 #include "internal.h"
 
 namespace msf {
@@ -162,6 +163,10 @@ extern "C" msf_status msf_plan_create(const msf_plan_desc* desc, msf_plan_t* out
         p->f32_tiles = f32_tiles;
         p->attn_max_ctas = (int)(tiles < msf::kAttnMaxCtas ? tiles : msf::kAttnMaxCtas);
     }
+    if (p->elem == 4 && !(p->order = msf::call_order_new())) {
+        delete p;
+        return MSF_ERR_INVALID_ARG;
+    }
     p->ws_bytes = msf::workspace_bytes(*p);
     p->hist_count = d.history_frames;
     p->hist_oldest = 0;
@@ -175,6 +180,7 @@ extern "C" void msf_plan_destroy_caches(msf_plan_t plan);
 extern "C" void msf_plan_destroy(msf_plan_t plan) {
     if (!plan) return;
     msf_plan_destroy_caches(plan);
+    msf::call_order_free(plan->order);
     delete plan;
 }
 
