@@ -159,19 +159,28 @@ def _ptr(t) -> Optional[int]:
     return t.data_ptr()
 
 
-_torch_c = None  # torch's C module once CUDA is initialised
+_current = None  # gives the current stream's handle, once CUDA is initialised
+
+
+def _current_handle():
+    import torch
+    torch.cuda.current_stream()  # initialises CUDA, or raises
+    # torch.cuda.current_stream() builds a Stream object: 2.9 us of a small
+    # call's 7 us on a Grace core. The handle alone takes 0.2 us, by two
+    # functions that are not part of torch's documented interface.
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    device = getattr(torch._C, "_cuda_getDevice", None)
+    if raw is None or device is None:
+        return lambda: torch.cuda.current_stream().cuda_stream
+    return lambda: raw(device())
 
 
 def _stream(stream) -> Optional[int]:
     if stream is None:
-        # torch.cuda.current_stream() builds a Stream object: 2.9 us of a
-        # small call's 7 us on a Grace core; the handle alone takes 0.2 us.
-        global _torch_c
-        if _torch_c is None:
-            import torch
-            torch.cuda.current_stream()  # initialises CUDA, or raises
-            _torch_c = torch._C
-        return _torch_c._cuda_getCurrentRawStream(_torch_c._cuda_getDevice())
+        global _current
+        if _current is None:
+            _current = _current_handle()
+        return _current()
     return stream if isinstance(stream, int) else stream.cuda_stream
 
 
