@@ -45,6 +45,12 @@ cudaError_t set_smem_attr(const void* fn, int bytes, int carveout, int regs) {
     return e;
 }
 
+cudaError_t device_sms(int* sms) {
+    int dev = 0;
+    const cudaError_t e = cudaGetDevice(&dev);
+    return e == cudaSuccess ? cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, dev) : e;
+}
+
 }  // namespace msf
 
 namespace {

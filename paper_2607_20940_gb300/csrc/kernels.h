@@ -19,6 +19,9 @@ namespace msf {
 // setmaxnreg split counts on. Thread-safe.
 cudaError_t set_smem_attr(const void* fn, int bytes, int carveout = -1, int regs = 0);
 
+// Number of SMs of the current device.
+cudaError_t device_sms(int* sms);
+
 // One block that waits, with the bounded wait of the tcgen05 kernels, on an
 // mbarrier nothing arrives at, then raises the TIMEOUT bit of *status.
 cudaError_t launch_wait_timeout_selftest(unsigned int* status, long long limit_cycles, cudaStream_t st);

@@ -25,6 +25,7 @@
 #include "msp_tc.h"
 #include "pool.cuh"
 #include "ptx.cuh"
+#include "sched.h"
 
 namespace msf {
 
@@ -907,31 +908,21 @@ cudaError_t launch_msp_embed(const MspEmbedRun* runs, int n, const MspShape& sh,
         for (int k = 0; k < pb.n; ++k) max_n = pb.j[k].out_n > max_n ? pb.j[k].out_n : max_n;
         p.pool_tasks = max_n * (pb.row_vecs / 2);
         const long long total = (long long)pb.n * p.pool_tasks;
-        // The tiles' idle warps take tasks while the pool CTAs do not all start
-        // at once (two CTAs per SM): one a thread on tiles of one K chunk and
-        // three on longer ones, or two and four, up to a third or a quarter of
-        // all tasks, so that no tile waits for them. Launch, us, none / one and
-        // three / two and four: 480p with the history 16.2 / 16.1 / 14.7, window
-        // only 11.5 / 10.9 / 11.7, four streams 79.8 / 74.4 / 72.5 and 51.8 / 46.8
-        // / 45.4; where every pool CTA starts at once they only cost (6.6 / 7.0 /
-        // 7.6), and at 410 CTAs still (5.65 / - / 5.8).
         auto share_of = [&](int one, int more) {
             long long x = 0;
             for (int i = 0; i < n; ++i)
                 x += 64ll * (p.run[i].K <= 64 ? one : more) * ((i + 1 < n ? p.run[i + 1].tile_base : tiles) - p.run[i].tile_base);
             return x;
         };
-        int one = 0, more = 0;
-        if (batch * (tiles + (total + kThreads - 1) / kThreads) > 3 * 152) {
-            if (4 * share_of(2, 4) <= total)
-                one = 2, more = 4;
-            else if (3 * share_of(1, 3) <= total)
-                one = 1, more = 3;
-        }
-        for (int i = 0; i < n && one > 0; ++i) {
+        int sms = 0;
+        const cudaError_t e = device_sms(&sms);
+        if (e != cudaSuccess) return e;
+        const IdleTasks idle = idle_tasks(batch * (tiles + (total + kThreads - 1) / kThreads), sms, total,
+                                          share_of(2, 4), share_of(1, 3));
+        for (int i = 0; i < n && idle.one > 0; ++i) {
             EmbedRun& R = p.run[i];
             R.pool_base = p.pool_first;
-            R.pool_per = R.K <= 64 ? one : more;
+            R.pool_per = R.K <= 64 ? idle.one : idle.more;
             p.pool_first += 64 * R.pool_per * ((i + 1 < n ? p.run[i + 1].tile_base : tiles) - R.tile_base);
         }
         p.pool_ctas = (int)((total - p.pool_first + kThreads - 1) / kThreads);

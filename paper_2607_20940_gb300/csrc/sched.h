@@ -1,4 +1,4 @@
-// Host estimate of when a launch's work ends.
+// Host rules on how a launch's work is placed.
 #pragma once
 
 namespace msf {
@@ -60,6 +60,31 @@ inline double lpt_end(WorkUnits* u, int n, int slots) {
     }
     for (int k = 0; k < nl; ++k) end = lv[k].load > end ? lv[k].load : end;
     return end;
+}
+
+// Pyramid tasks that a thread of the embedding tiles' idle warps takes: `one` on
+// tiles of one K chunk, `more` on longer ones (0: the pool CTAs take them all).
+struct IdleTasks {
+    int one, more;
+};
+
+// A launch of `ctas` CTAs (embedding tiles and pool CTAs, two on an SM), `total`
+// pool tasks, of which two and four a thread would give `two_four` to the idle
+// warps and one and three `one_three`: the larger up to a quarter of all tasks,
+// else the smaller up to a third, so that no tile waits for them. Where the pool
+// CTAs start early anyway they only cost the tiles: so from nine CTAs an SM on, and
+// from five if they take a fifth of the tasks. Over 250 launches against none: there
+// 10 % faster at best, 4 % on average and at worst 2 % slower; with fewer CTAs or
+// tasks, from three CTAs an SM on, 10 % faster to 19 % (2.9 us) slower.
+inline IdleTasks idle_tasks(long long ctas, int sms, long long total, long long two_four, long long one_three) {
+    IdleTasks t = {0, 0};
+    long long share = 0;
+    if (4 * two_four <= total)
+        t = {2, 4}, share = two_four;
+    else if (3 * one_three <= total)
+        t = {1, 3}, share = one_three;
+    if (ctas <= 5ll * sms || (5 * share < total && ctas <= 9ll * sms)) t = {0, 0};
+    return t;
 }
 
 }  // namespace msf
