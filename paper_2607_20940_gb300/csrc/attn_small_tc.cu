@@ -434,11 +434,14 @@ __global__ void __launch_bounds__(kThreads, 1)
 
 // The rule: the estimate of this kernel's end (its clusters placed longest
 // first; clusters of four and eight leave some SMs of a GPC over) against the
-// persistent kernel's. Microseconds fitted on a GB300 over 34 windows of 0.02 to
-// 203 GFLOP: here 6.5 and a step of two K/V tiles. 8 heads x 64, 24 tiles,
-// cluster 2: 14.2 us against 20.1; one query tile a head, 32 tiles, cluster 8:
-// 13.3 against 58.2; 96 query tiles of 49 K/V tiles: 50 against 38.4, which the
-// estimates tell apart. More than one round has to win by a tenth.
+// persistent kernel's. Microseconds fitted on a GB300 over 660 drawn windows of
+// 0.01 to 600 GFLOP, each timed in every form that it can take
+// (profiles/attention_routes.md): a start and a step of two K/V tiles. 8 heads x 64,
+// 24 tiles, cluster 2: 14.2 us against 20.1 of the even split; one query tile a
+// head, 32 tiles, cluster 8: 13.3 against 58.2; 96 query tiles of 49 K/V tiles: 50
+// against 38.4, which the estimates tell apart. More than one round has to win by a
+// tenth; of two sizes that end together the larger is taken (one pair of tiles: 9.2
+// us on one CTA, 8.6 on two).
 int attn_small_cluster(const TcGroup* g, int n_groups, int H, int B, int D, int sms, double persistent_us) {
     long long items = 0;  // 128-row query tiles
     int longest = 0;
@@ -448,18 +451,19 @@ int attn_small_cluster(const TcGroup* g, int n_groups, int H, int B, int D, int 
         longest = g[i].n_tiles > longest ? g[i].n_tiles : longest;
     }
     if (items > 2 * sms) return 0;
-    const double step = D == 64 ? 1.2 : 1.75;
+    const double step = D == 64 ? 1.34 : 1.67;
     double best = persistent_us;
     int cluster = 0;
     for (int c = 1; c <= kMaxCluster && (c == 1 || c <= longest); c *= 2) {
         const int places = (c <= 2 ? sms : sms * 5 / 6) / c;
         if (c > 1 && items > places) break;
+        const double start = D == 64 ? (c == 8 ? 7.1 : 5.7) : (c == 8 ? 9.8 : 7.7);
         WorkUnits u[MSF_MAX_GROUPS];
         for (int i = 0; i < n_groups; ++i)
-            u[i] = {6.5 + step * ((g[i].n_tiles + 2 * c - 1) / (2 * c)) + (c > 1 ? 0.5 : 0.0),
+            u[i] = {start + step * ((g[i].n_tiles + 2 * c - 1) / (2 * c)),
                     (long long)((g[i].q_end - g[i].q_begin + kBM - 1) / kBM) * H * B};
         const double t = lpt_end(u, n_groups, places) * (items > places ? 1.1 : 1.0);
-        if (t < best) {
+        if (t < best || (cluster > 0 && t == best)) {
             best = t;
             cluster = c;
         }

@@ -1168,8 +1168,7 @@ void tc_cache_invalidate(msf_plan_t plan) {
 }
 
 // Estimated end in us of the even (stream-K) split: the start and the merges, and
-// the SMs' equal shares of the 256 x 128 tiles (fitted over 34 windows of 0.02 to
-// 203 GFLOP).
+// the SMs' equal shares of the 256 x 128 tiles.
 static double split_us(const TcGroup* g, int n, int D, int sms) {
     double tiles = 0;
     for (int i = 0; i < n; ++i) tiles += (double)g[i].n_items * g[i].n_tiles;
@@ -1178,7 +1177,8 @@ static double split_us(const TcGroup* g, int n, int D, int sms) {
 
 // Whole blocks instead: CTA c takes the blocks of the sequence positions
 // [bound[c], bound[c + 1]), cut so that the longest share is shortest. Returns
-// the estimated end in us, 1e9 where there are too many blocks to count.
+// the estimated end in us (within 5 % for nine windows of ten,
+// profiles/attention_routes.md), 1e9 where there are too many blocks to count.
 static double whole_us(const TcGroup* g, int n, int D, int sms, int* bound, int* ctas) {
     long long items = 0;
     double longest = 0, sum = 0, cost[MSF_MAX_GROUPS];
@@ -1222,7 +1222,7 @@ static double whole_us(const TcGroup* g, int n, int D, int sms, int* bound, int*
         if (!cut(hi)) return 1e9;
         lo = hi;
     }
-    return 5.5 + lo;
+    return D == 64 ? 1.7 + 1.095 * lo : 3.1 + 1.011 * lo;
 }
 
 msf_status launch_attn_tc(msf_plan_t plan, const AttnArgs& a, cudaStream_t st, const PoolBatch* pool) {
@@ -1341,8 +1341,6 @@ msf_status launch_attn_tc(msf_plan_t plan, const AttnArgs& a, cudaStream_t st, c
     tp.total_tiles = total_tiles;
     if (total_tiles == 0) return MSF_OK;
     if (item_base > P.attn_items) return MSF_ERR_STATE;
-    // Small calls: one 128-row query tile per cluster (after the pyramid, if
-    // the launch was to build it).
     long long ncta = cache.num_sms;
     if (ncta > P.attn_max_ctas) ncta = P.attn_max_ctas;
     const double split = split_us(tp.g, tp.n_groups, P.D, cache.num_sms);
@@ -1352,9 +1350,12 @@ msf_status launch_attn_tc(msf_plan_t plan, const AttnArgs& a, cudaStream_t st, c
     // Whole blocks where they end first: the partial results and merges of the
     // even split cost about 10 us. Even / whole, us: 108 blocks of 12 tiles 30.1 /
     // 23.3, 208 of 5 to 14 38.5 / 26.5, 132 of up to 20 (D 64) 19.7 / 14.3, 22 of 40
-    // 42.7 / 117.5; over 220 windows the choice was never slower than the even
-    // split beyond what two runs of it differ, and up to 1.56 times faster.
+    // 42.7 / 117.5. Over 500 drawn windows the choice between the three forms was
+    // nowhere more than 0.6 % slower than the even split, and 1.4 times as fast on
+    // average (profiles/attention_routes.md).
     const bool by_item = whole < 0.97 * split;
+    // Small calls: one 128-row query tile per cluster (after the pyramid, if
+    // the launch was to build it).
     const int cluster =
         attn_small_cluster(tp.g, tp.n_groups, P.H, P.B, P.D, cache.num_sms, by_item ? whole : split);
     if (cluster > 0) {
