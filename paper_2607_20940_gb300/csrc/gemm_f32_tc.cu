@@ -208,13 +208,12 @@ __global__ void __launch_bounds__(kThreads, 2) gemm_f32_kernel(const __grid_cons
     ptx::cluster_sync();
     // ---- rows [split * R, split * R + R) of the tile, summed in split order
     const int R = kBM / p.splits;
-    for (int x = tid; x < R * (BN / 4); x += kThreads) {
-        const int row = split * R + x / (BN / 4), n = n0 + 4 * (x % (BN / 4)), m = m0 + row;
-        if (m >= g.M || n >= g.N) continue;
+    auto sum4 = [&](const float* src) {
+        if (p.splits == 1) return *reinterpret_cast<const float4*>(src);
         float4 v[kMaxSplits];
 #pragma unroll
         for (int s = 0; s < kMaxSplits; ++s)
-            if (s < p.splits) v[s] = ptx::ld_cluster_f4(part + row * C::kRow + n - n0, (uint32_t)s);
+            if (s < p.splits) v[s] = ptx::ld_cluster_f4(src, (uint32_t)s);
         float4 a = v[0];
 #pragma unroll
         for (int s = 1; s < kMaxSplits; ++s)
@@ -224,18 +223,47 @@ __global__ void __launch_bounds__(kThreads, 2) gemm_f32_kernel(const __grid_cons
                 a.z += v[s].z;
                 a.w += v[s].w;
             }
-        if (p.P == 0) {
-            *reinterpret_cast<float4*>(g.C + b * g.c_bstride + m * g.ldc + n) = a;
+        return a;
+    };
+    // Four features of a token from n on, into the latent from its first pixel.
+    const int P = p.P, PP = P * P;
+    auto scatter = [&](float* lat, int n, const float4& a) {
+        auto at = [&](int f) { return lat + (f / PP) * p.plane + (long long)(f % PP / P) * p.Wl + f % P; };
+        if (P % 4 == 0) {
+            *reinterpret_cast<float4*>(at(n)) = a;
+        } else if (P % 2 == 0) {
+            *reinterpret_cast<float2*>(at(n)) = make_float2(a.x, a.y);
+            *reinterpret_cast<float2*>(at(n + 2)) = make_float2(a.z, a.w);
         } else {
-            float* lat = g.C + b * g.c_bstride + (long long)(p.P * (m / p.gw)) * p.Wl + (long long)p.P * (m % p.gw);
-            const float y[4] = {a.x, a.y, a.z, a.w};
-            const int PP = p.P * p.P;
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const int f = n + e;
-                lat[(f / PP) * p.plane + (long long)(f % PP / p.P) * p.Wl + f % p.P] = y[e];
-            }
+            *at(n) = a.x;
+            *at(n + 1) = a.y;
+            *at(n + 2) = a.z;
+            *at(n + 3) = a.w;
         }
+    };
+    auto pixel = [&](int m) {
+        return g.C + b * g.c_bstride + (long long)(P * (m / p.gw)) * p.Wl + (long long)P * (m % p.gw);
+    };
+    if (P == 0 || p.splits > 2) {
+        for (int x = tid; x < R * (BN / 4); x += kThreads) {
+            const int row = split * R + x / (BN / 4), n = n0 + 4 * (x % (BN / 4)), m = m0 + row;
+            if (m >= g.M || n >= g.N) continue;
+            const float4 a = sum4(part + row * C::kRow + n - n0);
+            if (P == 0)
+                *reinterpret_cast<float4*>(g.C + b * g.c_bstride + m * g.ldc + n) = a;
+            else
+                scatter(pixel(m), n, a);
+        }
+    } else if (m0 + split * R + tid % R < g.M) {
+        // The sums of one or two CTAs into the latent, a token per thread: neighbouring
+        // tokens' pixels of a feature run lie side by side there, while a row's features
+        // go to a line each (one chunk, 96 tokens of patch edge 4: 17.2 us and 7.3).
+        // From four CTAs on the loads of the others' shared memory, a row's features in
+        // a run, weigh more (144 tokens, 8 chunks: 8.5 us as above, 9.6 this way).
+        const int row = split * R + tid % R;
+        float* lat = pixel(m0 + row);
+        for (int c = 4 * (tid / R); c < BN && n0 + c < g.N; c += 4 * (kThreads / R))
+            scatter(lat, n0 + c, sum4(part + row * C::kRow + c));
     }
     // No CTA leaves while another may still read its shared memory.
     ptx::cluster_sync();
@@ -262,7 +290,15 @@ cudaError_t launch_gemm_f32_tc(const GemmArgs* a, int n, int batch, unsigned int
         widest = a[i].N > widest ? a[i].N : widest;
         deepest = a[i].K > deepest ? a[i].K : deepest;
     }
-    const int bn = widest <= 64 ? 64 : 128;
+    int sms = 0;
+    cudaError_t e = device_sms(&sms);
+    if (e != cudaSuccess) return e;
+    const int chunks = (deepest + 63) / 64;
+    // Tiles of 64 columns where those of 128 would leave SMs idle and have little to
+    // multiply (36 tokens, K = 64, N = 256: 10.5 -> 7.2 us).
+    long long wide = 0;
+    for (int i = 0; i < n; ++i) wide += (long long)((a[i].M + kBM - 1) / kBM) * ((a[i].N + 127) / 128) * batch;
+    const int bn = widest <= 64 || (chunks <= 2 && wide <= sms) ? 64 : 128;
     int tiles = 0;
     for (int i = 0; i < n; ++i) {
         F32Problem& g = p.g[i];
@@ -280,13 +316,12 @@ cudaError_t launch_gemm_f32_tc(const GemmArgs* a, int n, int batch, unsigned int
     }
     // At most eight chunks (32 steps at full size) per CTA where the cluster
     // allows it, and more CTAs while the tiles leave half of the SMs idle.
-    const int chunks = (deepest + 63) / 64;
     int s = 1;
-    while (s < kMaxSplits && (chunks > 8 * s || ((long long)tiles * batch * s < 152 && chunks >= 4 * s))) s *= 2;
+    while (s < kMaxSplits && (chunks > 8 * s || ((long long)tiles * batch * s < sms && chunks >= 4 * s))) s *= 2;
     p.splits = s;
     const void* fn = bn == 64 ? (const void*)gemm_f32_kernel<64> : (const void*)gemm_f32_kernel<128>;
     const int smem = bn == 64 ? GCfg<64>::kSmem : GCfg<128>::kSmem;
-    cudaError_t e = set_smem_attr(fn, smem, 100);
+    e = set_smem_attr(fn, smem, 100);
     if (e != cudaSuccess) return e;
     const dim3 grid((unsigned)tiles, (unsigned)s, (unsigned)batch);
     return bn == 64 ? launch_pdl_cluster(gemm_f32_kernel<64>, grid, dim3(kThreads), smem, st, dim3(1, s, 1), p)

@@ -25,6 +25,18 @@ SHAPES = [
 ]
 
 
+# The ways into the latent: one, two (a token per thread) and four CTAs a tile (a
+# token's features over the threads), stores of 1, 2 and 4 pixels, 64- and 128-wide
+# tiles, a last tile of few tokens and features.
+INTO_LATENT = [
+    ((1, 2), (6, 22), 64, 3, 1, 2, 1),      # edge 1 and 2; N = 3 x 1 and 12: not vectors of four, then one
+    ((1, 2), (10, 14), 64, 4, 3, 1, 1),     # edge 3 and 6
+    ((1, 2, 4), (16, 24), 64, 16, 2, 3, 1),  # edge 2, 4, 8; N = 64, 256, 1024
+    ((1, 2), (12, 20), 320, 16, 3, 1, 2),   # two CTAs; N = 144 and 576
+    ((2, 4), (12, 20), 576, 5, 2, 2, 1),    # four CTAs; N = 80 and 320
+]
+
+
 def _run(shape, edit=None):
     scales, (gh, gw), E, C, patch, B, F = shape
     w = synth.Workload("p", len(scales), scales, gh, gw, 1, 64, 0, 0, 0, B, 70, latent_channels=C, patch=patch,
@@ -66,7 +78,8 @@ def _run(shape, edit=None):
     return tok.cpu(), torch.cat(toks, 1), back, lats
 
 
-@pytest.mark.parametrize("shape", SHAPES, ids=[f"{s[0]}-{s[1]}-E{s[2]}-C{s[3]}" for s in SHAPES])
+@pytest.mark.parametrize("shape", SHAPES + INTO_LATENT,
+                         ids=[f"{s[0]}-{s[1]}-E{s[2]}-C{s[3]}" for s in SHAPES + INTO_LATENT])
 def test_f32_projections(shape):
     tok, ref, back, lats = _run(shape)
     assert (tok.double() - ref).abs().max() <= 5e-6
