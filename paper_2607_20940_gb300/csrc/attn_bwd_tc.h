@@ -28,7 +28,7 @@ msf_status launch_bwd_tc(msf_plan_t plan, const BwdTcInput& in, cudaStream_t st)
 // fp32 plans (attn_bwd_f32_tc.cu): dq and the context-row gradients on the
 // tensor cores from three bf16 planes per value; dout_planes is scratch of
 // f32_part_bytes(kF32Q). *range receives what says whether the CUDA-core
-// kernels have to answer instead.
+// kernels have to answer instead (no condition: nothing was launched here).
 msf_status launch_bwd_f32_tc(msf_plan_t plan, const BwdCommon& c, const AttnArgs& a, const BwdGroup* bg, float* dq,
                              char* dout_planes, F32Range* range, cudaStream_t st);
 

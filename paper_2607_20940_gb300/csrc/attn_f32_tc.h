@@ -33,6 +33,8 @@ struct F32Maps {
     CUtensorMap k[kNumMaps];
     CUtensorMap v[kNumMaps];
 };
+// Keys of the longest context.
+int f32_longest_context(const AttnArgs& a);
 // Add the first `rows` rows per stream of a [B, .., H, D] fp32 tensor as planes
 // [B, 3, alloc, H, D] at `dst` to the split, and encode their tensor map.
 bool add_planes(const Plan& P, SplitParams& sp, int operand, const void* src, long long src_bstride_bytes, char* dst,

@@ -238,6 +238,29 @@ def test_f32_tensor_backward(w, mode):
     del ws
 
 
+@pytest.mark.parametrize("D,keys", [(64, 12), (64, 13), (64, 24), (64, 25), (128, 10), (128, 11), (128, 18), (128, 19)])
+def test_f32_few_keys(D, keys):
+    """On either side of the number of keys from which the tensor cores are ahead."""
+    from oracle import mssa_bwd as obwd
+    w = dataclasses.replace(CASES[0], grid_w=keys - 5, sink_tokens=5, heads=3, head_dim=D, batch=2)
+    x = synth.attention_inputs(w, F32)
+    out, lse, simt = _forward(w, x)
+    if keys <= (24 if D == 64 else 18):
+        assert torch.equal(out, simt)
+    mx, _ = err_stats(out, oracle_mssa(x, w))
+    assert mx <= 1.5e-5 and torch.isfinite(lse).all(), mx
+    dout, (got, again, simt) = _backward(w, x)
+    assert all(torch.equal(a, b) for a, b in zip(got, again))
+    if keys <= (12 if D == 64 else 10):
+        assert all(torch.equal(a, b) for a, b in zip(got, simt))
+    f = synth.to_f64
+    ref = obwd.mssa_backward(f(x["q"]), f(x["k_win"]), f(x["v_win"]), f(x["k_sink"]), f(x["v_sink"]), f(x["k_hist"]),
+                             f(x["v_hist"]), f(dout), w.scales, w.grid_h, w.grid_w)
+    for g, key in zip(got, ("dq", "dk_win", "dv_win")):
+        e = abs(g.double().cpu().numpy() - ref[key]).max() / abs(ref[key]).max()
+        assert e <= 1e-5, (key, e)
+
+
 @pytest.mark.parametrize("value", [float("inf"), float("nan"), torch.finfo(F32).min])
 @pytest.mark.parametrize("where", ["q", "k_win", "v_sink"])
 def test_f32_backward_values_the_planes_cannot_hold(value, where):
