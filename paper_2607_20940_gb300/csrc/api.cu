@@ -619,6 +619,28 @@ static msf_status mssa_backward(msf_plan_t plan, const void* q, const void* k_wi
     return cuda_status(msf::launch_bwd_gather(c, ga, dk_win, dv_win, bf16, s));
 }
 
+// Not part of msf.h: the forms that a bf16 plan's attention and gradient take on a
+// device with `sms` SMs, for tests that name one. Host only, bound or not. out: cluster
+// size of the small-call kernel (0: the persistent kernel), whole blocks, CTAs, rounds
+// of whole blocks and most pieces of a block of the persistent kernel; items of the
+// gradient, placed lists.
+extern "C" msf_status msf_test_routes(msf_plan_t plan, int32_t sms, int32_t* out) {
+    if (!plan || sms < 1 || !out) return MSF_ERR_INVALID_ARG;
+    const Plan& p = *plan;
+    if (p.elem != 2) return MSF_ERR_UNSUPPORTED;
+    msf::AttnArgs a;
+    build_attn_args(p, nullptr, nullptr, nullptr, nullptr, a);
+    msf::BwdGroup bg[MSF_MAX_GROUPS];
+    int crow = 0;
+    for (int gi = 0; gi < p.n_groups; ++gi) build_bwd_group(p, gi, nullptr, nullptr, bg[gi], crow);
+    const msf::AttnRoute r = msf::attn_route(p, a, sms);
+    msf::BwdRoute b;
+    msf::bwd_route(p, a, bg, sms, &b);
+    const int32_t all[] = {r.cluster, r.whole, r.ctas, r.dp_rounds, r.pieces, b.items, b.placed};
+    memcpy(out, all, sizeof(all));
+    return MSF_OK;
+}
+
 extern "C" msf_status msf_mssa_backward(msf_plan_t plan, const void* q, const void* k_win,
                                         const void* v_win, const void* out, const void* dout,
                                         const float* lse, void* dq, void* dk_win, void* dv_win,

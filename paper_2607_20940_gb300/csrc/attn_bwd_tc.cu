@@ -62,8 +62,7 @@ struct BSeg {
 };
 struct BGroupQ {
     int q_begin, q_end;
-    int n_qt;       // 128-row query tiles
-    int item_base;  // first item of this group
+    int n_qt;  // 128-row query tiles
     int n_seg, n_tiles;
     BSeg seg[kMaxSeg];
 };
@@ -73,8 +72,7 @@ struct BGrad {
 };
 struct BGroupK {
     int q_begin, q_end, n_qt;
-    int item_base;  // first item of this group
-    int n_kt;       // key tiles of this group (all runs)
+    int n_kt;  // key tiles of this group (all runs)
     int n_grad;
     BGrad gr[kMaxGradSeg];
 };
@@ -92,24 +90,15 @@ struct BwdTcParams {
     int dq_v8, ctx_v8;  // 32-byte aligned outputs: 32-byte stores
     int n_items;
     // dq work
-    int n_groups;
     BGroupQ g[MSF_MAX_GROUPS];
     // dK/dV work
-    int n_kgroups;
     BGroupK kg[MSF_MAX_GROUPS];
     // Item ranges, most expensive items first: kind 0 =
     // dq items of group g[group], kind 1 = dK/dV items of kg[group].
     int n_ranges;
     struct Range {
-        int kind, group, base, count;
+        int kind, group, base;
     } range[2 * MSF_MAX_GROUPS];
-};
-// The items of every CTA: CTA c takes item[first[c]], ..., item[first[c + 1] - 1].
-constexpr int kMaxOrderCtas = 160, kMaxOrderItems = 2048;
-struct BwdOrder {
-    int on;  // 0: rounds of alternating direction
-    uint16_t first[kMaxOrderCtas + 1];
-    uint16_t item[kMaxOrderItems];
 };
 struct BwdMaps {
     CUtensorMap q, dout;
@@ -852,79 +841,125 @@ bool encode_all(BwdMaps& m, const Plan& P, const BwdTcInput& in) {
     return true;
 }
 
-// Equal items of a launch.
-struct ItemClass {
-    int kind, group, count;
-    int blocks;  // MMA blocks of 128x128xD: 3 per K/V tile of a dq item, 4 per query tile of a dK/dV item
-    int ns;      // what an item takes, as measured
-    int base;    // its first item
-};
-
-// Gives every item, longest first, to the CTA that would be free first, where
-// that ends the launch at least a hundredth and a microsecond earlier than the
-// rounds of alternating direction: those keep neighbouring tiles of a head and
-// items of one kind together, and are near enough once a CTA has a dozen items.
-// New loads of a class only grow, so two sorted queues hold the CTAs and an item
-// costs the host a few nanoseconds. Forward and backward, rounds / placed: a fine
-// and a coarse state of 40 x 36 tokens, 16 heads x 128, 278.6 / 238.0 us (576
-// items); 46 x 26, three frames a state, 3 heads x 64, 239.7 / 220.0; 8 x 39, four
-// streams, 113.4 / 107.7 (480); 480p 508.0 / 506.4 (1032).
-void place_items(BwdOrder& o, const ItemClass* cl, int n, int total, int ctas) {
-    o.on = 0;
-    if (total <= ctas || total > kMaxOrderItems || ctas > kMaxOrderCtas) return;
-    struct Cta {
-        long long load;
-        int c;
-    };
-    Cta old[kMaxOrderCtas], grown[kMaxOrderItems], rest[kMaxOrderCtas];
-    long long rounds[kMaxOrderCtas];
-    uint8_t cta_of[kMaxOrderItems];  // by item
-    uint16_t taken[kMaxOrderItems];  // items, longest first
-    for (int c = 0; c < ctas; ++c) {
-        old[c] = {0, c};
-        rounds[c] = 0;
+// Every item of a gradient, host only: the groups, the ranges and the classes of
+// equal items; returns the number of classes.
+int fill_items(const Plan& P, const AttnArgs& a, const BwdGroup* bg, BwdTcParams& tp, ItemClass* rs) {
+    // dQ: every query tile of every group, longest contexts first.
+    int order[MSF_MAX_GROUPS];
+    int len[MSF_MAX_GROUPS];
+    for (int i = 0; i < a.n_groups; ++i) {
+        order[i] = i;
+        len[i] = 0;
+        for (int s = 0; s < a.g[i].n_seg; ++s) len[i] += a.g[i].seg[s].len;
     }
-    int by_ns[2 * MSF_MAX_GROUPS];
-    for (int k = 0; k < n; ++k) {
-        int at = k;
-        for (; at > 0 && cl[by_ns[at - 1]].ns < cl[k].ns; --at) by_ns[at] = by_ns[at - 1];
-        by_ns[at] = k;
-        for (int x = 0; x < cl[k].count; ++x) {
-            const int r = (cl[k].base + x) / ctas, c = (cl[k].base + x) % ctas;
-            rounds[r & 1 ? ctas - 1 - c : c] += cl[k].ns;
+    for (int i = 0; i < a.n_groups; ++i)
+        for (int k = i + 1; k < a.n_groups; ++k)
+            if (len[order[k]] > len[order[i]]) {
+                const int t = order[i];
+                order[i] = order[k];
+                order[k] = t;
+            }
+    for (int oi = 0; oi < a.n_groups; ++oi) {
+        const int gi = order[oi];
+        const AttnGroup& ag = a.g[gi];
+        BGroupQ& g = tp.g[oi];
+        g.q_begin = ag.q_begin;
+        g.q_end = ag.q_end;
+        g.n_qt = (ag.q_end - ag.q_begin + kBM - 1) / kBM;
+        g.n_seg = ag.n_seg;
+        g.n_tiles = 0;
+        for (int s = 0; s < ag.n_seg; ++s) {
+            const Segment& sg = ag.seg[s];
+            BSeg& bs = g.seg[s];
+            bs.map = sg.map_id == kMapPyr ? kMapPyr0 + gi : sg.map_id;
+            bs.row0 = sg.map_id == kMapPyr ? 0 : sg.row0;
+            bs.len = sg.len;
+            bs.tile0 = g.n_tiles;
+            g.n_tiles += (sg.len + kBM - 1) / kBM;
         }
     }
-    memset(o.first, 0, sizeof(o.first));
-    int done = 0;
-    for (int k = 0; k < n; ++k) {
-        const ItemClass& ic = cl[by_ns[k]];
-        int i = 0, head = 0, tail = 0;
-        auto lightest = [&] {
-            return head == tail || (i < ctas && old[i].load <= grown[head].load) ? old[i++] : grown[head++];
-        };
-        for (int x = 0; x < ic.count; ++x) {
-            Cta t = lightest();
-            t.load += ic.ns;
-            grown[tail++] = t;
-            cta_of[ic.base + x] = (uint8_t)t.c;
-            taken[done++] = (uint16_t)(ic.base + x);
-            ++o.first[t.c + 1];
+    // dK/dV: every group's window-derived rows in one launch, groups with
+    // the most query tiles first.
+    int korder[MSF_MAX_GROUPS];
+    int nk = 0;
+    for (int gi = 0; gi < a.n_groups; ++gi)
+        if (bg[gi].n_gseg > 0 && bg[gi].q_end > bg[gi].q_begin) korder[nk++] = gi;
+    for (int i = 0; i < nk; ++i)
+        for (int k = i + 1; k < nk; ++k)
+            if (bg[korder[k]].q_end - bg[korder[k]].q_begin >
+                bg[korder[i]].q_end - bg[korder[i]].q_begin) {
+                const int t = korder[i];
+                korder[i] = korder[k];
+                korder[k] = t;
+            }
+    for (int oi = 0; oi < nk; ++oi) {
+        const int gi = korder[oi];
+        const BwdGroup& b = bg[gi];
+        BGroupK& kg = tp.kg[oi];
+        kg.q_begin = b.q_begin;
+        kg.q_end = b.q_end;
+        kg.n_qt = (b.q_end - b.q_begin + kBM - 1) / kBM;
+        kg.n_grad = b.n_gseg;
+        int kt0 = 0;
+        for (int s = 0; s < b.n_gseg; ++s) {
+            const GradSeg& gs = b.gseg[s];
+            BGrad& g = kg.gr[s];
+            g.map = gs.map_id == kMapPyr ? kMapPyr0 + gi : gs.map_id;
+            // pyramid rows are addressed from the group's pyramid part, the
+            // ring from its first slot, the window from token 0
+            g.row0 = gs.map_id == kMapPyr ? gs.row0 - P.groups[gi].pyr_offset : gs.row0;
+            g.len = gs.len;
+            g.kt0 = kt0;
+            g.crow0 = gs.crow0;
+            kt0 += (gs.len + kBM - 1) / kBM;
         }
-        for (int m = 0; m < ctas; ++m) rest[m] = lightest();
-        memcpy(old, rest, sizeof(old));
+        kg.n_kt = kt0;
     }
-    long long end = 0;
-    for (int c = 0; c < ctas; ++c) end = rounds[c] > end ? rounds[c] : end;
-    const long long gain = end - old[ctas - 1].load;
-    if (gain < 1000 || 100 * gain < end) return;
-    o.on = 1;
-    for (int c = 0; c < ctas; ++c) o.first[c + 1] = (uint16_t)(o.first[c + 1] + o.first[c]);
-    uint16_t at[kMaxOrderCtas];
-    memcpy(at, o.first, sizeof(at));
-    for (int x = 0; x < total; ++x) o.item[at[cta_of[taken[x]]]++] = taken[x];
+    // Ranges with the most MMA blocks per item first; the times are from
+    // globaltimer stamps over eight windows of 1 to 175 tiles an item (within
+    // 8 % from two tiles on).
+    const bool d128 = P.D == 128;
+    int nr = 0;
+    for (int oi = 0; oi < a.n_groups; ++oi) {
+        const int n = tp.g[oi].n_tiles;
+        if (tp.g[oi].n_qt > 0)
+            rs[nr++] = {0, oi, tp.g[oi].n_qt * P.H * P.B, 3 * n, d128 ? 1200 + 1085 * n : 1500 + 710 * n, 0};
+    }
+    for (int oi = 0; oi < nk; ++oi) {
+        const int n = tp.kg[oi].n_qt;
+        if (tp.kg[oi].n_kt > 0)
+            rs[nr++] = {1, oi, tp.kg[oi].n_kt * P.H * P.B, 4 * n, d128 ? 4500 + 1355 * n : 2600 + 1110 * n, 0};
+    }
+    for (int i = 0; i < nr; ++i)
+        for (int k = i + 1; k < nr; ++k)
+            if (rs[k].blocks > rs[i].blocks) {
+                const ItemClass t = rs[i];
+                rs[i] = rs[k];
+                rs[k] = t;
+            }
+    int total = 0;
+    for (int i = 0; i < nr; ++i) {
+        tp.range[i].kind = rs[i].kind;
+        tp.range[i].group = rs[i].group;
+        tp.range[i].base = rs[i].base = total;
+        total += rs[i].count;
+    }
+    tp.n_ranges = nr;
+    tp.n_items = total;
+    return nr;
 }
 
 }  // namespace
+
+void bwd_route(const Plan& P, const AttnArgs& a, const BwdGroup* bg, int sms, BwdRoute* out) {
+    BwdTcParams tp;
+    memset(&tp, 0, sizeof(tp));
+    ItemClass rs[2 * MSF_MAX_GROUPS];
+    const int nr = fill_items(P, a, bg, tp, rs);
+    BwdOrder order;
+    place_items(order, rs, nr, tp.n_items, tp.n_items < sms ? tp.n_items : sms);
+    *out = {tp.n_items, order.on};
+}
 
 msf_status launch_bwd_tc(msf_plan_t plan, const BwdTcInput& in, cudaStream_t st) {
     const Plan& P = *plan;
@@ -950,128 +985,14 @@ msf_status launch_bwd_tc(msf_plan_t plan, const BwdTcInput& in, cudaStream_t st)
     tp.R = in.R;
     tp.status = a.status;
     tp.wait_limit = kWaitLimit;
-    // dQ: every query tile of every group, longest contexts first.
-    int order[MSF_MAX_GROUPS];
-    int len[MSF_MAX_GROUPS];
-    for (int i = 0; i < a.n_groups; ++i) {
-        order[i] = i;
-        len[i] = 0;
-        for (int s = 0; s < a.g[i].n_seg; ++s) len[i] += a.g[i].seg[s].len;
-    }
-    for (int i = 0; i < a.n_groups; ++i)
-        for (int k = i + 1; k < a.n_groups; ++k)
-            if (len[order[k]] > len[order[i]]) {
-                const int t = order[i];
-                order[i] = order[k];
-                order[k] = t;
-            }
-    int items = 0;
-    for (int oi = 0; oi < a.n_groups; ++oi) {
-        const int gi = order[oi];
-        const AttnGroup& ag = a.g[gi];
-        BGroupQ& g = tp.g[oi];
-        g.q_begin = ag.q_begin;
-        g.q_end = ag.q_end;
-        g.n_qt = (ag.q_end - ag.q_begin + kBM - 1) / kBM;
-        g.item_base = items;
-        g.n_seg = ag.n_seg;
-        g.n_tiles = 0;
-        for (int s = 0; s < ag.n_seg; ++s) {
-            const Segment& sg = ag.seg[s];
-            BSeg& bs = g.seg[s];
-            bs.map = sg.map_id == kMapPyr ? kMapPyr0 + gi : sg.map_id;
-            bs.row0 = sg.map_id == kMapPyr ? 0 : sg.row0;
-            bs.len = sg.len;
-            bs.tile0 = g.n_tiles;
-            g.n_tiles += (sg.len + kBM - 1) / kBM;
-        }
-        items += g.n_qt * P.H * P.B;
-    }
-    tp.n_groups = a.n_groups;
-    tp.n_groups = a.n_groups;
-    // dK/dV: every group's window-derived rows in one launch, groups with
-    // the most query tiles first.
-    int korder[MSF_MAX_GROUPS];
-    int nk = 0;
-    for (int gi = 0; gi < a.n_groups; ++gi)
-        if (in.g[gi].n_gseg > 0 && in.g[gi].q_end > in.g[gi].q_begin) korder[nk++] = gi;
-    for (int i = 0; i < nk; ++i)
-        for (int k = i + 1; k < nk; ++k)
-            if (in.g[korder[k]].q_end - in.g[korder[k]].q_begin >
-                in.g[korder[i]].q_end - in.g[korder[i]].q_begin) {
-                const int t = korder[i];
-                korder[i] = korder[k];
-                korder[k] = t;
-            }
-    int kitems = 0;
-    for (int oi = 0; oi < nk; ++oi) {
-        const int gi = korder[oi];
-        const BwdGroup& bg = in.g[gi];
-        BGroupK& kg = tp.kg[oi];
-        kg.q_begin = bg.q_begin;
-        kg.q_end = bg.q_end;
-        kg.n_qt = (bg.q_end - bg.q_begin + kBM - 1) / kBM;
-        kg.item_base = kitems;
-        kg.n_grad = bg.n_gseg;
-        int kt0 = 0;
-        for (int s = 0; s < bg.n_gseg; ++s) {
-            const GradSeg& gs = bg.gseg[s];
-            BGrad& g = kg.gr[s];
-            g.map = gs.map_id == kMapPyr ? kMapPyr0 + gi : gs.map_id;
-            // pyramid rows are addressed from the group's pyramid part, the
-            // ring from its first slot, the window from token 0
-            g.row0 = gs.map_id == kMapPyr ? gs.row0 - P.groups[gi].pyr_offset : gs.row0;
-            g.len = gs.len;
-            g.kt0 = kt0;
-            g.crow0 = gs.crow0;
-            kt0 += (gs.len + kBM - 1) / kBM;
-        }
-        kg.n_kt = kt0;
-        kitems += kt0 * P.H * P.B;
-    }
-    tp.n_kgroups = nk;
-    // Ranges with the most MMA blocks per item first; the times are from
-    // globaltimer stamps over eight windows of 1 to 175 tiles an item (within
-    // 8 % from two tiles on).
-    const bool d128 = P.D == 128;
     ItemClass rs[2 * MSF_MAX_GROUPS];
-    int nr = 0;
-    for (int oi = 0; oi < a.n_groups; ++oi) {
-        const int n = tp.g[oi].n_tiles;
-        if (tp.g[oi].n_qt > 0)
-            rs[nr++] = {0, oi, tp.g[oi].n_qt * P.H * P.B, 3 * n, d128 ? 1200 + 1085 * n : 1500 + 710 * n, 0};
-    }
-    for (int oi = 0; oi < nk; ++oi) {
-        const int n = tp.kg[oi].n_qt;
-        if (tp.kg[oi].n_kt > 0)
-            rs[nr++] = {1, oi, tp.kg[oi].n_kt * P.H * P.B, 4 * n, d128 ? 4500 + 1355 * n : 2600 + 1110 * n, 0};
-    }
-    for (int i = 0; i < nr; ++i)
-        for (int k = i + 1; k < nr; ++k)
-            if (rs[k].blocks > rs[i].blocks) {
-                const ItemClass t = rs[i];
-                rs[i] = rs[k];
-                rs[k] = t;
-            }
-    int total = 0;
-    for (int i = 0; i < nr; ++i) {
-        tp.range[i].kind = rs[i].kind;
-        tp.range[i].group = rs[i].group;
-        tp.range[i].base = rs[i].base = total;
-        tp.range[i].count = rs[i].count;
-        total += rs[i].count;
-    }
-    tp.n_ranges = nr;
-    tp.n_items = total;
-    (void)items;
-    (void)kitems;
+    const int nr = fill_items(P, a, in.g, tp, rs), total = tp.n_items;
     if (total == 0) return MSF_OK;
     // Rows of one head are a multiple of 32 bytes, so the bases decide.
     tp.dq_v8 = (uintptr_t)in.dq % 32 == 0;
     tp.ctx_v8 = (uintptr_t)in.dk_ctx % 32 == 0 && (uintptr_t)in.dv_ctx % 32 == 0;
-    int dev = 0, sms = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    int sms = 0;
+    cudaError_t e = device_sms(&sms);
     if (e != cudaSuccess) {
         set_cuda_error((int)e);
         return MSF_ERR_CUDA;
@@ -1079,6 +1000,7 @@ msf_status launch_bwd_tc(msf_plan_t plan, const BwdTcInput& in, cudaStream_t st)
     const int grid = total < sms ? total : sms;
     BwdOrder placed;
     place_items(placed, rs, nr, total, grid);
+    const bool d128 = P.D == 128;
     const int smem = d128 ? BCfg<128>::kSmem : BCfg<64>::kSmem;
     e = d128 ? set_smem_attr((const void*)bwd_tc_kernel<128>, BCfg<128>::kSmem)
              : set_smem_attr((const void*)bwd_tc_kernel<64>, BCfg<64>::kSmem);

@@ -25,6 +25,13 @@ struct BwdTcInput {
 // every group's window-derived context rows (one launch).
 msf_status launch_bwd_tc(msf_plan_t plan, const BwdTcInput& in, cudaStream_t st);
 
+// What such a launch does on a device with `sms` SMs (host only).
+struct BwdRoute {
+    int items;
+    int placed;  // 1: placed lists, 0: rounds of alternating direction
+};
+void bwd_route(const Plan& P, const AttnArgs& a, const BwdGroup* bg, int sms, BwdRoute* out);
+
 // fp32 plans (attn_bwd_f32_tc.cu): dq and the context-row gradients on the
 // tensor cores from three bf16 planes per value; dout_planes is scratch of
 // f32_part_bytes(kF32Q). *range receives what says whether the CUDA-core

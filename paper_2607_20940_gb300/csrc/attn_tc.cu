@@ -152,11 +152,11 @@ struct MergeJob {
     int stop;            // no more jobs
 };
 
-__device__ __forceinline__ long long cta_begin(long long c, long long T, long long n) {
+__host__ __device__ __forceinline__ long long cta_begin(long long c, long long T, long long n) {
     return c * T / n;
 }
 // The CTA whose range [cta_begin(c), cta_begin(c+1)) holds tile t.
-__device__ __forceinline__ long long cta_of(long long t, long long T, long long n) {
+__host__ __device__ __forceinline__ long long cta_of(long long t, long long T, long long n) {
     return ((t + 1) * n - 1) / T;
 }
 
@@ -1225,6 +1225,110 @@ static double whole_us(const TcGroup* g, int n, int D, int sms, int* bound, int*
     return D == 64 ? 1.7 + 1.095 * lo : 3.1 + 1.011 * lo;
 }
 
+// The groups by context length, longest first, host only; returns the length of the
+// tile sequence.
+static long long tc_groups(const Plan& P, const AttnArgs& a, TcGroup* g, int* items) {
+    int order[MSF_MAX_GROUPS];
+    for (int i = 0; i < a.n_groups; ++i) order[i] = i;
+    for (int i = 0; i < a.n_groups; ++i)
+        for (int k = i + 1; k < a.n_groups; ++k) {
+            int ni = 0, nk = 0;
+            for (int s = 0; s < a.g[order[i]].n_seg; ++s) ni += a.g[order[i]].seg[s].len;
+            for (int s = 0; s < a.g[order[k]].n_seg; ++s) nk += a.g[order[k]].seg[s].len;
+            if (nk > ni) {
+                int tmp = order[i];
+                order[i] = order[k];
+                order[k] = tmp;
+            }
+        }
+    long long total_tiles = 0;
+    int item_base = 0;
+    for (int oi = 0; oi < a.n_groups; ++oi) {
+        const int gi = order[oi];
+        const AttnGroup& ag = a.g[gi];
+        TcGroup& tg = g[oi];
+        tg.q_begin = ag.q_begin;
+        tg.q_end = ag.q_end;
+        tg.n_qb = (ag.q_end - ag.q_begin + 2 * kBlockM - 1) / (2 * kBlockM);
+        tg.n_items = tg.n_qb * P.H * P.B;
+        tg.n_seg = ag.n_seg;
+        tg.n_tiles = 0;
+        for (int s = 0; s < ag.n_seg; ++s) {
+            const Segment& sg = ag.seg[s];
+            TcSeg& ts = tg.seg[s];
+            const bool pyr = sg.map_id == kMapPyr;  // a map of the group's own pyramid part
+            ts.map = pyr ? kMapPyr0 + gi : sg.map_id;
+            ts.row0 = pyr ? 0 : sg.row0;
+            ts.len = sg.len;
+            ts.tile0 = tg.n_tiles;
+            tg.n_tiles += (sg.len + kBlockN - 1) / kBlockN;
+        }
+        tg.n_virt = tg.n_tiles + kItemLeadTiles;
+        tg.tile_base = total_tiles;
+        tg.item_base = item_base;
+        total_tiles += (long long)tg.n_items * tg.n_virt;
+        item_base += tg.n_items;
+    }
+    *items = item_base;
+    return total_tiles;
+}
+
+// Which form a call takes on `sms` SMs.
+static AttnRoute choose(const Plan& P, const TcGroup* g, int n, long long total_tiles, int sms, TcBounds& bounds) {
+    AttnRoute r = {0, 0, 0, 0, 0};
+    long long ncta = sms;
+    if (ncta > P.attn_max_ctas) ncta = P.attn_max_ctas;
+    const double split = split_us(g, n, P.D, sms);
+    int whole_ctas = 0;
+    const double whole = whole_us(g, n, P.D, (int)ncta, bounds.at, &whole_ctas);
+    // Whole blocks where they end first: the partial results and merges of the
+    // even split cost about 10 us. Even / whole, us: 108 blocks of 12 tiles 30.1 /
+    // 23.3, 208 of 5 to 14 38.5 / 26.5, 132 of up to 20 (D 64) 19.7 / 14.3, 22 of 40
+    // 42.7 / 117.5. Over 500 drawn windows the choice between the three forms was
+    // nowhere more than 0.6 % slower than the even split, and 1.4 times as fast on
+    // average (profiles/attention_routes.md).
+    const bool by_item = whole < 0.97 * split;
+    // Small calls: one 128-row query tile per cluster.
+    r.cluster = attn_small_cluster(g, n, P.H, P.B, P.D, sms, by_item ? whole : split);
+    if (r.cluster > 0) return r;
+    if (by_item) {
+        r.whole = 1;
+        r.ctas = whole_ctas;
+        return r;
+    }
+    if (ncta > total_tiles) ncta = total_tiles;
+    if (ncta < 1) ncta = 1;
+    r.ctas = (int)ncta;
+    // Data-parallel rounds: while the longest group has at least one item per
+    // CTA, each CTA first takes whole items of it (no partial results), and
+    // only the rest of the sequence is split evenly (stream-K).
+    r.dp_rounds = (int)(g[0].n_items / ncta);
+    // The split counts a piece for every CTA between an item's first and last:
+    // each must hold a tile, so a rest of fewer tiles than CTAs takes a round in.
+    const long long rest = total_tiles - r.dp_rounds * ncta * g[0].n_virt;
+    if (r.dp_rounds > 0 && rest > 0 && rest < ncta) --r.dp_rounds;
+    return r;
+}
+
+AttnRoute attn_route(const Plan& P, const AttnArgs& a, int sms) {
+    TcGroup g[MSF_MAX_GROUPS];
+    memset(g, 0, sizeof(g));
+    int items = 0;
+    TcBounds bounds;
+    const long long total = tc_groups(P, a, g, &items);
+    AttnRoute r = choose(P, g, a.n_groups, total, sms, bounds);
+    if (r.cluster > 0 || r.whole) return r;
+    const long long t_sk = (long long)r.dp_rounds * r.ctas * g[0].n_virt, rest = total - t_sk;
+    for (int i = 0; i < a.n_groups; ++i)
+        for (int k = 0; k < g[i].n_items; ++k) {
+            const long long at = g[i].tile_base + (long long)k * g[i].n_virt + kItemLeadTiles - t_sk;
+            if (at < 0) continue;
+            const int pieces = (int)(cta_of(at + g[i].n_tiles - 1, rest, r.ctas) - cta_of(at, rest, r.ctas)) + 1;
+            r.pieces = pieces > r.pieces ? pieces : r.pieces;
+        }
+    return r;
+}
+
 msf_status launch_attn_tc(msf_plan_t plan, const AttnArgs& a, cudaStream_t st, const PoolBatch* pool) {
     Plan& P = *plan;
     if (!P.tc_cache) {
@@ -1276,47 +1380,19 @@ msf_status launch_attn_tc(msf_plan_t plan, const AttnArgs& a, cudaStream_t st, c
         set_cuda_error((int)cudaErrorInvalidValue);
         return MSF_ERR_CUDA;
     }
-    // Order groups by context length, longest first.
-    int order[MSF_MAX_GROUPS];
-    for (int i = 0; i < a.n_groups; ++i) order[i] = i;
-    for (int i = 0; i < a.n_groups; ++i)
-        for (int k = i + 1; k < a.n_groups; ++k) {
-            int ni = 0, nk = 0;
-            for (int s = 0; s < a.g[order[i]].n_seg; ++s) ni += a.g[order[i]].seg[s].len;
-            for (int s = 0; s < a.g[order[k]].n_seg; ++s) nk += a.g[order[k]].seg[s].len;
-            if (nk > ni) {
-                int tmp = order[i];
-                order[i] = order[k];
-                order[k] = tmp;
-            }
-        }
-    long long total_tiles = 0;
-    int item_base = 0;
-    for (int oi = 0; oi < a.n_groups; ++oi) {
-        const int gi = order[oi];
-        const AttnGroup& ag = a.g[gi];
-        TcGroup& tg = tp.g[oi];
-        tg.q_begin = ag.q_begin;
-        tg.q_end = ag.q_end;
-        tg.n_qb = (ag.q_end - ag.q_begin + 2 * kBlockM - 1) / (2 * kBlockM);
-        tg.n_items = tg.n_qb * P.H * P.B;
-        tg.n_seg = ag.n_seg;
-        tg.n_tiles = 0;
-        for (int s = 0; s < ag.n_seg; ++s) {
-            const Segment& sg = ag.seg[s];
-            TcSeg& ts = tg.seg[s];
+    for (int gi = 0; gi < a.n_groups; ++gi)
+        for (int s = 0; s < a.g[gi].n_seg; ++s) {
+            const Segment& sg = a.g[gi].seg[s];
             int slot = sg.map_id;
             int rows_total = sg.rows_total;
             const char* kb = sg.k;
             const char* vb = sg.v;
-            int row0 = sg.row0;
             if (slot == kMapPyr) {
                 // per-group map starting at the group's pyramid part, extent = live rows
                 slot = kMapPyr0 + gi;
                 kb = sg.k + (size_t)sg.row0 * row;
                 vb = sg.v + (size_t)sg.row0 * row;
                 rows_total = sg.len;
-                row0 = 0;
             } else if (slot == kMapHist) {
                 rows_total = sg.len;  // live history frames only
             }
@@ -1325,65 +1401,27 @@ msf_status launch_attn_tc(msf_plan_t plan, const AttnArgs& a, cudaStream_t st, c
                 set_cuda_error((int)cudaErrorInvalidValue);
                 return MSF_ERR_CUDA;
             }
-            ts.map = slot;
-            ts.row0 = row0;
-            ts.len = sg.len;
-            ts.tile0 = tg.n_tiles;
-            tg.n_tiles += (sg.len + kBlockN - 1) / kBlockN;
         }
-        tg.n_virt = tg.n_tiles + kItemLeadTiles;
-        tg.tile_base = total_tiles;
-        tg.item_base = item_base;
-        total_tiles += (long long)tg.n_items * tg.n_virt;
-        item_base += tg.n_items;
-    }
+    int item_base = 0;
+    const long long total_tiles = tc_groups(P, a, tp.g, &item_base);
     tp.n_groups = a.n_groups;
     tp.total_tiles = total_tiles;
     if (total_tiles == 0) return MSF_OK;
     if (item_base > P.attn_items) return MSF_ERR_STATE;
-    long long ncta = cache.num_sms;
-    if (ncta > P.attn_max_ctas) ncta = P.attn_max_ctas;
-    const double split = split_us(tp.g, tp.n_groups, P.D, cache.num_sms);
     TcBounds bounds;
-    int ctas = 0;
-    const double whole = whole_us(tp.g, tp.n_groups, P.D, (int)ncta, bounds.at, &ctas);
-    // Whole blocks where they end first: the partial results and merges of the
-    // even split cost about 10 us. Even / whole, us: 108 blocks of 12 tiles 30.1 /
-    // 23.3, 208 of 5 to 14 38.5 / 26.5, 132 of up to 20 (D 64) 19.7 / 14.3, 22 of 40
-    // 42.7 / 117.5. Over 500 drawn windows the choice between the three forms was
-    // nowhere more than 0.6 % slower than the even split, and 1.4 times as fast on
-    // average (profiles/attention_routes.md).
-    const bool by_item = whole < 0.97 * split;
-    // Small calls: one 128-row query tile per cluster (after the pyramid, if
-    // the launch was to build it).
-    const int cluster =
-        attn_small_cluster(tp.g, tp.n_groups, P.H, P.B, P.D, cache.num_sms, by_item ? whole : split);
-    if (cluster > 0) {
+    const AttnRoute route = choose(P, tp.g, tp.n_groups, total_tiles, cache.num_sms, bounds);
+    if (route.cluster > 0) {  // after the pyramid, if the launch was to build it
         e = pool ? launch_pool(*pool, P.B, true, st) : cudaSuccess;
-        if (e == cudaSuccess) e = launch_attn_small(cache.maps, tp.g, tp.n_groups, P, a, cluster, st);
+        if (e == cudaSuccess) e = launch_attn_small(cache.maps, tp.g, tp.n_groups, P, a, route.cluster, st);
         if (e == cudaSuccess) return MSF_OK;
         set_cuda_error((int)e);
         return MSF_ERR_CUDA;
     }
-    if (ncta > total_tiles) ncta = total_tiles;
-    if (ncta < 1) ncta = 1;
-    // Data-parallel rounds: while the longest group has at least one item per
-    // CTA, each CTA first takes whole items of it (no partial results), and
-    // only the rest of the sequence is split evenly (stream-K).
-    tp.dp_rounds = 0;
-    if (tp.n_groups > 0) tp.dp_rounds = (int)(tp.g[0].n_items / ncta);
+    const bool by_item = route.whole != 0;
+    const int ctas = route.ctas;
+    tp.dp_rounds = route.dp_rounds;
     tp.dp_stride = tp.g[0].n_virt;
-    tp.t_sk = (long long)tp.dp_rounds * ncta * tp.dp_stride;
-    // The split counts a piece for every CTA between an item's first and last:
-    // each must hold a tile, so a rest of fewer tiles than CTAs takes a round in.
-    if (tp.dp_rounds > 0 && total_tiles > tp.t_sk && total_tiles - tp.t_sk < ncta) {
-        --tp.dp_rounds;
-        tp.t_sk -= ncta * tp.dp_stride;
-    }
-    if (by_item) {
-        tp.dp_rounds = 0;
-        tp.t_sk = 0;
-    }
+    tp.t_sk = (long long)route.dp_rounds * ctas * tp.dp_stride;
     // The launch's own pyramid (D = 128): vector-pair tasks of every job and
     // stream. Other head sizes run the pool kernel first.
     const bool own_pool = pool && pool->n > 0 && P.D == 128 && !by_item;
@@ -1431,7 +1469,7 @@ msf_status launch_attn_tc(msf_plan_t plan, const AttnArgs& a, cudaStream_t st, c
             set_cuda_error((int)e);
             return MSF_ERR_CUDA;
         }
-        e = launch_pdl(mssa_tc_pool_kernel, dim3((unsigned)ncta), dim3(kThreads), Cfg<128>::kSmem, st,
+        e = launch_pdl(mssa_tc_pool_kernel, dim3((unsigned)ctas), dim3(kThreads), Cfg<128>::kSmem, st,
                        cache.maps, tp, *pool);
     } else if (P.D == 128) {
         if (!cache.attr_set[1]) {
@@ -1450,7 +1488,7 @@ msf_status launch_attn_tc(msf_plan_t plan, const AttnArgs& a, cudaStream_t st, c
             set_cuda_error((int)e);
             return MSF_ERR_CUDA;
         }
-        e = launch_pdl(mssa_tc_kernel<128>, dim3((unsigned)ncta), dim3(kThreads), Cfg<128>::kSmem, st,
+        e = launch_pdl(mssa_tc_kernel<128>, dim3((unsigned)ctas), dim3(kThreads), Cfg<128>::kSmem, st,
                        cache.maps, tp);
     } else {
         if (!cache.attr_set[0]) {
@@ -1468,7 +1506,7 @@ msf_status launch_attn_tc(msf_plan_t plan, const AttnArgs& a, cudaStream_t st, c
             set_cuda_error((int)e);
             return MSF_ERR_CUDA;
         }
-        e = launch_pdl(mssa_tc_kernel<64>, dim3((unsigned)ncta), dim3(kThreads), Cfg<64>::kSmem, st,
+        e = launch_pdl(mssa_tc_kernel<64>, dim3((unsigned)ctas), dim3(kThreads), Cfg<64>::kSmem, st,
                        cache.maps, tp);
     }
     if (e == cudaSuccess) e = cudaGetLastError();

@@ -41,6 +41,16 @@ struct TcMaps {
     CUtensorMap v[kNumMaps];
 };
 
+// What a bf16 attention call does on a device with `sms` SMs (host only).
+struct AttnRoute {
+    int cluster;    // > 0: the small-call kernel with clusters of so many CTAs
+    int whole;      // 1: the persistent kernel on whole blocks, 0: on an even split
+    int ctas;       // CTAs of the persistent kernel
+    int dp_rounds;  // even split: rounds of whole blocks before it
+    int pieces;     // most pieces of a block of the split (attn_route only)
+};
+AttnRoute attn_route(const Plan& P, const AttnArgs& a, int sms);
+
 // With `pool` (bf16 jobs), the launch also builds that K/V pyramid: every CTA
 // pools a share of it first, and tiles of pyramid segments wait until all
 // shares are written.

@@ -65,3 +65,16 @@ def err_stats(got: torch.Tensor, ref: np.ndarray, heads=None):
 def bf16_round(x: np.ndarray) -> np.ndarray:
     """Round-to-nearest-even of fp64 values to bf16, returned as fp64."""
     return torch.from_numpy(np.ascontiguousarray(x)).to(torch.float32).to(BF16).to(torch.float64).numpy()
+
+
+def routes(plan, sms=None):
+    """The forms that the plan's bf16 attention and gradient take on `sms` SMs (the
+    current device's if None): cluster, whole, ctas, rounds, pieces, items, placed."""
+    import ctypes
+    if sms is None:
+        sms = torch.cuda.get_device_properties(torch.cuda.current_device()).multi_processor_count
+    lib = ctypes.CDLL(msf().LIB_PATH)
+    lib.msf_test_routes.argtypes = [ctypes.c_void_p, ctypes.c_int32, ctypes.POINTER(ctypes.c_int32)]
+    out = (ctypes.c_int32 * 7)()
+    assert lib.msf_test_routes(plan.handle, sms, out) == 0
+    return dict(zip(("cluster", "whole", "ctas", "rounds", "pieces", "items", "placed"), out))

@@ -2,9 +2,9 @@
 
 Every item (a query tile's dq, a key tile's dk/dv) is computed by one CTA, so
 which CTA takes it changes no bit: a call of several streams equals the calls of
-its parts that have no more items than an SM count and so are not placed, on the
-same forward results. Sizes: placed by time at both head widths, just below
-and just above the largest number of items that is placed.
+its streams, which are not placed, on the same forward results. Cases: placed by
+time at both head widths, just below the largest number of items that is placed,
+above it, and a call whose gain lies below the line.
 """
 import dataclasses
 
@@ -13,20 +13,28 @@ import torch
 
 from paper_2607_20940_gb300 import synth
 
-from helpers import BF16, bind, device_inputs, make_plan, msf
+from helpers import BF16, bind, device_inputs, make_plan, msf, routes
 from test_gpu_backward import _run
 
 pytestmark = pytest.mark.gpu
 
-D128 = synth.Workload("items_d128", 2, (1, 1), 8, 39, 12, 128, 250, 1, 1, 4, 61)     # 120 items a stream
-D64 = synth.Workload("items_d64", 4, (1, 2, 2, 4), 12, 60, 5, 64, 130, 1, 1, 2, 62)  # 140 items a stream
+D128 = synth.Workload("items_d128", 2, (1, 1), 8, 39, 12, 128, 250, 1, 1, 4, 61)
+CASES = {  # workload, items, placed
+    "d128": (synth.Workload("d128", 2, (1, 1), 20, 16, 2, 128, 0, 1, 1, 16, 62), 320, 1),
+    "d64": (synth.Workload("d64", 2, (1, 1), 30, 52, 3, 64, 0, 1, 1, 2, 63), 300, 1),
+    "d64_most": (synth.Workload("d64_most", 2, (1, 2), 34, 36, 5, 64, 250, 1, 1, 13, 64), 2015, 1),
+    "no_gain": (D128, 480, 0),
+    "too_many": (dataclasses.replace(D128, batch=18), 2160, 0),
+}
 
 
-@pytest.mark.parametrize("w", [D128, dataclasses.replace(D128, batch=17), dataclasses.replace(D128, batch=18), D64],
-                         ids=["d128_480", "d128_2040", "d128_2160", "d64_280"])
-def test_items_placed_anywhere_same_bits(w):
-    x, dout, out, lse, g, _ = _run(w, BF16)
+@pytest.mark.parametrize("name", CASES)
+def test_items_placed_anywhere_same_bits(name):
+    w, items, placed = CASES[name]
     one = dataclasses.replace(w, batch=1)
+    r = routes(make_plan(w))
+    assert (r["items"], r["placed"]) == (items, placed) and routes(make_plan(one))["placed"] == 0
+    x, dout, out, lse, g, _ = _run(w, BF16)
     for b in (0, w.batch - 1):
         dx = device_inputs({k: v[b:b + 1].contiguous() for k, v in x.items()}, w.history_capacity)
         plan = make_plan(one, BF16)

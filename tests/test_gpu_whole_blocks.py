@@ -9,7 +9,7 @@ import numpy as np
 import pytest
 import torch
 
-from helpers import BF16, bind, device_inputs, err_stats, make_plan, msf, oracle_mssa
+from helpers import BF16, bind, device_inputs, err_stats, make_plan, msf, oracle_mssa, routes
 from oracle import mssa as omssa
 from paper_2607_20940_gb300 import synth
 
@@ -28,6 +28,8 @@ def test_whole_blocks(w):
     x = synth.attention_inputs(w, BF16)
     dx = device_inputs(x, w.history_capacity)
     plan = make_plan(w, BF16)
+    taken = routes(plan)
+    assert taken["whole"] == 1 and taken["cluster"] == 0, taken
     bind(plan, dx)
     B, N = dx["q"].shape[:2]
     outs = [torch.full_like(dx["q"], float("nan")) for _ in range(3)]
