@@ -4,7 +4,8 @@ output, the pyramid and the staged head must equal, bit for bit, those of
 msf_kv_resample followed by msf_mssa_forward, whose own parity against the
 oracle the other GPU tests check; launches in a row and CUDA graph replays
 check that the launch's pyramid counts reset themselves. One case is also
-checked against the oracle directly.
+checked against the oracle directly. (Calls of the small-call kernel, of whole
+blocks and of 64-wide heads run the two launches; ONE says which cases take one.)
 """
 import dataclasses
 
@@ -13,15 +14,18 @@ import torch
 
 from paper_2607_20940_gb300 import synth
 
-from helpers import BF16, F32, bind, device_inputs, err_stats, make_plan, msf, oracle_mssa
+from helpers import BF16, F32, bind, device_inputs, err_stats, make_plan, msf, oracle_mssa, routes
 
 pytestmark = pytest.mark.gpu
 
 SMALL3 = synth.Workload("fr_t4_12x20", 4, (1, 1, 2, 4), 12, 20, 3, 128, 200, 2, 3, 2, 41)
+# ragged segments and pooled rows in one launch: every block cut in two
+SPLIT3 = synth.Workload("fr_split_t4_12x20", 4, (1, 1, 2, 4), 12, 20, 20, 128, 3000, 2, 3, 2, 46)
 RAGGED = synth.Workload("fr_ragged_t3_10x14_d64", 3, (1, 2, 2), 10, 14, 2, 64, 37, 1, 1, 1, 43)
 CASES = [
     ("tiny", synth.TINY),
     ("small3", SMALL3),
+    ("split3", SPLIT3),
     ("ragged_d64", RAGGED),
     ("layer_480p", synth.LAYER_480P),
     ("stream_b4", dataclasses.replace(synth.STREAM_480P, history_frames=3)),
@@ -30,7 +34,8 @@ CASES = [
     ("max_states", synth.Workload("fr_max_states_t16", 16, (1, 1, 2, 2, 4, 4, 8, 8) + (16,) * 8, 32, 48, 2,
                                   64, 40, 2, 3, 2, 45)),
 ]
-STRIDED_CASES = [("small3", SMALL3), ("layer_480p", synth.LAYER_480P), ("three_scale", synth.THREE_SCALE)]
+ONE = ("split3", "layer_480p", "stream_b4", "three_scale", "chunked")
+STRIDED_CASES = [("small3", SMALL3), ("split3", SPLIT3), ("layer_480p", synth.LAYER_480P), ("three_scale", synth.THREE_SCALE)]
 
 
 def _pyramid(plan, ws, w):
@@ -61,6 +66,8 @@ def test_one_launch_equals_resample_then_forward(name, w, flags):
     x = synth.attention_inputs(w)
     dx = device_inputs(x, w.history_capacity)
     plan = make_plan(w)
+    r = routes(plan)
+    assert (w.head_dim == 128 and not r["cluster"] and not r["whole"]) == (name in ONE), r
     ws = bind(plan, dx)
     # the history part of the pyramid must exist before a window-only pass
     plan.kv_resample(dx["k_win"], dx["v_win"], m.MSF_RESAMPLE_FULL)

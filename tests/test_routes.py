@@ -6,6 +6,7 @@ import dataclasses
 import pytest
 
 import test_gpu_backward_items as items
+import test_gpu_forward_resample as resample
 import test_gpu_merge_paths as merges
 import test_gpu_merge_rest as rest
 import test_gpu_small_calls as small
@@ -26,6 +27,12 @@ def test_merges(name):
     w, _, takes = merges.CASES[name]
     r = routes(make_plan(w), SMS)
     assert takes(r), r
+
+
+@pytest.mark.parametrize("name,w", resample.CASES, ids=[c[0] for c in resample.CASES])
+def test_one_launch(name, w):
+    r = routes(make_plan(w), SMS)
+    assert (w.head_dim == 128 and not r["cluster"] and not r["whole"]) == (name in resample.ONE), r
 
 
 @pytest.mark.parametrize("w", whole.CASES, ids=lambda w: w.name)
