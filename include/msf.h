@@ -130,7 +130,12 @@ typedef struct msf_plan_info {
                                          fused_append: the spare slot the head is staged in) */
     int32_t pyramid_tokens;           /* tokens per stream in the workspace pyramid */
     int32_t frames_per_state;         /* F (1 when desc.frames_per_state is 0) */
-    uint64_t workspace_bytes;         /* device workspace msf_plan_bind needs */
+    uint64_t workspace_bytes;         /* device workspace msf_plan_bind needs. fp32 plans hold
+                                         their operands as three bf16 planes there (6 bytes per
+                                         element of q, sink, ring, pyramid and window K and V) and
+                                         up to 128 MB of partial outputs: 383 MB for a 480p layer
+                                         (T = 5, 30 x 52 tokens, 12 heads x 128, history of 2),
+                                         1.47 GB for four streams and a history of 4 */
     uint64_t attention_flops;         /* 4*D*H*B*sum_g Nq_g*Nkv_g (current history) */
     uint64_t dense_flops;             /* same window with every s_l = 1 (no MSP, no MSSA) */
     uint64_t resample_bytes;          /* bytes read+written by a full msf_kv_resample */
@@ -333,9 +338,10 @@ msf_status msf_mssa_forward(msf_plan_t plan, const void* q, const void* k_win, c
  * segment; with fused_append also the history ring, which holds the staged
  * head) waits (bounded) until every CTA's share is written; the pyramid, the
  * staged head and out are
- * exactly those of the two calls. fp32 plans and small calls (those whose
- * attention gives every 128-row query tile its own thread-block cluster) run
- * the two calls. flags:
+ * exactly those of the two calls. fp32 plans, 64-wide heads, small calls
+ * (those whose attention gives every 128-row query tile its own thread-block
+ * cluster) and calls whose attention takes whole query blocks (no partial
+ * results to merge) run the two calls. flags:
  * MSF_RESAMPLE_FULL or MSF_RESAMPLE_WINDOW_ONLY. Errors: INVALID_ARG,
  * UNSUPPORTED (more pooling jobs than one launch takes), STATE (not bound),
  * CUDA; a wait that gives up raises TIMEOUT in the device status. */

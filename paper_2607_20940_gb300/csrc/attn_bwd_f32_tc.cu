@@ -20,11 +20,12 @@
 // TMEM columns: S [0,128), dP [128,256), output [192, 192 + D), own dP
 // operand's planes from 320 (64 each). The planes of dS (P) are written over
 // S (h, m) and [128,192) (l); the output takes dP's place once it is read.
-// Bound: the tensor pipe, 144 MMAs of ~69-82 cycles per tile pair for dQ and
-// dK, 96 for dV, plus the softmax between dP and the output (the exponentials
+// Bound: the tensor pipe, 144 MMAs of 64 cycles per tile pair for dQ and dK, 96
+// for dV, plus the softmax between dP and the output (the exponentials
 // run beside the dP MMAs). A small window (two 16 x 24 frames per state, 1008
 // tokens, 4 heads x 128) takes 86 us where the CUDA-core kernels take 1422 us,
 // with relative errors against 64 bits of 5.1-6.1e-7 (CUDA cores 6.5-8.5e-7).
+// At D = 128 ptxas spills 44 bytes of the 168 registers.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>

@@ -245,8 +245,9 @@ __device__ __forceinline__ void store_f32(float* dst, const uint32_t (&o)[32], f
 // phases per query tile keep the pipe busy: once P^T_i is written, dV_i and
 // S^T_{i+1} run while the softmax turns dP^T_i into dS^T_i; then dK_i and
 // dP^T_{i+1} run while it turns S^T_{i+1} into P^T_{i+1}. All MMAs are 128
-// columns wide: the two 64-query halves of the version before cost 62.6
-// cycles per 64-wide MMA (shared-memory reads bound it) against 82 per 128.
+// columns wide: the two 64-query halves of the version before had 64-wide ones
+// with both operands in shared memory, whose reads bound them (a probe that only
+// issues MMAs: 48 cycles against 64 of a 128-wide one).
 template <int D>
 __global__ void __launch_bounds__(kThreads, 1)
     bwd_tc_kernel(const __grid_constant__ BwdMaps maps, const __grid_constant__ BwdTcParams p,

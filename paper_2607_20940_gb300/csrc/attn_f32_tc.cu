@@ -25,8 +25,8 @@
 // merge_f32_kernel     sums the units of a split query tile.
 //
 // Bound: the tensor pipe, 96 MMAs per 128 x 128 pair tile at D = 128 (six
-// times the bf16 kernel's 16), about 7250 cycles with the measured 82 (both
-// operands in shared memory) and 69 cycles (P in TMEM) per MMA. The softmax
+// times the bf16 kernel's 16), 6144 cycles at 64 per MMA, which a probe that only
+// issues them reaches. The softmax
 // (exponentials, the three-way split of P, the read-out of O) takes about a
 // third of that and runs beside it: S of tile j+1 is issued before P V of
 // tile j, into the other S buffer.

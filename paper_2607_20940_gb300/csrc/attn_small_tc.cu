@@ -17,6 +17,7 @@
 // 3-deep rings), warp 1 MMA issuer, warp 2 TMEM, warps 4-7 softmax of the even
 // tiles, warps 8-11 of the odd ones (one thread per query row).
 // TMEM columns: S0 [0,128) S1 [128,256) O0 [256,256+D) O1 [384,384+D).
+// At 168 registers ptxas spills 8 bytes (stored once, 40 loaded).
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -435,8 +436,9 @@ __global__ void __launch_bounds__(kThreads, 1)
 // The rule: the estimate of this kernel's end (its clusters placed longest
 // first; clusters of four and eight leave some SMs of a GPC over) against the
 // persistent kernel's. Microseconds fitted on a GB300 over 660 drawn windows of
-// 0.01 to 600 GFLOP, each timed in every form that it can take
-// (profiles/attention_routes.md): a start and a step of two K/V tiles. 8 heads x 64,
+// 0.01 to 600 GFLOP, each timed in every form that it can take: a start and a step
+// of two K/V tiles (median 1.02 of the measured time, 0.95 to 1.2 for nine of ten of
+// 500 others). 8 heads x 64,
 // 24 tiles, cluster 2: 14.2 us against 20.1 of the even split; one query tile a
 // head, 32 tiles, cluster 8: 13.3 against 58.2; 96 query tiles of 49 K/V tiles: 50
 // against 38.4, which the estimates tell apart. More than one round has to win by a

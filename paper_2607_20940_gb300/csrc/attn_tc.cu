@@ -1177,8 +1177,7 @@ static double split_us(const TcGroup* g, int n, int D, int sms) {
 
 // Whole blocks instead: CTA c takes the blocks of the sequence positions
 // [bound[c], bound[c + 1]), cut so that the longest share is shortest. Returns
-// the estimated end in us (within 5 % for nine windows of ten,
-// profiles/attention_routes.md), 1e9 where there are too many blocks to count.
+// the estimated end in us (within 5 % for nine of ten of 500 drawn windows), 1e9 where there are too many blocks to count.
 static double whole_us(const TcGroup* g, int n, int D, int sms, int* bound, int* ctas) {
     long long items = 0;
     double longest = 0, sum = 0, cost[MSF_MAX_GROUPS];
@@ -1286,7 +1285,7 @@ static AttnRoute choose(const Plan& P, const TcGroup* g, int n, long long total_
     // 23.3, 208 of 5 to 14 38.5 / 26.5, 132 of up to 20 (D 64) 19.7 / 14.3, 22 of 40
     // 42.7 / 117.5. Over 500 drawn windows the choice between the three forms was
     // nowhere more than 0.6 % slower than the even split, and 1.4 times as fast on
-    // average (profiles/attention_routes.md).
+    // average.
     const bool by_item = whole < 0.97 * split;
     // Small calls: one 128-row query tile per cluster.
     r.cluster = attn_small_cluster(g, n, P.H, P.B, P.D, sms, by_item ? whole : split);
