@@ -148,3 +148,24 @@ def test_branches_of_a_capture():
             _pass(plan, d, c)
     _check(plan, calls, ref)
     del ws
+
+
+def test_while_another_stream_captures():
+    """Calls on a stream that is not captured, the plan's first among them, go on
+    while another one is, and neither side waits on the other's events."""
+    plan, d, ws, calls = _setup()
+    fresh, fd, fws, fcalls = _setup()
+    ref = _alone(plan, d, calls)
+    graph, main = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+    with torch.cuda.graph(graph, stream=main):
+        _pass(plan, d, calls[0])
+        for p, pd, c in ((plan, d, calls[1]), (fresh, fd, fcalls[2])):
+            with torch.cuda.stream(c["stream"]):
+                _pass(p, pd, c)
+        _pass(plan, d, calls[0])
+    torch.cuda.synchronize()
+    _check(plan, calls[1:2], ref[1:2])
+    _check(fresh, fcalls[2:], ref[2:])
+    graph.replay()
+    _check(plan, calls[:1], ref[:1])
+    del ws, fws
