@@ -989,7 +989,10 @@ cudaError_t launch_msp_deembed(const void* tokens, long long tok_bstride_elems, 
     // chain). Each split keeps at least one K chunk.
     const int clusters = (M + 127) / 128 * (F / kDeBN) * batch;
     const bool extras = lora || res;
-    int splits = clusters <= (extras ? 15 : 30) ? 8 : clusters <= 72 ? 4 : extras || clusters <= 152 ? 2 : 1;
+    int sms = 0;
+    cudaError_t e = device_sms(&sms);
+    if (e != cudaSuccess) return e;
+    int splits = clusters <= (extras ? 15 : 30) ? 8 : clusters <= 72 ? 4 : extras || clusters <= sms ? 2 : 1;
     while (splits > 1 && splits > nk_all) splits /= 2;
     DeembedParams p;
     memset(&p, 0, sizeof(p));
@@ -1016,12 +1019,12 @@ cudaError_t launch_msp_deembed(const void* tokens, long long tok_bstride_elems, 
         tp.up = (const __nv_bfloat16*)tier->up;
         tp.latent = (const __nv_bfloat16*)tier->latent;
         tp.latent_bstride = tier->latent_bstride;
-        cudaError_t e = set_smem_attr((const void*)msp_deembed_kernel<true, DeembedTierParams>, de_tier_smem(1), 100);
+        e = set_smem_attr((const void*)msp_deembed_kernel<true, DeembedTierParams>, de_tier_smem(1), 100);
         if (e != cudaSuccess) return e;
         return launch_pdl_cluster(msp_deembed_kernel<true, DeembedTierParams>, grid, dim3(kThreads),
                                   de_tier_smem(splits), st, cluster, maps, p, tp);
     }
-    cudaError_t e = set_smem_attr((const void*)msp_deembed_kernel<false, NoTier>, kDeSmem);
+    e = set_smem_attr((const void*)msp_deembed_kernel<false, NoTier>, kDeSmem);
     if (e != cudaSuccess) return e;
     return launch_pdl_cluster(msp_deembed_kernel<false, NoTier>, grid, dim3(kThreads), kDeSmem, st, cluster, maps, p,
                               NoTier{});
