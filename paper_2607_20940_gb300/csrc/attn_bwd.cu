@@ -297,7 +297,7 @@ __global__ void __launch_bounds__(128, 3)
                     T* dq, int dq_tiles, const F32Range unless) {
     ptx::grid_dep_wait();
     ptx::grid_dep_launch();
-    if (unless.words && planes_hold(unless)) return;
+    if (unless.words && planes_held(unless)) return;
     __shared__ float s0[32][D];
     __shared__ float s1[32][D];
     __shared__ float l[32], d[32];

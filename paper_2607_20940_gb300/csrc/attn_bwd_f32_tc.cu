@@ -526,7 +526,7 @@ __global__ void __launch_bounds__(256) bwd_f32_merge_kernel(const __grid_constan
     using C = FBCfg<D>;
     ptx::grid_dep_wait();
     ptx::grid_dep_launch();
-    if (!planes_hold(p.range)) return;
+    if (!planes_held(p.range)) return;
     int ci = 0;
     while (ci + 1 < p.n_classes && (p.c[ci].n_split == 1 || (int)blockIdx.x >= p.c[ci + 1].item_base)) ++ci;
     const FBClass& cl = p.c[ci];
@@ -678,10 +678,10 @@ msf_status launch_bwd_f32_tc(msf_plan_t plan, const BwdCommon& c, const AttnArgs
         }
     }
     if (slots > max_slots) return MSF_ERR_STATE;
+    if (units == 0) return MSF_OK;
     e = launch_split_planes(sp, c.scale_log2, &fp.range, st);
     if (e != cudaSuccess) return fail(e);
     *range = fp.range;
-    if (units == 0) return MSF_OK;
     const bool d128 = P.D == 128;
     const int smem = d128 ? FBCfg<128>::kSmem : FBCfg<64>::kSmem;
     const void* fn = d128 ? (const void*)bwd_f32_kernel<128> : (const void*)bwd_f32_kernel<64>;

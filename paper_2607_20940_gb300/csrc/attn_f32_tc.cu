@@ -452,7 +452,7 @@ __global__ void __launch_bounds__(256) merge_f32_kernel(const __grid_constant__ 
     using C = FCfg<D>;
     ptx::grid_dep_wait();
     ptx::grid_dep_launch();
-    if (!planes_hold(p.range)) return;
+    if (!planes_held(p.range)) return;
     int tile = blockIdx.x, gi = 0;
     for (; gi < p.n_groups; ++gi) {
         const int nt = p.g[gi].n_split > 1 ? p.g[gi].n_qt * p.H * p.B : 0;
@@ -628,6 +628,7 @@ bool add_context_planes(const Plan& P, const AttnArgs& a, SplitParams& sp, F32Ma
 cudaError_t launch_split_planes(const SplitParams& sp, float scale_log2, F32Range* range, cudaStream_t st) {
     const long long want = (sp.total + 255) / 256;
     range->words = sp.words;
+    range->answer = sp.words + kF32SplitBlocks;
     range->n = want < kF32SplitBlocks ? (int)want : kF32SplitBlocks;
     frexpf(scale_log2, &range->scale_exp);
     return launch_pdl(split_planes_kernel, dim3((unsigned)range->n), dim3(256), 0, st, sp);

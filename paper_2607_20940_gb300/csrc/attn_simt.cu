@@ -35,7 +35,7 @@ template <typename T, int D>
 __global__ void __launch_bounds__(128) attn_simt_kernel(const AttnArgs a) {
     ptx::grid_dep_wait();
     ptx::grid_dep_launch();
-    if (a.unless.words && planes_hold(a.unless)) return;
+    if (a.unless.words && planes_held(a.unless)) return;
     constexpr int DP = D / 4;
     constexpr int KT = 32;
     __shared__ float Ks[KT][D];

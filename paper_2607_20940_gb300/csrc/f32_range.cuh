@@ -25,12 +25,17 @@ __device__ __forceinline__ uint32_t block_codes(uint32_t m) {
     return warp_codes(lane < (int)blockDim.x / 32 ? of_warp[lane] : 0u);
 }
 
-// Whether the planes hold the operands of this call (every thread of the block).
+// Whether the planes hold the operands of this call, from the split's words (every
+// thread of the block); leaves the answer for the kernels behind this one.
 __device__ __forceinline__ bool planes_hold(const F32Range& r) {
     uint32_t m = 0;
-    for (int i = threadIdx.x; i < r.n; i += blockDim.x) m = __vmaxu4(m, __ldg(r.words + i));
-    return range_holds(block_codes(m), r.scale_exp);
+    for (int i = threadIdx.x; i < r.n; i += blockDim.x) m = __vmaxu4(m, __ldcg(r.words + i));
+    const bool holds = range_holds(block_codes(m), r.scale_exp);
+    if (blockIdx.x == 0 && threadIdx.x == 0) *r.answer = holds ? 1u : 0u;
+    return holds;
 }
+// The same from the answer.
+__device__ __forceinline__ bool planes_held(const F32Range& r) { return __ldcg(r.answer) != 0; }
 
 // The largest magnitude of four values, as bits.
 __device__ __forceinline__ uint32_t abs_bits4(const float4& x) {

@@ -68,9 +68,12 @@ MSF_RANGE_FN bool range_holds_gemm(uint32_t a, uint32_t b) {
 
 // What the plane split found in a call's operands: one word of codes per block.
 struct F32Range {
-    const unsigned int* words;  // NULL: no condition
+    unsigned int* words;  // NULL: no condition
     int n;
     int scale_exp;
+    // The kernel after the split leaves its answer here (1: the planes hold) for the
+    // ones behind it.
+    unsigned int* answer;
 };
 
 }  // namespace msf

@@ -108,7 +108,8 @@ constexpr int kTierCodeCols = 64;  // largest LoRA rank of a tier module
 // [B, 3, rows, H, D] for q and for k, v of the sink, the ring, each group's
 // pyramid part and the window; the output units of split query tiles, each
 // [128 rows][D] fp32 and the rows' running max and sum; and one word of range
-// codes per block of the kernel that writes the planes.
+// codes per block of the kernel that writes the planes, and the answer that
+// follows from them.
 enum : int { kF32Q = 0, kF32Sink = 1, kF32Ring = 2, kF32Pyr = 3, kF32Win = 4 };
 constexpr int kF32MaxSms = 160;
 constexpr int kF32MaxRounds = 6;       // rounds of units per SM when tiles are split
@@ -132,7 +133,7 @@ inline int f32_max_slots(const Plan& p) {
     return (int)(p.f32_tiles < n ? p.f32_tiles : n);
 }
 inline size_t f32_partial_bytes(const Plan& p) {
-    return p.elem == 4 ? round256((size_t)f32_max_slots(p) * 128 * (p.D + 2) * 4) + round256(kF32SplitBlocks * 4) : 0;
+    return p.elem == 4 ? round256((size_t)f32_max_slots(p) * 128 * (p.D + 2) * 4) + round256((kF32SplitBlocks + 1) * 4) : 0;
 }
 // Backward workspace (caller-provided per msf_mssa_backward call):
 // [delta fp32 [B, H, N] | dk_ctx fp32 [B, R, H, D] | dv_ctx fp32 [B, R, H, D] |
